@@ -124,10 +124,10 @@ typedef struct fmm_plan_s* fmm_plan;
  *              A and B are cubes of one size) or FMM_SPLIT_TARGET (split A
  *              then).  Alg. 1 always splits the larger cube; when that cell
  *              is a leaf the other one is split.
- *   p2p_tpl    P2P tile: target particles per lane of the one-warp pair kernel,
- *              0 (default: 2 when ncrit > 32, else 1), 1, or 2 (the two
- *              targets as the two halves of packed FP32x2 instructions).  The
- *              same pair terms either way; fmm_autotune_plan measures it.
+ *   p2p_tpl    P2P tile: 0 (default) or 2: tiles of 64 targets of a leaf, more
+ *              than 32 of them two per lane; 1: tiles of 32, one target per
+ *              lane.  The same pair terms either way; fmm_autotune_plan
+ *              measures it.
  */
 typedef struct {
   int32_t p;

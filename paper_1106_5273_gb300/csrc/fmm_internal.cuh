@@ -24,7 +24,40 @@ struct SegMac {  // traversal: image shift and regularisation MAC (Sec. 3.3)
   double blen, smax;
   float blenf, ksf, slack0, pad;
 };
-struct SegP2P {  // near field: core width, class bounds, dipole correction
+// erfcx(1/y) ~ sum c_k y^k on [1/4.6, 1] (gen_cutoff_fit.py, degree 3)
+constexpr float kE0 = -1.202012900e-02f, kE1 = 6.541014877e-01f, kE2 = -2.626216807e-01f,
+                kE3 = 4.812366022e-02f;
+
+// Constants of one core width sigma.  The polynomial H is stored negated
+// (hn = -H) so that S = 1/r^3 + q (hn / r^2) is one FMA.
+struct SigK {
+  float kq;   // -log2(e) / (2 sigma^2)
+  float kc;   // -sqrt(2/pi) / (3 sigma^3)   (T' = (S + kc q) / r^2)
+  float ku;   // 1 / sigma^2
+  float is3;  // 1 / sigma^3
+  float is5;  // -2 / (3 sigma^5)            (near series: T' = f'(u) is5)
+  float hn0;  // -sqrt(2/pi) / sigma          (constant term of -H)
+  float hn1, hn2, hn3, hn4;  // -e_0 .. -e_3,  e_k = c_k (sqrt2 sigma)^k
+};
+
+__host__ __device__ inline SigK make_sigk(float sigma) {
+  SigK k;
+  const double s = (double)sigma, ky = 1.4142135623730951 * s;
+  k.kq = (float)(-1.4426950408889634 / (2.0 * s * s));
+  k.kc = (float)(-0.79788456080286535588 / (3.0 * s * s * s));
+  k.ku = (float)(1.0 / (s * s));
+  k.is3 = (float)(1.0 / (s * s * s));
+  k.is5 = (float)(-2.0 / (3.0 * s * s * s * s * s));
+  k.hn0 = (float)(-0.79788456080286535588 / s);
+  k.hn1 = (float)(-(double)kE0);
+  k.hn2 = (float)(-(double)kE1 * ky);
+  k.hn3 = (float)(-(double)kE2 * ky * ky);
+  k.hn4 = (float)(-(double)kE3 * ky * ky * ky);
+  return k;
+}
+
+struct SegP2P {  // near field: core width and its constants, class bounds, dipole correction
+  SigK k;
   float sigma, smax, blen, margin;
   float dip[3], pad;
 };
@@ -92,7 +125,10 @@ struct fmm_plan_s {
   fmm::DBuf tcount, tmask, tscan0, tscan1, tscan2;    // per-item scratch
   fmm::DBuf p2p_raw, m2l_raw;                         // int4 (a,b,o,0)
   fmm::DBuf lk0, lk1, lv0, lv1;                       // list sort ping-pong
-  fmm::DBuf p2p_sorted, p2p_off;                      // int2 (b,o) by leaf, CSR offsets per leaf
+  fmm::DBuf p2p_sorted, p2p_off;                      // int2 (first source, image) by leaf, CSR offsets per leaf
+  fmm::DBuf p2p_pre;                                  // u32 scanned source counts of the list entries
+  fmm::DBuf p2p_items, p2p_islot, p2p_plan;           // pair kernel work items, their partial slots, per-leaf split
+  fmm::DBuf p2p_partial, p2p_sigk;                    // partial sums of split lists; per-particle core constants
   fmm::DBuf m2l_key, m2l_slot, ukeys;                 // per pair key, slot; unique keys
   fmm::DBuf T32, Tbf;                                 // M2L operator cache [slot]: FP32, BF16 hi/lo
   std::unordered_map<uint64_t, int> tcache;           // translation key -> cache slot
@@ -116,6 +152,7 @@ struct fmm_plan_s {
   int nlevels = 0;
   double cf_margin = 0.0;  // rounding margin of the FP32 cell copies (2e-6 x largest coordinate)
   int64_t n_p2p = 0, n_m2l = 0, n_keys = 0, n_steps = 0, p2p_pairs = 0;
+  int64_t n_p2p_items = 0, n_p2p_slots = 0;  // pair kernel work items and partial slots
   int64_t last_n = 0;
   int last_tc = 0;
   int m2l_stage_chunks = 0;  // K chunks per stage of the last tensor-core M2L
@@ -174,6 +211,9 @@ int eval_strengths(fmm_plan p, const float* gam, float* vel, float* dg, cudaStre
 // p2p.cu
 int p2p_near(fmm_plan p, int64_t n, float sig_u, int per_particle_sigma, double smax, float* vel, float* dg,
              cudaStream_t s);
+// work items of the pair kernel; counts (device) receives (items, partial slots)
+int p2p_tile(fmm_plan p);
+int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s);
 int p2p_direct_all(int64_t n, const float* pos, const float* gam, const float* sig, float sig_u, float* vel,
                    float* dg, cudaStream_t s);
 }  // namespace fmm

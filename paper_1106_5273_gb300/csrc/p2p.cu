@@ -20,9 +20,9 @@
 // self pair is skipped explicitly (its exact value is zero).  Periodic image
 // pairs form the exact FP32 difference first and then add the image shift.
 //
-// One warp per target leaf, two target particles per lane (one when ncrit <=
-// 32); the source leaves of the leaf's list are staged through shared memory
-// in double-buffered chunks.  Each staged source is classified by a lower
+// A CTA takes a tile of at most 64 targets of a leaf and a range of the leaf's
+// sources, which its four warps share; the sources are staged through shared
+// memory in chunks of 64 per warp.  Each staged source is classified by a lower
 // bound on its distance to every target of the tile (its distance to the
 // targets' bounding box, rounding margin off): the singular kernel where
 // g = 1 to FP32 precision (rho >= 6.5), the cutoff without the series test
@@ -37,9 +37,6 @@ namespace {
 constexpr int kMaxBlock = 128;
 constexpr float kInv4Pi = 0.0795774715459476679f;
 constexpr float kM3 = -3.f;  // T = -3 T': scales the stretching sums built from T'
-// erfcx(1/y) ~ sum c_k y^k on [1/4.6, 1] (gen_cutoff_fit.py, degree 3)
-constexpr float kE0 = -1.202012900e-02f, kE1 = 6.541014877e-01f, kE2 = -2.626216807e-01f,
-                kE3 = 4.812366022e-02f;
 // Source-leaf classes by a lower bound d_min on the pair distance:
 //   kFar : d_min >= 6.5 sigma_max: 1 - g < 4e-9 and exp(-rho^2/2) < 1e-9, so
 //          S = 1/r^3 and T = -3/r^5 exactly in FP32 (singular kernel);
@@ -68,34 +65,6 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// Constants of one core width sigma.  The polynomial H is stored negated
-// (hn = -H) so that S = 1/r^3 + q (hn / r^2) is one FMA.
-struct SigK {
-  float kq;   // -log2(e) / (2 sigma^2)
-  float kc;   // -sqrt(2/pi) / (3 sigma^3)   (T' = (S + kc q) / r^2)
-  float ku;   // 1 / sigma^2
-  float is3;  // 1 / sigma^3
-  float is5;  // -2 / (3 sigma^5)            (near series: T' = f'(u) is5)
-  float hn0;  // -sqrt(2/pi) / sigma          (constant term of -H)
-  float hn1, hn2, hn3, hn4;  // -e_0 .. -e_3,  e_k = c_k (sqrt2 sigma)^k
-};
-
-__host__ __device__ inline SigK make_sigk(float sigma) {
-  SigK k;
-  const double s = (double)sigma, ky = 1.4142135623730951 * s;
-  k.kq = (float)(-1.4426950408889634 / (2.0 * s * s));
-  k.kc = (float)(-0.79788456080286535588 / (3.0 * s * s * s));
-  k.ku = (float)(1.0 / (s * s));
-  k.is3 = (float)(1.0 / (s * s * s));
-  k.is5 = (float)(-2.0 / (3.0 * s * s * s * s * s));
-  k.hn0 = (float)(-0.79788456080286535588 / s);
-  k.hn1 = (float)(-(double)kE0);
-  k.hn2 = (float)(-(double)kE1 * ky);
-  k.hn3 = (float)(-(double)kE2 * ky * ky);
-  k.hn4 = (float)(-(double)kE3 * ky * ky * ky);
-  return k;
 }
 
 // The constants of make_sigk for the mixed core width of a pair,
@@ -178,95 +147,6 @@ __device__ __forceinline__ void pair_acc(float dx, float dy, float dz, const flo
   a.sx = fmaf(td, cx, a.sx);
   a.sy = fmaf(td, cy, a.sy);
   a.sz = fmaf(td, cz, a.sz);
-}
-
-// Leaf-relative form used by k_p2p: with X = x - c (c the target leaf centre;
-// image shifts folded into the source's X) and k_j = gamma_j x X_j staged per
-// source,  sum_j S (gamma_j x d) = A x X_i - B  and
-// sum_j T (gamma_i . d)(gamma_j x d) = C x X_i - D, where
-// A = sum S gamma_j, B = sum S k_j, C = sum td gamma_j, D = sum td k_j, td = T' (gamma_i . d)
-// (T' = -T/3, so the stretching is s = A x gamma_i - 3 (C x X_i - D)).
-// Transpose scheme: with m_i = X_i x gamma_i, w = T' gamma_i . (gamma_j x d) = T' (gamma_j . m_i -
-// gamma_i . k_j); C.x = sum w, D = sum w X_j, and s = gamma_i x A - 3 ((sum w) X_i - D).
-struct AccR {
-  float ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz;
-};
-
-// ST: 0 velocity only, 1 classical stretching, 2 transpose stretching.
-template <int MODE, int ST>
-__device__ __forceinline__ void pair_acc_rel(float dx, float dy, float dz, const float4& xj, const float4& gj,
-                                             const float4& kj, float gix, float giy, float giz, float mix,
-                                             float miy, float miz, const SigK& K, AccR& a) {
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  float S, T;
-  pair_ST<MODE, ST>(r2, K, S, T);
-  a.ax = fmaf(S, gj.x, a.ax);
-  a.ay = fmaf(S, gj.y, a.ay);
-  a.az = fmaf(S, gj.z, a.az);
-  a.bx = fmaf(S, kj.x, a.bx);
-  a.by = fmaf(S, kj.y, a.by);
-  a.bz = fmaf(S, kj.z, a.bz);
-  if (ST == 0) return;
-  if (ST == 2) {
-    const float e = fmaf(-giz, kj.z, fmaf(-giy, kj.y, fmaf(-gix, kj.x, fmaf(gj.x, mix, fmaf(gj.y, miy, gj.z * miz)))));
-    const float w = T * e;
-    a.cx += w;
-    a.dx = fmaf(w, xj.x, a.dx);
-    a.dy = fmaf(w, xj.y, a.dy);
-    a.dz = fmaf(w, xj.z, a.dz);
-    return;
-  }
-  const float td = T * fmaf(gix, dx, fmaf(giy, dy, giz * dz));
-  a.cx = fmaf(td, gj.x, a.cx);
-  a.cy = fmaf(td, gj.y, a.cy);
-  a.cz = fmaf(td, gj.z, a.cz);
-  a.dx = fmaf(td, kj.x, a.dx);
-  a.dy = fmaf(td, kj.y, a.dy);
-  a.dz = fmaf(td, kj.z, a.dz);
-}
-
-template <int TPT>
-struct TgtR {
-  float x[TPT], y[TPT], z[TPT], gx[TPT], gy[TPT], gz[TPT];  // X_i (leaf-relative) and gamma_i
-  float mx[TPT], my[TPT], mz[TPT];                          // m_i = X_i x gamma_i (transpose scheme)
-  float sg[TPT];                                            // sigma_i (mixed core width)
-  int self[TPT];
-  AccR a[TPT];
-};
-
-// MIX (PS only): the pair's core width is sigma_ij (sigk_mixed), not sigma_j.
-template <bool PS, int MODE, bool SELF, int TPT, int ST, bool MIX>
-__device__ __forceinline__ void run_chunk_rel(const float4* sA, const float4* sB, const float4* sC, const SigK* sK,
-                                              int jb, int je, TgtR<TPT>& t, const SigK& K0) {
-#pragma unroll 4
-  for (int j = jb; j < je; ++j) {
-    const float4 xj = sA[j];
-    const float4 gj = sB[j];
-    const float4 kj = sC[j];
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      if (SELF && j == t.self[q]) continue;
-      pair_acc_rel<MODE, ST>(t.x[q] - xj.x, t.y[q] - xj.y, t.z[q] - xj.z, xj, gj, kj, t.gx[q], t.gy[q], t.gz[q],
-                             t.mx[q], t.my[q], t.mz[q],
-                             MIX ? sigk_mixed(t.sg[q], xj.w) : (PS ? sK[j] : K0), t.a[q]);
-    }
-  }
-}
-
-// The groups of a staged chunk: sources [0, nf) far, [nf, nf + nm) mid, the
-// rest near; the self entry (not grouped) runs the near form with the self
-// pair skipped.
-template <bool PS, int TPT, int ST, bool MIX>
-__device__ __forceinline__ void dispatch_rel(bool self, int nf, int nm, const float4* sA, const float4* sB,
-                                             const float4* sC, const SigK* sK, int cnt, TgtR<TPT>& t,
-                                             const SigK& K0) {
-  if (self) {
-    run_chunk_rel<PS, kNear, true, TPT, ST, MIX>(sA, sB, sC, sK, 0, cnt, t, K0);
-    return;
-  }
-  if (nf > 0) run_chunk_rel<PS, kFar, false, TPT, ST, MIX>(sA, sB, sC, sK, 0, nf, t, K0);
-  if (nm > 0) run_chunk_rel<PS, kMid, false, TPT, ST, MIX>(sA, sB, sC, sK, nf, nf + nm, t, K0);
-  if (nf + nm < cnt) run_chunk_rel<PS, kNear, false, TPT, ST, MIX>(sA, sB, sC, sK, nf + nm, cnt, t, K0);
 }
 
 // Axis-aligned bounding box of the targets of one tile, relative to the leaf
@@ -354,16 +234,6 @@ __device__ __forceinline__ void group_slots(const int* cls, int lane, int* slot,
   }
 }
 
-// Pair counts by class of one warp, added to the evaluation's counters.
-__device__ __forceinline__ void add_class_counts(unsigned long long* cnt, unsigned long long c_near,
-                                                 unsigned long long c_mid, unsigned long long c_far) {
-  if (threadIdx.x == 0) {
-    if (c_near) atomicAdd(&cnt[0], c_near);
-    if (c_mid) atomicAdd(&cnt[1], c_mid);
-    if (c_far) atomicAdd(&cnt[2], c_far);
-  }
-}
-
 // Targets held by one thread.
 template <int TPT>
 struct Tgt {
@@ -393,218 +263,43 @@ __device__ __forceinline__ void run_chunk(const float4* sA, const float4* sB, co
   }
 }
 
-
-
-// One warp per target leaf, TPT targets per lane; source chunks of 32*TPT
-// particles double-buffered (the next chunk is loaded into registers while the
-// current one is computed from shared memory).  Coordinates are relative to
-// the target leaf centre.
-// SEG: a batch of problems; the leaf's problem supplies sigma, the class
-// bounds, the image shift and the dipole correction instead of the arguments.
-// ST: 0 velocity only (dg is not written), 1 classical, 2 transpose stretching.
-template <bool PS, int TPT, bool SEG, int ST, bool MIX>
-__global__ void __launch_bounds__(32) k_p2p(const int* __restrict__ leaves, const int2* __restrict__ off,
-                                            const int2* __restrict__ list, const int* __restrict__ begin,
-                                            const int* __restrict__ end, const float4* __restrict__ cf,
-                                            const float4* __restrict__ A, const float4* __restrict__ B,
-                                            const float* __restrict__ far_u, const float* __restrict__ far_s,
-                                            const uint32_t* __restrict__ sidx, float blen, float smax, float margin0,
-                                            SigK K0, const double* __restrict__ dip, const int* __restrict__ cseg,
-                                            const SegP2P* __restrict__ sp, float* __restrict__ vel,
-                                            float* __restrict__ dg, unsigned long long* __restrict__ ccount) {
-  constexpr int CH = 32 * TPT;
-  __shared__ float4 sA[2][CH], sB[2][CH], sC[2][CH];
-  __shared__ SigK sK[2][PS ? CH : 1];
-  const int lane = threadIdx.x;
-  const int leaf = leaves[blockIdx.x];
-  const int tb = begin[leaf], te = end[leaf];
-  const int2 rg = off[blockIdx.x];
-  const float4 lc = cf[leaf];
-  float dux = dip ? (float)dip[0] : 0.f, duy = dip ? (float)dip[1] : 0.f, duz = dip ? (float)dip[2] : 0.f;
-  if (SEG) {
-    const SegP2P q = sp[cseg[leaf]];
-    if (!PS) K0 = make_sigk(q.sigma);
-    blen = q.blen;
-    smax = q.smax;
-    margin0 = q.margin;
-    dux = q.dip[0];
-    duy = q.dip[1];
-    duz = q.dip[2];
-  }
-  float4 ra[TPT], rb[TPT];
-  unsigned long long c_near = 0, c_mid = 0, c_far = 0;
-  TileBox box;
-  // source j of entry e, staged as X_j = (x_j - c) - shift, gamma_j, k_j = gamma_j x X_j,
-  // grouped by class (the self entry in source order)
-  auto stage = [&](int bb, int cnt, int img, bool self_entry, int& nf, int& nm) {
-    const float shx = -(float)(img / 9 - 1) * blen, shy = -(float)((img / 3) % 3 - 1) * blen,
-                shz = -(float)(img % 3 - 1) * blen;
-    float X[TPT], Y[TPT], Z[TPT];
-    int cls[TPT], slot[TPT];
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int j = lane + 32 * q;
-      X[q] = (ra[q].x - lc.x) - shx;
-      Y[q] = (ra[q].y - lc.y) - shy;
-      Z[q] = (ra[q].z - lc.z) - shz;
-      cls[q] = j >= cnt ? -1 : self_entry ? kNear : source_class(X[q], Y[q], Z[q], box, lc.w, smax, margin0);
-    }
-    group_slots<TPT>(cls, lane, slot, nf, nm);
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int k = slot[q];
-      if (k >= 0) {
-        const float4 g = rb[q];
-        sA[bb][k] = make_float4(X[q], Y[q], Z[q], ra[q].w);
-        sB[bb][k] = g;
-        sC[bb][k] = make_float4(g.y * Z[q] - g.z * Y[q], g.z * X[q] - g.x * Z[q], g.x * Y[q] - g.y * X[q], 0.f);
-        if (PS) sK[bb][k] = make_sigk(ra[q].w);
-      }
-    }
-  };
-  for (int t0 = tb; t0 < te; t0 += CH) {
-    TgtR<TPT> t;
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int i = t0 + lane + 32 * q;
-      float4 xi = i < te ? A[i] : lc;
-      float4 gi = i < te ? B[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      t.x[q] = xi.x - lc.x;
-      t.y[q] = xi.y - lc.y;
-      t.z[q] = xi.z - lc.z;
-      t.gx[q] = gi.x;
-      t.gy[q] = gi.y;
-      t.gz[q] = gi.z;
-      t.sg[q] = xi.w;
-      t.mx[q] = t.y[q] * gi.z - t.z[q] * gi.y;
-      t.my[q] = t.z[q] * gi.x - t.x[q] * gi.z;
-      t.mz[q] = t.x[q] * gi.y - t.y[q] * gi.x;
-      t.a[q] = AccR{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    }
-    {
-      bool valid[TPT];
-#pragma unroll
-      for (int q = 0; q < TPT; ++q) valid[q] = t0 + lane + 32 * q < te;
-      box = tile_box<TPT>(t.x, t.y, t.z, valid);
-    }
-    const unsigned long long nt = (unsigned long long)min(CH, te - t0);
-    int cur_e = rg.x, cur_c0 = rg.x < rg.y ? begin[list[rg.x].x] : 0, cur_cnt = 0, cur_nf = 0, cur_nm = 0;
-    int buf = 0;
-    if (cur_e < rg.y) {
-      cur_cnt = min(CH, end[list[cur_e].x] - cur_c0);
-#pragma unroll
-      for (int q = 0; q < TPT; ++q) {
-        const int j = lane + 32 * q;
-        if (j < cur_cnt) {
-          ra[q] = A[cur_c0 + j];
-          rb[q] = B[cur_c0 + j];
-        }
-      }
-      const int2 e0 = list[cur_e];
-      stage(0, cur_cnt, e0.y, e0.x == leaf && e0.y == kImageZero, cur_nf, cur_nm);
-    }
-    __syncwarp();
-    while (cur_e < rg.y) {
-      int ne = cur_e, nc0 = cur_c0 + CH;
-      if (nc0 >= end[list[ne].x]) {
-        ++ne;
-        nc0 = ne < rg.y ? begin[list[ne].x] : 0;
-      }
-      int ncnt = 0;
-      if (ne < rg.y) {
-        ncnt = min(CH, end[list[ne].x] - nc0);
-#pragma unroll
-        for (int q = 0; q < TPT; ++q) {
-          const int j = lane + 32 * q;
-          if (j < ncnt) {
-            ra[q] = A[nc0 + j];
-            rb[q] = B[nc0 + j];
-          }
-        }
-      }
-      const int2 ent = list[cur_e];
-      const bool self = (ent.x == leaf) && ent.y == kImageZero;
-#pragma unroll
-      for (int q = 0; q < TPT; ++q) t.self[q] = self ? (t0 + lane + 32 * q) - cur_c0 : -1;
-      dispatch_rel<PS, TPT, ST, PS && MIX>(self, cur_nf, cur_nm, sA[buf], sB[buf], sC[buf], sK[buf], cur_cnt, t,
-                                           K0);
-      c_far += nt * (unsigned long long)cur_nf;
-      c_mid += nt * (unsigned long long)cur_nm;
-      c_near += nt * (unsigned long long)(cur_cnt - cur_nf - cur_nm);
-      __syncwarp();
-      buf ^= 1;
-      int nnf = 0, nnm = 0;
-      if (ne < rg.y) {
-        const int2 en = list[ne];
-        stage(buf, ncnt, en.y, en.x == leaf && en.y == kImageZero, nnf, nnm);
-      }
-      __syncwarp();
-      cur_e = ne;
-      cur_c0 = nc0;
-      cur_cnt = ncnt;
-      cur_nf = nnf;
-      cur_nm = nnm;
-    }
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int i = t0 + lane + 32 * q;
-      if (i >= te) continue;
-      const AccR& a = t.a[q];
-      const float X = t.x[q], Y = t.y[q], Z = t.z[q];
-      const uint32_t o = sidx[i];
-      if (vel) {  // u = A x X_i - B
-        vel[3 * o] = far_u[3 * i] + kInv4Pi * ((a.ay * Z - a.az * Y) - a.bx) + dux;
-        vel[3 * o + 1] = far_u[3 * i + 1] + kInv4Pi * ((a.az * X - a.ax * Z) - a.by) + duy;
-        vel[3 * o + 2] = far_u[3 * i + 2] + kInv4Pi * ((a.ax * Y - a.ay * X) - a.bz) + duz;
-      }
-      if (ST == 1 && dg) {  // s = A x gamma_i + C x X_i - D
-        const float gx = t.gx[q], gy = t.gy[q], gz = t.gz[q];
-        dg[3 * o] = far_s[3 * i] + kInv4Pi * ((a.ay * gz - a.az * gy) + kM3 * ((a.cy * Z - a.cz * Y) - a.dx));
-        dg[3 * o + 1] = far_s[3 * i + 1] + kInv4Pi * ((a.az * gx - a.ax * gz) + kM3 * ((a.cz * X - a.cx * Z) - a.dy));
-        dg[3 * o + 2] = far_s[3 * i + 2] + kInv4Pi * ((a.ax * gy - a.ay * gx) + kM3 * ((a.cx * Y - a.cy * X) - a.dz));
-      }
-      if (ST == 2 && dg) {  // s = gamma_i x A + W X_i - D (W = C.x)
-        const float gx = t.gx[q], gy = t.gy[q], gz = t.gz[q];
-        dg[3 * o] = far_s[3 * i] + kInv4Pi * ((gy * a.az - gz * a.ay) + kM3 * (a.cx * X - a.dx));
-        dg[3 * o + 1] = far_s[3 * i + 1] + kInv4Pi * ((gz * a.ax - gx * a.az) + kM3 * (a.cx * Y - a.dy));
-        dg[3 * o + 2] = far_s[3 * i + 2] + kInv4Pi * ((gx * a.ay - gy * a.ax) + kM3 * (a.cx * Z - a.dz));
-      }
-    }
-  }
-  add_class_counts(ccount, c_near, c_mid, c_far);
-}
-
-// ---- Packed form: the two targets of a lane as float2 lanes of the FP32x2
-// instructions (fma/mul/add .f32x2).  The FMA pipe does the same work per
-// clock either way; the packed form halves the issue slots per pair, which
-// is what bounds the scalar kernel.  Every element sees the same operations in
-// the same order as pair_acc_rel (subtractions as additions of staged
-// negated values), so each element is rounded exactly as in the scalar form.
+// ---- The pair kernel.  Two pairs at a time run as the two lanes of the
+// FP32x2 instructions (fma/mul/add .f32x2): the FMA pipe does the same work
+// per clock as with scalars, in half the issue slots.
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 
-// SigK with every constant duplicated into both lanes.
+// The constants of two pairs.
 struct SigK2 {
   float2 kq, kc, ku, is3, is5, hn0, hn1, hn2, hn3, hn4;
 };
 
-__device__ __forceinline__ SigK2 make_sigk2(const SigK& K) {
+__device__ __forceinline__ SigK2 make_sigk2(const SigK& a, const SigK& b) {
   SigK2 k;
-  k.kq = dup2(K.kq);
-  k.kc = dup2(K.kc);
-  k.ku = dup2(K.ku);
-  k.is3 = dup2(K.is3);
-  k.is5 = dup2(K.is5);
-  k.hn0 = dup2(K.hn0);
-  k.hn1 = dup2(K.hn1);
-  k.hn2 = dup2(K.hn2);
-  k.hn3 = dup2(K.hn3);
-  k.hn4 = dup2(K.hn4);
+  k.kq = make_float2(a.kq, b.kq);
+  k.kc = make_float2(a.kc, b.kc);
+  k.ku = make_float2(a.ku, b.ku);
+  k.is3 = make_float2(a.is3, b.is3);
+  k.is5 = make_float2(a.is5, b.is5);
+  k.hn0 = make_float2(a.hn0, b.hn0);
+  k.hn1 = make_float2(a.hn1, b.hn1);
+  k.hn2 = make_float2(a.hn2, b.hn2);
+  k.hn3 = make_float2(a.hn3, b.hn3);
+  k.hn4 = make_float2(a.hn4, b.hn4);
   return k;
 }
 
+// Sums of two chains in the leaf-relative form: with X = x - c (c the target
+// leaf's centre, image shifts folded into the source's X) and k_j =
+// gamma_j x X_j staged per source,  sum_j S (gamma_j x d) = A x X_i - B  and
+// sum_j T (gamma_i . d)(gamma_j x d) = C x X_i - D, where A = sum S gamma_j,
+// B = sum S k_j, C = sum td gamma_j, D = sum td k_j, td = T' (gamma_i . d)
+// (T' = -T/3, so the stretching is s = A x gamma_i - 3 (C x X_i - D)).
+// Transpose scheme: with m_i = X_i x gamma_i, w = T' gamma_i . (gamma_j x d) =
+// T' (gamma_j . m_i - gamma_i . k_j); cx holds W = sum w and D = sum w (-X_j)
+// (the staged coordinates are negated); s = gamma_i x A - 3 (W X_i + D).
 struct AccR2 {
   float2 ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz;
 };
@@ -648,284 +343,663 @@ __device__ __forceinline__ void pair_ST2(float2 r2, const SigK2& K, float2& S, f
   }
 }
 
-// Transpose scheme (ST = 2): cx accumulates W = sum w and dx, dy, dz the sum
-// of w (-X_j) (the staged coordinates are negated), mx.. = m_i, ngx.. = -gamma_i.
-struct TgtT2 {
-  float2 mx, my, mz, ngx, ngy, ngz;
+// The targets of a lane's two chains (narrow tiles: the same target twice).
+struct Tgt2 {
+  float2 x, y, z, gx, gy, gz;    // X_i and gamma_i
+  float2 mx, my, mz, ngx, ngy, ngz;  // m_i = X_i x gamma_i and -gamma_i (transpose scheme)
+  float2 sg;                     // sigma_i (mixed core width)
+  int id0, id1;                  // their sorted positions
 };
 
-// One staged source (v0..v4) against the two targets of one FP32x2 chain.
-// self_lo / self_hi: the staged index of each target itself (self pair
-// skipped), or -1.
-template <int MODE, bool SELF, int ST>
-__device__ __forceinline__ void pair_x2(const float4& v0, const float4& v1, const float4& v2, const float4& v3,
-                                        const float2& v4, int j, float2 tx, float2 ty, float2 tz, float2 gix,
-                                        float2 giy, float2 giz, const TgtT2& tt, int self_lo, int self_hi,
-                                        const SigK2& K, AccR2& a) {
-  const float2 dx = add2(tx, make_float2(v0.x, v0.y));
-  const float2 dy = add2(ty, make_float2(v0.z, v0.w));
-  const float2 dz = add2(tz, make_float2(v1.x, v1.y));
-  const float2 gjx = make_float2(v1.z, v1.w), gjy = make_float2(v2.x, v2.y), gjz = make_float2(v2.z, v2.w);
-  const float2 kjx = make_float2(v3.x, v3.y), kjy = make_float2(v3.z, v3.w), kjz = v4;
-  const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-  float2 S, T;
-  pair_ST2<MODE, ST>(r2, K, S, T);
-  float2 td = dup2(0.f);
-  if (ST == 1) td = mul2(T, fma2(gix, dx, fma2(giy, dy, mul2(giz, dz))));
-  if (ST == 2)
-    td = mul2(T, fma2(tt.ngz, kjz, fma2(tt.ngy, kjy, fma2(tt.ngx, kjx, fma2(gjx, tt.mx, fma2(gjy, tt.my,
-                                                                                          mul2(gjz, tt.mz)))))));
-  if (SELF) {
-    if (j == self_lo) {
-      S.x = 0.f;
-      td.x = 0.f;
-    }
-    if (j == self_hi) {
-      S.y = 0.f;
-      td.y = 0.f;
-    }
-  }
-  a.ax = fma2(S, gjx, a.ax);
-  a.ay = fma2(S, gjy, a.ay);
-  a.az = fma2(S, gjz, a.az);
-  a.bx = fma2(S, kjx, a.bx);
-  a.by = fma2(S, kjy, a.by);
-  a.bz = fma2(S, kjz, a.bz);
-  if (ST == 0) return;
-  if (ST == 2) {  // td holds w
-    a.cx = add2(a.cx, td);
-    a.dx = fma2(td, make_float2(v0.x, v0.y), a.dx);
-    a.dy = fma2(td, make_float2(v0.z, v0.w), a.dy);
-    a.dz = fma2(td, make_float2(v1.x, v1.y), a.dz);
-    return;
-  }
-  a.cx = fma2(td, gjx, a.cx);
-  a.cy = fma2(td, gjy, a.cy);
-  a.cz = fma2(td, gjz, a.cz);
-  a.dx = fma2(td, kjx, a.dx);
-  a.dy = fma2(td, kjy, a.dy);
-  a.dz = fma2(td, kjz, a.dz);
+constexpr int kCh = 64;        // sources staged at a time
+constexpr int kChPad = 72;     // slots of a staged narrow chunk (padded to a whole unit of 2, 4 or 8)
+
+// The staged sources, every value once.  PAIR (narrow tiles): rows of kChPad
+// floats (-X, -Y, -Z, gamma, k), read as float2 = two sources.  Wide tiles:
+// (-X, -Y, -Z, gamma_x), (gamma_y, gamma_z, k_x, k_y), k_z per source, each
+// value copied to both halves of its register pair after the load: the loop
+// is bound by the FMA pipe and the shared-memory reads together, and storing
+// every value twice (two and a half times the wavefronts) measured 73 instead
+// of 66 cycles per 64 far pairs and warp scheduler, 92 instead of 87 mid.
+// id = the source's sorted position (-1 for an image: never the target
+// itself).  k (PS = 1): the constants of SigK, PAIR as rows kq kc hn0 hn2 hn3
+// hn4 ku is3 is5, wide as two float4 rows and is5; (PS = 2): sigma_j.  The
+// next chunk's loads go through shared memory (cp.async) and the targets' box
+// is kept there, which leaves the registers to the pair loops.
+template <int PS>
+struct Stage {
+  float4 v[9 * kChPad / 4];
+  float4 k[PS == 1 ? 9 * kChPad / 4 : (PS == 2 ? kChPad / 4 : 1)];
+  int id[kChPad];
+  // the next chunk on its way (each lane reads back its own two sources)
+  float4 raw[PS == 1 ? 5 : 2][kCh];
+  int rid[kCh], rimg[kCh];
+  TileBox box;
+  float4 centre;
+};
+
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
 
-template <int MODE, bool SELF, int ST>
-__device__ __forceinline__ void run_chunk_x2(const float4* s0, const float4* s1, const float4* s2, const float4* s3,
-                                             const float2* s4, int jb, int je, float2 tx, float2 ty, float2 tz,
-                                             float2 gix, float2 giy, float2 giz, const TgtT2& tt, int self_lo,
-                                             int self_hi, const SigK2& K, AccR2& a) {
-#pragma unroll 4
-  for (int j = jb; j < je; ++j)
-    pair_x2<MODE, SELF, ST>(s0[j], s1[j], s2[j], s3[j], s4[j], j, tx, ty, tz, gix, giy, giz, tt, self_lo, self_hi,
-                            K, a);
+// Sources [jb, je) of a staged chunk in form MODE (PAIR: units of two sources,
+// in steps of `step` units).  The near form skips the self pair.
+// PS: 0 one core width, 1 sigma_j of the source, 2 the mixed width sigma_ij.
+// ST: 0 velocity only, 1 classical stretching, 2 transpose stretching.
+template <int MODE, bool PAIR, int PS, int ST>
+__device__ __forceinline__ void run_group(const Stage<PS>& sm, int jb, int je, int step, const Tgt2& t,
+                                          const SigK2& K0, AccR2& a) {
+#pragma unroll(MODE == kNear ? 2 : 4)
+  for (int j = jb; j < je; j += PAIR ? step : 1) {
+    float2 nx, ny, nz, gjx, gjy, gjz, kjx, kjy, kjz;
+    if (PAIR) {
+      const float2* r = reinterpret_cast<const float2*>(sm.v) + j;
+      constexpr int S = kChPad / 2;
+      nx = r[0];
+      ny = r[S];
+      nz = r[2 * S];
+      gjx = r[3 * S];
+      gjy = r[4 * S];
+      gjz = r[5 * S];
+      kjx = r[6 * S];
+      kjy = r[7 * S];
+      kjz = r[8 * S];
+    } else {
+      const float4 v0 = sm.v[j], v1 = sm.v[kCh + j];
+      nx = dup2(v0.x);
+      ny = dup2(v0.y);
+      nz = dup2(v0.z);
+      gjx = dup2(v0.w);
+      gjy = dup2(v1.x);
+      gjz = dup2(v1.y);
+      kjx = dup2(v1.z);
+      kjy = dup2(v1.w);
+      kjz = dup2(reinterpret_cast<const float*>(sm.v + 2 * kCh)[j]);
+    }
+    SigK2 K = K0;
+    if constexpr (PS == 1 && MODE != kFar) {
+      if constexpr (PAIR) {
+        const float2* r = reinterpret_cast<const float2*>(sm.k) + j;
+        constexpr int S = kChPad / 2;
+        K.kq = r[0];
+        K.kc = r[S];
+        K.hn0 = r[2 * S];
+        K.hn2 = r[3 * S];
+        K.hn3 = r[4 * S];
+        K.hn4 = r[5 * S];
+        if (MODE == kNear) {
+          K.ku = r[6 * S];
+          K.is3 = r[7 * S];
+          K.is5 = r[8 * S];
+        }
+      } else {
+        const float4 a0 = sm.k[j], a1 = sm.k[kChPad + j];
+        K.kq = dup2(a0.x);
+        K.kc = dup2(a0.y);
+        K.hn0 = dup2(a0.z);
+        K.hn2 = dup2(a0.w);
+        K.hn3 = dup2(a1.x);
+        K.hn4 = dup2(a1.y);
+        if (MODE == kNear) {
+          K.ku = dup2(a1.z);
+          K.is3 = dup2(a1.w);
+          K.is5 = dup2(reinterpret_cast<const float*>(sm.k + 2 * kChPad)[j]);
+        }
+      }
+    }
+    if constexpr (PS == 2 && MODE != kFar) {
+      float s0, s1;
+      if (PAIR) {
+        const float2 s = reinterpret_cast<const float2*>(sm.k)[j];
+        s0 = s.x;
+        s1 = s.y;
+      } else {
+        s0 = s1 = reinterpret_cast<const float*>(sm.k)[j];
+      }
+      K = make_sigk2(sigk_mixed(t.sg.x, s0), sigk_mixed(t.sg.y, s1));
+    }
+    const float2 dx = add2(t.x, nx), dy = add2(t.y, ny), dz = add2(t.z, nz);
+    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    float2 S, T;
+    pair_ST2<MODE, ST>(r2, K, S, T);
+    float2 td = dup2(0.f);
+    if (ST == 1) td = mul2(T, fma2(t.gx, dx, fma2(t.gy, dy, mul2(t.gz, dz))));
+    if (ST == 2)
+      td = mul2(T, fma2(t.ngz, kjz,
+                        fma2(t.ngy, kjy, fma2(t.ngx, kjx, fma2(gjx, t.mx, fma2(gjy, t.my, mul2(gjz, t.mz)))))));
+    if (MODE == kNear) {
+      const int i0 = PAIR ? sm.id[2 * j] : sm.id[j], i1 = PAIR ? sm.id[2 * j + 1] : i0;
+      if (i0 == t.id0) {
+        S.x = 0.f;
+        td.x = 0.f;
+      }
+      if (i1 == t.id1) {
+        S.y = 0.f;
+        td.y = 0.f;
+      }
+    }
+    a.ax = fma2(S, gjx, a.ax);
+    a.ay = fma2(S, gjy, a.ay);
+    a.az = fma2(S, gjz, a.az);
+    a.bx = fma2(S, kjx, a.bx);
+    a.by = fma2(S, kjy, a.by);
+    a.bz = fma2(S, kjz, a.bz);
+    if (ST == 1) {
+      a.cx = fma2(td, gjx, a.cx);
+      a.cy = fma2(td, gjy, a.cy);
+      a.cz = fma2(td, gjz, a.cz);
+      a.dx = fma2(td, kjx, a.dx);
+      a.dy = fma2(td, kjy, a.dy);
+      a.dz = fma2(td, kjz, a.dz);
+    }
+    if (ST == 2) {
+      a.cx = add2(a.cx, td);
+      a.dx = fma2(td, nx, a.dx);
+      a.dy = fma2(td, ny, a.dy);
+      a.dz = fma2(td, nz, a.dz);
+    }
+  }
 }
 
-// k_p2p for a uniform core width and two targets per lane, in the packed
-// form.  Same lists, classes, staging order and output as k_p2p<false, 2, SEG>;
-// the staged source holds its negated coordinates and every value twice.
-template <bool SEG, int ST>
-__global__ void __launch_bounds__(32) k_p2p_x2(const int* __restrict__ leaves, const int2* __restrict__ off,
-                                               const int2* __restrict__ list, const int* __restrict__ begin,
-                                               const int* __restrict__ end, const float4* __restrict__ cf,
-                                               const float4* __restrict__ A, const float4* __restrict__ B,
-                                               const float* __restrict__ far_u, const float* __restrict__ far_s,
-                                               const uint32_t* __restrict__ sidx, float blen, float smax,
-                                               float margin0, SigK K0, const double* __restrict__ dip,
-                                               const int* __restrict__ cseg, const SegP2P* __restrict__ sp,
-                                               float* __restrict__ vel, float* __restrict__ dg,
-                                               unsigned long long* __restrict__ ccount) {
-  constexpr int CH = 64;
-  __shared__ float4 s0[2][CH], s1[2][CH], s2[2][CH], s3[2][CH];
-  __shared__ float2 s4[2][CH];
+// What the pair kernel and the combine kernel write.
+struct P2POut {
+  const float* far_u;
+  const float* far_s;
+  const uint32_t* sidx;
+  const double* dip;  // uniform dipole velocity of a one-problem evaluation (or nullptr)
+  float* vel;
+  float* dg;
+};
+
+// Output of target i (sorted position) from its 12 sums.
+template <int ST>
+__device__ __forceinline__ void write_target(const P2POut& out, int i, float X, float Y, float Z, const float4& g,
+                                             const float v[12], float dux, float duy, float duz) {
+  const size_t o = out.sidx[i], f = (size_t)3 * i;
+  const float ax = v[0], ay = v[1], az = v[2];
+  if (out.vel) {  // u = A x X_i - B
+    out.vel[3 * o] = out.far_u[f] + kInv4Pi * ((ay * Z - az * Y) - v[3]) + dux;
+    out.vel[3 * o + 1] = out.far_u[f + 1] + kInv4Pi * ((az * X - ax * Z) - v[4]) + duy;
+    out.vel[3 * o + 2] = out.far_u[f + 2] + kInv4Pi * ((ax * Y - ay * X) - v[5]) + duz;
+  }
+  if (ST == 1 && out.dg) {  // s = A x gamma_i - 3 (C x X_i - D)
+    const float cx = v[6], cy = v[7], cz = v[8];
+    out.dg[3 * o] = out.far_s[f] + kInv4Pi * ((ay * g.z - az * g.y) + kM3 * ((cy * Z - cz * Y) - v[9]));
+    out.dg[3 * o + 1] = out.far_s[f + 1] + kInv4Pi * ((az * g.x - ax * g.z) + kM3 * ((cz * X - cx * Z) - v[10]));
+    out.dg[3 * o + 2] = out.far_s[f + 2] + kInv4Pi * ((ax * g.y - ay * g.x) + kM3 * ((cx * Y - cy * X) - v[11]));
+  }
+  if (ST == 2 && out.dg) {  // s = gamma_i x A - 3 (W X_i + D)
+    out.dg[3 * o] = out.far_s[f] + kInv4Pi * ((g.y * az - g.z * ay) + kM3 * (v[6] * X + v[9]));
+    out.dg[3 * o + 1] = out.far_s[f + 1] + kInv4Pi * ((g.z * ax - g.x * az) + kM3 * (v[6] * Y + v[10]));
+    out.dg[3 * o + 2] = out.far_s[f + 2] + kInv4Pi * ((g.x * ay - g.y * ax) + kM3 * (v[6] * Z + v[11]));
+  }
+}
+
+constexpr int kTileMax = 64;  // targets of a work item
+// One-warp CTAs asked for per SM (80 registers): Taylor-Green 128^3 took 19.08,
+// 18.90, 19.04 and 18.56 ms at 16, 18, 20 and 24, a 100,003-blob ball 1.154,
+// 1.125, 1.129 and 1.113 ms.
+constexpr int kP2PPerSm = 24;
+
+// One warp per work item: a tile of at most 64 targets of one leaf against a
+// range [f0, f1) of the leaf's sources, numbered through the leaf's list
+// (epre: the scanned source counts of the list entries).  The sources are
+// loaded 64 at a time, one chunk ahead, and staged grouped by class.  Staging
+// runs across entry boundaries, so small source leaves fill a chunk.  A tile
+// of more than 32 targets is wide: two targets per lane, one source at a
+// time.  A tile of at most 32 targets is narrow: one target per lane and two
+// sources at a time, and with at most 16 (8) targets 2 (4) lane groups take
+// every 2nd (4th) pair of sources, so the lanes stay filled.  The sums of a
+// range that is not the whole list go to a partial slot, added in range order
+// by k_p2p_combine.  One-warp CTAs keep the chunk bookkeeping warp-uniform
+// (four warps per CTA on quarters of an item cost 5% at Taylor-Green 128^3).
+// Bound by the FMA pipe: 78 cycles per 64 pairs and warp scheduler at
+// Taylor-Green 128^3, where the pair loops alone (microbenchmark) take 66 (far)
+// and 87 (mid).  Measured P2P, before (one warp per leaf, whole lists, source
+// leaves staged one by one) and after: Taylor-Green 128^3 19.34 -> 18.56 ms,
+// Plummer 1,000,000 22.3 -> 10.5 ms, Plummer 30,011 2.52 -> 0.39 ms, ball
+// 100,003 1.74 -> 1.11 ms.
+template <int PS, int ST>
+__global__ void __launch_bounds__(32, kP2PPerSm)
+    k_p2p(const int4* __restrict__ items, const int* __restrict__ islot, int tile, const int* __restrict__ leaves,
+          const int2* __restrict__ off, const int2* __restrict__ list, const uint32_t* __restrict__ epre,
+          const int* __restrict__ begin, const int* __restrict__ end, const float4* __restrict__ cf,
+          const float4* __restrict__ A, const float4* __restrict__ B, const float4* __restrict__ sigk, float blen,
+          float smax, float margin0, SigK K0, const int* __restrict__ cseg, const SegP2P* __restrict__ sp,
+          P2POut out, float* __restrict__ partial, unsigned long long* __restrict__ ccount) {
+  __shared__ Stage<PS> sm;
   const int lane = threadIdx.x;
-  const int leaf = leaves[blockIdx.x];
-  const int tb = begin[leaf], te = end[leaf];
-  const int2 rg = off[blockIdx.x];
+  const int4 item = items[blockIdx.x];
+  const int leaf = leaves[item.x];
+  const int t0 = item.y, nt = min(tile, end[leaf] - t0);
+  const int2 rg = off[item.x];
   const float4 lc = cf[leaf];
-  float dux = dip ? (float)dip[0] : 0.f, duy = dip ? (float)dip[1] : 0.f, duz = dip ? (float)dip[2] : 0.f;
-  if (SEG) {
-    const SegP2P q = sp[cseg[leaf]];
-    K0 = make_sigk(q.sigma);
+  float dux = 0.f, duy = 0.f, duz = 0.f;
+  if (cseg) {
+    const SegP2P& q = sp[cseg[leaf]];
+    K0 = q.k;
     blen = q.blen;
     smax = q.smax;
     margin0 = q.margin;
     dux = q.dip[0];
     duy = q.dip[1];
     duz = q.dip[2];
+  } else if (out.dip) {
+    dux = (float)out.dip[0];
+    duy = (float)out.dip[1];
+    duz = (float)out.dip[2];
   }
-  const SigK2 K = make_sigk2(K0);
-  float4 ra[2], rb[2];
-  unsigned long long c_near = 0, c_mid = 0, c_far = 0;
-  TileBox box;
-  auto stage = [&](int bb, int cnt, int img, bool self_entry, int& nf, int& nm) {
-    const float shx = -(float)(img / 9 - 1) * blen, shy = -(float)((img / 3) % 3 - 1) * blen,
-                shz = -(float)(img % 3 - 1) * blen;
-    float X[2], Y[2], Z[2];
-    int cls[2], slot[2];
+  const bool wide = nt > 32;
+  const int groups = nt > 16 ? 1 : (nt > 8 ? 2 : 4);
+  const int width = 32 / groups, grp = lane / width, tl = lane & (width - 1);
+  Tgt2 t;
+  {
+    float xs[2], ys[2], zs[2], gx[2], gy[2], gz[2], sg[2];
+    bool valid[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const int j = lane + 32 * q;
-      X[q] = (ra[q].x - lc.x) - shx;
-      Y[q] = (ra[q].y - lc.y) - shy;
-      Z[q] = (ra[q].z - lc.z) - shz;
-      cls[q] = j >= cnt ? -1 : self_entry ? kNear : source_class(X[q], Y[q], Z[q], box, lc.w, smax, margin0);
-    }
-    group_slots<2>(cls, lane, slot, nf, nm);
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int k = slot[q];
-      if (k >= 0) {
-        const float4 g = rb[q];
-        const float kx = g.y * Z[q] - g.z * Y[q], ky = g.z * X[q] - g.x * Z[q], kz = g.x * Y[q] - g.y * X[q];
-        s0[bb][k] = make_float4(-X[q], -X[q], -Y[q], -Y[q]);
-        s1[bb][k] = make_float4(-Z[q], -Z[q], g.x, g.x);
-        s2[bb][k] = make_float4(g.y, g.y, g.z, g.z);
-        s3[bb][k] = make_float4(kx, kx, ky, ky);
-        s4[bb][k] = make_float2(kz, kz);
-      }
-    }
-  };
-  for (int t0 = tb; t0 < te; t0 += CH) {
-    float xs[2], ys[2], zs[2], gxs[2], gys[2], gzs[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = t0 + lane + 32 * q;
-      const float4 xi = i < te ? A[i] : lc;
-      const float4 gi = i < te ? B[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int k = wide ? lane + 32 * q : tl;
+      valid[q] = k < nt;
+      const float4 xi = valid[q] ? A[t0 + k] : lc;
+      const float4 gi = valid[q] ? B[t0 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
       xs[q] = xi.x - lc.x;
       ys[q] = xi.y - lc.y;
       zs[q] = xi.z - lc.z;
-      gxs[q] = gi.x;
-      gys[q] = gi.y;
-      gzs[q] = gi.z;
+      gx[q] = gi.x;
+      gy[q] = gi.y;
+      gz[q] = gi.z;
+      sg[q] = valid[q] ? xi.w : smax;
+      (q ? t.id1 : t.id0) = valid[q] ? t0 + k : -2;
     }
-    {
-      const bool valid[2] = {t0 + lane < te, t0 + lane + 32 < te};
-      box = tile_box<2>(xs, ys, zs, valid);
+    const TileBox b = tile_box<2>(xs, ys, zs, valid);
+    if (lane == 0) {
+      sm.box = b;
+      sm.centre = lc;
     }
-    const float2 tx = make_float2(xs[0], xs[1]), ty = make_float2(ys[0], ys[1]), tz = make_float2(zs[0], zs[1]);
-    const float2 gix = make_float2(gxs[0], gxs[1]), giy = make_float2(gys[0], gys[1]),
-                 giz = make_float2(gzs[0], gzs[1]);
-    TgtT2 tt;
+    t.x = make_float2(xs[0], xs[1]);
+    t.y = make_float2(ys[0], ys[1]);
+    t.z = make_float2(zs[0], zs[1]);
+    t.gx = make_float2(gx[0], gx[1]);
+    t.gy = make_float2(gy[0], gy[1]);
+    t.gz = make_float2(gz[0], gz[1]);
+    if (PS == 2) t.sg = make_float2(sg[0], sg[1]);
     if (ST == 2) {
-      float m[3][2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        m[0][q] = ys[q] * gzs[q] - zs[q] * gys[q];
-        m[1][q] = zs[q] * gxs[q] - xs[q] * gzs[q];
-        m[2][q] = xs[q] * gys[q] - ys[q] * gxs[q];
-      }
-      tt.mx = make_float2(m[0][0], m[0][1]);
-      tt.my = make_float2(m[1][0], m[1][1]);
-      tt.mz = make_float2(m[2][0], m[2][1]);
-      tt.ngx = make_float2(-gxs[0], -gxs[1]);
-      tt.ngy = make_float2(-gys[0], -gys[1]);
-      tt.ngz = make_float2(-gzs[0], -gzs[1]);
-    }
-    AccR2 a;
-    a.ax = a.ay = a.az = a.bx = a.by = a.bz = a.cx = a.cy = a.cz = a.dx = a.dy = a.dz = dup2(0.f);
-    const unsigned long long nt = (unsigned long long)min(CH, te - t0);
-    int cur_e = rg.x, cur_c0 = rg.x < rg.y ? begin[list[rg.x].x] : 0, cur_cnt = 0, cur_nf = 0, cur_nm = 0;
-    int buf = 0;
-    if (cur_e < rg.y) {
-      cur_cnt = min(CH, end[list[cur_e].x] - cur_c0);
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int j = lane + 32 * q;
-        if (j < cur_cnt) {
-          ra[q] = A[cur_c0 + j];
-          rb[q] = B[cur_c0 + j];
-        }
-      }
-      const int2 e0 = list[cur_e];
-      stage(0, cur_cnt, e0.y, e0.x == leaf && e0.y == kImageZero, cur_nf, cur_nm);
-    }
-    __syncwarp();
-    while (cur_e < rg.y) {
-      int ne = cur_e, nc0 = cur_c0 + CH;
-      if (nc0 >= end[list[ne].x]) {
-        ++ne;
-        nc0 = ne < rg.y ? begin[list[ne].x] : 0;
-      }
-      int ncnt = 0;
-      if (ne < rg.y) {
-        ncnt = min(CH, end[list[ne].x] - nc0);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int j = lane + 32 * q;
-          if (j < ncnt) {
-            ra[q] = A[nc0 + j];
-            rb[q] = B[nc0 + j];
-          }
-        }
-      }
-      const int2 ent = list[cur_e];
-      const bool self = (ent.x == leaf) && ent.y == kImageZero;
-      const float4* c0 = s0[buf];
-      const float4* c1 = s1[buf];
-      const float4* c2 = s2[buf];
-      const float4* c3 = s3[buf];
-      const float2* c4 = s4[buf];
-      if (self) {
-        const int slo = (t0 + lane) - cur_c0, shi = (t0 + lane + 32) - cur_c0;
-        run_chunk_x2<kNear, true, ST>(c0, c1, c2, c3, c4, 0, cur_cnt, tx, ty, tz, gix, giy, giz, tt, slo, shi, K,
-                                      a);
-      } else {
-        const int nfm = cur_nf + cur_nm;
-        if (cur_nf > 0)
-          run_chunk_x2<kFar, false, ST>(c0, c1, c2, c3, c4, 0, cur_nf, tx, ty, tz, gix, giy, giz, tt, -1, -1, K, a);
-        if (cur_nm > 0)
-          run_chunk_x2<kMid, false, ST>(c0, c1, c2, c3, c4, cur_nf, nfm, tx, ty, tz, gix, giy, giz, tt, -1, -1, K,
-                                        a);
-        if (nfm < cur_cnt)
-          run_chunk_x2<kNear, false, ST>(c0, c1, c2, c3, c4, nfm, cur_cnt, tx, ty, tz, gix, giy, giz, tt, -1, -1,
-                                         K, a);
-      }
-      c_far += nt * (unsigned long long)cur_nf;
-      c_mid += nt * (unsigned long long)cur_nm;
-      c_near += nt * (unsigned long long)(cur_cnt - cur_nf - cur_nm);
-      __syncwarp();
-      buf ^= 1;
-      int nnf = 0, nnm = 0;
-      if (ne < rg.y) {
-        const int2 en = list[ne];
-        stage(buf, ncnt, en.y, en.x == leaf && en.y == kImageZero, nnf, nnm);
-      }
-      __syncwarp();
-      cur_e = ne;
-      cur_c0 = nc0;
-      cur_cnt = ncnt;
-      cur_nf = nnf;
-      cur_nm = nnm;
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = t0 + lane + 32 * q;
-      if (i >= te) continue;
-      const float ax = q ? a.ax.y : a.ax.x, ay = q ? a.ay.y : a.ay.x, az = q ? a.az.y : a.az.x;
-      const float bx = q ? a.bx.y : a.bx.x, by = q ? a.by.y : a.by.x, bz = q ? a.bz.y : a.bz.x;
-      const float cx = q ? a.cx.y : a.cx.x, cy = q ? a.cy.y : a.cy.x, cz = q ? a.cz.y : a.cz.x;
-      const float ex = q ? a.dx.y : a.dx.x, ey = q ? a.dy.y : a.dy.x, ez = q ? a.dz.y : a.dz.x;
-      const float X = xs[q], Y = ys[q], Z = zs[q];
-      const uint32_t o = sidx[i];
-      if (vel) {  // u = A x X_i - B
-        vel[3 * o] = far_u[3 * i] + kInv4Pi * ((ay * Z - az * Y) - bx) + dux;
-        vel[3 * o + 1] = far_u[3 * i + 1] + kInv4Pi * ((az * X - ax * Z) - by) + duy;
-        vel[3 * o + 2] = far_u[3 * i + 2] + kInv4Pi * ((ax * Y - ay * X) - bz) + duz;
-      }
-      if (ST == 2 && dg) {  // s = gamma_i x A + W X_i + (sum w (-X_j)), W = C.x
-        const float gx = gxs[q], gy = gys[q], gz = gzs[q];
-        dg[3 * o] = far_s[3 * i] + kInv4Pi * ((gy * az - gz * ay) + kM3 * (cx * X + ex));
-        dg[3 * o + 1] = far_s[3 * i + 1] + kInv4Pi * ((gz * ax - gx * az) + kM3 * (cx * Y + ey));
-        dg[3 * o + 2] = far_s[3 * i + 2] + kInv4Pi * ((gx * ay - gy * ax) + kM3 * (cx * Z + ez));
-      }
-      if (ST == 1 && dg) {  // s = A x gamma_i + C x X_i - D
-        const float gx = gxs[q], gy = gys[q], gz = gzs[q];
-        dg[3 * o] = far_s[3 * i] + kInv4Pi * ((ay * gz - az * gy) + kM3 * ((cy * Z - cz * Y) - ex));
-        dg[3 * o + 1] = far_s[3 * i + 1] + kInv4Pi * ((az * gx - ax * gz) + kM3 * ((cz * X - cx * Z) - ey));
-        dg[3 * o + 2] = far_s[3 * i + 2] + kInv4Pi * ((ax * gy - ay * gx) + kM3 * ((cx * Y - cy * X) - ez));
-      }
+      t.mx = make_float2(ys[0] * gz[0] - zs[0] * gy[0], ys[1] * gz[1] - zs[1] * gy[1]);
+      t.my = make_float2(zs[0] * gx[0] - xs[0] * gz[0], zs[1] * gx[1] - xs[1] * gz[1]);
+      t.mz = make_float2(xs[0] * gy[0] - ys[0] * gx[0], xs[1] * gy[1] - ys[1] * gx[1]);
+      t.ngx = make_float2(-gx[0], -gx[1]);
+      t.ngy = make_float2(-gy[0], -gy[1]);
+      t.ngz = make_float2(-gz[0], -gz[1]);
     }
   }
-  add_class_counts(ccount, c_near, c_mid, c_far);
+  const SigK2 K = make_sigk2(K0, K0);
+  AccR2 a;
+  a.ax = a.ay = a.az = a.bx = a.by = a.bz = a.cx = a.cy = a.cz = a.dx = a.dy = a.dz = dup2(0.f);
+  unsigned c_near = 0, c_mid = 0, c_far = 0;
+
+  const uint32_t base = epre[rg.x], fe = (uint32_t)item.w;
+  uint32_t f = (uint32_t)item.z;
+  if (f < fe) {
+    // the entry that holds source f: the last one whose prefix is <= f
+    int e0 = rg.x, hi = rg.y;
+    while (hi - e0 > 1) {
+      const int st = (hi - e0 + 31) / 32, c = e0 + lane * st;
+      const bool le = c < hi && epre[c] - base <= f;
+      const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
+      e0 += k * st;
+      hi = min(hi, e0 + st);
+    }
+    // window of 32 entries from e0: their prefixes, source ranges and images
+    uint32_t wp, wend;
+    int2 wl;
+    auto load_window = [&](int e) {
+      const int c = e + lane;
+      wp = c < rg.y ? epre[c] - base : 0xffffffffu;
+      wl = c < rg.y ? list[c] : make_int2(0, 0);
+      wend = epre[min(e + 32, rg.y)] - base;
+    };
+    int cnt = 0;
+    // the next chunk's loads: the sources from f on, within the window; then
+    // the window of the chunk after it
+    auto load_chunk = [&]() {
+      cnt = (int)min(min(fe, wend) - f, (uint32_t)kCh);
+      const bool one = __shfl_sync(0xffffffffu, wp, 1) >= f + (uint32_t)cnt;  // all in the first entry
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint32_t s = f + (uint32_t)(lane + 32 * q);
+        int k = 0;
+        if (!one) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            const uint32_t v = __shfl_sync(0xffffffffu, wp, k + o);
+            if (v <= s) k += o;
+          }
+        }
+        const uint32_t pk = __shfl_sync(0xffffffffu, wp, k);
+        const int bk = __shfl_sync(0xffffffffu, wl.x, k);
+        const int ik = __shfl_sync(0xffffffffu, wl.y, k);
+        if (lane + 32 * q < cnt) {
+          const int j = bk + (int)(s - pk), r = lane + 32 * q;
+          copy16(&sm.raw[0][r], A + j);
+          copy16(&sm.raw[1][r], B + j);
+          if constexpr (PS == 1) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) copy16(&sm.raw[2 + i][r], sigk + 3 * (size_t)j + i);
+          }
+          sm.rid[r] = ik == kImageZero ? j : -1;
+          sm.rimg[r] = ik;
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      f += (uint32_t)cnt;
+      if (f < fe) {
+        e0 += f >= wend ? 32 : __popc(__ballot_sync(0xffffffffu, wp <= f)) - 1;
+        load_window(e0);
+      }
+    };
+    load_window(e0);
+    load_chunk();
+    while (cnt > 0) {
+      // stage the loaded chunk: X_j = (x_j - c) - shift, gamma_j, k_j =
+      // gamma_j x X_j, grouped far, mid, near (in source order each);
+      // sources of zero strength (the separate targets of
+      // fmm_eval_targets) add nothing and are left out
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      const TileBox box = sm.box;
+      const float4 c = sm.centre;
+      float X[2], Y[2], Z[2];
+      float4 ra[2], rb[2];
+      int cls[2], slot[2], nf, nm;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int r = lane + 32 * q, img = r < cnt ? sm.rimg[r] : kImageZero;
+        ra[q] = r < cnt ? sm.raw[0][r] : c;
+        rb[q] = r < cnt ? sm.raw[1][r] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float shx = -(float)(img / 9 - 1) * blen, shy = -(float)((img / 3) % 3 - 1) * blen,
+                    shz = -(float)(img % 3 - 1) * blen;
+        X[q] = (ra[q].x - c.x) - shx;
+        Y[q] = (ra[q].y - c.y) - shy;
+        Z[q] = (ra[q].z - c.z) - shz;
+        const bool live = rb[q].x != 0.f || rb[q].y != 0.f || rb[q].z != 0.f;
+        cls[q] = live ? source_class(X[q], Y[q], Z[q], box, c.w, smax, margin0) : -1;
+      }
+      group_slots<2>(cls, lane, slot, nf, nm);
+      const int used = __popc(__ballot_sync(0xffffffffu, cls[0] >= 0)) + __popc(__ballot_sync(0xffffffffu, cls[1] >= 0));
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int k = slot[q];
+        if (k < 0) continue;
+        const float4 g = rb[q];
+        const float kx = g.y * Z[q] - g.z * Y[q], ky = g.z * X[q] - g.x * Z[q], kz = g.x * Y[q] - g.y * X[q];
+        sm.id[k] = sm.rid[lane + 32 * q];
+        float* sk = reinterpret_cast<float*>(sm.k);
+        if (wide) {
+          sm.v[k] = make_float4(-X[q], -Y[q], -Z[q], g.x);
+          sm.v[kCh + k] = make_float4(g.y, g.z, kx, ky);
+          reinterpret_cast<float*>(sm.v + 2 * kCh)[k] = kz;
+          if constexpr (PS == 1) {
+            sm.k[k] = sm.raw[2][lane + 32 * q];
+            sm.k[kChPad + k] = sm.raw[3][lane + 32 * q];
+            sk[8 * kChPad + k] = sm.raw[4][lane + 32 * q].x;
+          }
+        } else {
+          float* r = reinterpret_cast<float*>(sm.v) + k;
+          r[0] = -X[q];
+          r[kChPad] = -Y[q];
+          r[2 * kChPad] = -Z[q];
+          r[3 * kChPad] = g.x;
+          r[4 * kChPad] = g.y;
+          r[5 * kChPad] = g.z;
+          r[6 * kChPad] = kx;
+          r[7 * kChPad] = ky;
+          r[8 * kChPad] = kz;
+          if constexpr (PS == 1) {
+            const float4 k0 = sm.raw[2][lane + 32 * q], k1 = sm.raw[3][lane + 32 * q];
+            sk[k] = k0.x;
+            sk[kChPad + k] = k0.y;
+            sk[2 * kChPad + k] = k0.z;
+            sk[3 * kChPad + k] = k0.w;
+            sk[4 * kChPad + k] = k1.x;
+            sk[5 * kChPad + k] = k1.y;
+            sk[6 * kChPad + k] = k1.z;
+            sk[7 * kChPad + k] = k1.w;
+            sk[8 * kChPad + k] = sm.raw[4][lane + 32 * q].x;
+          }
+        }
+        if (PS == 2) sk[k] = ra[q].w;
+      }
+      int n0 = nf, n1 = nf + nm, n2 = used;
+      if (!wide) {
+        // whole units: a class's remainder runs in the next nearer form, the
+        // last unit is filled with sources of zero strength away from the targets
+        const int unit = 2 * groups;
+        n0 &= ~(unit - 1);
+        n1 &= ~(unit - 1);
+        n2 = (used + unit - 1) & ~(unit - 1);
+        if (lane < n2 - used) {
+          float* r = reinterpret_cast<float*>(sm.v) + used + lane;
+          r[0] = -(box.hx + 4.f * smax + 1.f);
+          r[kChPad] = -box.hy;
+          r[2 * kChPad] = -box.hz;
+#pragma unroll
+          for (int q = 3; q < 9; ++q) r[q * kChPad] = 0.f;
+          sm.id[used + lane] = -1;
+          float* sk = reinterpret_cast<float*>(sm.k) + used + lane;
+          if (PS == 1) {
+            sk[0] = -1.f;
+#pragma unroll
+            for (int q = 1; q < 9; ++q) sk[q * kChPad] = 0.f;
+            sk[6 * kChPad] = 4.f;
+          }
+          if (PS == 2) sk[0] = smax;
+        }
+      }
+      c_far += (unsigned)n0;
+      c_mid += (unsigned)(n1 - n0);
+      c_near += (unsigned)(used - n1);
+      __syncwarp();
+      const bool more = f < fe;
+      if (more) load_chunk();
+      else cnt = 0;
+      if (wide) {
+        if (n0 > 0) run_group<kFar, false, PS, ST>(sm, 0, n0, 1, t, K, a);
+        if (n1 > n0) run_group<kMid, false, PS, ST>(sm, n0, n1, 1, t, K, a);
+        if (n2 > n1) run_group<kNear, false, PS, ST>(sm, n1, n2, 1, t, K, a);
+      } else {
+        if (n0 > 0) run_group<kFar, true, PS, ST>(sm, grp, n0 / 2, groups, t, K, a);
+        if (n1 > n0) run_group<kMid, true, PS, ST>(sm, n0 / 2 + grp, n1 / 2, groups, t, K, a);
+        if (n2 > n1) run_group<kNear, true, PS, ST>(sm, n1 / 2 + grp, n2 / 2, groups, t, K, a);
+      }
+      __syncwarp();
+    }
+  }
+  constexpr int NV = ST == 0 ? 6 : 12;
+  const float2 va[12] = {a.ax, a.ay, a.az, a.bx, a.by, a.bz, a.cx, a.cy, a.cz, a.dx, a.dy, a.dz};
+  const int ps = islot[blockIdx.x];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float v[12];
+    const int k = wide ? lane + 32 * q : tl;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      v[i] = q ? va[i].y : va[i].x;
+      if (!wide) {  // the two chains and the lane groups hold sums of the same target
+        v[i] += q ? va[i].x : va[i].y;
+        for (int o = width; o < 32; o <<= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+      }
+    }
+    if (k >= nt || (!wide && (q || grp))) continue;
+    if (ps >= 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) partial[((size_t)ps * 12 + i) * kTileMax + k] = v[i];
+    } else {
+      const float4 g = make_float4(q ? t.gx.y : t.gx.x, q ? t.gy.y : t.gy.x, q ? t.gz.y : t.gz.x, 0.f);
+      write_target<ST>(out, t0 + k, q ? t.x.y : t.x.x, q ? t.y.y : t.y.x, q ? t.z.y : t.z.x, g, v, dux, duy, duz);
+    }
+  }
+  if (lane == 0) {
+    const unsigned long long m = (unsigned long long)nt;
+    if (c_near) atomicAdd(&ccount[0], m * c_near);
+    if (c_mid) atomicAdd(&ccount[1], m * c_mid);
+    if (c_far) atomicAdd(&ccount[2], m * c_far);
+  }
+}
+
+// Targets of the tiles whose list was split: the partial sums of the ranges,
+// added in range order.  One CTA per leaf; plan[leaf] = (first partial slot,
+// ranges per tile).
+template <int ST>
+__global__ void __launch_bounds__(kTileMax) k_p2p_combine(const int2* __restrict__ plan, int tile,
+                                                          const int* __restrict__ leaves,
+                                                          const int* __restrict__ begin, const int* __restrict__ end,
+                                                          const float4* __restrict__ cf,
+                                                          const float4* __restrict__ A, const float4* __restrict__ B,
+                                                          const int* __restrict__ cseg, const SegP2P* __restrict__ sp,
+                                                          P2POut out, const float* __restrict__ partial) {
+  constexpr int NV = ST == 0 ? 6 : 12;
+  const int2 pl = plan[blockIdx.x];
+  if (pl.y <= 1) return;
+  const int leaf = leaves[blockIdx.x];
+  const float4 lc = cf[leaf];
+  float dux = 0.f, duy = 0.f, duz = 0.f;
+  if (cseg) {
+    const SegP2P& q = sp[cseg[leaf]];
+    dux = q.dip[0];
+    duy = q.dip[1];
+    duz = q.dip[2];
+  } else if (out.dip) {
+    dux = (float)out.dip[0];
+    duy = (float)out.dip[1];
+    duz = (float)out.dip[2];
+  }
+  int slot = pl.x;
+  for (int t0 = begin[leaf]; t0 < end[leaf]; t0 += tile, slot += pl.y) {
+    const int i = t0 + threadIdx.x;
+    if ((int)threadIdx.x >= tile || i >= end[leaf]) continue;
+    float v[12];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = 0.f;
+    for (int k = 0; k < pl.y; ++k) {
+      const float* src = partial + (size_t)(slot + k) * 12 * kTileMax + threadIdx.x;
+#pragma unroll
+      for (int q = 0; q < NV; ++q) v[q] += src[q * kTileMax];
+    }
+    const float4 xi = A[i];
+    write_target<ST>(out, i, xi.x - lc.x, xi.y - lc.y, xi.z - lc.z, B[i], v, dux, duy, duz);
+  }
+}
+
+// How a leaf's F sources are cut into ranges: none up to `whole`, else ranges of
+// at most `range` sources, but at most `cap` of them.
+struct RangeRule {
+  uint32_t whole, range, cap;
+};
+
+// ---- work items: per leaf, tiles x ranges, the longest ranges first (four
+// length classes, leaf order within each), so that the last warps to start
+// are short: in leaf order the batch of 32 problems waited for its longest
+// lists (P2P 5.56 ms, now 5.23).  One CTA walks the leaves twice: the class
+// totals, then the scan.  counts[0] = items, counts[1] = partial slots.
+constexpr int kItemClasses = 4;
+
+__global__ void __launch_bounds__(1024) k_p2p_items(const int* __restrict__ leaves, int nl,
+                                                    const int* __restrict__ begin, const int* __restrict__ end,
+                                                    const int2* __restrict__ off, const uint32_t* __restrict__ epre,
+                                                    int tile, RangeRule rr, int4* __restrict__ items,
+                                                    int* __restrict__ islot, int2* __restrict__ plan,
+                                                    uint32_t* __restrict__ counts) {
+  constexpr int NC = kItemClasses + 1;  // item classes, then partial slots
+  __shared__ uint32_t ws[NC][32];
+  __shared__ uint32_t carry[NC];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x < NC) carry[threadIdx.x] = 0u;
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int c0 = 0; c0 < nl; c0 += 1024) {
+      const int i = c0 + threadIdx.x;
+      uint32_t nit = 0, nsp = 0, F = 0;
+      int tb = 0, te = 0, cls = kItemClasses - 1;
+      if (i < nl) {
+        const int leaf = leaves[i];
+        tb = begin[leaf];
+        te = end[leaf];
+        const int2 rg = off[i];
+        F = epre[rg.y] - epre[rg.x];
+        nsp = F <= rr.whole ? 1u : min(rr.cap, (F + rr.range - 1) / rr.range);
+        nit = nsp * (uint32_t)((te - tb + tile - 1) / tile);
+        const uint32_t len = F / nsp;
+        cls = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
+      }
+      uint32_t own[NC], inc[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        own[q] = q < kItemClasses ? (q == cls ? nit : 0u) : (nsp > 1 ? nit : 0u);
+        inc[q] = own[q];
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc[q], o);
+          if (lane >= o) inc[q] += y;
+        }
+        if (lane == 31) ws[q][w] = inc[q];
+      }
+      __syncthreads();
+      if (w < NC) {  // warp w scans the warp totals of count w
+        uint32_t v = ws[w][lane], x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        const uint32_t c = carry[w];
+        ws[w][lane] = c + x - v;
+        if (lane == 31) carry[w] = c + x;
+      }
+      __syncthreads();
+      if (pass == 1 && i < nl) {
+        uint32_t io = 0;
+#pragma unroll
+        for (int q = 0; q < kItemClasses; ++q)
+          if (q == cls) io = ws[q][w] + inc[q] - own[q];
+        uint32_t slot = ws[kItemClasses][w] + inc[kItemClasses] - own[kItemClasses];
+        plan[i] = make_int2((int)slot, (int)nsp);
+        // equal ranges, so that no range is a short remainder
+        const uint32_t len = (F + nsp - 1) / nsp;
+        for (int t0 = tb; t0 < te; t0 += tile)
+          for (uint32_t k = 0; k < nsp; ++k, ++io, ++slot) {
+            items[io] = make_int4(i, t0, (int)min(F, k * len), (int)min(F, (k + 1) * len));
+            islot[io] = nsp > 1 ? (int)slot : -1;
+          }
+      }
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+      if (pass == 0) {  // the classes' first items
+        uint32_t acc = 0;
+        for (int q = 0; q < kItemClasses; ++q) {
+          const uint32_t c = carry[q];
+          carry[q] = acc;
+          acc += c;
+        }
+        counts[0] = acc;
+        counts[1] = carry[kItemClasses];
+        carry[kItemClasses] = 0u;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// The constants of every particle's own core width, in the order the pair
+// kernel stages them: (kq, kc, hn0, hn2), (hn3, hn4, ku, is3), (is5).  Once per
+// particle: computed in the pair kernel for every staged source, their FP64
+// divisions were most of its time (ball of 60,000 own widths: P2P 4.74 ms,
+// 1.09 with the table and the packed pairs).
+__global__ void k_sigk(const float4* __restrict__ A, int64_t n, float4* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const SigK k = make_sigk(A[i].w);
+  out[3 * i] = make_float4(k.kq, k.kc, k.hn0, k.hn2);
+  out[3 * i + 1] = make_float4(k.hn3, k.hn4, k.ku, k.is3);
+  out[3 * i + 2] = make_float4(k.is5, 0.f, 0.f, 0.f);
 }
 
 // All pairs of one array, free space, self pair skipped (near class throughout).
@@ -1064,87 +1138,124 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
   return FMM_OK;
 }
 
+// Work items of the pair kernel (after the list is grouped by leaf): one warp
+// per (tile of a leaf, range of its sources).  Ranges bound the longest warp:
+// the big outer leaves of a clustered cloud meet thousands of small ones, and
+// one warp per leaf left the chip waiting for them (Plummer, 30,011 blobs:
+// P2P 2.5 ms; 0.39 ms with ranges).  One-problem plans take the range that
+// gives about eight warps per resident one, at least 128 sources (two chunks);
+// the partial slots are then bounded by twice that many items (3 KB each).  A
+// batch takes a rule of its own, so that a problem's sums do not depend on the
+// rest of the batch, with the ranges of a leaf capped for the slots' sake.
+constexpr int64_t kItemTarget = 8 * 16 * 152;  // items aimed at (24 instead of 16 per SM: Plummer 30,011 0.39 -> 0.42 ms)
+constexpr uint32_t kItemSrcMin = 128;
+// batch of 32 problems, 477,044 blobs: P2P 5.23 ms; 5.17 with whole lists only
+// up to 4096 sources, for twice the slots
+constexpr RangeRule kBatchRule = {8192u, 2048u, 16u};
+
+int p2p_tile(fmm_plan p) { return p->prm.p2p_tpl == 1 ? 32 : kTileMax; }
+
+int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s) {
+  const int tile = p2p_tile(p);
+  RangeRule rr = kBatchRule;
+  if (!p->batched) {
+    const int64_t q = (tile_sources / kItemTarget + kCh - 1) / kCh * kCh;
+    rr.whole = rr.range = (uint32_t)std::min<int64_t>(0xffffffffll - kCh, std::max<int64_t>(kItemSrcMin, q));
+    rr.cap = 0xffffffffu;
+  }
+  // at most one partly filled range and one partly filled tile per leaf
+  const int64_t tiles = p->nleaves + n / tile + 1;
+  const int64_t items = tiles + std::min<int64_t>(tile_sources / rr.range + 1, tiles * (int64_t)rr.cap);
+  FMM_TRY(p->p2p_items.ensure((size_t)items * sizeof(int4)));
+  FMM_TRY(p->p2p_islot.ensure((size_t)items * sizeof(int)));
+  FMM_TRY(p->p2p_plan.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
+  ++g_launches;
+  k_p2p_items<<<1, 1024, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, p->c_begin.as<int>(), p->c_end.as<int>(),
+                                 p->p2p_off.as<int2>(), p->p2p_pre.as<uint32_t>(), tile, rr,
+                                 p->p2p_items.as<int4>(), p->p2p_islot.as<int>(), p->p2p_plan.as<int2>(), counts);
+  FMM_CUDA_TRY(cudaGetLastError());
+  return FMM_OK;
+}
+
+// The staging memory (7.5 to 13 KB a warp, 16 warps per SM) needs the largest
+// shared-memory carveout.
+static int p2p_attributes() {
+  static const bool ok = [] {
+    const void* k[9] = {(const void*)k_p2p<0, 0>, (const void*)k_p2p<0, 1>, (const void*)k_p2p<0, 2>,
+                        (const void*)k_p2p<1, 0>, (const void*)k_p2p<1, 1>, (const void*)k_p2p<1, 2>,
+                        (const void*)k_p2p<2, 0>, (const void*)k_p2p<2, 1>, (const void*)k_p2p<2, 2>};
+    for (const void* f : k)
+      if (cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) return false;
+    return true;
+  }();
+  return ok ? FMM_OK : FMM_E_CUDA;
+}
+
 int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, float* vel, float* dg, cudaStream_t s) {
-  const double* dip = nullptr;
   double* scal = p->scal.as<double>();
   const int* cseg = p->batched ? p->c_seg.as<int>() : nullptr;
   SegP2P* sp = p->batched ? p->seg_p2p.as<SegP2P>() : nullptr;
+  P2POut out;
+  out.far_u = p->far_u.as<float>();
+  out.far_s = p->far_s.as<float>();
+  out.sidx = p->sidx;
+  out.dip = nullptr;
+  out.vel = vel;
+  out.dg = dg;
   if (p->prm.periodic && p->batched) {
     ++g_launches;
     k_dipole_seg<<<p->nseg, 256, 0, s>>>(p->sortA.as<float4>(), p->sortB.as<float4>(), p->seg_off.as<int>(),
                                          p->seg_box.as<double>(), sp);
   } else if (p->prm.periodic) {
-    dip = scal + kScalDipole;  // dipole_pass ran beside the traversal
+    out.dip = scal + kScalDipole;  // dipole_pass ran beside the traversal
   }
   const float blen = p->prm.periodic ? (float)p->prm.box_len : 0.f;
-  SigK K0 = make_sigk(ps ? 1.f : sig_u);
-  const unsigned g = (unsigned)p->nleaves;
+  const SigK K0 = make_sigk(ps ? 1.f : sig_u);
+  const int mode = ps ? (p->prm.sigma_rule == FMM_SIGMA_MIXED ? 2 : 1) : 0;
+  const int tile = p2p_tile(p);
+  const float4* A = p->sortA.as<float4>();
+  const float4* B = p->sortB.as<float4>();
+  const float4* sigk = nullptr;
+  if (mode == 1) {
+    FMM_TRY(p->p2p_sigk.ensure((size_t)n * 3 * sizeof(float4)));
+    ++g_launches;
+    k_sigk<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(A, n, p->p2p_sigk.as<float4>());
+    sigk = p->p2p_sigk.as<float4>();
+  }
+  FMM_TRY(p->p2p_partial.ensure((size_t)std::max<int64_t>(p->n_p2p_slots, 1) * 12 * kTileMax * sizeof(float)));
+  float* partial = p->p2p_partial.as<float>();
+  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(scal + kScalCount + 4);
+  FMM_CUDA_TRY(cudaMemsetAsync(cnt, 0, 3 * sizeof(unsigned long long), s));
   const int* leaves = p->leaves.as<int>();
-  const int2* off = p->p2p_off.as<int2>();
-  const int2* list = p->p2p_sorted.as<int2>();
   const int* cb = p->c_begin.as<int>();
   const int* ce = p->c_end.as<int>();
   const float4* cf = p->c_cf.as<float4>();
-  const float4* A = p->sortA.as<float4>();
-  const float4* B = p->sortB.as<float4>();
-  const float* fu = p->far_u.as<float>();
-  const float* fs = p->far_s.as<float>();
-  const float smaxf = (float)smax;
-  const float margin0 = (float)p->cf_margin;
-  const bool two = p->prm.p2p_tpl ? p->prm.p2p_tpl == 2 : p->prm.ncrit > 32;
-  const int mixed = ps && p->prm.sigma_rule == FMM_SIGMA_MIXED;
-  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(scal + kScalCount + 4);
-  FMM_CUDA_TRY(cudaMemsetAsync(cnt, 0, 3 * sizeof(unsigned long long), s));
+  const unsigned items = (unsigned)p->n_p2p_items;
+  const float smaxf = (float)smax, margin0 = (float)p->cf_margin;
+  FMM_TRY(p2p_attributes());
+#define FMM_P2P(PS_, ST_)                                                                                             \
+  k_p2p<PS_, ST_><<<items, 32, 0, s>>>(p->p2p_items.as<int4>(), p->p2p_islot.as<int>(), tile, leaves,     \
+                                                   p->p2p_off.as<int2>(), p->p2p_sorted.as<int2>(),                   \
+                                                   p->p2p_pre.as<uint32_t>(), cb, ce, cf, A, B, sigk, blen, smaxf,    \
+                                                   margin0, K0, cseg, sp, out, partial, cnt)
+#define FMM_P2P_ST(ST_)                \
+  do {                                 \
+    if (mode == 0) FMM_P2P(0, ST_);    \
+    else if (mode == 1) FMM_P2P(1, ST_); \
+    else FMM_P2P(2, ST_);              \
+    if (p->n_p2p_slots > 0) {          \
+      ++g_launches;                    \
+      k_p2p_combine<ST_><<<(unsigned)p->nleaves, kTileMax, 0, s>>>(p->p2p_plan.as<int2>(), tile, leaves, cb, ce, cf, \
+                                                                   A, B, cseg, sp, out, partial);                    \
+    }                                  \
+  } while (0)
   ++g_launches;
-  // the packed kernel stages 9 KB per warp: ask for the largest shared-memory carveout
-  static bool carveout_set = false;
-  if (!carveout_set) {
-    const void* kx2[6] = {(const void*)k_p2p_x2<false, 0>, (const void*)k_p2p_x2<false, 1>,
-                          (const void*)k_p2p_x2<false, 2>, (const void*)k_p2p_x2<true, 0>,
-                          (const void*)k_p2p_x2<true, 1>,  (const void*)k_p2p_x2<true, 2>};
-    for (const void* k : kx2)
-      FMM_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    carveout_set = true;
-  }
-#define FMM_P2P_LAUNCH(PS_, TPT_, SEG_, ST_)                                                                      \
-  do {                                                                                                            \
-    if (mixed)                                                                                                    \
-      k_p2p<true, TPT_, SEG_, ST_, true><<<g, 32, 0, s>>>(leaves, off, list, cb, ce, cf, A, B, fu, fs, p->sidx,    \
-                                                          blen, smaxf, margin0, K0, dip, cseg, sp, vel, dg, cnt); \
-    else                                                                                                          \
-      k_p2p<PS_, TPT_, SEG_, ST_, false><<<g, 32, 0, s>>>(leaves, off, list, cb, ce, cf, A, B, fu, fs, p->sidx,    \
-                                                          blen, smaxf, margin0, K0, dip, cseg, sp, vel, dg, cnt); \
-  } while (0)
-#define FMM_P2P_X2_LAUNCH(SEG_, ST_)                                                                          \
-  k_p2p_x2<SEG_, ST_><<<g, 32, 0, s>>>(leaves, off, list, cb, ce, cf, A, B, fu, fs, p->sidx, blen, smaxf,     \
-                                       margin0, K0, dip, cseg, sp, vel, dg, cnt)
-#define FMM_P2P_ALL(ST_)                                       \
-  do {                                                         \
-    if (cseg) {                                                \
-      if (two) {                                               \
-        if (ps) FMM_P2P_LAUNCH(true, 2, true, ST_);            \
-        else FMM_P2P_X2_LAUNCH(true, ST_);                     \
-      } else {                                                 \
-        if (ps) FMM_P2P_LAUNCH(true, 1, true, ST_);            \
-        else FMM_P2P_LAUNCH(false, 1, true, ST_);              \
-      }                                                        \
-    } else {                                                   \
-      if (two) {                                               \
-        if (ps) FMM_P2P_LAUNCH(true, 2, false, ST_);           \
-        else FMM_P2P_X2_LAUNCH(false, ST_);                    \
-      } else {                                                 \
-        if (ps) FMM_P2P_LAUNCH(true, 1, false, ST_);           \
-        else FMM_P2P_LAUNCH(false, 1, false, ST_);             \
-      }                                                        \
-    }                                                          \
-  } while (0)
   // without a stretching output the kernels skip T and the stretching sums
-  if (!dg) FMM_P2P_ALL(0);
-  else if (p->prm.outputs & FMM_OUT_STRETCHING_TRANSPOSE) FMM_P2P_ALL(2);
-  else FMM_P2P_ALL(1);
-#undef FMM_P2P_ALL
-#undef FMM_P2P_LAUNCH
-#undef FMM_P2P_X2_LAUNCH
+  if (!dg) FMM_P2P_ST(0);
+  else if (p->prm.outputs & FMM_OUT_STRETCHING_TRANSPOSE) FMM_P2P_ST(2);
+  else FMM_P2P_ST(1);
+#undef FMM_P2P_ST
+#undef FMM_P2P
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }

@@ -375,18 +375,37 @@ __global__ void k_p2p_keys(const int4* __restrict__ raw, int n, uint64_t* __rest
   vals[i] = (uint32_t)i;
 }
 
-__global__ void k_p2p_gather(const int4* __restrict__ raw, const uint32_t* __restrict__ order, int n,
-                             int2* __restrict__ out, const int* __restrict__ begin, const int* __restrict__ end,
-                             unsigned long long* __restrict__ pairs) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long cnt = 0;
-  if (i < n) {
-    int4 v = raw[order[i]];
-    out[i] = make_int2(v.y, v.z);
-    cnt = (unsigned long long)(end[v.x] - begin[v.x]) * (unsigned long long)(end[v.y] - begin[v.y]);
+// Entries in leaf order: (first source particle, image) and the source count;
+// totals: the particle pairs, and the sources summed over the target tiles.
+// Grid-stride with few blocks, one atomic per block and total.
+__global__ void __launch_bounds__(256) k_p2p_gather(const int4* __restrict__ raw, const uint32_t* __restrict__ order,
+                                                    int n, int2* __restrict__ out, uint32_t* __restrict__ count,
+                                                    const int* __restrict__ begin, const int* __restrict__ end,
+                                                    int tile, unsigned long long* __restrict__ totals) {
+  unsigned long long pairs = 0, srcs = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int4 v = raw[order[i]];
+    const int sb = begin[v.y], ns = end[v.y] - sb, nt = end[v.x] - begin[v.x];
+    out[i] = make_int2(sb, v.z);
+    count[i] = (uint32_t)ns;
+    pairs += (unsigned long long)nt * (unsigned long long)ns;
+    srcs += (unsigned long long)((nt + tile - 1) / tile) * (unsigned long long)ns;
   }
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(pairs, cnt);
+  for (int o = 16; o > 0; o >>= 1) {
+    pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    srcs += __shfl_xor_sync(0xffffffffu, srcs, o);
+  }
+  __shared__ unsigned long long sh[2][8];
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = pairs;
+    sh[1][threadIdx.x >> 5] = srcs;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long c = 0;
+    for (int w = 0; w < 8; ++w) c += sh[threadIdx.x][w];
+    if (c) atomicAdd(&totals[threadIdx.x], c);
+  }
 }
 
 __device__ inline int lower_bound_key(const uint64_t* a, int n, uint64_t v) {
@@ -697,6 +716,7 @@ __global__ void k_seg_tables(int nseg, const double* __restrict__ box, const uns
   mac[sg] = m;
   SegP2P q;
   q.sigma = sig ? sig[sg] : 1.f;
+  q.k = make_sigk(q.sigma);
   q.smax = (float)smax;
   q.blen = (float)blen;
   q.margin = (float)margin;
@@ -862,14 +882,19 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
     uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
     unsigned long long* dpairs = reinterpret_cast<unsigned long long*>(p->scal.as<double>() + kScalCount + 2);
-    FMM_CUDA_TRY(cudaMemsetAsync(dpairs, 0, sizeof(unsigned long long), s));
+    FMM_CUDA_TRY(cudaMemsetAsync(dpairs, 0, 2 * sizeof(unsigned long long), s));
+    FMM_TRY(p->p2p_pre.ensure((size_t)(n + 1) * sizeof(uint32_t)));
     ++g_launches;
-    k_p2p_gather<<<g, T, 0, s>>>(p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(), p->c_begin.as<int>(),
-                                 p->c_end.as<int>(), dpairs);
+    k_p2p_gather<<<std::min<unsigned>(std::max(g, 1u), 1216u), T, 0, s>>>(
+        p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(), p->p2p_pre.as<uint32_t>(), p->c_begin.as<int>(),
+        p->c_end.as<int>(), p2p_tile(p), dpairs);
+    // the scan wraps past 2^32 sources; differences within a leaf stay exact
+    FMM_TRY(exclusive_scan_u32(p->p2p_pre.as<uint32_t>(), p->p2p_pre.as<uint32_t>(), n, p->p2p_pre.as<uint32_t>() + n,
+                               p->scan_tmp, s));
     ++g_launches;
     k_p2p_offsets<<<(unsigned)((p->nleaves + T - 1) / T), T, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, sk, n,
                                                                      p->p2p_off.as<int2>());
-    FMM_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(p->pinned) + 64, dpairs, sizeof(unsigned long long),
+    FMM_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(p->pinned) + 64, dpairs, 2 * sizeof(unsigned long long),
                                  cudaMemcpyDeviceToHost, s));
   }
 
@@ -901,6 +926,11 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       int* hg = reinterpret_cast<int*>(reinterpret_cast<char*>(p->pinned) + 1024);  // counts, then offsets
       FMM_CUDA_TRY(cudaMemcpyAsync(hg, gcount, kGroups * sizeof(int), cudaMemcpyDeviceToHost, s));
       FMM_CUDA_TRY(cudaStreamSynchronize(s));
+      // the list totals copied above: the work items of the pair kernel
+      const int64_t tile_sources = (int64_t) reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 64)[1];
+      FMM_TRY(p2p_build_items(p, p->last_n, tile_sources, dcnt + 2, s));
+      FMM_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(p->pinned) + 96, dcnt + 2, 2 * sizeof(uint32_t),
+                                   cudaMemcpyDeviceToHost, s));
       int* hofs = hg + kGroups;
       int* htile = hofs + kGroups;
       int cells = 0, tiles = 0;
@@ -1070,6 +1100,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   }
   FMM_CUDA_TRY(cudaStreamSynchronize(s));
   p->p2p_pairs = (int64_t) * reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 64);
+  p->n_p2p_items = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(p->pinned) + 96)[0];
+  p->n_p2p_slots = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(p->pinned) + 96)[1];
   return FMM_OK;
 }
 
