@@ -42,13 +42,14 @@ struct SigK {
 
 __host__ __device__ inline SigK make_sigk(float sigma) {
   SigK k;
-  const double s = (double)sigma, ky = 1.4142135623730951 * s;
-  k.kq = (float)(-1.4426950408889634 / (2.0 * s * s));
-  k.kc = (float)(-0.79788456080286535588 / (3.0 * s * s * s));
-  k.ku = (float)(1.0 / (s * s));
-  k.is3 = (float)(1.0 / (s * s * s));
-  k.is5 = (float)(-2.0 / (3.0 * s * s * s * s * s));
-  k.hn0 = (float)(-0.79788456080286535588 / s);
+  // one FP64 division (k_sigk and k_direct evaluate this per particle)
+  const double s = (double)sigma, ky = 1.4142135623730951 * s, i = 1.0 / s, i2 = i * i, i3 = i2 * i;
+  k.kq = (float)(-0.72134752044448170 * i2);
+  k.kc = (float)(-0.79788456080286535588 / 3.0 * i3);
+  k.ku = (float)i2;
+  k.is3 = (float)i3;
+  k.is5 = (float)(-2.0 / 3.0 * (i3 * i2));
+  k.hn0 = (float)(-0.79788456080286535588 * i);
   k.hn1 = (float)(-(double)kE0);
   k.hn2 = (float)(-(double)kE1 * ky);
   k.hn3 = (float)(-(double)kE2 * ky * ky);

@@ -28,13 +28,14 @@
 // g = 1 to FP32 precision (rho >= 6.5), the cutoff without the series test
 // (rho^2 >= 2), or the full form; a chunk is staged grouped by class, so each
 // group runs its own branch-free loop.
+#include <cooperative_groups.h>
+
 #include "fmm_internal.cuh"
 
 namespace fmm {
 
 namespace {
 
-constexpr int kMaxBlock = 128;
 constexpr float kInv4Pi = 0.0795774715459476679f;
 constexpr float kM3 = -3.f;  // T = -3 T': scales the stretching sums built from T'
 // Source-leaf classes by a lower bound d_min on the pair distance:
@@ -88,65 +89,6 @@ __device__ __forceinline__ SigK sigk_mixed(float si, float sj) {
   k.hn3 = -kE2 * 2.f * s2;
   k.hn4 = -kE3 * 2.82842712474619030f * s2 * sg;
   return k;
-}
-
-// S = g/r^3 and T' = -S'(r)/(3r) for one pair (see the file header); ST = 0:
-// S only (velocity without stretching).
-template <int MODE, int ST = 1>
-__device__ __forceinline__ void pair_ST(float r2, const SigK& K, float& S, float& T) {
-  const float rinv = rsqrt_approx(r2);
-  const float rinv2 = rinv * rinv;
-  T = 0.f;
-  if (MODE == kFar) {
-    S = rinv2 * rinv;
-    if (ST) T = S * rinv2;
-    return;
-  }
-  const float rinv3 = rinv2 * rinv;
-  const float q = ex2_approx(r2 * K.kq);
-  // beyond the fit range (x > 4.6) exp(-x^2) < 8e-10 multiplies a bounded
-  // polynomial, so g = 1 to FP32 precision without clamping
-  const float hn = fmaf(fmaf(fmaf(fmaf(K.hn4, rinv, K.hn3), rinv, K.hn2), rinv, K.hn1), rinv, K.hn0);
-  S = fmaf(q, rinv2 * hn, rinv3);
-  if (ST) T = fmaf(K.kc, q, S) * rinv2;
-  if (MODE == kNear) {
-    const float u = r2 * K.ku;
-    if (u < 2.f) {
-      float sS = cSer[kSerTerms - 1], sT = (float)(kSerTerms - 1) * cSer[kSerTerms - 1];
-#pragma unroll
-      for (int k = kSerTerms - 2; k >= 0; --k) {
-        sS = fmaf(sS, u, cSer[k]);
-        if (ST && k >= 1) sT = fmaf(sT, u, (float)k * cSer[k]);
-      }
-      S = sS * K.is3;
-      if (ST) T = sT * K.is5;
-    }
-  }
-}
-
-struct Acc {
-  float ux, uy, uz, sx, sy, sz, ax, ay, az;
-};
-
-template <int MODE>
-__device__ __forceinline__ void pair_acc(float dx, float dy, float dz, const float4& gj, float gix, float giy,
-                                         float giz, const SigK& K, Acc& a) {
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  float S, T;
-  pair_ST<MODE>(r2, K, S, T);
-  const float cx = fmaf(gj.y, dz, -gj.z * dy);
-  const float cy = fmaf(gj.z, dx, -gj.x * dz);
-  const float cz = fmaf(gj.x, dy, -gj.y * dx);
-  a.ux = fmaf(S, cx, a.ux);
-  a.uy = fmaf(S, cy, a.uy);
-  a.uz = fmaf(S, cz, a.uz);
-  a.ax = fmaf(S, gj.x, a.ax);
-  a.ay = fmaf(S, gj.y, a.ay);
-  a.az = fmaf(S, gj.z, a.az);
-  const float td = T * fmaf(gix, dx, fmaf(giy, dy, giz * dz));
-  a.sx = fmaf(td, cx, a.sx);
-  a.sy = fmaf(td, cy, a.sy);
-  a.sz = fmaf(td, cz, a.sz);
 }
 
 // Axis-aligned bounding box of the targets of one tile, relative to the leaf
@@ -234,35 +176,6 @@ __device__ __forceinline__ void group_slots(const int* cls, int lane, int* slot,
   }
 }
 
-// Targets held by one thread.
-template <int TPT>
-struct Tgt {
-  float x[TPT], y[TPT], z[TPT], gx[TPT], gy[TPT], gz[TPT];
-  int self[TPT];  // staged index of the target itself in the current chunk, or -1
-  Acc a[TPT];
-};
-
-template <bool PS, int MODE, bool SHIFT, bool SELF, int TPT>
-__device__ __forceinline__ void run_chunk(const float4* sA, const float4* sB, const SigK* sK, int cnt, Tgt<TPT>& t,
-                                          float shx, float shy, float shz, const SigK& K0) {
-#pragma unroll 2
-  for (int j = 0; j < cnt; ++j) {
-    const float4 xj = sA[j];
-    const float4 gj = sB[j];
-#pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      float dx = t.x[q] - xj.x, dy = t.y[q] - xj.y, dz = t.z[q] - xj.z;
-      if (SHIFT) {
-        dx += shx;
-        dy += shy;
-        dz += shz;
-      }
-      if (SELF && j == t.self[q]) continue;
-      pair_acc<MODE>(dx, dy, dz, gj, t.gx[q], t.gy[q], t.gz[q], PS ? sK[j] : K0, t.a[q]);
-    }
-  }
-}
-
 // ---- The pair kernel.  Two pairs at a time run as the two lanes of the
 // FP32x2 instructions (fma/mul/add .f32x2): the FMA pipe does the same work
 // per clock as with scalars, in half the issue slots.
@@ -304,7 +217,8 @@ struct AccR2 {
   float2 ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz;
 };
 
-// S and T of two pairs (see pair_ST).
+// S = g/r^3 and T' = -S'(r)/(3r) of two pairs (see the file header); ST = 0: S
+// only (velocity without stretching).
 template <int MODE, int ST>
 __device__ __forceinline__ void pair_ST2(float2 r2, const SigK2& K, float2& S, float2& T) {
   const float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
@@ -318,6 +232,8 @@ __device__ __forceinline__ void pair_ST2(float2 r2, const SigK2& K, float2& S, f
   const float2 rinv3 = mul2(rinv2, rinv);
   const float2 qa = mul2(r2, K.kq);
   const float2 q = make_float2(ex2_approx(qa.x), ex2_approx(qa.y));
+  // beyond the fit range (x > 4.6) exp(-x^2) < 8e-10 multiplies a bounded
+  // polynomial, so g = 1 to FP32 precision without clamping
   const float2 hn = fma2(fma2(fma2(fma2(K.hn4, rinv, K.hn3), rinv, K.hn2), rinv, K.hn1), rinv, K.hn0);
   S = fma2(q, mul2(rinv2, hn), rinv3);
   if (ST) T = mul2(fma2(K.kc, q, S), rinv2);
@@ -1002,55 +918,166 @@ __global__ void k_sigk(const float4* __restrict__ A, int64_t n, float4* __restri
   out[3 * i + 2] = make_float4(k.is5, 0.f, 0.f, 0.f);
 }
 
-// All pairs of one array, free space, self pair skipped (near class throughout).
+// All pairs of one array, free space, self pair skipped.  A cluster of eight
+// CTAs of four warps takes 64 targets (two per lane, as the two halves of the
+// FP32x2 operations); each of its 32 warps sums a contiguous 32nd of the
+// sources, staged 32 at a time in its own shared memory, and the partial sums
+// meet in distributed shared memory, added in source order.  The split keeps
+// the chip filled at any n without a workspace: 20,000 blobs took 1.75 ms as
+// 157 CTAs of 128 targets with scalar pairs, 0.67 ms now (100,000: 19.3 ->
+// 14.1 ms; the error against FP64 2.5e-6 -> 5.2e-7).  Bound by the FMA
+// pipe (38 operations per pair).  The targets keep absolute coordinates, so a
+// pair takes gamma_j x d of the exact difference.
+constexpr int kDirCluster = 8, kDirWarps = 4, kDirTile = 64;
+
+struct DirStage {
+  float4 a[32];  // -x, -y, -z, gamma_x
+  float2 b[32];  // gamma_y, gamma_z
+};
+struct DirStageK {  // constants of the source's own core width
+  float4 k0[32], k1[32];  // kq kc hn0 hn2, hn3 hn4 ku is3
+  float is5[32];
+};
+
 template <bool PS>
-__global__ void __launch_bounds__(kMaxBlock) k_direct(int64_t n, const float* __restrict__ pos,
-                                                      const float* __restrict__ gam, const float* __restrict__ sig,
-                                                      SigK K0, float* __restrict__ vel, float* __restrict__ dg) {
-  __shared__ float4 sA[kMaxBlock], sB[kMaxBlock];
-  __shared__ SigK sK[PS ? kMaxBlock : 1];
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = i < n;
-  Tgt<1> t;
-  t.x[0] = t.y[0] = t.z[0] = t.gx[0] = t.gy[0] = t.gz[0] = 0.f;
-  if (valid) {
-    t.x[0] = pos[3 * i];
-    t.y[0] = pos[3 * i + 1];
-    t.z[0] = pos[3 * i + 2];
-    t.gx[0] = gam[3 * i];
-    t.gy[0] = gam[3 * i + 1];
-    t.gz[0] = gam[3 * i + 2];
+__global__ void __cluster_dims__(kDirCluster, 1, 1) __launch_bounds__(32 * kDirWarps, 6)
+    k_direct(int64_t n, const float* __restrict__ pos, const float* __restrict__ gam, const float* __restrict__ sig,
+             SigK K0, float* __restrict__ vel, float* __restrict__ dg) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ DirStage st[kDirWarps];
+  __shared__ DirStageK stk[PS ? kDirWarps : 1];
+  __shared__ float red[kDirWarps][9][kDirTile];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = (int)cluster.block_rank();
+  const int64_t i0 = (int64_t)(blockIdx.x / kDirCluster) * kDirTile;
+  float2 tx, ty, tz, gx, gy, gz;
+  {
+    float v[2][6];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int64_t i = min(i0 + lane + 32 * q, n - 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        v[q][a] = pos[3 * i + a];
+        v[q][3 + a] = gam[3 * i + a];
+      }
+    }
+    tx = make_float2(v[0][0], v[1][0]);
+    ty = make_float2(v[0][1], v[1][1]);
+    tz = make_float2(v[0][2], v[1][2]);
+    gx = make_float2(v[0][3], v[1][3]);
+    gy = make_float2(v[0][4], v[1][4]);
+    gz = make_float2(v[0][5], v[1][5]);
   }
-  t.a[0] = Acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int64_t c0 = 0; c0 < n; c0 += blockDim.x) {
-    const int cnt = (int)min((int64_t)blockDim.x, n - c0);
-    __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-      int64_t j = c0 + threadIdx.x;
-      float s = PS ? sig[j] : 0.f;
-      sA[threadIdx.x] = make_float4(pos[3 * j], pos[3 * j + 1], pos[3 * j + 2], s);
-      sB[threadIdx.x] = make_float4(gam[3 * j], gam[3 * j + 1], gam[3 * j + 2], 0.f);
-      if (PS) sK[threadIdx.x] = make_sigk(s);
+  const SigK2 K1 = make_sigk2(K0, K0);
+  float2 acc[9];  // sum S gamma_j x d, sum T' (gamma_i . d) gamma_j x d, sum S gamma_j
+#pragma unroll
+  for (int q = 0; q < 9; ++q) acc[q] = dup2(0.f);
+  const int64_t per = (n + kDirCluster * kDirWarps - 1) / (kDirCluster * kDirWarps);
+  const int64_t j0 = min(n, (int64_t)(rank * kDirWarps + warp) * per), j1 = min(n, j0 + per);
+  float r[7];
+  auto load = [&](int64_t c) {
+    const int64_t j = c + lane;
+    if (j < j1) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        r[a] = pos[3 * j + a];
+        r[3 + a] = gam[3 * j + a];
+      }
+      r[6] = PS ? sig[j] : 0.f;
     }
-    __syncthreads();
-    if (valid) {
-      const bool self = i >= c0 && i < c0 + cnt;
-      t.self[0] = self ? (int)(i - c0) : -1;
-      if (self) run_chunk<PS, kNear, false, true, 1>(sA, sB, sK, cnt, t, 0.f, 0.f, 0.f, K0);
-      else run_chunk<PS, kNear, false, false, 1>(sA, sB, sK, cnt, t, 0.f, 0.f, 0.f, K0);
+  };
+  load(j0);
+  for (int64_t c = j0; c < j1; c += 32) {
+    const int cnt = (int)min((int64_t)32, j1 - c);
+    if (lane < cnt) {
+      st[warp].a[lane] = make_float4(-r[0], -r[1], -r[2], r[3]);
+      st[warp].b[lane] = make_float2(r[4], r[5]);
+      if (PS) {
+        const SigK k = make_sigk(r[6]);
+        stk[PS ? warp : 0].k0[lane] = make_float4(k.kq, k.kc, k.hn0, k.hn2);
+        stk[PS ? warp : 0].k1[lane] = make_float4(k.hn3, k.hn4, k.ku, k.is3);
+        stk[PS ? warp : 0].is5[lane] = k.is5;
+      }
     }
+    __syncwarp();
+    load(c + 32);
+    // staged index of each target itself, if any
+    const int64_t d = i0 + lane - c;
+    const int self0 = d >= 0 && d < 32 ? (int)d : -1, self1 = d + 32 >= 0 && d < 0 ? (int)d + 32 : -1;
+#pragma unroll 2
+    for (int j = 0; j < cnt; ++j) {
+      const float4 a = st[warp].a[j];
+      const float2 b = st[warp].b[j];
+      SigK2 K = K1;
+      if (PS) {
+        const float4 a0 = stk[PS ? warp : 0].k0[j], a1 = stk[PS ? warp : 0].k1[j];
+        K.kq = dup2(a0.x);
+        K.kc = dup2(a0.y);
+        K.hn0 = dup2(a0.z);
+        K.hn2 = dup2(a0.w);
+        K.hn3 = dup2(a1.x);
+        K.hn4 = dup2(a1.y);
+        K.ku = dup2(a1.z);
+        K.is3 = dup2(a1.w);
+        K.is5 = dup2(stk[PS ? warp : 0].is5[j]);
+      }
+      const float2 dx = add2(tx, dup2(a.x)), dy = add2(ty, dup2(a.y)), dz = add2(tz, dup2(a.z));
+      const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+      float2 S, T;
+      pair_ST2<kNear, 1>(r2, K, S, T);
+      if (j == self0) S.x = T.x = 0.f;
+      if (j == self1) S.y = T.y = 0.f;
+      const float2 jx = dup2(a.w), jy = dup2(b.x), jz = dup2(b.y);
+      const float2 cx = fma2(jy, dz, mul2(dup2(-b.y), dy));
+      const float2 cy = fma2(jz, dx, mul2(dup2(-a.w), dz));
+      const float2 cz = fma2(jx, dy, mul2(dup2(-b.x), dx));
+      const float2 td = mul2(T, fma2(gx, dx, fma2(gy, dy, mul2(gz, dz))));
+      acc[0] = fma2(S, cx, acc[0]);
+      acc[1] = fma2(S, cy, acc[1]);
+      acc[2] = fma2(S, cz, acc[2]);
+      acc[3] = fma2(td, cx, acc[3]);
+      acc[4] = fma2(td, cy, acc[4]);
+      acc[5] = fma2(td, cz, acc[5]);
+      acc[6] = fma2(S, jx, acc[6]);
+      acc[7] = fma2(S, jy, acc[7]);
+      acc[8] = fma2(S, jz, acc[8]);
+    }
+    __syncwarp();
   }
-  if (valid) {
-    const Acc& a = t.a[0];
-    if (vel) {
-      vel[3 * i] = kInv4Pi * a.ux;
-      vel[3 * i + 1] = kInv4Pi * a.uy;
-      vel[3 * i + 2] = kInv4Pi * a.uz;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    red[warp][q][lane] = acc[q].x;
+    red[warp][q][lane + 32] = acc[q].y;
+  }
+  cluster.sync();
+  // each CTA finishes eight of the targets: the 32 partial sums of each value
+  // in source order
+  const int t = threadIdx.x / 9, q = threadIdx.x % 9;
+  const int k = rank * (kDirTile / kDirCluster) + t;
+  __shared__ float fin[kDirTile / kDirCluster][9];
+  if (t < kDirTile / kDirCluster) {
+    float v = 0.f;
+    for (int b = 0; b < kDirCluster; ++b) {
+      const float* src = cluster.map_shared_rank(&red[0][q][k], b);
+      for (int w = 0; w < kDirWarps; ++w) v += src[w * 9 * kDirTile];
     }
-    if (dg) {
-      dg[3 * i] = kInv4Pi * (kM3 * a.sx + (a.ay * t.gz[0] - a.az * t.gy[0]));
-      dg[3 * i + 1] = kInv4Pi * (kM3 * a.sy + (a.az * t.gx[0] - a.ax * t.gz[0]));
-      dg[3 * i + 2] = kInv4Pi * (kM3 * a.sz + (a.ax * t.gy[0] - a.ay * t.gx[0]));
+    fin[t][q] = v;
+  }
+  cluster.sync();  // the other CTAs' sums have been read
+  if (threadIdx.x < kDirTile / kDirCluster) {
+    const int64_t i = i0 + rank * (kDirTile / kDirCluster) + threadIdx.x;
+    const float* v = fin[threadIdx.x];
+    if (i < n) {
+      if (vel)
+        for (int a = 0; a < 3; ++a) vel[3 * i + a] = kInv4Pi * v[a];
+      if (dg) {
+        const float x = gam[3 * i], y = gam[3 * i + 1], z = gam[3 * i + 2];
+        dg[3 * i] = kInv4Pi * (kM3 * v[3] + (v[7] * z - v[8] * y));
+        dg[3 * i + 1] = kInv4Pi * (kM3 * v[4] + (v[8] * x - v[6] * z));
+        dg[3 * i + 2] = kInv4Pi * (kM3 * v[5] + (v[6] * y - v[7] * x));
+      }
     }
   }
 }
@@ -1262,12 +1289,13 @@ int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, float* vel
 
 int p2p_direct_all(int64_t n, const float* pos, const float* gam, const float* sig, float sig_u, float* vel, float* dg,
                    cudaStream_t s) {
-  const int bs = 128;
-  unsigned g = (unsigned)((n + bs - 1) / bs);
-  SigK K0 = make_sigk(sig ? 1.f : sig_u);
+  const int64_t tiles = (n + kDirTile - 1) / kDirTile;
+  if (tiles * kDirCluster > 0x7fffffffll) return FMM_E_INVAL;
+  const unsigned g = (unsigned)(tiles * kDirCluster);
+  const SigK K0 = make_sigk(sig ? 1.f : sig_u);
   ++g_launches;
-  if (sig) k_direct<true><<<g, bs, 0, s>>>(n, pos, gam, sig, K0, vel, dg);
-  else k_direct<false><<<g, bs, 0, s>>>(n, pos, gam, sig, K0, vel, dg);
+  if (sig) k_direct<true><<<g, 32 * kDirWarps, 0, s>>>(n, pos, gam, sig, K0, vel, dg);
+  else k_direct<false><<<g, 32 * kDirWarps, 0, s>>>(n, pos, gam, sig, K0, vel, dg);
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }

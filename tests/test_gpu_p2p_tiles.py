@@ -64,3 +64,29 @@ def test_pair_sums_at_tile_edges(sums, ncrit, kind):
             assert rel_l2(u.cpu().numpy(), ud) < 2e-5, (tpl, tr)
             assert rel_l2(s.cpu().numpy(), sd) < 5e-5, (tpl, tr)
             plan.close()
+
+
+@pytest.mark.parametrize("kind", ["one", "each"])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 63, 64, 65, 1023, 1025, 2049])
+def test_direct_sum_at_tile_and_share_edges(n, kind):
+    """The all-pairs kernel where a 64-target tile or a warp's 32nd of the
+    sources is empty, partly filled or one past full, against the FP64 pair
+    sum; rel-L2 2e-6 (u) and 5e-6 (s), the tolerances of the all-pairs parity
+    test (FP32 unit roundoff times the growth of sums of a few thousand terms
+    of exact differences)."""
+    import torch
+    from oracle import pairs
+    from paper_1106_5273_gb300 import direct
+    w = workloads.uniform_ball(n)
+    sig = (w["sigma"] * np.linspace(0.7, 1.3, n)).astype(np.float32) if kind == "each" else None
+    u, s = direct(to_dev(w["pos"]), to_dev(w["gamma"]), sigma=None if sig is None else to_dev(sig),
+                  sigma_uniform=float(w["sigma"]))
+    torch.cuda.synchronize()
+    x, g = w["pos"].astype(np.float64), w["gamma"].astype(np.float64)
+    sg = np.full(n, float(w["sigma"])) if sig is None else sig.astype(np.float64)
+    ud, sd = pairs.pair_sum(x, g, x, g, sg, None, np.eye(n, dtype=bool))
+    if n == 1:
+        assert not u.cpu().numpy().any() and not s.cpu().numpy().any()
+    else:
+        assert rel_l2(u.cpu().numpy(), ud) < 2e-6
+        assert rel_l2(s.cpu().numpy(), sd) < 5e-6
