@@ -41,7 +41,7 @@ std::vector<DBuf*> plan_buffers(fmm_plan p) {
           &p->tile_cells, &p->tile_first, &p->tile_groups, &p->c_ijk, &p->t_pos, &p->t_gam, &p->t_sig, &p->t_vel, &p->leaves, &p->M, &p->L, &p->Mbf, &p->fr0, &p->fr1, &p->tcount, &p->tmask,
           &p->tscan0, &p->tscan1, &p->tscan2, &p->p2p_raw, &p->m2l_raw, &p->lk0, &p->lk1, &p->lv0, &p->lv1,
           &p->p2p_sorted, &p->p2p_off, &p->p2p_pre, &p->p2p_items, &p->p2p_islot, &p->p2p_plan, &p->p2p_partial, &p->p2p_sigk, &p->m2l_key, &p->m2l_slot, &p->ukeys, &p->T32, &p->Tbf,
-          &p->tmiss_keys, &p->tmiss_slots, &p->tslot_map, &p->st_tile, &p->st_slot, &p->st_src, &p->bin_flag, &p->bin_scan, &p->bin_flag2, &p->bin_scan2, &p->st_ckey,
+          &p->tc_key, &p->tc_slot, &p->tmiss_keys, &p->tmiss_slots, &p->tslot_map, &p->st_tile, &p->st_slot, &p->st_src, &p->bin_flag, &p->bin_scan, &p->bin_flag2, &p->bin_scan2, &p->st_ckey,
           &p->st_fkey, &p->m2l_items, &p->m2l_partial, &p->tile_range, &p->scan_tmp, &p->sort_hist, &p->scal,
           &p->flags, &p->seg_off, &p->seg_box, &p->seg_sig, &p->seg_smax, &p->seg_mac, &p->seg_p2p, &p->c_seg};
 }
@@ -63,6 +63,7 @@ int ensure_aux_stream(fmm_plan p) {
   FMM_CUDA_TRY(cudaStreamCreateWithFlags(&p->s_up, cudaStreamNonBlocking));
   FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
   FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
+  FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_read, cudaEventDisableTiming));
   return FMM_OK;
 }
 
@@ -127,7 +128,6 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
     smax = (double)f;
   }
   FMM_TRY(traverse(p, smax, s));
-  FMM_TRY(build_m2l_operators(p, s));
   tm.mark();
   FMM_CUDA_TRY(cudaStreamWaitEvent(s, p->ev_join, 0));
   join_guard.joined = true;
@@ -282,6 +282,7 @@ void fmm_plan_destroy(fmm_plan p) {
     for (int i = 0; i < 8; ++i) cudaEventDestroy(p->ev[i]);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
+  if (p->ev_read) cudaEventDestroy(p->ev_read);
   if (p->s_up) cudaStreamDestroy(p->s_up);
   delete p;
 }

@@ -2,7 +2,6 @@
 #pragma once
 
 #include <algorithm>
-#include <unordered_map>
 #include <vector>
 
 #include "common.cuh"
@@ -132,11 +131,10 @@ struct fmm_plan_s {
   fmm::DBuf p2p_partial, p2p_sigk;                    // partial sums of split lists; per-particle core constants
   fmm::DBuf m2l_key, m2l_slot, ukeys;                 // per pair key, slot; unique keys
   fmm::DBuf T32, Tbf;                                 // M2L operator cache [slot]: FP32, BF16 hi/lo
-  std::unordered_map<uint64_t, int> tcache;           // translation key -> cache slot
-  int64_t tcache_cap = 0;
+  fmm::DBuf tc_key, tc_slot;                          // operator cache: open-addressing table key -> slot
+  int64_t tc_cap = 0, tc_size = 0;                    // table entries; operators in it
+  int64_t tcache_cap = 0;                             // operators T32 / Tbf have room for
   fmm::DBuf tmiss_keys, tmiss_slots, tslot_map;       // keys to build, their slots; unique key -> slot
-  std::vector<uint64_t> h_keys;
-  std::vector<int> h_map;
   int64_t n_built = 0;                                // operators built by the last evaluation
   fmm::DBuf st_tile, st_slot, st_src, tile_range;     // M2L steps
   fmm::DBuf bin_flag, bin_scan, bin_flag2, bin_scan2;  // binned step build: key and bin tables
@@ -178,6 +176,7 @@ struct fmm_plan_s {
   // caller's stream (both read only the tree); fork / join by events
   cudaStream_t s_up = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaEvent_t ev_read = nullptr;  // the host's reads of list sizes
 };
 
 namespace fmm {
@@ -190,7 +189,10 @@ int build_forest(fmm_plan p, int64_t n, const float* pos, const float* gam, cons
                  cudaStream_t s);
 // operators.cu
 int build_constant_operators(fmm_plan p);
-int build_m2l_operators(fmm_plan p, cudaStream_t s);
+int find_m2l_operators(fmm_plan p, uint32_t* miss, uint32_t* rank, uint32_t* nmiss, cudaStream_t s);
+int build_m2l_operators(fmm_plan p, int64_t nmiss, uint32_t* miss, uint32_t* rank, uint32_t* nmiss_dev,
+                        cudaStream_t s);
+int remap_step_slots(fmm_plan p, cudaStream_t s);
 int apply_lattice(fmm_plan p, cudaStream_t s);
 int lattice_operator_host(int p, int images, double* out);
 // lattice.cu

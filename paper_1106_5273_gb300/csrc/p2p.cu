@@ -831,26 +831,31 @@ __global__ void __launch_bounds__(1024) k_p2p_items(const int* __restrict__ leav
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x < NC) carry[threadIdx.x] = 0u;
   __syncthreads();
+  constexpr int R = 4;  // leaves per thread and round (independent loads in flight)
   for (int pass = 0; pass < 2; ++pass) {
-    for (int c0 = 0; c0 < nl; c0 += 1024) {
-      const int i = c0 + threadIdx.x;
-      uint32_t nit = 0, nsp = 0, F = 0;
-      int tb = 0, te = 0, cls = kItemClasses - 1;
-      if (i < nl) {
-        const int leaf = leaves[i];
-        tb = begin[leaf];
-        te = end[leaf];
-        const int2 rg = off[i];
-        F = epre[rg.y] - epre[rg.x];
-        nsp = F <= rr.whole ? 1u : min(rr.cap, (F + rr.range - 1) / rr.range);
-        nit = nsp * (uint32_t)((te - tb + tile - 1) / tile);
-        const uint32_t len = F / nsp;
-        cls = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
+    for (int c0 = 0; c0 < nl; c0 += 1024 * R) {
+      const int i0 = c0 + threadIdx.x * R;
+      uint32_t nit[R], nsp[R], F[R];
+      int cls[R];
+      uint32_t own[NC] = {0u, 0u, 0u, 0u, 0u}, inc[NC];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        nit[r] = nsp[r] = F[r] = 0;
+        cls[r] = kItemClasses - 1;
+        if (i0 + r < nl) {
+          const int leaf = leaves[i0 + r];
+          const int2 rg = off[i0 + r];
+          F[r] = epre[rg.y] - epre[rg.x];
+          nsp[r] = F[r] <= rr.whole ? 1u : min(rr.cap, (F[r] + rr.range - 1) / rr.range);
+          nit[r] = nsp[r] * (uint32_t)((end[leaf] - begin[leaf] + tile - 1) / tile);
+          const uint32_t len = F[r] / nsp[r];
+          cls[r] = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) own[q] += (q < kItemClasses ? q == cls[r] : nsp[r] > 1) ? nit[r] : 0u;
       }
-      uint32_t own[NC], inc[NC];
 #pragma unroll
       for (int q = 0; q < NC; ++q) {
-        own[q] = q < kItemClasses ? (q == cls ? nit : 0u) : (nsp > 1 ? nit : 0u);
         inc[q] = own[q];
         for (int o = 1; o < 32; o <<= 1) {
           const uint32_t y = __shfl_up_sync(0xffffffffu, inc[q], o);
@@ -870,20 +875,29 @@ __global__ void __launch_bounds__(1024) k_p2p_items(const int* __restrict__ leav
         if (lane == 31) carry[w] = c + x;
       }
       __syncthreads();
-      if (pass == 1 && i < nl) {
-        uint32_t io = 0;
+      if (pass == 1) {
+        uint32_t at[NC];
 #pragma unroll
-        for (int q = 0; q < kItemClasses; ++q)
-          if (q == cls) io = ws[q][w] + inc[q] - own[q];
-        uint32_t slot = ws[kItemClasses][w] + inc[kItemClasses] - own[kItemClasses];
-        plan[i] = make_int2((int)slot, (int)nsp);
-        // equal ranges, so that no range is a short remainder
-        const uint32_t len = (F + nsp - 1) / nsp;
-        for (int t0 = tb; t0 < te; t0 += tile)
-          for (uint32_t k = 0; k < nsp; ++k, ++io, ++slot) {
-            items[io] = make_int4(i, t0, (int)min(F, k * len), (int)min(F, (k + 1) * len));
-            islot[io] = nsp > 1 ? (int)slot : -1;
-          }
+        for (int q = 0; q < NC; ++q) at[q] = ws[q][w] + inc[q] - own[q];
+        for (int r = 0; r < R && i0 + r < nl; ++r) {
+          const int leaf = leaves[i0 + r], tb = begin[leaf], te = end[leaf];
+          uint32_t io = 0, slot = at[kItemClasses];
+#pragma unroll
+          for (int q = 0; q < kItemClasses; ++q)
+            if (q == cls[r]) {
+              io = at[q];
+              at[q] += nit[r];
+            }
+          if (nsp[r] > 1) at[kItemClasses] += nit[r];
+          plan[i0 + r] = make_int2((int)slot, (int)nsp[r]);
+          // equal ranges, so that no range is a short remainder
+          const uint32_t len = (F[r] + nsp[r] - 1) / nsp[r];
+          for (int t0 = tb; t0 < te; t0 += tile)
+            for (uint32_t k = 0; k < nsp[r]; ++k, ++io, ++slot) {
+              items[io] = make_int4(i0 + r, t0, (int)min(F[r], k * len), (int)min(F[r], (k + 1) * len));
+              islot[io] = nsp[r] > 1 ? (int)slot : -1;
+            }
+        }
       }
       __syncthreads();
     }

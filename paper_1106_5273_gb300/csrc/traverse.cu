@@ -584,11 +584,12 @@ __global__ void k_bin_mark(const int2* __restrict__ raw, const uint64_t* __restr
 }
 
 __global__ void k_bin_steps(const uint32_t* __restrict__ bflag, const uint32_t* __restrict__ bstep, int64_t nb,
-                            int nkeys, int* __restrict__ st_tile, int* __restrict__ st_slot) {
+                            int nkeys, const int* __restrict__ map, int* __restrict__ st_tile,
+                            int* __restrict__ st_slot) {
   int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb || !bflag[b]) return;
   st_tile[bstep[b]] = (int)(b / nkeys);
-  st_slot[bstep[b]] = (int)(b % nkeys);
+  st_slot[bstep[b]] = map[b % nkeys];  // unique key -> operator slot
 }
 
 __global__ void k_bin_fill(const int2* __restrict__ raw, const uint32_t* __restrict__ pbin, int n,
@@ -649,24 +650,57 @@ __global__ void k_unique_flags(const uint64_t* __restrict__ k, int n, uint32_t* 
 // relative interaction lists in a uniform region, so a tile's steps are
 // nearly full; a tile never mixes octants, so a coarse level is split into
 // its octants instead of one long tile.
-__global__ void k_tile_order_keys(const int* __restrict__ level, const uint64_t* __restrict__ ckey, int nc,
-                                  uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                  int* __restrict__ gcount) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nc) return;
-  const int oct = (int)(ckey[c] & 7ull);
-  // the sort is stable, so cells of a group keep their (Morton) index order
-  keys[c] = ((uint64_t)level[c] << 3) | (uint64_t)oct;
-  vals[c] = (uint32_t)c;
-  atomicAdd(&gcount[level[c] * 8 + oct], 1);
+constexpr int kGroups = (kMaxLevel + 1) * 8;
+__global__ void __launch_bounds__(256) k_tile_order_keys(const int* __restrict__ level,
+                                                         const uint64_t* __restrict__ ckey, int nc,
+                                                         uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                         int* __restrict__ gcount) {
+  __shared__ int h[kGroups];
+  for (int g = threadIdx.x; g < kGroups; g += blockDim.x) h[g] = 0;
+  __syncthreads();
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < nc) {
+    const int g = level[c] * 8 + (int)(ckey[c] & 7ull);
+    // the sort is stable, so cells of a group keep their (Morton) index order
+    keys[c] = (uint64_t)g;
+    vals[c] = (uint32_t)c;
+    atomicAdd(&h[g], 1);
+  }
+  __syncthreads();
+  for (int g = threadIdx.x; g < kGroups; g += blockDim.x)
+    if (h[g]) atomicAdd(&gcount[g], h[g]);
 }
 
 // gofs[g] = first sorted position of (level, octant) group g, gtile[g] = its
-// first tile.
-__global__ void k_cell_tiles(int nc, int ntiles, const uint32_t* __restrict__ order, const int* __restrict__ level,
-                             const uint64_t* __restrict__ ckey, const int* __restrict__ gofs,
-                             const int* __restrict__ gtile, int* __restrict__ ctile, int* __restrict__ tcell,
-                             int* __restrict__ tfirst) {
+// first tile; *ntiles the number of tiles.  Also starts the key ranges.
+__global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int* __restrict__ gofs,
+                                                     int* __restrict__ gtile, uint32_t* __restrict__ ntiles,
+                                                     int* __restrict__ rng) {
+  __shared__ int cells[256], tiles[256];
+  const int g = threadIdx.x;
+  const int c = g < kGroups ? gcount[g] : 0, t = (c + kTile - 1) / kTile;
+  cells[g] = c;
+  tiles[g] = t;
+  __syncthreads();
+  for (int o = 1; o < 256; o <<= 1) {
+    const int x = g >= o ? cells[g - o] : 0, y = g >= o ? tiles[g - o] : 0;
+    __syncthreads();
+    cells[g] += x;
+    tiles[g] += y;
+    __syncthreads();
+  }
+  if (g < kGroups) {
+    gofs[g] = cells[g] - c;
+    gtile[g] = tiles[g] - t;
+  }
+  if (g == 255) *ntiles = (uint32_t)tiles[255];
+  if (g < 8) rng[g] = (g & 1) ? INT_MIN : INT_MAX;
+}
+
+__global__ void k_cell_tiles(int nc, const uint32_t* __restrict__ ntiles, const uint32_t* __restrict__ order,
+                             const int* __restrict__ level, const uint64_t* __restrict__ ckey,
+                             const int* __restrict__ gofs, const int* __restrict__ gtile, int* __restrict__ ctile,
+                             int* __restrict__ tcell, int* __restrict__ tfirst) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nc) return;
   const int c = (int)order[q];
@@ -676,7 +710,7 @@ __global__ void k_cell_tiles(int nc, int ntiles, const uint32_t* __restrict__ or
   ctile[c] = t * kTile + r % kTile;
   tcell[q] = c;
   if (r % kTile == 0) tfirst[t] = q;
-  if (q == 0) tfirst[ntiles] = nc;
+  if (q == 0) tfirst[*ntiles] = nc;
 }
 
 __global__ void k_step_flags(const uint64_t* __restrict__ k, int n, uint32_t* __restrict__ f) {
@@ -743,6 +777,80 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
   return FMM_OK;
 }
 
+// Tiles: at most 64 cells of one (level, octant) group each; and the cells'
+// integer coordinates.  ntiles and the key ranges stay on the device.
+static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
+  const int T = 256;
+  const int nc = (int)p->ncells;
+  FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
+  FMM_TRY(p->tile_cells.ensure((nc + 1) * sizeof(int)));
+  FMM_TRY(p->tile_groups.ensure(3 * kGroups * sizeof(int)));
+  FMM_TRY(p->tile_first.ensure((size_t)(nc / kTile + kGroups + 1) * sizeof(int)));
+  FMM_TRY(p->c_ijk.ensure((size_t)(nc + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->lk0.ensure((nc + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->lk1.ensure((nc + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->lv0.ensure((nc + 1) * sizeof(uint32_t)));
+  FMM_TRY(p->lv1.ensure((nc + 1) * sizeof(uint32_t)));
+  int* gcount = p->tile_groups.as<int>();
+  int* gofs = gcount + kGroups;
+  int* gtile = gofs + kGroups;
+  FMM_CUDA_TRY(cudaMemsetAsync(gcount, 0, kGroups * sizeof(int), s));
+  const unsigned gc = (unsigned)((nc + T - 1) / T);
+  ++g_launches;
+  k_tile_order_keys<<<gc, T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc, p->lk0.as<uint64_t>(),
+                                     p->lv0.as<uint32_t>(), gcount);
+  int second = 0;
+  FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
+                         nc, 0, 8, &second, p->sort_hist, p->scan_tmp, s));
+  ++g_launches;
+  k_tile_groups<<<1, 256, 0, s>>>(gcount, gofs, gtile, ntiles, rng);
+  ++g_launches;
+  k_cell_tiles<<<gc, T, 0, s>>>(nc, ntiles, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
+                                p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs, gtile, p->c_tile.as<int>(),
+                                p->tile_cells.as<int>(), p->tile_first.as<int>());
+  ++g_launches;
+  k_cell_ijk<<<gc, T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc, p->c_ijk.as<uint64_t>());
+  FMM_CUDA_TRY(cudaGetLastError());
+  return FMM_OK;
+}
+
+// P2P entries grouped by target leaf (CSR) with the scanned source counts;
+// totals (host, valid once the stream has passed): particle pairs, and sources
+// summed over the target tiles.
+static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t s) {
+  const int T = 256;
+  FMM_TRY(p->lk0.ensure((size_t)(n + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->lk1.ensure((size_t)(n + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->lv0.ensure((size_t)(n + 1) * sizeof(uint32_t)));
+  FMM_TRY(p->lv1.ensure((size_t)(n + 1) * sizeof(uint32_t)));
+  FMM_TRY(p->p2p_sorted.ensure((size_t)(n + 1) * sizeof(int2)));
+  FMM_TRY(p->p2p_off.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
+  FMM_TRY(p->p2p_pre.ensure((size_t)(n + 1) * sizeof(uint32_t)));
+  unsigned long long* dpairs = reinterpret_cast<unsigned long long*>(p->scal.as<double>() + kScalCount + 2);
+  FMM_CUDA_TRY(cudaMemsetAsync(dpairs, 0, 2 * sizeof(unsigned long long), s));
+  const unsigned g = std::max(1u, (unsigned)((n + T - 1) / T));
+  ++g_launches;
+  k_p2p_keys<<<g, T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+  int second = 0;
+  FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
+                         n, 0, bits_for(p->ncells), &second, p->sort_hist, p->scan_tmp, s));
+  uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
+  uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
+  ++g_launches;
+  k_p2p_gather<<<std::min(g, 1216u), T, 0, s>>>(p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(),
+                                                p->p2p_pre.as<uint32_t>(), p->c_begin.as<int>(), p->c_end.as<int>(),
+                                                p2p_tile(p), dpairs);
+  FMM_CUDA_TRY(cudaMemcpyAsync(totals, dpairs, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  // the scan wraps past 2^32 sources; differences within a leaf stay exact
+  FMM_TRY(exclusive_scan_u32(p->p2p_pre.as<uint32_t>(), p->p2p_pre.as<uint32_t>(), n, p->p2p_pre.as<uint32_t>() + n,
+                             p->scan_tmp, s));
+  ++g_launches;
+  k_p2p_offsets<<<(unsigned)((p->nleaves + T - 1) / T), T, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, sk, n,
+                                                                   p->p2p_off.as<int2>());
+  FMM_CUDA_TRY(cudaGetLastError());
+  return FMM_OK;
+}
+
 int traverse(fmm_plan p, double smax, cudaStream_t s) {
   const int T = 256;
   const int nc = (int)p->ncells;
@@ -784,6 +892,19 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   const int img0 = p->prm.periodic ? 0 : kImageZero;
   uint32_t* hc = reinterpret_cast<uint32_t*>(p->pinned);
   uint32_t* dcnt = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount);
+  int* drng = reinterpret_cast<int*>(p->scal.as<double>() + kScalCount + 8);
+  // device counts: tiles, translations, steps, missing operators, P2P items and partial slots
+  uint32_t* dmisc = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount + 12);
+  char* pin = reinterpret_cast<char*>(p->pinned);
+  uint32_t* hmisc = reinterpret_cast<uint32_t*>(pin + 288);
+  int* hrng = reinterpret_cast<int*>(pin + 256);
+  // the host reads `bytes` of device counts: enqueue the copy, mark it, and
+  // (after more work is enqueued behind it) wait for the mark
+  auto read_mark = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
+    FMM_CUDA_TRY(cudaMemcpyAsync(dst_h, src_d, bytes, cudaMemcpyDeviceToHost, s));
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_read, s));
+    return FMM_OK;
+  };
 
   // Frontier loop: one cooperative launch for all levels; the host reads the
   // list sizes once.  A launch that stops because a buffer is too small is
@@ -837,7 +958,10 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_trav_loop, dim3(G), dim3(kTravThreads), args, 0, s));
     TravState hs;
     FMM_CUDA_TRY(cudaMemcpyAsync(hc, dst, sizeof(TravState), cudaMemcpyDeviceToHost, s));
-    FMM_CUDA_TRY(cudaStreamSynchronize(s));
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_read, s));
+    // the M2L tiles need the tree alone: they run while the host reads the sizes
+    if (launch == 0) FMM_TRY(cell_tiles(p, dmisc, drng, s));
+    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
     memcpy(&hs, hc, sizeof(TravState));
     if (hs.abort) return FMM_E_TIMEOUT;
     if (hs.overflow) {  // grow what was too small (x1.25, contents kept) and resume
@@ -864,244 +988,185 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   p->n_m2l = nm;
   p->n_p2p = np;
 
-  // ---- P2P: group by target leaf
-  {
-    const int n = (int)np;
-    FMM_TRY(p->lk0.ensure((n + 1) * sizeof(uint64_t)));
-    FMM_TRY(p->lk1.ensure((n + 1) * sizeof(uint64_t)));
-    FMM_TRY(p->lv0.ensure((n + 1) * sizeof(uint32_t)));
-    FMM_TRY(p->lv1.ensure((n + 1) * sizeof(uint32_t)));
-    FMM_TRY(p->p2p_sorted.ensure((n + 1) * sizeof(int2)));
-    FMM_TRY(p->p2p_off.ensure((p->nleaves + 1) * sizeof(int2)));
-    unsigned g = (unsigned)((n + T - 1) / T);
+  // ---- M2L: translation keys and their field ranges; the P2P grouping runs
+  // while the host reads the ranges
+  const int n = (int)nm;
+  const unsigned g = (unsigned)((n + T - 1) / T);
+  if (n > 0) {
+    FMM_TRY(p->m2l_key.ensure((size_t)(n + 1) * sizeof(uint64_t)));
     ++g_launches;
-    k_p2p_keys<<<g, T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
-    int second = 0;
-    FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                           p->lv1.as<uint32_t>(), n, 0, bits_for(nc), &second, p->sort_hist, p->scan_tmp, s));
-    uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
-    uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
-    unsigned long long* dpairs = reinterpret_cast<unsigned long long*>(p->scal.as<double>() + kScalCount + 2);
-    FMM_CUDA_TRY(cudaMemsetAsync(dpairs, 0, 2 * sizeof(unsigned long long), s));
-    FMM_TRY(p->p2p_pre.ensure((size_t)(n + 1) * sizeof(uint32_t)));
-    ++g_launches;
-    k_p2p_gather<<<std::min<unsigned>(std::max(g, 1u), 1216u), T, 0, s>>>(
-        p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(), p->p2p_pre.as<uint32_t>(), p->c_begin.as<int>(),
-        p->c_end.as<int>(), p2p_tile(p), dpairs);
-    // the scan wraps past 2^32 sources; differences within a leaf stay exact
-    FMM_TRY(exclusive_scan_u32(p->p2p_pre.as<uint32_t>(), p->p2p_pre.as<uint32_t>(), n, p->p2p_pre.as<uint32_t>() + n,
-                               p->scan_tmp, s));
-    ++g_launches;
-    k_p2p_offsets<<<(unsigned)((p->nleaves + T - 1) / T), T, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, sk, n,
-                                                                     p->p2p_off.as<int2>());
-    FMM_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(p->pinned) + 64, dpairs, 2 * sizeof(unsigned long long),
-                                 cudaMemcpyDeviceToHost, s));
+    k_m2l_keys<<<std::min<unsigned>(g, 2048u), T, 0, s>>>(p->m2l_raw.as<int2>(), n, p->c_level.as<int>(),
+                                                          p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
+                                                          p->flags.as<int>());
   }
-
-  // ---- M2L: keys, unique operators, steps per (tile, key)
-  {
-    const int n = (int)nm;
-    // tiles: at most 64 cells of one (level, octant) group each
-    constexpr int kGroups = (kMaxLevel + 1) * 8;
-    FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
-    FMM_TRY(p->tile_cells.ensure((nc + 1) * sizeof(int)));
-    FMM_TRY(p->tile_groups.ensure(3 * kGroups * sizeof(int)));
-    FMM_TRY(p->lk0.ensure((nc + 1) * sizeof(uint64_t)));
-    FMM_TRY(p->lk1.ensure((nc + 1) * sizeof(uint64_t)));
-    FMM_TRY(p->lv0.ensure((nc + 1) * sizeof(uint32_t)));
-    FMM_TRY(p->lv1.ensure((nc + 1) * sizeof(uint32_t)));
-    {
-      int* gcount = p->tile_groups.as<int>();
-      int* gofs = gcount + kGroups;
-      int* gtile = gofs + kGroups;
-      FMM_CUDA_TRY(cudaMemsetAsync(gcount, 0, kGroups * sizeof(int), s));
-      unsigned gc = (unsigned)((nc + T - 1) / T);
-      ++g_launches;
-      k_tile_order_keys<<<gc, T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc, p->lk0.as<uint64_t>(),
-                                         p->lv0.as<uint32_t>(), gcount);
-      int second = 0;
-      FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), nc, 0, 8, &second, p->sort_hist, p->scan_tmp, s));
-      uint32_t* ord = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
-      int* hg = reinterpret_cast<int*>(reinterpret_cast<char*>(p->pinned) + 1024);  // counts, then offsets
-      FMM_CUDA_TRY(cudaMemcpyAsync(hg, gcount, kGroups * sizeof(int), cudaMemcpyDeviceToHost, s));
-      FMM_CUDA_TRY(cudaStreamSynchronize(s));
-      // the list totals copied above: the work items of the pair kernel
-      const int64_t tile_sources = (int64_t) reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 64)[1];
-      FMM_TRY(p2p_build_items(p, p->last_n, tile_sources, dcnt + 2, s));
-      FMM_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(p->pinned) + 96, dcnt + 2, 2 * sizeof(uint32_t),
-                                   cudaMemcpyDeviceToHost, s));
-      int* hofs = hg + kGroups;
-      int* htile = hofs + kGroups;
-      int cells = 0, tiles = 0;
-      for (int g = 0; g < kGroups; ++g) {
-        hofs[g] = cells;
-        htile[g] = tiles;
-        cells += hg[g];
-        tiles += (hg[g] + kTile - 1) / kTile;
-      }
-      p->ntiles = tiles;
-      FMM_CUDA_TRY(cudaMemcpyAsync(gofs, hofs, 2 * kGroups * sizeof(int), cudaMemcpyHostToDevice, s));
-      FMM_TRY(p->tile_first.ensure((p->ntiles + 1) * sizeof(int)));
-      ++g_launches;
-      k_cell_tiles<<<gc, T, 0, s>>>(nc, (int)p->ntiles, ord, p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs,
-                                    gtile, p->c_tile.as<int>(), p->tile_cells.as<int>(), p->tile_first.as<int>());
+  FMM_CUDA_TRY(cudaMemcpyAsync(hrng, drng, 8 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  FMM_TRY(read_mark(hmisc, dmisc, sizeof(uint32_t)));
+  FMM_TRY(group_p2p(p, (int)np, reinterpret_cast<unsigned long long*>(pin + 64), s));
+  p->n_keys = 0;
+  p->n_steps = 0;
+  p->n_built = 0;
+  // the work items of the pair kernel, once the list totals are on the host
+  auto p2p_items = [&]() -> int {
+    const unsigned long long* tot = reinterpret_cast<unsigned long long*>(pin + 64);
+    p->p2p_pairs = (int64_t)tot[0];
+    FMM_TRY(p2p_build_items(p, p->last_n, (int64_t)tot[1], dmisc + 4, s));
+    return FMM_OK;
+  };
+  auto p2p_counts = [&]() {
+    p->n_p2p_items = hmisc[4];
+    p->n_p2p_slots = hmisc[5];
+  };
+  FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+  p->ntiles = hmisc[0];
+  FMM_TRY(p->tile_range.ensure((p->ntiles + 1) * sizeof(int2)));
+  FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (p->ntiles + 1) * sizeof(int2), s));
+  if (n == 0) {
+    FMM_CUDA_TRY(cudaStreamSynchronize(s));
+    FMM_TRY(p2p_items());
+    FMM_TRY(read_mark(hmisc + 4, dmisc + 4, 2 * sizeof(uint32_t)));
+    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+    p2p_counts();
+  } else {
+    FMM_TRY(p->lv0.ensure((n + 1) * sizeof(uint32_t)));
+    FMM_TRY(p->tcount.ensure((n + 1) * sizeof(uint32_t)));
+    FMM_TRY(p->tscan0.ensure((n + 1) * sizeof(uint32_t)));
+    KeyPack kp;
+    int sh = 0;
+    for (int q = 3; q >= 0; --q) {
+      kp.lo[q] = hrng[2 * q];
+      int range = hrng[2 * q + 1] - hrng[2 * q];
+      int b = 0;
+      while ((1ll << b) <= (long long)range) ++b;
+      kp.shift[q] = sh;
+      kp.width[q] = b;
+      sh += b;
     }
-    FMM_TRY(p->tile_range.ensure((p->ntiles + 1) * sizeof(int2)));
-    FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (p->ntiles + 1) * sizeof(int2), s));
-    p->n_keys = 0;
-    p->n_steps = 0;
-    if (n > 0) {
-      FMM_TRY(p->lk0.ensure((n + 1) * sizeof(uint64_t)));
-      FMM_TRY(p->lk1.ensure((n + 1) * sizeof(uint64_t)));
-      FMM_TRY(p->lv0.ensure((n + 1) * sizeof(uint32_t)));
-      FMM_TRY(p->lv1.ensure((n + 1) * sizeof(uint32_t)));
-      FMM_TRY(p->m2l_key.ensure((n + 1) * sizeof(uint64_t)));
-      FMM_TRY(p->tcount.ensure((n + 1) * sizeof(uint32_t)));
-      FMM_TRY(p->tscan0.ensure((n + 1) * sizeof(uint32_t)));
-      unsigned g = (unsigned)((n + T - 1) / T);
-      int* flag = p->flags.as<int>();
-      // 1. full translation keys and their field ranges
+    kp.bits = sh;
+    int tb = 1;
+    while ((1ll << tb) < (long long)p->ntiles) ++tb;
+    if (tb + kp.bits > 63) return FMM_E_DEPTH;
+    const int64_t K = 1ll << kp.bits;
+    bool binned = false;
+    if (kp.bits <= kBinKeyBits && !(p->prm.m2l_mode & FMM_M2L_SORT_STEPS)) {
+      // the steps from flag tables (no sort) when the tables are small
+      FMM_TRY(p->bin_flag.ensure((size_t)(K + 1) * sizeof(uint32_t)));
+      FMM_TRY(p->bin_scan.ensure((size_t)(K + 1) * sizeof(uint32_t)));
+      uint32_t* kflag = p->bin_flag.as<uint32_t>();
+      uint32_t* kslot = p->bin_scan.as<uint32_t>();
+      FMM_CUDA_TRY(cudaMemsetAsync(kflag, 0, (size_t)K * sizeof(uint32_t), s));
       ++g_launches;
-      FMM_TRY(p->c_ijk.ensure((size_t)(nc + 1) * sizeof(uint64_t)));
-      ++g_launches;
-      k_cell_ijk<<<(unsigned)((nc + T - 1) / T), T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc,
-                                                           p->c_ijk.as<uint64_t>());
-      int* drng = reinterpret_cast<int*>(p->scal.as<double>() + kScalCount + 8);
-      const int init[8] = {INT_MAX, INT_MIN, INT_MAX, INT_MIN, INT_MAX, INT_MIN, INT_MAX, INT_MIN};
-      int* hr = reinterpret_cast<int*>(reinterpret_cast<char*>(p->pinned) + 256);
-      memcpy(hr, init, sizeof(init));
-      FMM_CUDA_TRY(cudaMemcpyAsync(drng, hr, sizeof(init), cudaMemcpyHostToDevice, s));
-      k_m2l_keys<<<std::min<unsigned>(g, 2048u), T, 0, s>>>(p->m2l_raw.as<int2>(), n, p->c_level.as<int>(),
-                                                            p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
-                                                            flag);
-      FMM_CUDA_TRY(cudaMemcpyAsync(hr, drng, sizeof(init), cudaMemcpyDeviceToHost, s));
-      FMM_CUDA_TRY(cudaStreamSynchronize(s));
-      KeyPack kp;
-      int sh = 0;
-      for (int q = 3; q >= 0; --q) {
-        kp.lo[q] = hr[2 * q];
-        int range = hr[2 * q + 1] - hr[2 * q];
-        int b = 0;
-        while ((1ll << b) <= (long long)range) ++b;
-        kp.shift[q] = sh;
-        kp.width[q] = b;
-        sh += b;
-      }
-      kp.bits = sh;
-      int tb = 1;
-      while ((1ll << tb) < (long long)p->ntiles) ++tb;
-      if (tb + kp.bits > 63) return FMM_E_DEPTH;
-      const int64_t K = 1ll << kp.bits;
-      bool binned = false;
-      if (kp.bits <= kBinKeyBits && !(p->prm.m2l_mode & FMM_M2L_SORT_STEPS)) {
-        // 2'. the steps from flag tables (no sort) when the tables are small
-        FMM_TRY(p->bin_flag.ensure((size_t)(K + 1) * sizeof(uint32_t)));
-        FMM_TRY(p->bin_scan.ensure((size_t)(K + 1) * sizeof(uint32_t)));
-        uint32_t* kflag = p->bin_flag.as<uint32_t>();
-        uint32_t* kslot = p->bin_scan.as<uint32_t>();
-        FMM_CUDA_TRY(cudaMemsetAsync(kflag, 0, (size_t)K * sizeof(uint32_t), s));
+      k_key_mark<<<g, T, 0, s>>>(p->m2l_key.as<uint64_t>(), n, kp, kflag);
+      FMM_TRY(exclusive_scan_u32(kflag, kslot, K, dmisc + 1, p->scan_tmp, s));
+      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
+      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      const int64_t nkeys = hmisc[1];
+      const int64_t nb = nkeys * (int64_t)p->ntiles;
+      if (nb <= kBinMax) {
+        binned = true;
+        p->n_keys = nkeys;
+        FMM_TRY(p->ukeys.ensure((size_t)(nkeys + 1) * sizeof(uint64_t)));
         ++g_launches;
-        k_key_mark<<<g, T, 0, s>>>(p->m2l_key.as<uint64_t>(), n, kp, kflag);
-        FMM_TRY(exclusive_scan_u32(kflag, kslot, K, dcnt, p->scan_tmp, s));
-        FMM_CUDA_TRY(cudaMemcpyAsync(hc, dcnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        FMM_CUDA_TRY(cudaStreamSynchronize(s));
-        const int64_t nkeys = hc[0];
-        const int64_t nb = nkeys * (int64_t)p->ntiles;
-        if (nb <= kBinMax) {
-          binned = true;
-          p->n_keys = nkeys;
-          FMM_TRY(p->ukeys.ensure((size_t)(nkeys + 1) * sizeof(uint64_t)));
-          ++g_launches;
-          k_key_unpack<<<(unsigned)((K + T - 1) / T), T, 0, s>>>(kflag, kslot, K, kp, p->ukeys.as<uint64_t>());
-          // the key tables stay live: bins go to bin_flag2 / bin_scan2
-          FMM_TRY(p->bin_flag2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
-          FMM_TRY(p->bin_scan2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
-          uint32_t* bflag = p->bin_flag2.as<uint32_t>();
-          uint32_t* bstep = p->bin_scan2.as<uint32_t>();
-          uint32_t* pbin = p->lv0.as<uint32_t>();
-          FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), s));
-          ++g_launches;
-          k_bin_mark<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
-                                     kslot, (int)nkeys, bflag, pbin);
-          FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dcnt, p->scan_tmp, s));
-          FMM_CUDA_TRY(cudaMemcpyAsync(hc, dcnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-          FMM_CUDA_TRY(cudaStreamSynchronize(s));
-          p->n_steps = hc[0];
-          const int64_t ns = p->n_steps;
-          FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
-          FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
-          FMM_TRY(p->st_src.ensure((ns + 1) * kTile * sizeof(int)));
-          FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * kTile * sizeof(int), s));
-          ++g_launches;
-          k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, s>>>(bflag, bstep, nb, (int)nkeys, p->st_tile.as<int>(),
-                                                                 p->st_slot.as<int>());
-          ++g_launches;
-          k_bin_fill<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(),
-                                     p->st_src.as<int>());
-          ++g_launches;
-          k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns,
-                                                                  p->tile_range.as<int2>());
-          FMM_CUDA_TRY(cudaGetLastError());
-        }
-      }
-      if (!binned) {
-        // 2. sort pairs by (tile, compact key): consecutive runs are the steps
+        k_key_unpack<<<(unsigned)((K + T - 1) / T), T, 0, s>>>(kflag, kslot, K, kp, p->ukeys.as<uint64_t>());
+        uint32_t* miss = p->tcount.as<uint32_t>();
+        uint32_t* rank = p->tscan0.as<uint32_t>();
+        FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, s));
+        // the key tables stay live: bins go to bin_flag2 / bin_scan2
+        FMM_TRY(p->bin_flag2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
+        FMM_TRY(p->bin_scan2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
+        uint32_t* bflag = p->bin_flag2.as<uint32_t>();
+        uint32_t* bstep = p->bin_scan2.as<uint32_t>();
+        uint32_t* pbin = p->lv0.as<uint32_t>();
+        FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), s));
         ++g_launches;
-        k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
-                                     p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
-        int second = 0;
-        FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                               p->lv1.as<uint32_t>(), n, 0, tb + kp.bits, &second, p->sort_hist, p->scan_tmp, s));
-        uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
-        uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
-        ++g_launches;
-        k_step_flags<<<g, T, 0, s>>>(sk, n, p->tcount.as<uint32_t>());
-        FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dcnt, p->scan_tmp, s));
-        FMM_CUDA_TRY(cudaMemcpyAsync(hc, dcnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        FMM_CUDA_TRY(cudaStreamSynchronize(s));
-        p->n_steps = hc[0];
+        k_bin_mark<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
+                                   kslot, (int)nkeys, bflag, pbin);
+        FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, s));
+        FMM_TRY(p2p_items());
+        FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 4 * sizeof(uint32_t)));
+        FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+        p2p_counts();
+        p->n_steps = hmisc[2];
         const int64_t ns = p->n_steps;
         FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_src.ensure((ns + 1) * kTile * sizeof(int)));
-        FMM_TRY(p->st_ckey.ensure((ns + 1) * sizeof(uint64_t)));
-        FMM_TRY(p->st_fkey.ensure((ns + 1) * sizeof(uint64_t)));
+        FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, s));
         FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * kTile * sizeof(int), s));
         ++g_launches;
-        k_step_write2<<<g, T, 0, s>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
-                                      p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), kp.bits,
-                                      p->st_tile.as<int>(),
-                                      p->st_ckey.as<uint64_t>(), p->st_fkey.as<uint64_t>(), p->st_src.as<int>());
+        k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, s>>>(bflag, bstep, nb, (int)nkeys, p->tslot_map.as<int>(),
+                                                               p->st_tile.as<int>(), p->st_slot.as<int>());
         ++g_launches;
-        k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns, p->tile_range.as<int2>());
-        // 3. distinct translations among the steps -> operator slots
-        FMM_TRY(p->ukeys.ensure((ns + 1) * sizeof(uint64_t)));
-        unsigned gs = (unsigned)((ns + T - 1) / T);
+        k_bin_fill<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(), p->st_src.as<int>());
         ++g_launches;
-        k_copy_u64_iota<<<gs, T, 0, s>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
-        FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                               p->lv1.as<uint32_t>(), ns, 0, std::max(kp.bits, 1), &second, p->sort_hist, p->scan_tmp,
-                               s));
-        sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
-        sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
-        ++g_launches;
-        k_unique_flags<<<gs, T, 0, s>>>(sk, (int)ns, p->tcount.as<uint32_t>());
-        FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dcnt, p->scan_tmp, s));
-        ++g_launches;
-        k_step_slots<<<gs, T, 0, s>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
-                                      p->st_fkey.as<uint64_t>(), p->ukeys.as<uint64_t>(), p->st_slot.as<int>());
-        FMM_CUDA_TRY(cudaMemcpyAsync(hc, dcnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        FMM_CUDA_TRY(cudaStreamSynchronize(s));
-        p->n_keys = hc[0];
+        k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns,
+                                                                p->tile_range.as<int2>());
         FMM_CUDA_TRY(cudaGetLastError());
       }
     }
+    if (!binned) {
+      FMM_TRY(p->lk0.ensure((n + 1) * sizeof(uint64_t)));
+      FMM_TRY(p->lk1.ensure((n + 1) * sizeof(uint64_t)));
+      FMM_TRY(p->lv1.ensure((n + 1) * sizeof(uint32_t)));
+      // sort pairs by (tile, compact key): consecutive runs are the steps
+      ++g_launches;
+      k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
+                                   p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+      int second = 0;
+      FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                             p->lv1.as<uint32_t>(), n, 0, tb + kp.bits, &second, p->sort_hist, p->scan_tmp, s));
+      uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
+      uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
+      ++g_launches;
+      k_step_flags<<<g, T, 0, s>>>(sk, n, p->tcount.as<uint32_t>());
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, s));
+      FMM_TRY(read_mark(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
+      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      p->n_steps = hmisc[2];
+      const int64_t ns = p->n_steps;
+      FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
+      FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
+      FMM_TRY(p->st_src.ensure((ns + 1) * kTile * sizeof(int)));
+      FMM_TRY(p->st_ckey.ensure((ns + 1) * sizeof(uint64_t)));
+      FMM_TRY(p->st_fkey.ensure((ns + 1) * sizeof(uint64_t)));
+      FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * kTile * sizeof(int), s));
+      ++g_launches;
+      k_step_write2<<<g, T, 0, s>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
+                                    p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), kp.bits,
+                                    p->st_tile.as<int>(),
+                                    p->st_ckey.as<uint64_t>(), p->st_fkey.as<uint64_t>(), p->st_src.as<int>());
+      ++g_launches;
+      k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns, p->tile_range.as<int2>());
+      // distinct translations among the steps -> operator slots
+      FMM_TRY(p->ukeys.ensure((ns + 1) * sizeof(uint64_t)));
+      unsigned gs = (unsigned)((ns + T - 1) / T);
+      ++g_launches;
+      k_copy_u64_iota<<<gs, T, 0, s>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+      FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                             p->lv1.as<uint32_t>(), ns, 0, std::max(kp.bits, 1), &second, p->sort_hist, p->scan_tmp,
+                             s));
+      sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
+      sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
+      ++g_launches;
+      k_unique_flags<<<gs, T, 0, s>>>(sk, (int)ns, p->tcount.as<uint32_t>());
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dmisc + 1, p->scan_tmp, s));
+      ++g_launches;
+      k_step_slots<<<gs, T, 0, s>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
+                                    p->st_fkey.as<uint64_t>(), p->ukeys.as<uint64_t>(), p->st_slot.as<int>());
+      FMM_TRY(p2p_items());
+      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, 5 * sizeof(uint32_t)));
+      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      p2p_counts();
+      p->n_keys = hmisc[1];
+      uint32_t* miss = p->tcount.as<uint32_t>();
+      uint32_t* rank = p->tscan0.as<uint32_t>();
+      FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, s));
+      FMM_TRY(read_mark(hmisc + 3, dmisc + 3, sizeof(uint32_t)));
+      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, s));
+      FMM_TRY(remap_step_slots(p, s));
+      FMM_CUDA_TRY(cudaGetLastError());
+    }
   }
-  FMM_CUDA_TRY(cudaStreamSynchronize(s));
-  p->p2p_pairs = (int64_t) * reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 64);
-  p->n_p2p_items = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(p->pinned) + 96)[0];
-  p->n_p2p_slots = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(p->pinned) + 96)[1];
   return FMM_OK;
 }
 
