@@ -35,12 +35,12 @@ int check_params(const fmm_params* q) {
 
 std::vector<DBuf*> plan_buffers(fmm_plan p) {
   return {&p->m2m_T, &p->l2l_T, &p->l2p_tab, &p->lattice, &p->keys0, &p->keys1, &p->vals0, &p->vals1,
-          &p->sortA, &p->sortB, &p->far_u, &p->far_s, &p->leaf_of, &p->in_pos, &p->in_gam, &p->in_sig,
+          &p->sortA, &p->sortB, &p->far_u, &p->far_s, &p->c_clo, &p->tree_state, &p->in_pos, &p->in_gam, &p->in_sig,
           &p->out_vel, &p->out_dg, &p->c_begin, &p->c_end, &p->c_level, &p->c_parent, &p->c_child,
           &p->c_nchild, &p->c_key, &p->c_center, &p->c_radius2, &p->c_radius, &p->dip_part, &p->c_cf, &p->c_tile,
           &p->tile_cells, &p->tile_first, &p->tile_groups, &p->c_ijk, &p->t_pos, &p->t_gam, &p->t_sig, &p->t_vel, &p->leaves, &p->M, &p->L, &p->Mbf, &p->fr0, &p->fr1, &p->tcount, &p->tmask,
           &p->tscan0, &p->tscan1, &p->tscan2, &p->p2p_raw, &p->m2l_raw, &p->lk0, &p->lk1, &p->lv0, &p->lv1,
-          &p->p2p_sorted, &p->p2p_off, &p->p2p_pre, &p->p2p_items, &p->p2p_islot, &p->p2p_plan, &p->p2p_partial, &p->p2p_sigk, &p->m2l_key, &p->m2l_slot, &p->ukeys, &p->T32, &p->Tbf,
+          &p->p2p_sorted, &p->p2p_off, &p->p2p_pre, &p->p2p_items, &p->p2p_islot, &p->p2p_plan, &p->p2p_bar, &p->p2p_partial, &p->p2p_sigk, &p->m2l_key, &p->m2l_slot, &p->ukeys, &p->T32, &p->Tbf,
           &p->tc_key, &p->tc_slot, &p->tmiss_keys, &p->tmiss_slots, &p->tslot_map, &p->st_tile, &p->st_slot, &p->st_src, &p->bin_flag, &p->bin_scan, &p->bin_flag2, &p->bin_scan2, &p->st_ckey,
           &p->st_fkey, &p->m2l_items, &p->m2l_partial, &p->tile_range, &p->scan_tmp, &p->sort_hist, &p->scal,
           &p->flags, &p->seg_off, &p->seg_box, &p->seg_sig, &p->seg_smax, &p->seg_mac, &p->seg_p2p, &p->c_seg};
@@ -86,6 +86,7 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
   const int m2l_kind = p->prm.m2l_mode & 3;
   p->last_tc = (m2l_kind == FMM_M2L_SIMT) ? 0 : p->tc_ok;
   if ((m2l_kind == FMM_M2L_TENSOR || m2l_kind == FMM_M2L_TENSOR_TF32) && !p->tc_ok) return FMM_E_INVAL;
+  FMM_TRY(ensure_aux_stream(p));
   Timer tm{p, s};
   tm.mark();
   if (sg) FMM_TRY(build_forest(p, n, pos, gam, sig, *sg, s));
@@ -93,7 +94,6 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
   tm.mark();
   // Fork: P2M / M2M on the plan's second stream while the traversal (which
   // reads only the tree) runs on the caller's stream; join before M2L.
-  FMM_TRY(ensure_aux_stream(p));
   FMM_CUDA_TRY(cudaEventRecord(p->ev_fork, s));
   FMM_CUDA_TRY(cudaStreamWaitEvent(p->s_up, p->ev_fork, 0));
   {
@@ -252,7 +252,7 @@ int fmm_plan_create(const fmm_params* prm, int64_t n_max, fmm_plan* out) {
     if ((rc = build_constant_operators(p)) != FMM_OK) break;
     if ((rc = p->keys0.ensure(nn * 8)) || (rc = p->keys1.ensure(nn * 8)) || (rc = p->vals0.ensure(nn * 4)) ||
         (rc = p->vals1.ensure(nn * 4)) || (rc = p->sortA.ensure(nn * 16)) || (rc = p->sortB.ensure(nn * 16)) ||
-        (rc = p->leaf_of.ensure(nn * 4)) || (rc = p->scal.ensure(64 * sizeof(double))) ||
+        (rc = p->scal.ensure(64 * sizeof(double))) ||
         (rc = p->flags.ensure(16 * sizeof(int))))
       break;
     if (cudaMallocHost(&p->pinned, 4096) != cudaSuccess) {

@@ -104,7 +104,8 @@ struct fmm_plan_s {
   uint32_t* sidx = nullptr;              // sorted position -> input index
   fmm::DBuf sortA, sortB;                // float4 (x,y,z,sigma), (gx,gy,gz,0) in sorted order
   fmm::DBuf far_u, far_s;                // [n][3] far field, sorted order
-  fmm::DBuf leaf_of;                     // [n]
+  fmm::DBuf c_clo;                       // float4 low part of the centre, then u32 FP32 squared radius
+  fmm::DBuf tree_state;                  // state and block totals of the octree kernel
   fmm::DBuf in_pos, in_gam, in_sig, out_vel, out_dg;  // staging of the _host entry point
   fmm::DBuf t_pos, t_gam, t_sig, t_vel;                // sources + zero-strength targets (fmm_eval_targets)
   // cells
@@ -128,7 +129,7 @@ struct fmm_plan_s {
   fmm::DBuf p2p_sorted, p2p_off;                      // int2 (first source, image) by leaf, CSR offsets per leaf
   fmm::DBuf p2p_pre;                                  // u32 scanned source counts of the list entries
   fmm::DBuf p2p_items, p2p_islot, p2p_plan;           // pair kernel work items, their partial slots, per-leaf split
-  fmm::DBuf p2p_partial, p2p_sigk;                    // partial sums of split lists; per-particle core constants
+  fmm::DBuf p2p_bar, p2p_partial, p2p_sigk;                    // partial sums of split lists; per-particle core constants
   fmm::DBuf m2l_key, m2l_slot, ukeys;                 // per pair key, slot; unique keys
   fmm::DBuf T32, Tbf;                                 // M2L operator cache [slot]: FP32, BF16 hi/lo
   fmm::DBuf tc_key, tc_slot;                          // operator cache: open-addressing table key -> slot
@@ -147,6 +148,7 @@ struct fmm_plan_s {
   void* pinned = nullptr;  // host pinned scratch (counts)
   // host mirror of the last tree / lists
   std::vector<int> level_begin;  // cells of level l: [level_begin[l], level_begin[l+1])
+  int64_t cell_cap = 0;          // cells the arrays were asked to hold
   int64_t ncells = 0, nleaves = 0, ntiles = 0;
   int nlevels = 0;
   double cf_margin = 0.0;  // rounding margin of the FP32 cell copies (2e-6 x largest coordinate)

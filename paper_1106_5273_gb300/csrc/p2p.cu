@@ -815,104 +815,123 @@ struct RangeRule {
 // ---- work items: per leaf, tiles x ranges, the longest ranges first (four
 // length classes, leaf order within each), so that the last warps to start
 // are short: in leaf order the batch of 32 problems waited for its longest
-// lists (P2P 5.56 ms, now 5.23).  One CTA walks the leaves twice: the class
-// totals, then the scan.  counts[0] = items, counts[1] = partial slots.
-constexpr int kItemClasses = 4;
+// lists (P2P 5.56 ms, now 5.23).  One cooperative launch: the blocks own
+// contiguous ranges of the leaves, take their class totals, meet at a bounded
+// grid barrier and write (one CTA over all leaves took 153 us at Taylor-Green
+// 128^3).  counts[0] = items, counts[1] = partial slots.
+constexpr int kItemClasses = 4, kItemThreads = 256, kItemBlocks = 128;
 
-__global__ void __launch_bounds__(1024) k_p2p_items(const int* __restrict__ leaves, int nl,
-                                                    const int* __restrict__ begin, const int* __restrict__ end,
-                                                    const int2* __restrict__ off, const uint32_t* __restrict__ epre,
-                                                    int tile, RangeRule rr, int4* __restrict__ items,
-                                                    int* __restrict__ islot, int2* __restrict__ plan,
-                                                    uint32_t* __restrict__ counts) {
+__global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restrict__ leaves, int nl,
+                                                            const int* __restrict__ begin,
+                                                            const int* __restrict__ end,
+                                                            const int2* __restrict__ off,
+                                                            const uint32_t* __restrict__ epre, int tile, RangeRule rr,
+                                                            int4* __restrict__ items, int* __restrict__ islot,
+                                                            int2* __restrict__ plan, uint32_t* __restrict__ counts,
+                                                            uint32_t* blk, GridBar* bar) {
   constexpr int NC = kItemClasses + 1;  // item classes, then partial slots
-  __shared__ uint32_t ws[NC][32];
+  __shared__ uint32_t ws[NC][kItemThreads / 32];
   __shared__ uint32_t carry[NC];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x < NC) carry[threadIdx.x] = 0u;
-  __syncthreads();
-  constexpr int R = 4;  // leaves per thread and round (independent loads in flight)
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int c0 = 0; c0 < nl; c0 += 1024 * R) {
-      const int i0 = c0 + threadIdx.x * R;
-      uint32_t nit[R], nsp[R], F[R];
-      int cls[R];
-      uint32_t own[NC] = {0u, 0u, 0u, 0u, 0u}, inc[NC];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        nit[r] = nsp[r] = F[r] = 0;
-        cls[r] = kItemClasses - 1;
-        if (i0 + r < nl) {
-          const int leaf = leaves[i0 + r];
-          const int2 rg = off[i0 + r];
-          F[r] = epre[rg.y] - epre[rg.x];
-          nsp[r] = F[r] <= rr.whole ? 1u : min(rr.cap, (F[r] + rr.range - 1) / rr.range);
-          nit[r] = nsp[r] * (uint32_t)((end[leaf] - begin[leaf] + tile - 1) / tile);
-          const uint32_t len = F[r] / nsp[r];
-          cls[r] = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
-        }
-#pragma unroll
-        for (int q = 0; q < NC; ++q) own[q] += (q < kItemClasses ? q == cls[r] : nsp[r] > 1) ? nit[r] : 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        inc[q] = own[q];
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, inc[q], o);
-          if (lane >= o) inc[q] += y;
-        }
-        if (lane == 31) ws[q][w] = inc[q];
-      }
-      __syncthreads();
-      if (w < NC) {  // warp w scans the warp totals of count w
-        uint32_t v = ws[w][lane], x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-          if (lane >= o) x += y;
-        }
-        const uint32_t c = carry[w];
-        ws[w][lane] = c + x - v;
-        if (lane == 31) carry[w] = c + x;
-      }
-      __syncthreads();
-      if (pass == 1) {
-        uint32_t at[NC];
-#pragma unroll
-        for (int q = 0; q < NC; ++q) at[q] = ws[q][w] + inc[q] - own[q];
-        for (int r = 0; r < R && i0 + r < nl; ++r) {
-          const int leaf = leaves[i0 + r], tb = begin[leaf], te = end[leaf];
-          uint32_t io = 0, slot = at[kItemClasses];
-#pragma unroll
-          for (int q = 0; q < kItemClasses; ++q)
-            if (q == cls[r]) {
-              io = at[q];
-              at[q] += nit[r];
-            }
-          if (nsp[r] > 1) at[kItemClasses] += nit[r];
-          plan[i0 + r] = make_int2((int)slot, (int)nsp[r]);
-          // equal ranges, so that no range is a short remainder
-          const uint32_t len = (F[r] + nsp[r] - 1) / nsp[r];
-          for (int t0 = tb; t0 < te; t0 += tile)
-            for (uint32_t k = 0; k < nsp[r]; ++k, ++io, ++slot) {
-              items[io] = make_int4(i0 + r, t0, (int)min(F[r], k * len), (int)min(F[r], (k + 1) * len));
-              islot[io] = nsp[r] > 1 ? (int)slot : -1;
-            }
-        }
-      }
-      __syncthreads();
+  const int G = (int)gridDim.x, b = (int)blockIdx.x;
+  const int chunk = (nl + G - 1) / G, l0 = min(nl, b * chunk), l1 = min(nl, l0 + chunk);
+  struct Leaf {
+    uint32_t nit, nsp, F;
+    int cls, tb, te;
+  };
+  auto read = [&](int i) {
+    Leaf q{0u, 0u, 0u, kItemClasses - 1, 0, 0};
+    if (i < l1) {
+      const int leaf = leaves[i];
+      const int2 rg = off[i];
+      q.tb = begin[leaf];
+      q.te = end[leaf];
+      q.F = epre[rg.y] - epre[rg.x];
+      q.nsp = q.F <= rr.whole ? 1u : min(rr.cap, (q.F + rr.range - 1) / rr.range);
+      q.nit = q.nsp * (uint32_t)((q.te - q.tb + tile - 1) / tile);
+      const uint32_t len = q.F / q.nsp;
+      q.cls = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
     }
-    if (threadIdx.x == 0) {
-      if (pass == 0) {  // the classes' first items
-        uint32_t acc = 0;
-        for (int q = 0; q < kItemClasses; ++q) {
-          const uint32_t c = carry[q];
-          carry[q] = acc;
-          acc += c;
-        }
-        counts[0] = acc;
-        counts[1] = carry[kItemClasses];
-        carry[kItemClasses] = 0u;
+    return q;
+  };
+  uint32_t sum[NC] = {0u, 0u, 0u, 0u, 0u};
+  for (int i = l0 + threadIdx.x; i < l1; i += kItemThreads) {
+    const Leaf q = read(i);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) sum[k] += (k < kItemClasses ? k == q.cls : q.nsp > 1) ? q.nit : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+    if (lane == 0) ws[k][w] = sum[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < NC) {
+    uint32_t x = 0;
+    for (int i = 0; i < kItemThreads / 32; ++i) x += ws[threadIdx.x][i];
+    blk[b * NC + threadIdx.x] = x;
+  }
+  if (!grid_barrier(bar, (unsigned)G)) return;
+  if (threadIdx.x < NC) {  // this block's first item of each class, and its first slot
+    uint32_t pre = 0, all = 0;
+    for (int j = 0; j < G; ++j) {
+      const uint32_t x = ((volatile uint32_t*)blk)[j * NC + threadIdx.x];
+      if (j < b) pre += x;
+      all += x;
+    }
+    carry[threadIdx.x] = pre;
+    ws[threadIdx.x][0] = all;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t acc = 0;
+    for (int k = 0; k < kItemClasses; ++k) {
+      carry[k] += acc;
+      acc += ws[k][0];
+    }
+    if (b == 0) {
+      counts[0] = acc;
+      counts[1] = ws[kItemClasses][0];
+    }
+  }
+  __syncthreads();
+  for (int c0 = l0; c0 < l1; c0 += kItemThreads) {
+    const int i = c0 + threadIdx.x;
+    const Leaf q = read(i);
+    uint32_t at[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const uint32_t own = (k < kItemClasses ? k == q.cls : q.nsp > 1) ? q.nit : 0u;
+      uint32_t inc = own;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
       }
+      if (lane == 31) ws[k][w] = inc;
+      at[k] = inc - own;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      at[k] += carry[k];
+      for (int j = 0; j < w; ++j) at[k] += ws[k][j];
+    }
+    __syncthreads();
+    if (threadIdx.x < NC)
+      for (int j = 0; j < kItemThreads / 32; ++j) carry[threadIdx.x] += ws[threadIdx.x][j];
+    if (i < l1) {
+      uint32_t io = 0, slot = at[kItemClasses];
+#pragma unroll
+      for (int k = 0; k < kItemClasses; ++k)
+        if (k == q.cls) io = at[k];
+      plan[i] = make_int2((int)slot, (int)q.nsp);
+      // equal ranges, so that no range is a short remainder
+      const uint32_t len = (q.F + q.nsp - 1) / q.nsp;
+      for (int t0 = q.tb; t0 < q.te; t0 += tile)
+        for (uint32_t k = 0; k < q.nsp; ++k, ++io, ++slot) {
+          items[io] = make_int4(i, t0, (int)min(q.F, k * len), (int)min(q.F, (k + 1) * len));
+          islot[io] = q.nsp > 1 ? (int)slot : -1;
+        }
     }
     __syncthreads();
   }
@@ -1210,10 +1229,23 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* count
   FMM_TRY(p->p2p_items.ensure((size_t)items * sizeof(int4)));
   FMM_TRY(p->p2p_islot.ensure((size_t)items * sizeof(int)));
   FMM_TRY(p->p2p_plan.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
+  FMM_TRY(p->p2p_bar.ensure(sizeof(GridBar) + (size_t)kItemBlocks * (kItemClasses + 1) * sizeof(uint32_t)));
+  GridBar* bar = p->p2p_bar.as<GridBar>();
+  uint32_t* blk = reinterpret_cast<uint32_t*>(bar + 1);
+  FMM_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar), s));
+  const int* leaves = p->leaves.as<int>();
+  const int* cb = p->c_begin.as<int>();
+  const int* ce = p->c_end.as<int>();
+  const int2* off = p->p2p_off.as<int2>();
+  const uint32_t* pre = p->p2p_pre.as<uint32_t>();
+  int4* it = p->p2p_items.as<int4>();
+  int* is = p->p2p_islot.as<int>();
+  int2* plan = p->p2p_plan.as<int2>();
+  int nl = (int)p->nleaves, tl = tile;
+  const unsigned G = (unsigned)std::min<int64_t>(kItemBlocks, (nl + kItemThreads - 1) / kItemThreads);
+  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &rr, &it, &is, &plan, &counts, &blk, &bar};
   ++g_launches;
-  k_p2p_items<<<1, 1024, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, p->c_begin.as<int>(), p->c_end.as<int>(),
-                                 p->p2p_off.as<int2>(), p->p2p_pre.as<uint32_t>(), tile, rr,
-                                 p->p2p_items.as<int4>(), p->p2p_islot.as<int>(), p->p2p_plan.as<int2>(), counts);
+  FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_p2p_items, dim3(G), dim3(kItemThreads), args, 0, s));
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }

@@ -171,39 +171,11 @@ __device__ inline void split_of(const TravArgs& t, int a, int b, bool& split_a, 
 
 constexpr int kTravThreads = 256;
 constexpr int kTravMaxIter = 128;         // > 2 x the 22 levels a pair can descend
-constexpr long long kGridSpin = 1ll << 24;
 
-// state[]: 0 nm, 1 np, 2 nf, 3 overflow, 4 need_m, 5 need_p, 6 need_f, 7 iterations,
-// 8 barrier arrivals, 9 barrier generation, 10 abort
 struct TravState {
-  uint32_t nm, np, nf, cur_b, overflow, need_m, need_p, need_f, iters, bar_count, bar_gen, abort;
+  uint32_t nm, np, nf, cur_b, overflow, need_m, need_p, need_f, iters;
+  GridBar bar;
 };
-
-__device__ bool grid_barrier(TravState* st, unsigned nblocks) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile uint32_t* gen = &st->bar_gen;
-    volatile uint32_t* ab = &st->abort;
-    const uint32_t g = *gen;
-    __threadfence();
-    if (atomicAdd(&st->bar_count, 1u) == nblocks - 1) {
-      atomicExch(&st->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&st->bar_gen, 1u);
-    } else {
-      for (long long i = 0; *gen == g; ++i) {
-        if (*ab) break;
-        if (i > kGridSpin) {
-          atomicExch(&st->abort, 1u);
-          break;
-        }
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ((volatile uint32_t*)&st->abort)[0] == 0u;
-}
 
 // Exclusive block scan of three counts (thread order); returns the block totals.
 __device__ inline void block_scan3(uint32_t v[3], uint32_t tot[3]) {
@@ -283,7 +255,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
         blk[3 * b + threadIdx.x] = x;
       }
     }
-    if (!grid_barrier(st, G)) return;
+    if (!grid_barrier(&st->bar, G)) return;
     // offsets of this block (sum of the earlier blocks) and the level totals
     if (threadIdx.x < 6) bases[threadIdx.x] = 0u;
     __syncthreads();
@@ -354,7 +326,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
     int4* sw = cur;
     cur = nxt;
     nxt = sw;
-    if (!grid_barrier(st, G)) return;
+    if (!grid_barrier(&st->bar, G)) return;
   }
   if (b == 0 && threadIdx.x == 0) {  // where the lists stand (and, if stopped, where to resume)
     st->nm = nm;
@@ -928,7 +900,9 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trav_loop, kTravThreads, 0));
     grid_blocks[dev] = std::max(1, sms * std::min(per_sm, 4));
   }
-  const unsigned G = (unsigned)grid_blocks[dev];
+  // few blocks for a small tree: a barrier of the whole chip costs more than
+  // its frontier (1000 blobs, 68 cells: traversal 0.27 -> 0.25 ms)
+  const unsigned G = (unsigned)std::min<int64_t>(grid_blocks[dev], std::max<int64_t>(16, nc / 8));
   FMM_TRY(p->fr0.ensure(cap_fr * sizeof(int4)));
   FMM_TRY(p->fr1.ensure(cap_fr * sizeof(int4)));
   FMM_TRY(p->m2l_raw.ensure(cap_m * sizeof(int2)));
@@ -963,7 +937,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     if (launch == 0) FMM_TRY(cell_tiles(p, dmisc, drng, s));
     FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
     memcpy(&hs, hc, sizeof(TravState));
-    if (hs.abort) return FMM_E_TIMEOUT;
+    if (hs.bar.abort) return FMM_E_TIMEOUT;
     if (hs.overflow) {  // grow what was too small (x1.25, contents kept) and resume
       if ((int64_t)hs.need_m > cap_m) cap_m = (int64_t)hs.need_m + hs.need_m / 4 + 1024;
       if ((int64_t)hs.need_p > cap_p) cap_p = (int64_t)hs.need_p + hs.need_p / 4 + 1024;
