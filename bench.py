@@ -166,12 +166,20 @@ def p2p_roofline(st, p2p_ms, traffic=None):
                          "maximum clock)"}
 
 
-def m2l_roofline(st, p):
+def m2l_mma_cols(p):
+    """Columns of the tensor-core M2L's MMAs: 192 (64 cells x 3 components) with the operator's
+    rows as MMA rows (64 < P <= 128), else P rounded up to 16 with 42 cells x 3 as the 128 rows."""
+    P = int(p) ** 2
+    return 192 if 64 < P <= 128 else (P + 15) // 16 * 16
+
+
+def m2l_roofline(st, p, mma_cols=None):
     """Tensor roofline of the M2L phase: the products issued per M2L pair are
     2 P x 3 components x (3 K3 + (P - K3)), K3 = the source coefficients that take
     all three split products (the rest take hi x hi only); peak = the dense BF16 rate.
-    `issued` counts what the tensor pipe executes instead: every MMA of 128 rows x 192
-    columns x 16 (BF16 path), padding rows above P and empty tile slots included."""
+    `issued` counts what the tensor pipe executes instead: every MMA of 128 rows x
+    mma_cols columns x 16 (BF16 path), padding and empty tile slots included; without
+    mma_cols, of 128 operator rows x 192 columns with one block of rows per 128 of P."""
     P = int(p) ** 2
     if not (st.ms_m2l > 0 and st.m2l_tensor):
         return None
@@ -184,10 +192,12 @@ def m2l_roofline(st, p):
     if k3 % 16 == 0 or k3 == P:  # BF16 path: K steps of 16
         ks = (P + 15) // 16
         k3s = min(ks, (k3 + 15) // 16)
-        mmas = (3 * k3s + (ks - k3s)) * ((P + 127) // 128)
-        iss = 2.0 * 128 * 192 * 16 * mmas * st.m2l_steps / (st.ms_m2l * 1e-3) / 1e12
+        mmas = 3 * k3s + (ks - k3s)
+        if mma_cols is None:
+            mma_cols, mmas = 192, mmas * ((P + 127) // 128)
+        iss = 2.0 * 128 * mma_cols * 16 * mmas * st.m2l_steps / (st.ms_m2l * 1e-3) / 1e12
         out["issued"] = {"achieved": iss, "frac": iss / peak, "mmas_per_step": mmas,
-                         "what": "2 x 128 x 192 x 16 per MMA x MMAs per step x steps"}
+                         "what": "2 x 128 x %d x 16 per MMA x MMAs per step x steps" % mma_cols}
     return out
 
 
@@ -632,7 +642,7 @@ def run_config3(args, steps=3, warmup=1):
            "phases_ms": {k: float(np.mean([getattr(x, k) for x in sts])) for k in PHASES},
            "work": {k: getattr(st, k) for k in WORK},
            "roofline": p2p_roofline(st, float(np.mean([x.ms_p2p for x in sts]))),
-           "roofline_m2l": m2l_roofline(st, 10),
+           "roofline_m2l": m2l_roofline(st, 10, m2l_mma_cols(10)),
            "accuracy": {"rel_l2_u": eu, "rel_l2_s": es, "targets": 4096,
                         "reference": "exact blob field of the generating Fourier modes (oracle)"},
            "device_bytes": plan.device_bytes(), "input_generation_s": gen_s, "clocks": clk,
@@ -766,7 +776,7 @@ def main():
                               "ms_per_launch": probe_ms, "clocks": pc,
                               "what": "fmm_probe_fp32_rate: independent FFMA2 chains, 8 CTAs x 256 threads per SM, "
                                       "1000 launches timed with CUDA events"}
-    roof_m2l = m2l_roofline(st, w["p"])
+    roof_m2l = m2l_roofline(st, w["p"], m2l_mma_cols(w["p"]))
     reuse = None
     if rank == 0 and not args.no_reuse:
         reuse = run_tree_reuse(plan, pos, gam, sig, vel, dg, flush, stream, max(3, args.steps // 2), w)

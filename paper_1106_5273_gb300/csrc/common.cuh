@@ -17,7 +17,9 @@ extern std::atomic<int64_t> g_launches;
 constexpr int kMaxLevel = 21;      // 63-bit Morton keys, 3 bits per level (Sec. 3.2)
 constexpr int kPMax = 16;          // expansion degrees 0..15
 constexpr int kNCoefMax = kPMax * kPMax;
-constexpr int kTile = 64;          // target cells per M2L tile
+constexpr int kTileCells = 42;     // target cells per M2L tile, cells as MMA rows (3 components each: 126 of 128)
+constexpr int kTileRows = 64;      // ... and with the operator's rows as MMA rows (192 columns)
+constexpr int kKeyBuckets = 8;     // groups of translations a batch's M2L tile is split into
 constexpr int kImageZero = 13;     // image index of the zero shift, (ox+1)*9+(oy+1)*3+(oz+1)
 
 #define FMM_CUDA_TRY(expr)                         \

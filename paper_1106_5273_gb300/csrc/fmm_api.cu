@@ -128,6 +128,7 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
     smax = (double)f;
   }
   FMM_TRY(traverse(p, smax, s));
+  FMM_TRY(m2l_build_items(p, s));
   tm.mark();
   FMM_CUDA_TRY(cudaStreamWaitEvent(s, p->ev_join, 0));
   join_guard.joined = true;

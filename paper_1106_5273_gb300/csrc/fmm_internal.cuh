@@ -208,6 +208,7 @@ int traverse(fmm_plan p, double sigma_max_host, cudaStream_t s);
 int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s);
 // m2l.cu
 int m2l_simt(fmm_plan p, cudaStream_t s);
+int m2l_build_items(fmm_plan p, cudaStream_t s);  // once per tree
 int m2l_tensor(fmm_plan p, cudaStream_t s);
 // downward.cu
 int downward_pass(fmm_plan p, int64_t n, cudaStream_t s);
@@ -274,8 +275,17 @@ __host__ __device__ inline int m2l_split_chunks(int P, int kind, float theta, bo
   const float t2 = theta * theta, t8 = t2 * t2 * t2 * t2;
   return (kind == 0 && !full && t8 <= 1.0f / 1024.0f) ? 1 : nkc;
 }
-// Blocks of 128 output rows (one MMA M) covering P outputs.
-__host__ __device__ inline int m2l_rowblocks(int P) { return (P + 127) / 128; }
+// Output coefficients padded to the columns of an MMA (N a multiple of 16).
+__host__ __device__ inline int m2l_cols(int P) { return (P + 15) & ~15; }
+// Target cells per M2L tile.  With 64 < P <= 128 the operator's P rows are the
+// MMA's 128 rows (64 cells x 3 components as columns); otherwise the cells are
+// the rows and the P coefficients the columns, which fits any P (both forms
+// measured: m2l_tc.cu).
+__host__ __device__ inline int m2l_tile(int P) { return P > 64 && P <= 128 ? kTileRows : kTileCells; }
+// Bucket of a translation: a hash of its key, so that it depends on nothing else.
+__host__ __device__ inline int m2l_bucket(uint64_t key) {
+  return (int)((key * 0x9E3779B97F4A7C15ull) >> 61) & (kKeyBuckets - 1);
+}
 
 // Level / tile layout of the current tree, passed to kernels by value.
 }  // namespace fmm

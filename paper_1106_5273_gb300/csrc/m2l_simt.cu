@@ -1,5 +1,5 @@
 // M2L on CUDA cores, FP32 (Sec. 3.1; the reference path for the tensor-core
-// kernel).  Work is grouped into steps: one step = one 64-cell target tile
+// kernel).  Work is grouped into steps: one step = one target tile
 // of a level and one translation operator T (P x P), applied to the
 // multipoles of the tile's source cells:  L[:, t] += T M[:, src(t)].  One CTA
 // owns a tile, accumulates all its steps in registers and writes each target
@@ -12,17 +12,25 @@ namespace {
 
 constexpr int kRC = 32;  // output rows per pass
 
-__global__ void __launch_bounds__(192) k_m2l_simt(const int2* __restrict__ tile_range, const int* __restrict__ tfirst,
+// nsub: step ranges per tile (the key buckets of a batch; contiguous).
+__global__ void __launch_bounds__(3 * kTileRows) k_m2l_simt(const int2* __restrict__ tile_range, int nsub, int tsz,
+                                                  const int* __restrict__ tfirst,
                                                   const int* __restrict__ st_slot, const int* __restrict__ st_src,
                                                   const float* __restrict__ T32, const float* __restrict__ M, int P,
                                                   const int* __restrict__ tcell, float* __restrict__ L) {
   extern __shared__ float sT[];  // [kRC][P]
   const int tile = blockIdx.x;
-  const int2 rg = tile_range[tile];
+  int2 rg = make_int2(0, 0);
+  for (int q = 0; q < nsub; ++q) {
+    const int2 r = tile_range[tile * nsub + q];
+    if (r.y <= r.x) continue;
+    if (rg.y == 0) rg.x = r.x;
+    rg.y = r.y;
+  }
   if (rg.y <= rg.x) return;
   const int first = tfirst[tile];
   const int ncell = tfirst[tile + 1] - first;
-  const int comp = threadIdx.x / kTile, slot = threadIdx.x % kTile;
+  const int comp = threadIdx.x / tsz, slot = threadIdx.x % tsz;
   for (int r0 = 0; r0 < P; r0 += kRC) {
     const int nr = min(kRC, P - r0);
     float acc[kRC];
@@ -32,7 +40,7 @@ __global__ void __launch_bounds__(192) k_m2l_simt(const int2* __restrict__ tile_
       const float* T = T32 + (size_t)st_slot[st] * P * P;
       for (int i = threadIdx.x; i < nr * P; i += blockDim.x) sT[i] = T[(size_t)r0 * P + i];
       __syncthreads();
-      const int src = st_src[(size_t)st * kTile + slot];
+      const int src = st_src[(size_t)st * tsz + slot];
       if (src >= 0) {
         const float* m = M + ((size_t)src * 3 + comp) * P;
         for (int k = 0; k < P; ++k) {
@@ -57,7 +65,9 @@ int m2l_simt(fmm_plan p, cudaStream_t s) {
   size_t sh = (size_t)kRC * p->P * sizeof(float);
   if (sh > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2l_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
   ++g_launches;
-  k_m2l_simt<<<(unsigned)p->ntiles, 3 * kTile, sh, s>>>(p->tile_range.as<int2>(), p->tile_first.as<int>(),
+  k_m2l_simt<<<(unsigned)p->ntiles, 3 * m2l_tile(p->P), sh, s>>>(p->tile_range.as<int2>(),
+                                                         p->batched ? kKeyBuckets : 1, m2l_tile(p->P),
+                                                         p->tile_first.as<int>(),
                                                          p->st_slot.as<int>(),
                                                          p->st_src.as<int>(), p->T32.as<float>(), p->M.as<float>(),
                                                          p->P, p->tile_cells.as<int>(), p->L.as<float>());

@@ -3,35 +3,36 @@
 // translation vector).
 //
 // A step applies one translation operator T (P x P, P = p^2) to the
-// multipoles of the 64 source cells paired with a tile of 64 target cells:
-//   D[128 x 192] += T[128 x K] . B[K x 192],  B column (comp, slot) = M~ of
-// the slot's source for that potential component (zero if the slot has no
-// source under this translation).  T = T_hi + T_lo and B = B_hi + B_lo in
-// BF16; D accumulates T_hi B_hi + T_hi B_lo + T_lo B_hi (the lo.lo term is
-// below FP32 resolution of the sum).  The K chunks from m2l_split_chunks on
-// (source degrees 8 and up) take T_hi B_hi only: under the MAC their terms
-// are at most theta^8 / (1 - theta) of the leading one, which keeps the
-// 2^-8 error of one BF16 product there under 7e-6 for theta <= 0.42.  D lives in TMEM for all steps of the
-// tile; each target local expansion is written once.  P > 128 output rows
-// take a second CTA per tile (blockIdx.y = block of 128 rows), which gathers
-// the same B and its own rows of T.
+// multipoles of the source cells paired with a tile of target cells.  Cells as
+// MMA rows (k_m2l_cells), 42 to a tile:
+//   D[128 x N] += B[128 x K] . T^T[K x N],  row (slot, comp) of B = M~ of the
+// slot's source for that potential component (zero if the slot has no source
+// under this translation; rows 126 and 127 are unused), N = P rounded up to 16.
+// The cells are the rows and the coefficients the columns: P need not fill the
+// 128 rows of an MMA (with the operator as the 128-row operand half of them
+// were idle at p = 8, and P = 144 took a second block of 128 rows for its last
+// 16).  T = T_hi + T_lo and B = B_hi + B_lo in BF16; D accumulates T_hi B_hi +
+// T_hi B_lo + T_lo B_hi (the lo.lo term is below FP32 resolution of the sum).
+// The K chunks from m2l_split_chunks on (source degrees 8 and up) take
+// T_hi B_hi only: under the MAC their terms are at most theta^8 / (1 - theta)
+// of the leading one, which keeps the 2^-8 error of one BF16 product there
+// under 7e-6 for theta <= 0.42.  D lives in TMEM for all steps of an item.
 //
-// Per stage (one step, one 64-wide K chunk): A (T hi/lo, pre-swizzled in
-// global memory in the 128B-swizzle K-major layout) arrives by two 1-D bulk
-// copies on mbarrier fullA; 8 producer warps gather the B rows (128 B each)
-// and store them swizzled, then arrive on fullB; one thread issues the MMAs
-// and commits them to the stage's empty barrier.  One stage per CTA and two
-// CTAs per SM (81 KB of shared memory and 256 TMEM columns each): while one
-// CTA waits on its gathers and barriers the other's MMAs keep the tensor pipe
-// busy.  The producers load a stage's rows into registers before they wait
-// for its buffer.  Measured at 2M blobs: 5.6 ms, against 6.6 ms without the
-// early loads and 7.8 ms for two stages in one CTA per SM.  When a step has
-// two K chunks and the second takes one product (p = 9, 10 at theta <= 0.42)
-// the stage holds the whole step instead (three operator blocks of the rows
-// below P and three B blocks, 111 KB at p = 10, still two CTAs per SM), so
-// the operator-copy latency is paid once per step.  Every wait is
-// bounded; on expiry the kernel records FMM_E_TIMEOUT, waits (bounded) for
-// its own bulk copies, frees its tensor memory and returns.
+// A stage is one step and one 64-wide K chunk: the operator (rows pre-swizzled
+// in global memory in the 128-byte-swizzle K-major layout) arrives by 1-D bulk
+// copies on mbarrier fullA, issued by a warp of their own; 8 producer warps
+// gather the rows of B (128 B each) by 16-byte cp.async into the same swizzle and
+// arrive on fullB; one thread issues the MMAs and commits them to the stage's
+// empty barrier.  Every wait is bounded; on expiry the kernel records
+// FMM_E_TIMEOUT, waits (bounded) for its own copies, frees its tensor memory
+// and returns.
+//
+// With 64 < P <= 128 the roles are the other way round (k_m2l_rows: operator
+// rows as MMA rows, 64 cells x 3 components as 192 columns): P fills most of
+// the 128 rows, and an MMA costs about 20-40 cycles on top of N / 2, so fewer
+// and wider MMAs win (Taylor-Green 128^3, p = 10: 4.09 ms against 4.74 with the
+// cells as rows).  Elsewhere the cells win: Plummer 1,000,000 at p = 12 38.3 ->
+// 26.3 ms, Plummer 30,011 at p = 8 0.89 -> 0.56 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -42,18 +43,26 @@ namespace fmm {
 
 namespace {
 
-constexpr int kN = 3 * kTile;                               // 192 columns
-constexpr int kStages = 1;  // pipeline stages per CTA (the loop also runs with 2)
+constexpr int kRows = 128;                  // rows of D: (slot, component), 3 kTileCells of them used
 constexpr int kProducerWarps = 8;
-constexpr int kProducers = kProducerWarps * 32;
-constexpr int kThreads = kProducers + 32;                   // + control warp
-constexpr uint32_t kABytes = 128 * 128;                     // 128 rows x 64 bf16
-constexpr uint32_t kBBytes = kN * 128;                      // 192 rows x 64 bf16
-constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;  // 80 KB
-constexpr uint32_t kBarOff = kStages * kStageBytes;
-constexpr int kTmemCols = 256;
+constexpr int kThreads = (kProducerWarps + 2) * 32;  // + MMA warp, + operator copy warp
+constexpr int kMmaWarp = kProducerWarps, kCopyWarp = kProducerWarps + 1;
+constexpr uint32_t kBBytes = kRows * 128;   // one K chunk of the gathered rows, hi or lo
+constexpr int kStagesMax = 2;
 constexpr long long kSpin = 1ll << 24;
-constexpr int kGather = (2 * kN * 8) / kProducers;          // 16-byte items per producer thread (12)
+static_assert(3 * kTileCells <= kRows, "a tile's rows fit one MMA");
+// operator-row form
+constexpr int kColsB = 3 * kTileRows;                       // 192 columns
+constexpr int kRowStages = 1;                               // pipeline stages per CTA (the loop also runs with 2)
+constexpr int kProducers = kProducerWarps * 32;
+constexpr int kRowThreads = kProducers + 32;                // + control warp
+constexpr uint32_t kRowABytes = 128 * 128;                  // 128 rows x 64 bf16
+constexpr uint32_t kColBytes = kColsB * 128;                // 192 rows x 64 bf16
+constexpr uint32_t kRowStageBytes = 2 * kRowABytes + 2 * kColBytes;  // 80 KB
+constexpr uint32_t kBarOff = kRowStages * kRowStageBytes;
+constexpr int kRowTmemCols = 256;
+constexpr int kRowLd = 128;                                 // coefficients per row of its partial sums
+constexpr int kGather = (2 * kColsB * 8) / kProducers;      // 16-byte items per producer thread (12)
 // Work items of one-problem plans: S = steps / kItemTarget (about four items
 // per concurrent CTA, 2 per SM x 152 SMs) clamped to [kItemMinSteps,
 // kItemMaxSteps], then raised if needed so that there are at most kItemsMax
@@ -62,9 +71,10 @@ constexpr int kGather = (2 * kN * 8) / kProducers;          // 16-byte items per
 // MMAs into one sum) measured 4x the M2L error of sums over at most a few
 // hundred steps added in FP32 afterwards.
 constexpr int64_t kItemMinSteps = 64;
-constexpr int64_t kItemMaxSteps = 256;
+constexpr int64_t kItemMaxSteps = 128;
 constexpr int64_t kItemTarget = 4 * 2 * 152;
 constexpr int64_t kItemsMax = 1 << 15;
+constexpr int64_t kItemSortSteps = 1 << 18;  // the sort costs 0.04 ms: below, it is not worth it
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -118,24 +128,28 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   d |= (uint64_t)2 << 61;
   return d;
 }
-// Instruction descriptors: D f32, both operands K-major, N = 192, M = 128;
+// Instruction descriptor: D f32, both operands K-major, M = 128, N columns;
 // kind::f16 with A and B BF16 (format 1), kind::tf32 with A and B TF32 (format 2).
-constexpr uint32_t kIdescBf16 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kN >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t kIdescTf32 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kN >> 3) << 17) | ((128u >> 4) << 24);
+__device__ __forceinline__ uint32_t idesc(int kind, int N) {
+  const uint32_t fmt = kind ? 2u : 1u;
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
+}
+
+__device__ __forceinline__ uint32_t kRowIdesc(int kind) { return idesc(kind, kColsB); }
 
 template <int KIND>
-__device__ __forceinline__ void umma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void umma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   if (KIND == 0)
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
             tmem),
-        "l"(a), "l"(b), "r"(kIdescBf16), "r"(acc)
+        "l"(a), "l"(b), "r"(id), "r"(acc)
         : "memory");
   else
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(
             tmem),
-        "l"(a), "l"(b), "r"(kIdescTf32), "r"(acc)
+        "l"(a), "l"(b), "r"(id), "r"(acc)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -154,47 +168,310 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 16-byte asynchronous copy to shared memory; zeros if !live.
+__device__ __forceinline__ void gather16(uint32_t dst, const uint8_t* src, bool live) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+
+// ---- Cell rows (P <= 64 or P > 128).
 // KIND 0: BF16 operands (64 per 128-byte row, K step 16); KIND 1: TF32 (32
 // per row, K step 8).  Tb / Mb hold 128-byte rows: a K chunk of one operator
-// row or one (cell, hi/lo, component) multipole row.
-// items == nullptr: CTA x runs all steps of tile x and writes its local
-// expansions.  Otherwise CTA x runs work item x (tile, first step, end step,
-// partial slot) of *nitems: a tile's steps in runs of at most S; a tile split
-// into several items writes each item's D to its partial slot, summed later
-// by k_m2l_combine.
-template <int KIND, bool M2>
-__global__ void __launch_bounds__(kThreads, 2)
-    k_m2l_tc(const int2* __restrict__ tile_range, const int4* __restrict__ items, const uint32_t* __restrict__ nitems,
-             const int* __restrict__ tfirst, const int* __restrict__ st_slot, const int* __restrict__ st_src,
-             const uint8_t* __restrict__ Tb, const uint8_t* __restrict__ Mb, int P, int nkc, int nkc3, int ksteps_last,
-             int nrh,
+// row or one (cell, hi/lo, component) multipole row.  Operators: [slot][hi/lo]
+// [K chunk][N rows].
+// CTA x runs work item x (tile, first step, end step, partial slot) of *nitems:
+// a tile's steps in runs of at most S; an item that is its tile's only one
+// writes the local expansions (slot -1), the others write D to their partial
+// slot, summed by k_m2l_combine.  items == nullptr (batches): CTA x runs the
+// steps of range range0 + x, i.e. of one key bucket of one tile, into slot x.
+template <int KIND>
+__global__ void __launch_bounds__(kThreads, 3)
+    k_m2l_cells(const int2* __restrict__ tile_range, int range0, const int4* __restrict__ items,
+             const uint32_t* __restrict__ nitems, const uint32_t* __restrict__ order, const int* __restrict__ tfirst, const int* __restrict__ st_slot,
+             const int* __restrict__ st_src, const uint8_t* __restrict__ Tb, const uint8_t* __restrict__ Mb, int P,
+             int N, int nkc, int nkc3, int ksteps_last, int nstages, uint32_t tmem_cols,
              const int* __restrict__ tcell, float* __restrict__ L, float* __restrict__ partial,
              int* __restrict__ flag) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  int tile = blockIdx.x, pslot = -1;
+  int tile, pslot;
   int2 rg;
   if (items) {
     if (blockIdx.x >= *nitems) return;  // beyond the items of this evaluation
-    const int4 w = items[blockIdx.x];
+    const int4 w = items[order ? order[blockIdx.x] : blockIdx.x];
     tile = w.x;
     rg = make_int2(w.y, w.z);
     pslot = w.w;
   } else {
-    rg = tile_range[tile];
+    rg = tile_range[range0 + blockIdx.x];
+    tile = (range0 + (int)blockIdx.x) / kKeyBuckets;
+    pslot = (int)blockIdx.x;
   }
-  const int rh = blockIdx.y;  // block of 128 output rows
-  if (rg.y <= rg.x) return;  // no M2L for this tile: the whole CTA leaves before any barrier
+  if (rg.y <= rg.x) return;  // no M2L here: the whole CTA leaves before any barrier
+  constexpr int NB = 2;  // blocks of each operand per stage: hi and lo
+  const uint32_t abytes = (uint32_t)N * 128u;
+  const uint32_t stage_bytes = (uint32_t)NB * (kBBytes + abytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nstages * stage_bytes);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStagesMax + 1);
+  volatile int* abort = reinterpret_cast<volatile int*>(bars + 3 * kStagesMax + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar0 = smem_u32(bars);
+  auto fullA = [&](int s) { return bar0 + 8u * (uint32_t)s; };
+  auto fullB = [&](int s) { return bar0 + 8u * (uint32_t)(kStagesMax + s); };
+  auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(2 * kStagesMax + s); };
+  const uint32_t done = bar0 + 8u * (uint32_t)(3 * kStagesMax);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < nstages; ++s) {
+      mbar_init(fullA(s), 1);
+      mbar_init(fullB(s), kProducerWarps);
+      mbar_init(empty(s), 1);
+    }
+    mbar_init(done, 1);
+    *abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int niter = (rg.y - rg.x) * nkc;
+
+  if (warp < kProducerWarps) {
+    // ---- producers: thread t copies 16-byte chunk j = t % 8 of rows t/8 + 32 q
+    // (q = 0..3), i.e. of component row % 3 of the source in slot row / 3
+    const int j = threadIdx.x & 7, r0 = threadIdx.x >> 3;
+    int src[4], nxt[4];
+    // pieces of the ring that hold a source's values: a piece without a source
+    // is cleared only if it does (adaptive trees pair few of a tile's cells
+    // under one translation)
+    uint32_t dirty[kStagesMax];
+#pragma unroll
+    for (int q = 0; q < kStagesMax; ++q) dirty[q] = 0xffffffffu;
+    auto sources = [&](int st, int* v) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + 32 * q;
+        v[q] = r < 3 * kTileCells ? __ldg(st_src + (size_t)st * kTileCells + r / 3) : -1;
+      }
+    };
+    sources(rg.x, nxt);
+    const int ahead = nstages - 1;  // iterations in flight behind the one being loaded
+    int st = rg.x, kc = 0, stage = 0, astage = 0;
+    uint32_t ph = 0u;
+    bool ok = true;
+    for (int it = 0; it < niter + ahead; ++it) {
+      if (it < niter) {
+        if (kc == 0) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) src[q] = nxt[q];
+          if (st + 1 < rg.y) sources(st + 1, nxt);
+        }
+        // the warp goes on or gives up as one
+        if (!__all_sync(0xffffffffu, mbar_wait(empty(stage), ph ^ 1u, abort))) {
+          ok = false;
+          break;
+        }
+        const uint32_t dst = sbase + (uint32_t)stage * stage_bytes + (uint32_t)r0 * 128u + (uint32_t)((j ^ (r0 & 7)) << 4);
+        uint32_t held = 0u;
+#pragma unroll
+        for (int q = 0; q < kStagesMax; ++q)
+          if (q == stage) held = dirty[q];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          const bool need = (b == 0 || kc < nkc3) && j < 2 * (kc == nkc - 1 ? ksteps_last : 4);
+          if (!need) continue;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = r0 + 32 * q;
+            if (r >= 3 * kTileCells) continue;
+            const bool live = src[q] >= 0;
+            const uint32_t bit = 1u << (b * 4 + q);
+            if (!live && !(held & bit)) continue;
+            held = live ? held | bit : held & ~bit;
+            const uint8_t* p = Mb + ((((size_t)(live ? src[q] : 0) * 2 + b) * 3 + r % 3) * nkc + kc) * 128 + j * 16;
+            gather16(dst + (uint32_t)b * kBBytes + (uint32_t)q * 4096u, p, live);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kStagesMax; ++q)
+          if (q == stage) dirty[q] = held;
+        if (++kc == nkc) {
+          kc = 0;
+          ++st;
+        }
+        if (++stage == nstages) {
+          stage = 0;
+          ph ^= 1u;
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (it >= ahead) {  // the rows of iteration it - ahead have landed
+        if (ahead == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+        else asm volatile("cp.async.wait_group 1;" ::: "memory");
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(fullB(astage));
+        if (++astage == nstages) astage = 0;
+      }
+    }
+    if (!ok) asm volatile("cp.async.wait_group 0;" ::: "memory");
+  } else if (warp == kCopyWarp) {
+    // ---- operator copies
+    if (lane == 0) {
+      int issued = 0, stage = 0, st = rg.x, kc = 0;
+      uint32_t ph = 0u;
+      bool ok = true;
+      for (int it = 0; it < niter; ++it) {
+        if (!mbar_wait(empty(stage), ph ^ 1u, abort)) {
+          ok = false;
+          break;
+        }
+        const uint8_t* T = Tb + (size_t)st_slot[st] * 2 * nkc * abytes;
+        const uint32_t a0 = sbase + (uint32_t)stage * stage_bytes + (uint32_t)NB * kBBytes;
+        const bool lo = kc < nkc3;  // chunks from nkc3 on take the hi.hi product only
+        mbar_arrive_tx(fullA(stage), lo ? 2u * abytes : abytes);
+        bulk_g2s(a0, T + (size_t)kc * abytes, abytes, fullA(stage));
+        if (lo) bulk_g2s(a0 + abytes, T + (size_t)(nkc + kc) * abytes, abytes, fullA(stage));
+        issued = it + 1;
+        if (++kc == nkc) {
+          kc = 0;
+          ++st;
+        }
+        if (++stage == nstages) {
+          stage = 0;
+          ph ^= 1u;
+        }
+      }
+      if (!ok) {  // let the copies in flight land before the CTA exits
+        volatile int never = 0;
+        for (int it = issued > nstages ? issued - nstages : 0; it < issued; ++it)
+          mbar_wait(fullA(it % nstages), (uint32_t)(it / nstages) & 1u, &never);
+      }
+    }
+  } else if (lane == 0) {
+    // ---- MMA issue
+    const uint32_t id = idesc(KIND, N);
+    int stage = 0, kc = 0;
+    uint32_t ph = 0u;
+    bool ok = true;
+    for (int it = 0; it < niter; ++it) {
+      if (!mbar_wait(fullA(stage), ph, abort) || !mbar_wait(fullB(stage), ph, abort)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t b_hi = sbase + (uint32_t)stage * stage_bytes, b_lo = b_hi + kBBytes;
+      const uint32_t a_hi = b_hi + (uint32_t)NB * kBBytes, a_lo = a_hi + abytes;
+      const int ks = (kc == nkc - 1) ? ksteps_last : 4;
+      const bool three = kc < nkc3;
+      for (int kk = 0; kk < ks; ++kk) {
+        const uint32_t off = (uint32_t)kk * 32u;
+        umma<KIND>(tmem, sw128_desc(b_hi + off), sw128_desc(a_hi + off), id, (it > 0 || kk > 0) ? 1u : 0u);
+        if (three) {
+          umma<KIND>(tmem, sw128_desc(b_lo + off), sw128_desc(a_hi + off), id, 1u);
+          umma<KIND>(tmem, sw128_desc(b_hi + off), sw128_desc(a_lo + off), id, 1u);
+        }
+      }
+      if (++kc == nkc) kc = 0;
+      umma_commit(empty(stage));
+      if (++stage == nstages) {
+        stage = 0;
+        ph ^= 1u;
+      }
+    }
+    umma_commit(done);
+    if (!ok) {
+      // our MMAs finish before the tensor memory is freed
+      *abort = 1;
+      volatile int never = 0;
+      mbar_wait(done, 0u, &never);
+      atomicExch(flag, FMM_E_TIMEOUT);
+    }
+  }
+  // ---- epilogue: warps 0-3 own TMEM lanes 0-127 (row = slot, component)
+  if (warp < 4) {
+    if (__all_sync(0xffffffffu, mbar_wait(done, 0u, abort))) {
+      tc_fence_after();
+      const int first = tfirst[tile];
+      const int ncell = tfirst[tile + 1] - first;
+      const int row = warp * 32 + lane;
+      const bool live = row < 3 * ncell;
+      float* dst = pslot >= 0 ? partial + ((size_t)pslot * kRows + row) * N
+                              : L + ((size_t)(live ? tcell[first + row / 3] : 0) * 3 + row % 3) * P;
+      const int cols = pslot >= 0 ? N : P;
+      const bool vec = (cols & 3) == 0;  // rows of whole 16-byte groups
+#pragma unroll 1
+      for (int cb = 0; cb < N; cb += 16) {
+        float v[16];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cb, v);
+        if (!live) continue;
+        if (vec) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            if (cb + i < cols) *reinterpret_cast<float4*>(dst + cb + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (cb + i < cols) dst[cb + i] = v[i];
+        }
+      }
+    } else {
+      atomicExch(flag, FMM_E_TIMEOUT);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+  }
+}
+
+// ---- Operator rows (64 < P <= 128): D[128 x 192] += T[128 x K] . B[K x 192],
+// column (comp, slot) = M~ of the slot's source.  One stage per CTA and two
+// CTAs per SM (81 KB, a whole step 111 KB at p = 10, and 256 TMEM columns each):
+// while one CTA waits on its gathers and barriers the other's MMAs keep the
+// tensor pipe busy.  The producers load a stage's rows into registers before
+// they wait for its buffer.
+template <int KIND, bool M2>
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_m2l_rows(const int2* __restrict__ tile_range, int range0, const int4* __restrict__ items,
+             const uint32_t* __restrict__ nitems, const uint32_t* __restrict__ order, const int* __restrict__ tfirst, const int* __restrict__ st_slot, const int* __restrict__ st_src,
+             const uint8_t* __restrict__ Tb, const uint8_t* __restrict__ Mb, int P, int N, int nkc, int nkc3,
+             int ksteps_last, const int* __restrict__ tcell, float* __restrict__ L, float* __restrict__ partial,
+             int* __restrict__ flag) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  int tile, pslot;
+  int2 rg;
+  if (items) {
+    if (blockIdx.x >= *nitems) return;  // beyond the items of this evaluation
+    const int4 w = items[order ? order[blockIdx.x] : blockIdx.x];
+    tile = w.x;
+    rg = make_int2(w.y, w.z);
+    pslot = w.w;
+  } else {
+    rg = tile_range[range0 + blockIdx.x];
+    tile = (range0 + (int)blockIdx.x) / kKeyBuckets;
+    pslot = (int)blockIdx.x;
+  }
+  if (rg.y <= rg.x) return;  // no M2L here: the whole CTA leaves before any barrier
   // Only the operator rows below P are copied (whole 8-row swizzle groups):
   // the rows above feed only output rows that the epilogue never stores.
-  const uint32_t arows = (uint32_t)min(128, ((P - rh * 128) + 7) & ~7);
-  const uint32_t abytes = arows * 128u;
+  const uint32_t abytes = (uint32_t)((P + 7) & ~7) * 128u;
+  const size_t chunk = (size_t)N * 128;  // bytes of one (operator, hi/lo, K chunk) block
   // M2 (two K chunks, the second with one product, P <= 128): the stage holds
   // a whole step, A buffers of abytes (chunk 0 hi, chunk 0 lo, chunk 1 hi;
   // the MMA's rows past arows read the next buffer and feed discarded output
   // rows) followed by the B buffers (chunk 0 hi, chunk 0 lo, chunk 1 hi).
-  const uint32_t abuf = M2 ? abytes : kABytes;
-  const uint32_t stage_bytes = M2 ? 3u * abuf + 3u * kBBytes : kStageBytes;
+  const uint32_t abuf = M2 ? abytes : kRowABytes;
+  const uint32_t stage_bytes = M2 ? 3u * abuf + 3u * kColBytes : kRowStageBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + stage_bytes);
   // bars: fullA[2], fullB[2], empty[2], done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
@@ -207,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(4 + s); };
   const uint32_t done = bar0 + 8u * 6u;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kRowStages; ++s) {
       mbar_init(fullA(s), 1);
       mbar_init(fullB(s), kProducers);
       mbar_init(empty(s), 1);
@@ -218,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   if (warp == kProducerWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(kTmemCols)
+                 "r"(kRowTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -236,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     for (int it = 0; it < niter; ++it) {
       const uint32_t ph = (uint32_t)it & 1u;
       const int st = rg.x + it;
-      const int srcA = __ldg(st_src + (size_t)st * kTile + r0), srcB = __ldg(st_src + (size_t)st * kTile + r0 + 32);
+      const int srcA = __ldg(st_src + (size_t)st * kTileRows + r0), srcB = __ldg(st_src + (size_t)st * kTileRows + r0 + 32);
       uint4 v[G];
 #pragma unroll
       for (int q = 0; q < G; ++q) {
@@ -252,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int q = 0; q < G; ++q) {
         const int bsel = q / 6, n = r0 + 32 * (q % 6);
-        *reinterpret_cast<uint4*>(smem + 3 * abuf + bsel * kBBytes + n * 128 + ((j ^ (n & 7)) << 4)) = v[q];
+        *reinterpret_cast<uint4*>(smem + 3 * abuf + bsel * kColBytes + n * 128 + ((j ^ (n & 7)) << 4)) = v[q];
       }
       fence_proxy_async();
       mbar_arrive(fullB(0));
@@ -262,7 +539,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     // 12 MMAs for chunk 0 (three products) and ksteps_last for chunk 1 (hi x hi)
     int issued = 0, consumed = 0;
     bool ok = true;
-    const size_t chunk = (size_t)128 * 128;  // bytes of one (operator, hi/lo, K chunk) block (nrh == 1)
     for (int it = 0; it < niter; ++it) {
       const uint32_t ph = (uint32_t)it & 1u;
       if (!mbar_wait(empty(0), ph ^ 1u, abort)) {
@@ -290,13 +566,13 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         const uint32_t off = (uint32_t)kk * 32u;
-        umma<KIND>(tmem, sw128_desc(a0 + off), sw128_desc(b0 + off), (it > 0 || kk > 0) ? 1u : 0u);
-        umma<KIND>(tmem, sw128_desc(a0 + off), sw128_desc(b0 + kBBytes + off), 1u);
-        umma<KIND>(tmem, sw128_desc(a0 + abuf + off), sw128_desc(b0 + off), 1u);
+        umma<KIND>(tmem, sw128_desc(a0 + off), sw128_desc(b0 + off), kRowIdesc(KIND), (it > 0 || kk > 0) ? 1u : 0u);
+        umma<KIND>(tmem, sw128_desc(a0 + off), sw128_desc(b0 + kColBytes + off), kRowIdesc(KIND), 1u);
+        umma<KIND>(tmem, sw128_desc(a0 + abuf + off), sw128_desc(b0 + off), kRowIdesc(KIND), 1u);
       }
       for (int kk = 0; kk < ksteps_last; ++kk) {
         const uint32_t off = (uint32_t)kk * 32u;
-        umma<KIND>(tmem, sw128_desc(a0 + 2 * abuf + off), sw128_desc(b0 + 2 * kBBytes + off), 1u);
+        umma<KIND>(tmem, sw128_desc(a0 + 2 * abuf + off), sw128_desc(b0 + 2 * kColBytes + off), kRowIdesc(KIND), 1u);
       }
       umma_commit(empty(0));
     }
@@ -316,14 +592,14 @@ __global__ void __launch_bounds__(kThreads, 2)
     // ---- producers: thread t stores 16-byte chunk j = t % 8 of rows n = t/8 + 32k
     // (k = 0..5) of both halves, i.e. of the sources in slots t/8 and t/8 + 32;
     // the rows are loaded before the stage's buffer is waited for.
-    static_assert(kGather == 12 && kProducers == 256 && kN == 192, "producer row mapping");
+    static_assert(kGather == 12 && kProducers == 256 && kColsB == 192, "producer row mapping");
     const int j = threadIdx.x & 7, r0 = threadIdx.x >> 3;
     for (int it = 0; it < niter; ++it) {
-      const int stage = it % kStages;
-      const uint32_t ph = (uint32_t)(it / kStages) & 1u;
+      const int stage = it % kRowStages;
+      const uint32_t ph = (uint32_t)(it / kRowStages) & 1u;
       const int st = rg.x + it / nkc, kc = it % nkc;
       const bool lo = kc < nkc3;  // chunks from nkc3 on take the hi.hi product only
-      const int srcA = __ldg(st_src + (size_t)st * kTile + r0), srcB = __ldg(st_src + (size_t)st * kTile + r0 + 32);
+      const int srcA = __ldg(st_src + (size_t)st * kTileRows + r0), srcB = __ldg(st_src + (size_t)st * kTileRows + r0 + 32);
       uint4 v[kGather];
 #pragma unroll
       for (int q = 0; q < kGather; ++q) {
@@ -339,7 +615,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       for (int q = 0; q < kGather; ++q) {
         const int h = q / 6, n = r0 + 32 * (q % 6);
         if (h == 0 || lo)
-          *reinterpret_cast<uint4*>(smem + stage * kStageBytes + 2 * kABytes + h * kBBytes + n * 128 +
+          *reinterpret_cast<uint4*>(smem + stage * kRowStageBytes + 2 * kRowABytes + h * kColBytes + n * 128 +
                                     ((j ^ (n & 7)) << 4)) = v[q];
       }
       fence_proxy_async();
@@ -349,30 +625,29 @@ __global__ void __launch_bounds__(kThreads, 2)
     // ---- control thread: operator copies and MMAs
     int issued = 0;  // A copies issued for iterations [0, issued)
     auto issue_A = [&](int it) -> bool {
-      const int stage = it % kStages;
-      const uint32_t ph = (uint32_t)(it / kStages) & 1u;
+      const int stage = it % kRowStages;
+      const uint32_t ph = (uint32_t)(it / kRowStages) & 1u;
       if (!mbar_wait(empty(stage), ph ^ 1u, abort)) return false;
       const int st = rg.x + it / nkc, kc = it % nkc;
       const size_t key = (size_t)st_slot[st];
-      const size_t chunk = (size_t)nrh * 128 * 128, row0 = (size_t)rh * 128 * 128;  // bytes
-      const uint8_t* hi = Tb + ((key * 2 + 0) * nkc + kc) * chunk + row0;
-      const uint8_t* lo = Tb + ((key * 2 + 1) * nkc + kc) * chunk + row0;
-      const uint32_t a0 = sbase + stage * kStageBytes;
+      const uint8_t* hi = Tb + ((key * 2 + 0) * nkc + kc) * chunk;
+      const uint8_t* lo = Tb + ((key * 2 + 1) * nkc + kc) * chunk;
+      const uint32_t a0 = sbase + stage * kRowStageBytes;
       const bool with_lo = kc < nkc3;
       mbar_arrive_tx(fullA(stage), with_lo ? 2 * abytes : abytes);
       bulk_g2s(a0, hi, abytes, fullA(stage));
-      if (with_lo) bulk_g2s(a0 + kABytes, lo, abytes, fullA(stage));
+      if (with_lo) bulk_g2s(a0 + kRowABytes, lo, abytes, fullA(stage));
       issued = it + 1;
       return true;
     };
-    // operator copies run kStages - 1 iterations ahead of the MMAs
-    constexpr int kAhead = kStages - 1;
+    // operator copies run kRowStages - 1 iterations ahead of the MMAs
+    constexpr int kAhead = kRowStages - 1;
     bool ok = true;
     for (int k = 0; ok && k < kAhead && k < niter; ++k) ok = issue_A(k);
     int consumed = 0;  // iterations whose A copy was observed complete
     for (int it = 0; ok && it < niter; ++it) {
-      const int stage = it % kStages;
-      const uint32_t ph = (uint32_t)(it / kStages) & 1u;
+      const int stage = it % kRowStages;
+      const uint32_t ph = (uint32_t)(it / kRowStages) & 1u;
       if (it + kAhead < niter && !issue_A(it + kAhead)) {
         ok = false;
         break;
@@ -389,15 +664,15 @@ __global__ void __launch_bounds__(kThreads, 2)
       tc_fence_after();
       const int kc = it % nkc;
       const int ks = (kc == nkc - 1) ? ksteps_last : 4;
-      const uint32_t a_hi = sbase + stage * kStageBytes, a_lo = a_hi + kABytes;
-      const uint32_t b_hi = a_hi + 2 * kABytes, b_lo = b_hi + kBBytes;
+      const uint32_t a_hi = sbase + stage * kRowStageBytes, a_lo = a_hi + kRowABytes;
+      const uint32_t b_hi = a_hi + 2 * kRowABytes, b_lo = b_hi + kColBytes;
       const bool three = kc < nkc3;
       for (int kk = 0; kk < ks; ++kk) {
         const uint32_t off = (uint32_t)kk * 32u;
-        umma<KIND>(tmem, sw128_desc(a_hi + off), sw128_desc(b_hi + off), (it > 0 || kk > 0) ? 1u : 0u);
+        umma<KIND>(tmem, sw128_desc(a_hi + off), sw128_desc(b_hi + off), kRowIdesc(KIND), (it > 0 || kk > 0) ? 1u : 0u);
         if (three) {
-          umma<KIND>(tmem, sw128_desc(a_hi + off), sw128_desc(b_lo + off), 1u);
-          umma<KIND>(tmem, sw128_desc(a_lo + off), sw128_desc(b_hi + off), 1u);
+          umma<KIND>(tmem, sw128_desc(a_hi + off), sw128_desc(b_lo + off), kRowIdesc(KIND), 1u);
+          umma<KIND>(tmem, sw128_desc(a_lo + off), sw128_desc(b_hi + off), kRowIdesc(KIND), 1u);
         }
       }
       umma_commit(empty(stage));
@@ -410,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       // the tensor memory is freed and the CTA exits
       volatile int never = 0;
       for (int it = consumed; it < issued; ++it)
-        mbar_wait(fullA(it % kStages), (uint32_t)(it / kStages) & 1u, &never);
+        mbar_wait(fullA(it % kRowStages), (uint32_t)(it / kRowStages) & 1u, &never);
       umma_commit(done);
       mbar_wait(done, 0u, &never);
       atomicExch(flag, FMM_E_TIMEOUT);
@@ -422,18 +697,19 @@ __global__ void __launch_bounds__(kThreads, 2)
       tc_fence_after();
       const int first = tfirst[tile];
       const int ncell = tfirst[tile + 1] - first;
-      const int r = rh * 128 + warp * 32 + lane;  // output coefficient of this TMEM lane
-      float* pdst = pslot >= 0 ? partial + ((size_t)pslot * nrh + rh) * (size_t)kN * 128 : nullptr;
+      const int r = warp * 32 + lane;  // output coefficient of this TMEM lane
+      float* pdst = pslot >= 0 ? partial + (size_t)pslot * kColsB * kRowLd : nullptr;
 #pragma unroll 1
-      for (int cb = 0; cb < kN / 16; ++cb) {
+      for (int cb = 0; cb < kColsB / 16; ++cb) {
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cb * 16), v);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int n = cb * 16 + i;
-          const int comp = n / kTile, slot = n % kTile;
-          if (pdst) pdst[(size_t)n * 128 + warp * 32 + lane] = v[i];  // [column][row of the block]
-          else if (r < P && slot < ncell) L[((size_t)tcell[first + slot] * 3 + comp) * P + r] = v[i];
+          const int comp = n / kTileRows, slot = n % kTileRows;
+          if (r >= P || slot >= ncell) continue;
+          if (pdst) pdst[(size_t)(slot * 3 + comp) * kRowLd + r] = v[i];
+          else L[((size_t)tcell[first + slot] * 3 + comp) * P + r] = v[i];
         }
       }
     } else {
@@ -444,7 +720,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   if (warp == kProducerWarps) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kRowTmemCols) : "memory");
   }
 }
 
@@ -460,6 +736,19 @@ __global__ void k_m2l_item_count(const int2* __restrict__ tr, int ntiles, int S,
   pcnt[t] = k > 1 ? k : 0u;
 }
 
+// Items in the order of their first operator, for CTAs that run side by side to
+// read the same operators out of L2: with 10^5 steps and more the operators a
+// problem touches outgrow it (Plummer 1,000,000 at p = 12: 49,141 operators,
+// 5.4 GB; M2L 26.3 -> 24.2 ms, Taylor-Green 128^3 4.09 -> 3.86 ms).
+__global__ void k_m2l_item_keys(const int4* __restrict__ items, const uint32_t* __restrict__ nitems, int cap,
+                                const int* __restrict__ st_slot, uint64_t* __restrict__ keys,
+                                uint32_t* __restrict__ vals) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= cap) return;
+  keys[i] = i < (int)*nitems ? (uint64_t)st_slot[items[i].y] : 0xffffffffull;
+  vals[i] = (uint32_t)i;
+}
+
 __global__ void k_m2l_item_fill(const int2* __restrict__ tr, int ntiles, int S, const uint32_t* __restrict__ cnt,
                                 const uint32_t* __restrict__ ioff, const uint32_t* __restrict__ poff,
                                 int4* __restrict__ items) {
@@ -473,22 +762,46 @@ __global__ void k_m2l_item_fill(const int2* __restrict__ tr, int ntiles, int S, 
 }
 
 // Local expansions of the split tiles: the partial sums of their items, added
-// in item order (a fixed order, so the result is deterministic).
+// in item order (a fixed order, so the result is deterministic).  Partial
+// sums: [slot][row = cell slot, component][N coefficients].
 __global__ void k_m2l_combine(const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ poff,
-                              const int* __restrict__ tfirst, const int* __restrict__ tcell, int P, int nrh,
+                              const int* __restrict__ tfirst, const int* __restrict__ tcell, int P, int rows, int N,
                               const float* __restrict__ partial, float* __restrict__ L) {
   const int t = blockIdx.x;
   const uint32_t k = cnt[t];
   if (k <= 1) return;
   const int first = tfirst[t], ncell = tfirst[t + 1] - first;
-  const size_t per = (size_t)nrh * kN * 128;  // floats per partial slot
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < nrh * kN * 128; e += gridDim.y * blockDim.x) {
-    const int r = e & 127, n = (e >> 7) % kN, rh = e / (kN * 128);
-    const int row = rh * 128 + r, slot = n % kTile, comp = n / kTile;
-    if (row >= P || slot >= ncell) continue;
+  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < 3 * ncell * P; e += gridDim.y * blockDim.x) {
+    const int row = e / P, c = e % P;
     float acc = 0.f;
-    for (uint32_t q = 0; q < k; ++q) acc += partial[(size_t)(poff[t] + q) * per + (size_t)e];
-    L[((size_t)tcell[first + slot] * 3 + comp) * P + row] = acc;
+    for (uint32_t q = 0; q < k; ++q) acc += partial[((size_t)(poff[t] + q) * rows + row) * N + c];
+    L[((size_t)tcell[first + row / 3] * 3 + row % 3) * P + c] = acc;
+  }
+}
+
+// The same for the tiles [t0, t0 + gridDim.x) of a batch: the sums of the
+// tile's key buckets, in bucket order (empty buckets add nothing, so a problem's
+// sums are those it has alone).
+__global__ void k_m2l_combine_buckets(const int2* __restrict__ ranges, int t0, const int* __restrict__ tfirst,
+                                      const int* __restrict__ tcell, int P, int rows, int N,
+                                      const float* __restrict__ partial, float* __restrict__ L) {
+  const int t = t0 + blockIdx.x;
+  bool some[kKeyBuckets], any = false;
+#pragma unroll
+  for (int q = 0; q < kKeyBuckets; ++q) {
+    const int2 r = ranges[t * kKeyBuckets + q];
+    some[q] = r.y > r.x;
+    any = any || some[q];
+  }
+  if (!any) return;
+  const int first = tfirst[t], ncell = tfirst[t + 1] - first;
+  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < 3 * ncell * P; e += gridDim.y * blockDim.x) {
+    const int row = e / P, c = e % P;
+    float acc = 0.f;
+#pragma unroll
+    for (int q = 0; q < kKeyBuckets; ++q)
+      if (some[q]) acc += partial[((size_t)(blockIdx.x * kKeyBuckets + q) * rows + row) * N + c];
+    L[((size_t)tcell[first + row / 3] * 3 + row % 3) * P + c] = acc;
   }
 }
 
@@ -509,6 +822,115 @@ __global__ void k_wait_selftest(long long spins, int arrive, int* status) {
 
 }  // namespace
 
+// Kernel, launch shape and partial-sum layout of a plan's tensor-core M2L.
+struct M2lForm {
+  const void* kern;
+  size_t smem;
+  int threads, nstages, rows, ld;
+  uint32_t tmem_cols;
+  bool m2;
+};
+
+static M2lForm m2l_form(fmm_plan p, int nkc, int nkc3) {
+  const int kind = p->tc_kind;
+  const int N = m2l_cols(p->P);
+  M2lForm f{};
+  // A whole step per stage when it has two BF16 K chunks, the second with one
+  // product (p = 9 and 10 at theta <= 0.42): one operator-copy latency per
+  // step instead of one per chunk.
+  f.m2 = kind == 0 && nkc == 2 && nkc3 == 1 && !(p->prm.m2l_mode & FMM_M2L_CHUNK_STAGES);
+  if (m2l_tile(p->P) == kTileRows) {
+    f.kern = f.m2 ? (const void*)k_m2l_rows<0, true>
+                  : (kind ? (const void*)k_m2l_rows<1, false> : (const void*)k_m2l_rows<0, false>);
+    f.smem = (f.m2 ? 3 * (size_t)((p->P + 7) & ~7) * 128 + 3 * (size_t)kColBytes : (size_t)kBarOff) + 128 + 1024;
+    f.threads = kRowThreads;
+    f.rows = kColsB;
+    f.ld = kRowLd;
+    return f;
+  }
+  f.m2 = false;
+  f.kern = kind ? (const void*)k_m2l_cells<1> : (const void*)k_m2l_cells<0>;
+  f.tmem_cols = 32;
+  while ((int)f.tmem_cols < N) f.tmem_cols *= 2;
+  const size_t stage = 2 * (kBBytes + (size_t)N * 128);
+  // One stage per CTA and as many CTAs per SM as registers, TMEM and the stage
+  // memory allow (three at p <= 8, two at p >= 12): the CTAs hide each other's
+  // gathers, and more gathering threads run.  Rings of 2 and 3 stages in fewer
+  // CTAs were slower: Plummer 1,000,000 at p = 12 26.3 / 34.1 / 34.4 ms for 1 /
+  // 2 / 3 stages, the batch of 32 at p = 8 1.17 / 1.42 / 2.39 ms.
+  f.nstages = 1;
+  f.smem = f.nstages * stage + (3 * kStagesMax + 4) * 8 + 1024;
+  f.threads = kThreads;
+  f.rows = kRows;
+  f.ld = N;
+  return f;
+}
+
+// The work items of a one-problem plan and their place in p->m2l_items.
+struct M2lItems {
+  int64_t S, max_items, max_split;
+  int4* items;
+  uint32_t *order, *cnt, *pcnt, *ioff, *poff, *totals;  // totals: items, partial slots
+  size_t bytes;
+};
+
+static M2lItems m2l_items(fmm_plan p) {
+  const int64_t nt = p->ntiles;
+  M2lItems w{};
+  w.S = std::min(kItemMaxSteps, std::max(kItemMinSteps, (p->n_steps + kItemTarget - 1) / kItemTarget));
+  w.S = std::max(w.S, (p->n_steps + kItemsMax - 1) / kItemsMax);
+  w.max_items = nt + p->n_steps / w.S + 1;
+  w.max_split = 2 * (p->n_steps / w.S) + 1;
+  uint8_t* base = p->m2l_items.as<uint8_t>();
+  w.items = reinterpret_cast<int4*>(base);
+  uint32_t* u = reinterpret_cast<uint32_t*>(base + (size_t)w.max_items * sizeof(int4));
+  w.cnt = u;
+  w.pcnt = w.cnt + (nt + 1);
+  w.ioff = w.pcnt + (nt + 1);
+  w.poff = w.ioff + (nt + 1);
+  w.totals = w.poff + (nt + 1);
+  uint32_t* order = w.totals + 2;
+  w.bytes = (size_t)w.max_items * (sizeof(int4) + sizeof(uint32_t)) + (4 * (size_t)(nt + 1) + 2) * sizeof(uint32_t);
+  w.order = p->n_steps >= kItemSortSteps ? order : nullptr;
+  return w;
+}
+
+// One-problem plans split the tiles into work items of at most S steps:
+// with Alg. 1's printed rule the coarse target tiles collect many more steps
+// than the rest, and one CTA per tile left a long tail (and long tensor-memory
+// sums).  Built once per tree.
+int m2l_build_items(fmm_plan p, cudaStream_t s) {
+  if (p->n_steps == 0 || p->batched || !p->last_tc) return FMM_OK;
+  const int nt = (int)p->ntiles, T = 256;
+  FMM_TRY(p->m2l_items.ensure(m2l_items(p).bytes));
+  const M2lItems w = m2l_items(p);
+  const int2* ranges = p->tile_range.as<int2>();
+  const unsigned gt = (unsigned)((nt + T - 1) / T);
+  ++g_launches;
+  k_m2l_item_count<<<gt, T, 0, s>>>(ranges, nt, (int)w.S, w.cnt, w.pcnt);
+  FMM_TRY(exclusive_scan_u32(w.cnt, w.ioff, nt, w.totals, p->scan_tmp, s));
+  FMM_TRY(exclusive_scan_u32(w.pcnt, w.poff, nt, w.totals + 1, p->scan_tmp, s));
+  ++g_launches;
+  k_m2l_item_fill<<<gt, T, 0, s>>>(ranges, nt, (int)w.S, w.cnt, w.ioff, w.poff, w.items);
+  if (w.order) {
+    const size_t k = (size_t)w.max_items;
+    FMM_TRY(p->lk0.ensure(k * sizeof(uint64_t)));
+    FMM_TRY(p->lk1.ensure(k * sizeof(uint64_t)));
+    FMM_TRY(p->lv0.ensure(k * sizeof(uint32_t)));
+    FMM_TRY(p->lv1.ensure(k * sizeof(uint32_t)));
+    ++g_launches;
+    k_m2l_item_keys<<<(unsigned)((k + T - 1) / T), T, 0, s>>>(w.items, w.totals, (int)k, p->st_slot.as<int>(),
+                                                              p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+    int second = 0;
+    FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                           p->lv1.as<uint32_t>(), (int64_t)k, 0, 32, &second, p->sort_hist, p->scan_tmp, s));
+    FMM_CUDA_TRY(cudaMemcpyAsync(w.order, second ? p->lv1.ptr : p->lv0.ptr, k * sizeof(uint32_t),
+                                 cudaMemcpyDeviceToDevice, s));
+  }
+  FMM_CUDA_TRY(cudaGetLastError());
+  return FMM_OK;
+}
+
 int m2l_tensor(fmm_plan p, cudaStream_t s) {
   if (p->n_steps == 0) return FMM_OK;
   const int kind = p->tc_kind;
@@ -516,118 +938,70 @@ int m2l_tensor(fmm_plan p, cudaStream_t s) {
   const int nkc = m2l_kchunks(p->P, kind);
   const int last = ksteps - 4 * (nkc - 1);
   const int nkc3 = m2l_split_chunks(p->P, kind, p->prm.theta, p->prm.m2l_mode & FMM_M2L_FULL_SPLIT);
-  const size_t sh = (size_t)kBarOff + 128 + 1024;
-  static bool attr_set[2] = {false, false};
-  if (!attr_set[kind]) {
-    FMM_CUDA_TRY(cudaFuncSetAttribute(kind ? k_m2l_tc<1, false> : k_m2l_tc<0, false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-    attr_set[kind] = true;
-  }
-  const int nrh = m2l_rowblocks(p->P);
-  // A whole step per stage when it has two BF16 K chunks, the second with one
-  // product, in one block of output rows, and two such CTAs still fit an SM
-  // (p = 9 and 10 at theta <= 0.42): one operator-copy latency per step
-  // instead of one per chunk.
-  bool m2 = false;
-  size_t sh2 = 0;
-  if (kind == 0 && nkc == 2 && nkc3 == 1 && nrh == 1 && !(p->prm.m2l_mode & FMM_M2L_CHUNK_STAGES)) {
-    const size_t arows = (size_t)std::min(128, (p->P + 7) & ~7);
-    sh2 = 3 * arows * 128 + 3 * (size_t)kBBytes + 128 + 1024;
-    static int m2_ok = -1;  // 1: two CTAs per SM at the largest stage (P = 128 rows would not fit)
-    static size_t m2_sh = 0;
-    if (m2_ok < 0 || m2_sh != sh2) {
-      // Two CTAs per SM by shared memory (each with the per-block reserve) and
-      // registers, from the device and kernel attributes; the occupancy query
-      // reports one CTA per SM for both forms of this kernel, although two
-      // run (ncu: 17.5 of 18 warps active per SM).  Two such CTAs need the
-      // largest shared-memory carveout.
-      int dev = 0, smem_sm = 0, resv = 0, regs_sm = 0;
-      cudaFuncAttributes fa{};
-      m2_ok = cudaGetDevice(&dev) == cudaSuccess &&
-                      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) ==
-                          cudaSuccess &&
-                      cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess &&
-                      cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) == cudaSuccess &&
-                      cudaFuncGetAttributes(&fa, k_m2l_tc<0, true>) == cudaSuccess &&
-                      cudaFuncSetAttribute(k_m2l_tc<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh2) ==
-                          cudaSuccess &&
-                      cudaFuncSetAttribute(k_m2l_tc<0, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100) ==
-                          cudaSuccess &&
-                      2 * (sh2 + (size_t)resv + fa.sharedSizeBytes) <= (size_t)smem_sm &&
-                      2 * (size_t)fa.numRegs * kThreads <= (size_t)regs_sm
-                  ? 1
-                  : 0;
-      cudaGetLastError();
-      m2_sh = sh2;
-    }
-    m2 = m2_ok == 1;
-  }
-  p->m2l_stage_chunks = m2 ? 2 : 1;
+  const int N = m2l_cols(p->P);
+  const M2lForm f = m2l_form(p, nkc, nkc3);
+  p->m2l_stage_chunks = f.m2 ? 2 : 1;
+  static const bool attr_ok = [] {
+    const void* k[5] = {(const void*)k_m2l_cells<1>, (const void*)k_m2l_cells<0>,
+                        (const void*)k_m2l_rows<0, true>, (const void*)k_m2l_rows<1, false>,
+                        (const void*)k_m2l_rows<0, false>};
+    for (const void* q : k)
+      if (cudaFuncSetAttribute(q, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess ||
+          cudaFuncSetAttribute(q, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
+        return false;
+    return true;
+  }();
+  if (!attr_ok) return FMM_E_CUDA;
   const int nt = (int)p->ntiles;
   const int T = 256;
-  // One-problem plans split the tiles into work items of at most S steps:
-  // with Alg. 1's printed rule the coarse target tiles collect many more
-  // steps than the rest, and one CTA per tile left a long tail (and long
-  // tensor-memory sums).  Batches keep one CTA per tile: their tiles mix
-  // problems, and items cut at fixed step counts would make a problem's sums
-  // depend on the other problems of the batch.
-  const int4* items = nullptr;
-  const uint32_t* nitems = nullptr;
-  uint32_t *cnt = nullptr, *poff = nullptr;
-  unsigned grid = (unsigned)nt;
-  if (!p->batched) {
-    int64_t S = std::min(kItemMaxSteps, std::max(kItemMinSteps, (p->n_steps + kItemTarget - 1) / kItemTarget));
-    S = std::max(S, (p->n_steps + kItemsMax - 1) / kItemsMax);
-    const int64_t max_items = nt + p->n_steps / S + 1;
-    const int64_t max_split = 2 * (p->n_steps / S) + 1;
-    const size_t b_items = (size_t)max_items * sizeof(int4), b_arr = (size_t)(nt + 1) * sizeof(uint32_t);
-    FMM_TRY(p->m2l_items.ensure(b_items + 4 * b_arr + 64));
-    FMM_TRY(p->m2l_partial.ensure((size_t)max_split * nrh * kN * 128 * sizeof(float)));
-    uint8_t* base = p->m2l_items.as<uint8_t>();
-    int4* it = reinterpret_cast<int4*>(base);
-    cnt = reinterpret_cast<uint32_t*>(base + b_items);
-    uint32_t* pcnt = cnt + (nt + 1);
-    uint32_t* ioff = pcnt + (nt + 1);
-    poff = ioff + (nt + 1);
-    uint32_t* totals = poff + (nt + 1);  // [0] items, [1] partial slots
-    const unsigned gt = (unsigned)((nt + T - 1) / T);
+  const int2* ranges = p->tile_range.as<int2>();
+  const int* tfirst = p->tile_first.as<int>();
+  const int* tcell = p->tile_cells.as<int>();
+  float* L = p->L.as<float>();
+  const uint32_t* order = nullptr;
+  auto launch = [&](unsigned grid, int range0, const int4* items, const uint32_t* nitems) -> int {
+    const int* slot = p->st_slot.as<int>();
+    const int* src = p->st_src.as<int>();
+    const uint8_t* Tb = p->Tbf.as<uint8_t>();
+    const uint8_t* Mb = p->Mbf.as<uint8_t>();
+    float* partial = p->m2l_partial.as<float>();
+    int* flag = p->flags.as<int>();
+    int P = p->P, NN = N, a = nkc, b = nkc3, c = last, d = f.nstages;
+    uint32_t e = f.tmem_cols;
+    void* cells[] = {&ranges, &range0, &items, &nitems, &order, &tfirst, &slot, &src, &Tb, &Mb, &P, &NN,
+                     &a, &b, &c, &d, &e, &tcell, &L, &partial, &flag};
+    void* rows[] = {&ranges, &range0, &items, &nitems, &order, &tfirst, &slot, &src, &Tb, &Mb, &P, &NN,
+                    &a, &b, &c, &tcell, &L, &partial, &flag};
     ++g_launches;
-    k_m2l_item_count<<<gt, T, 0, s>>>(p->tile_range.as<int2>(), nt, (int)S, cnt, pcnt);
-    FMM_TRY(exclusive_scan_u32(cnt, ioff, nt, totals, p->scan_tmp, s));
-    FMM_TRY(exclusive_scan_u32(pcnt, poff, nt, totals + 1, p->scan_tmp, s));
-    ++g_launches;
-    k_m2l_item_fill<<<gt, T, 0, s>>>(p->tile_range.as<int2>(), nt, (int)S, cnt, ioff, poff, it);
+    FMM_CUDA_TRY(cudaLaunchKernel(f.kern, dim3(grid), dim3(f.threads), f.nstages ? cells : rows, f.smem, s));
+    return FMM_OK;
+  };
+  if (p->batched) {
+    // Batches: one CTA per (tile, key bucket), in rounds that bound the partial
+    // sums; a tile's buckets are cut by the translation alone, so a problem's
+    // sums do not depend on the rest of the batch.  One CTA per tile made the
+    // longest tile the time of the phase (32 problems: 4.7 ms, now 1.17).
+    const int round = std::min(nt, 1024);
+    FMM_TRY(p->m2l_partial.ensure((size_t)round * kKeyBuckets * f.rows * f.ld * sizeof(float)));
+    for (int t0 = 0; t0 < nt; t0 += round) {
+      const int k = std::min(round, nt - t0);
+      FMM_TRY(launch((unsigned)(k * kKeyBuckets), t0 * kKeyBuckets, nullptr, nullptr));
+      ++g_launches;
+      k_m2l_combine_buckets<<<dim3((unsigned)k, 4), T, 0, s>>>(ranges, t0, tfirst, tcell, p->P, f.rows, f.ld,
+                                                               p->m2l_partial.as<float>(), L);
+    }
     FMM_CUDA_TRY(cudaGetLastError());
-    items = it;
-    nitems = totals;
-    grid = (unsigned)max_items;
+    return FMM_OK;
   }
+  const M2lItems w = m2l_items(p);
+  order = w.order;
+  FMM_TRY(p->m2l_partial.ensure((size_t)w.max_split * f.rows * f.ld * sizeof(float)));
+  FMM_TRY(launch((unsigned)w.max_items, 0, w.items, w.totals));
   ++g_launches;
-  const dim3 g3(grid, (unsigned)nrh);
-  if (m2)
-    k_m2l_tc<0, true><<<g3, kThreads, sh2, s>>>(p->tile_range.as<int2>(), items, nitems, p->tile_first.as<int>(),
-                                                p->st_slot.as<int>(), p->st_src.as<int>(), p->Tbf.as<uint8_t>(),
-                                                p->Mbf.as<uint8_t>(), p->P, nkc, nkc3, last, nrh,
-                                                p->tile_cells.as<int>(), p->L.as<float>(), p->m2l_partial.as<float>(),
-                                                p->flags.as<int>());
-  else if (kind)
-    k_m2l_tc<1, false><<<g3, kThreads, sh, s>>>(p->tile_range.as<int2>(), items, nitems, p->tile_first.as<int>(),
-                                         p->st_slot.as<int>(), p->st_src.as<int>(), p->Tbf.as<uint8_t>(),
-                                         p->Mbf.as<uint8_t>(), p->P, nkc, nkc3, last, nrh, p->tile_cells.as<int>(),
-                                         p->L.as<float>(), p->m2l_partial.as<float>(), p->flags.as<int>());
-  else
-    k_m2l_tc<0, false><<<g3, kThreads, sh, s>>>(p->tile_range.as<int2>(), items, nitems, p->tile_first.as<int>(),
-                                         p->st_slot.as<int>(), p->st_src.as<int>(), p->Tbf.as<uint8_t>(),
-                                         p->Mbf.as<uint8_t>(), p->P, nkc, nkc3, last, nrh, p->tile_cells.as<int>(),
-                                         p->L.as<float>(), p->m2l_partial.as<float>(), p->flags.as<int>());
+  // a tile's rows over 8 CTAs (the split tiles are a few hundred)
+  k_m2l_combine<<<dim3((unsigned)nt, 8), T, 0, s>>>(w.cnt, w.poff, tfirst, tcell, p->P, f.rows, f.ld,
+                                                    p->m2l_partial.as<float>(), L);
   FMM_CUDA_TRY(cudaGetLastError());
-  if (items) {
-    ++g_launches;
-    // a tile's D block over 8 CTAs (the split tiles are a few hundred)
-    k_m2l_combine<<<dim3((unsigned)nt, 8), T, 0, s>>>(cnt, poff, p->tile_first.as<int>(), p->tile_cells.as<int>(),
-                                                      p->P, nrh, p->m2l_partial.as<float>(), p->L.as<float>());
-    FMM_CUDA_TRY(cudaGetLastError());
-  }
   return FMM_OK;
 }
 

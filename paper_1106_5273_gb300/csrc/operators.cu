@@ -175,7 +175,7 @@ __global__ void k_build_m2l(const uint64_t* __restrict__ keys, const int* __rest
     nu[r] = nu_d(n, m);
   }
   if (threadIdx.x < (unsigned)p) rp[threadIdx.x] = ldexp(1.0, delta * (int)threadIdx.x);
-  const int rows = 128 * m2l_rowblocks(P);  // output rows of the BF16 tiles
+  const int rows = m2l_cols(P);  // output rows of the operator tiles
   const size_t chunk_bytes = (size_t)rows * 128;
   if (nkc) {  // zero this slot's tiles (padding rows and columns stay zero)
     uint4* z = reinterpret_cast<uint4*>(Tb + (size_t)key_id * 2 * nkc * chunk_bytes);
@@ -427,7 +427,7 @@ int build_m2l_operators(fmm_plan p, int64_t nmiss, uint32_t* miss, uint32_t* ran
     int64_t cap = std::max<int64_t>(need, p->tcache_cap * 2);
     if (!tc) FMM_TRY(p->T32.grow_copy((size_t)cap * P * P * sizeof(float), s));
     if (tc)
-      FMM_TRY(p->Tbf.grow_copy((size_t)cap * 2 * m2l_kchunks(P, p->tc_kind) * 128 * m2l_rowblocks(P) * 128, s));
+      FMM_TRY(p->Tbf.grow_copy((size_t)cap * 2 * m2l_kchunks(P, p->tc_kind) * m2l_cols(P) * 128, s));
     p->tcache_cap = cap;
   }
   FMM_TRY(p->tmiss_keys.ensure((size_t)nmiss * sizeof(uint64_t)));

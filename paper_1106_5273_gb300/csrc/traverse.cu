@@ -14,7 +14,7 @@
 // in FP64 with explicitly rounded operations in a fixed order.
 //
 // Outputs: P2P entries grouped by target leaf (CSR), and M2L entries grouped
-// into steps = (tile of 64 consecutive target cells of one level, translation
+// into steps = (tile of target cells of one level, translation
 // key), each step carrying the source cell of every tile slot (or -1).
 #include <algorithm>
 #include <climits>
@@ -510,15 +510,15 @@ __device__ inline uint64_t compact_key(uint64_t k, const KeyPack& kp) {
   return c;
 }
 
-// (tile, compact key) sort keys of the M2L pairs: a run of equal keys is one
-// step.  A target has at most one source per translation, so the pairs of a
+// (tile, compact key) sort keys of the M2L pairs (batches: tile and key
+// bucket): a run of equal keys is one step.  A target has at most one source per translation, so the pairs of a
 // step have distinct slots and their order within the run does not matter.
 __global__ void k_step_keys2(const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys, int n,
-                             const int* __restrict__ ctile, KeyPack kp, uint64_t* __restrict__ keys,
+                             const int* __restrict__ ctile, int tsz, KeyPack kp, int nsub, uint64_t* __restrict__ keys,
                              uint32_t* __restrict__ vals) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const uint64_t tile = (uint64_t)(ctile[raw[i].x] / kTile);
+  const uint64_t tile = (uint64_t)(ctile[raw[i].x] / tsz) * nsub + (nsub > 1 ? m2l_bucket(fkeys[i]) : 0);
   keys[i] = (tile << kp.bits) | compact_key(fkeys[i], kp);
   vals[i] = (uint32_t)i;
 }
@@ -544,39 +544,60 @@ __global__ void k_key_unpack(const uint32_t* __restrict__ kflag, const uint32_t*
   ukeys[kslot[c]] = m2l_key_encode(f[0], f[1], f[2], f[3]);
 }
 
+// Batches number the translations by (bucket, key) instead of key, so that the
+// steps of a tile come bucket by bucket.
+__global__ void k_bucket_keys(const uint64_t* __restrict__ ukeys, int nk, uint64_t* __restrict__ keys,
+                              uint32_t* __restrict__ vals) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nk) return;
+  keys[i] = (uint64_t)m2l_bucket(ukeys[i]);
+  vals[i] = (uint32_t)i;
+}
+
+__global__ void k_bucket_order(const uint64_t* __restrict__ ukeys, const uint32_t* __restrict__ order, int nk,
+                               uint64_t* __restrict__ out, uint32_t* __restrict__ perm) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nk) return;
+  out[i] = ukeys[order[i]];
+  perm[order[i]] = (uint32_t)i;
+}
+
 // bin of pair i = tile * nkeys + slot; flags the bin and keeps it per pair.
 __global__ void k_bin_mark(const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys, int n,
-                           const int* __restrict__ ctile, KeyPack kp, const uint32_t* __restrict__ kslot, int nkeys,
-                           uint32_t* __restrict__ bflag, uint32_t* __restrict__ pbin) {
+                           const int* __restrict__ ctile, int tsz, KeyPack kp, const uint32_t* __restrict__ kslot,
+                           const uint32_t* __restrict__ perm, int nkeys, uint32_t* __restrict__ bflag,
+                           uint32_t* __restrict__ pbin) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const uint32_t b = (uint32_t)(ctile[raw[i].x] / kTile) * (uint32_t)nkeys + kslot[compact_key(fkeys[i], kp)];
+  uint32_t slot = kslot[compact_key(fkeys[i], kp)];
+  if (perm) slot = perm[slot];
+  const uint32_t b = (uint32_t)(ctile[raw[i].x] / tsz) * (uint32_t)nkeys + slot;
   bflag[b] = 1u;
   pbin[i] = b;
 }
 
 __global__ void k_bin_steps(const uint32_t* __restrict__ bflag, const uint32_t* __restrict__ bstep, int64_t nb,
-                            int nkeys, const int* __restrict__ map, int* __restrict__ st_tile,
-                            int* __restrict__ st_slot) {
+                            int nkeys, const int* __restrict__ map, const uint64_t* __restrict__ ukeys, int nsub,
+                            int* __restrict__ st_tile, int* __restrict__ st_slot) {
   int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb || !bflag[b]) return;
-  st_tile[bstep[b]] = (int)(b / nkeys);
+  st_tile[bstep[b]] = (int)(b / nkeys) * nsub + (nsub > 1 ? m2l_bucket(ukeys[b % nkeys]) : 0);
   st_slot[bstep[b]] = map[b % nkeys];  // unique key -> operator slot
 }
 
 __global__ void k_bin_fill(const int2* __restrict__ raw, const uint32_t* __restrict__ pbin, int n,
-                           const uint32_t* __restrict__ bstep, const int* __restrict__ ctile,
+                           const uint32_t* __restrict__ bstep, const int* __restrict__ ctile, int tsz,
                            int* __restrict__ st_src) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int2 v = raw[i];
-  st_src[(size_t)bstep[pbin[i]] * kTile + (ctile[v.x] % kTile)] = m2l_src(v);
+  st_src[(size_t)bstep[pbin[i]] * tsz + (ctile[v.x] % tsz)] = m2l_src(v);
 }
 
 __global__ void k_step_write2(const uint64_t* __restrict__ k, const uint32_t* __restrict__ idx, int n,
                               const uint32_t* __restrict__ f, const uint32_t* __restrict__ e,
                               const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys,
-                              const int* __restrict__ ctile, int kbits, int* __restrict__ st_tile,
+                              const int* __restrict__ ctile, int tsz, int kbits, int* __restrict__ st_tile,
                               uint64_t* __restrict__ st_ckey, uint64_t* __restrict__ st_fkey,
                               int* __restrict__ st_src) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -589,7 +610,7 @@ __global__ void k_step_write2(const uint64_t* __restrict__ k, const uint32_t* __
     st_fkey[s] = fkeys[idx[i]];
   }
   const int2 v = raw[idx[i]];
-  st_src[(size_t)s * kTile + (ctile[v.x] % kTile)] = m2l_src(v);
+  st_src[(size_t)s * tsz + (ctile[v.x] % tsz)] = m2l_src(v);
 }
 
 __global__ void k_step_slots(const uint64_t* __restrict__ sk, const uint32_t* __restrict__ sidx, int ns,
@@ -618,7 +639,7 @@ __global__ void k_unique_flags(const uint64_t* __restrict__ k, int n, uint32_t* 
 }
 
 // Tiles group the cells of one level and one child octant (in Morton order),
-// at most 64 per tile: cells at the same octant position have the same
+// 42 or 64 per tile (m2l_tile): cells at the same octant position have the same
 // relative interaction lists in a uniform region, so a tile's steps are
 // nearly full; a tile never mixes octants, so a coarse level is split into
 // its octants instead of one long tile.
@@ -645,12 +666,12 @@ __global__ void __launch_bounds__(256) k_tile_order_keys(const int* __restrict__
 
 // gofs[g] = first sorted position of (level, octant) group g, gtile[g] = its
 // first tile; *ntiles the number of tiles.  Also starts the key ranges.
-__global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int* __restrict__ gofs,
+__global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int tsz, int* __restrict__ gofs,
                                                      int* __restrict__ gtile, uint32_t* __restrict__ ntiles,
                                                      int* __restrict__ rng) {
   __shared__ int cells[256], tiles[256];
   const int g = threadIdx.x;
-  const int c = g < kGroups ? gcount[g] : 0, t = (c + kTile - 1) / kTile;
+  const int c = g < kGroups ? gcount[g] : 0, t = (c + tsz - 1) / tsz;
   cells[g] = c;
   tiles[g] = t;
   __syncthreads();
@@ -669,7 +690,7 @@ __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gco
   if (g < 8) rng[g] = (g & 1) ? INT_MIN : INT_MAX;
 }
 
-__global__ void k_cell_tiles(int nc, const uint32_t* __restrict__ ntiles, const uint32_t* __restrict__ order,
+__global__ void k_cell_tiles(int nc, int tsz, const uint32_t* __restrict__ ntiles, const uint32_t* __restrict__ order,
                              const int* __restrict__ level, const uint64_t* __restrict__ ckey,
                              const int* __restrict__ gofs, const int* __restrict__ gtile, int* __restrict__ ctile,
                              int* __restrict__ tcell, int* __restrict__ tfirst) {
@@ -678,10 +699,10 @@ __global__ void k_cell_tiles(int nc, const uint32_t* __restrict__ ntiles, const 
   const int c = (int)order[q];
   const int g = level[c] * 8 + (int)(ckey[c] & 7ull);
   const int r = q - gofs[g];
-  const int t = gtile[g] + r / kTile;
-  ctile[c] = t * kTile + r % kTile;
+  const int t = gtile[g] + r / tsz;
+  ctile[c] = t * tsz + r % tsz;
   tcell[q] = c;
-  if (r % kTile == 0) tfirst[t] = q;
+  if (r % tsz == 0) tfirst[t] = q;
   if (q == 0) tfirst[*ntiles] = nc;
 }
 
@@ -749,15 +770,15 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
   return FMM_OK;
 }
 
-// Tiles: at most 64 cells of one (level, octant) group each; and the cells'
+// Tiles: at most m2l_tile cells of one (level, octant) group each; and the cells'
 // integer coordinates.  ntiles and the key ranges stay on the device.
 static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
   const int T = 256;
-  const int nc = (int)p->ncells;
+  const int nc = (int)p->ncells, tsz = m2l_tile(p->P);
   FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
   FMM_TRY(p->tile_cells.ensure((nc + 1) * sizeof(int)));
   FMM_TRY(p->tile_groups.ensure(3 * kGroups * sizeof(int)));
-  FMM_TRY(p->tile_first.ensure((size_t)(nc / kTile + kGroups + 1) * sizeof(int)));
+  FMM_TRY(p->tile_first.ensure((size_t)(nc / tsz + kGroups + 1) * sizeof(int)));
   FMM_TRY(p->c_ijk.ensure((size_t)(nc + 1) * sizeof(uint64_t)));
   FMM_TRY(p->lk0.ensure((nc + 1) * sizeof(uint64_t)));
   FMM_TRY(p->lk1.ensure((nc + 1) * sizeof(uint64_t)));
@@ -775,9 +796,9 @@ static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
   FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
                          nc, 0, 8, &second, p->sort_hist, p->scan_tmp, s));
   ++g_launches;
-  k_tile_groups<<<1, 256, 0, s>>>(gcount, gofs, gtile, ntiles, rng);
+  k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, ntiles, rng);
   ++g_launches;
-  k_cell_tiles<<<gc, T, 0, s>>>(nc, ntiles, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
+  k_cell_tiles<<<gc, T, 0, s>>>(nc, tsz, ntiles, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
                                 p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs, gtile, p->c_tile.as<int>(),
                                 p->tile_cells.as<int>(), p->tile_first.as<int>());
   ++g_launches;
@@ -992,8 +1013,10 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   };
   FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
   p->ntiles = hmisc[0];
-  FMM_TRY(p->tile_range.ensure((p->ntiles + 1) * sizeof(int2)));
-  FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (p->ntiles + 1) * sizeof(int2), s));
+  // step ranges: one per tile, in a batch one per tile and key bucket
+  const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p->P);
+  FMM_TRY(p->tile_range.ensure((size_t)(p->ntiles + 1) * nsub * sizeof(int2)));
+  FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (size_t)(p->ntiles + 1) * nsub * sizeof(int2), s));
   if (n == 0) {
     FMM_CUDA_TRY(cudaStreamSynchronize(s));
     FMM_TRY(p2p_items());
@@ -1017,7 +1040,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     }
     kp.bits = sh;
     int tb = 1;
-    while ((1ll << tb) < (long long)p->ntiles) ++tb;
+    while ((1ll << tb) < (long long)p->ntiles * nsub) ++tb;
     if (tb + kp.bits > 63) return FMM_E_DEPTH;
     const int64_t K = 1ll << kp.bits;
     bool binned = false;
@@ -1041,6 +1064,27 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
         FMM_TRY(p->ukeys.ensure((size_t)(nkeys + 1) * sizeof(uint64_t)));
         ++g_launches;
         k_key_unpack<<<(unsigned)((K + T - 1) / T), T, 0, s>>>(kflag, kslot, K, kp, p->ukeys.as<uint64_t>());
+        const uint32_t* perm = nullptr;
+        if (nsub > 1) {
+          FMM_TRY(p->lk0.ensure((nkeys + 1) * sizeof(uint64_t)));
+          FMM_TRY(p->lk1.ensure((nkeys + 1) * sizeof(uint64_t)));
+          FMM_TRY(p->lv1.ensure((nkeys + 1) * sizeof(uint32_t)));
+          FMM_TRY(p->m2l_slot.ensure((nkeys + 1) * sizeof(uint32_t)));
+          const unsigned gk = (unsigned)((nkeys + T - 1) / T);
+          g_launches += 2;
+          k_bucket_keys<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(), (int)nkeys, p->lk0.as<uint64_t>(),
+                                         p->lv0.as<uint32_t>());
+          int second = 0;
+          FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                                 p->lv1.as<uint32_t>(), nkeys, 0, 3, &second, p->sort_hist, p->scan_tmp, s));
+          // the sorted bucket numbers are not needed: their buffer takes the keys in the new order
+          uint64_t* out = second ? p->lk0.as<uint64_t>() : p->lk1.as<uint64_t>();
+          k_bucket_order<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(),
+                                          second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(), (int)nkeys, out,
+                                          p->m2l_slot.as<uint32_t>());
+          FMM_CUDA_TRY(cudaMemcpyAsync(p->ukeys.ptr, out, (size_t)nkeys * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+          perm = p->m2l_slot.as<uint32_t>();
+        }
         uint32_t* miss = p->tcount.as<uint32_t>();
         uint32_t* rank = p->tscan0.as<uint32_t>();
         FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, s));
@@ -1052,8 +1096,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
         uint32_t* pbin = p->lv0.as<uint32_t>();
         FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), s));
         ++g_launches;
-        k_bin_mark<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
-                                   kslot, (int)nkeys, bflag, pbin);
+        k_bin_mark<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
+                                   kslot, perm, (int)nkeys, bflag, pbin);
         FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, s));
         FMM_TRY(p2p_items());
         FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 4 * sizeof(uint32_t)));
@@ -1063,14 +1107,16 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
         const int64_t ns = p->n_steps;
         FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
-        FMM_TRY(p->st_src.ensure((ns + 1) * kTile * sizeof(int)));
+        FMM_TRY(p->st_src.ensure((ns + 1) * tsz * sizeof(int)));
         FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, s));
-        FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * kTile * sizeof(int), s));
+        FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), s));
         ++g_launches;
         k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, s>>>(bflag, bstep, nb, (int)nkeys, p->tslot_map.as<int>(),
-                                                               p->st_tile.as<int>(), p->st_slot.as<int>());
+                                                               p->ukeys.as<uint64_t>(), nsub, p->st_tile.as<int>(),
+                                                               p->st_slot.as<int>());
         ++g_launches;
-        k_bin_fill<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(), p->st_src.as<int>());
+        k_bin_fill<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(), tsz,
+                                     p->st_src.as<int>());
         ++g_launches;
         k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns,
                                                                 p->tile_range.as<int2>());
@@ -1083,8 +1129,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       FMM_TRY(p->lv1.ensure((n + 1) * sizeof(uint32_t)));
       // sort pairs by (tile, compact key): consecutive runs are the steps
       ++g_launches;
-      k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), kp,
-                                   p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+      k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
+                                   nsub, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       int second = 0;
       FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
                              p->lv1.as<uint32_t>(), n, 0, tb + kp.bits, &second, p->sort_hist, p->scan_tmp, s));
@@ -1099,13 +1145,13 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       const int64_t ns = p->n_steps;
       FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
       FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
-      FMM_TRY(p->st_src.ensure((ns + 1) * kTile * sizeof(int)));
+      FMM_TRY(p->st_src.ensure((ns + 1) * tsz * sizeof(int)));
       FMM_TRY(p->st_ckey.ensure((ns + 1) * sizeof(uint64_t)));
       FMM_TRY(p->st_fkey.ensure((ns + 1) * sizeof(uint64_t)));
-      FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * kTile * sizeof(int), s));
+      FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), s));
       ++g_launches;
       k_step_write2<<<g, T, 0, s>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
-                                    p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), kp.bits,
+                                    p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), tsz, kp.bits,
                                     p->st_tile.as<int>(),
                                     p->st_ckey.as<uint64_t>(), p->st_fkey.as<uint64_t>(), p->st_src.as<int>());
       ++g_launches;
