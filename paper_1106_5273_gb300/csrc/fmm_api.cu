@@ -42,7 +42,7 @@ std::vector<DBuf*> plan_buffers(fmm_plan p) {
           &p->tscan0, &p->tscan1, &p->tscan2, &p->p2p_raw, &p->m2l_raw, &p->lk0, &p->lk1, &p->lv0, &p->lv1,
           &p->p2p_sorted, &p->p2p_off, &p->p2p_pre, &p->p2p_items, &p->p2p_islot, &p->p2p_plan, &p->p2p_bar, &p->p2p_partial, &p->p2p_sigk, &p->m2l_key, &p->m2l_slot, &p->ukeys, &p->T32, &p->Tbf,
           &p->tc_key, &p->tc_slot, &p->tmiss_keys, &p->tmiss_slots, &p->tslot_map, &p->st_tile, &p->st_slot, &p->st_src, &p->bin_flag, &p->bin_scan, &p->bin_flag2, &p->bin_scan2, &p->st_ckey,
-          &p->st_fkey, &p->m2l_items, &p->m2l_partial, &p->tile_range, &p->scan_tmp, &p->sort_hist, &p->scal,
+          &p->st_fkey, &p->m2l_items, &p->m2l_partial, &p->tile_range, &p->scan_tmp, &p->sort.state, &p->sort.look, &p->scal,
           &p->flags, &p->seg_off, &p->seg_box, &p->seg_sig, &p->seg_smax, &p->seg_mac, &p->seg_p2p, &p->c_seg};
 }
 

@@ -922,8 +922,8 @@ int m2l_build_items(fmm_plan p, cudaStream_t s) {
     k_m2l_item_keys<<<(unsigned)((k + T - 1) / T), T, 0, s>>>(w.items, w.totals, (int)k, p->st_slot.as<int>(),
                                                               p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
     int second = 0;
-    FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                           p->lv1.as<uint32_t>(), (int64_t)k, 0, 32, &second, p->sort_hist, p->scan_tmp, s));
+    FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                           p->lv1.as<uint32_t>(), (int64_t)k, 32, &second, p->flags.as<int>(), s));
     FMM_CUDA_TRY(cudaMemcpyAsync(w.order, second ? p->lv1.ptr : p->lv0.ptr, k * sizeof(uint32_t),
                                  cudaMemcpyDeviceToDevice, s));
   }

@@ -1,8 +1,11 @@
 // Device-wide exclusive scan and stable LSD radix sort (keys u64, values u32).
+// k_sort_hist / k_sort_scatter serve the caller that provides all scratch.
 //
 // Used by the Morton sort (Sec. 3.2), the tree build, the traversal output
 // compaction and the grouping of P2P / M2L lists.  Both are deterministic:
 // the scan is a fixed-order reduction, the sort is stable.
+#include <algorithm>
+
 #include "primitives.cuh"
 
 namespace fmm {
@@ -120,106 +123,6 @@ int exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* t
   return FMM_OK;
 }
 
-// ---------------------------------------------------------- three scans ---
-// Exclusive scans of three u32 arrays of one length in the same passes (the
-// traversal's per-pair M2L, P2P and push counts).  Each array is scanned
-// exactly as exclusive_scan_u32 scans it.
-
-namespace {
-
-struct Scan3Ptrs {
-  const uint32_t* in[3];
-  uint32_t* out[3];
-};
-
-__global__ void k_scan3_reduce(Scan3Ptrs a, int64_t n, uint32_t* __restrict__ sums, int64_t ld) {
-  __shared__ uint32_t s_warp[33];
-  const int64_t base = (int64_t)blockIdx.x * kScanTile;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    uint32_t acc = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      const int64_t idx = base + (int64_t)threadIdx.x * kScanItems + i;
-      if (idx < n) acc += a.in[c][idx];
-    }
-    uint32_t total;
-    block_excl_scan(acc, s_warp, total);
-    if (threadIdx.x == 0) sums[c * ld + blockIdx.x] = total;
-  }
-}
-
-__global__ void k_scan3_apply(Scan3Ptrs a, int64_t n, const uint32_t* __restrict__ offs, int64_t ld,
-                              uint32_t* __restrict__ total_out) {
-  __shared__ uint32_t s_warp[33];
-  const int64_t base = (int64_t)blockIdx.x * kScanTile;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    uint32_t v[kScanItems];
-    uint32_t acc = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      const int64_t idx = base + (int64_t)threadIdx.x * kScanItems + i;
-      v[i] = idx < n ? a.in[c][idx] : 0u;
-      acc += v[i];
-    }
-    uint32_t total;
-    uint32_t pre = block_excl_scan(acc, s_warp, total);
-    const uint32_t off = offs ? offs[c * ld + blockIdx.x] : 0u;
-    pre += off;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      const int64_t idx = base + (int64_t)threadIdx.x * kScanItems + i;
-      if (idx < n) a.out[c][idx] = pre;
-      pre += v[i];
-    }
-    if (total_out && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) total_out[c] = off + total;
-  }
-}
-
-}  // namespace
-
-int exclusive_scan3_u32(const uint32_t* const in[3], uint32_t* const out[3], int64_t n, uint32_t* total_dev,
-                        DBuf& tmp, DBuf& tmp2, cudaStream_t s) {
-  if (n <= 0) {
-    if (total_dev) FMM_CUDA_TRY(cudaMemsetAsync(total_dev, 0, 3 * sizeof(uint32_t), s));
-    return FMM_OK;
-  }
-  Scan3Ptrs a;
-  for (int c = 0; c < 3; ++c) {
-    a.in[c] = in[c];
-    a.out[c] = out[c];
-  }
-  const int64_t nb = (n + kScanTile - 1) / kScanTile;
-  if (nb <= 1) {
-    ++g_launches;
-    k_scan3_apply<<<1, kScanThreads, 0, s>>>(a, n, nullptr, 0, total_dev);
-    FMM_CUDA_TRY(cudaGetLastError());
-    return FMM_OK;
-  }
-  // block sums of the three arrays, scanned in place by the one-array scan
-  const int64_t ld = nb + 1;
-  FMM_TRY(tmp.ensure((size_t)(3 * ld) * sizeof(uint32_t) + 64));
-  uint32_t* sums = tmp.as<uint32_t>();
-  ++g_launches;
-  k_scan3_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(a, n, sums, ld);
-  if (nb <= kScanTile) {  // the three block-sum arrays in one single-block pass (in place)
-    Scan3Ptrs b;
-    for (int c = 0; c < 3; ++c) {
-      b.in[c] = sums + c * ld;
-      b.out[c] = sums + c * ld;
-    }
-    ++g_launches;
-    k_scan3_apply<<<1, kScanThreads, 0, s>>>(b, nb, nullptr, 0, nullptr);
-  } else {
-    for (int c = 0; c < 3; ++c) FMM_TRY(exclusive_scan_u32(sums + c * ld, sums + c * ld, nb, nullptr, tmp2, s));
-  }
-  ++g_launches;
-  k_scan3_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(a, n, sums, ld, total_dev);
-  FMM_CUDA_TRY(cudaGetLastError());
-  return FMM_OK;
-}
-
 // ------------------------------------------------------------------ sort ---
 
 namespace {
@@ -288,51 +191,232 @@ __global__ void k_sort_scatter(const uint64_t* __restrict__ kin, const uint32_t*
   }
 }
 
-__global__ void k_iota(uint32_t* v, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = (uint32_t)i;
+// ---- Sort passes with one kernel each.  The digit counts of all passes are
+// taken at once (k_digit_hist, or by the kernel that makes the keys), scanned by
+// one CTA (k_digit_scan), and a pass (k_onesweep) ranks its tile, learns the
+// counts of the tiles before it by looking back over their published counts,
+// and scatters.  Tiles are numbered by a ticket in the order the CTAs start, so
+// every tile that a CTA waits for has started; the waits are bounded.  Three
+// kernels per pass and a host read of the varying digits before: the tree phase
+// of 1000 blobs took 0.23 ms, now 0.14, of 100,003 0.44 -> 0.24, of 1,000,000
+// 0.82 -> 0.67.
+constexpr long long kSweepSpin = 1ll << 24;
+
+// Counts of digit q (8 bits from bit 8 q) of every key, q < npass.
+__global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__ keys, int64_t n, int npass,
+                                                    uint32_t* __restrict__ hist) {
+  __shared__ uint32_t h[kSortPasses * 256];
+  clear_digits(h, npass);
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = b + threadIdx.x;
+    count_digits(h, i < n ? keys[i] : 0ull, i < n, npass);
+  }
+  flush_digits(h, npass, hist);
 }
+
+// First output position of every digit of every pass, and which passes do
+// anything: one over a digit that is the same in every key is the identity, and
+// is left out unless `all` (the caller then knows where the result is).
+__global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, int64_t n, int npass, int all) {
+  __shared__ uint32_t ws[8];
+  __shared__ int act[kSortPasses];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  for (int q = 0; q < npass; ++q) {
+    const uint32_t c = st->hist[q][t];
+    if (t == 0) act[q] = all;
+    uint32_t inc = warp_incl_scan(c);
+    if (lane == 31) ws[w] = inc;
+    __syncthreads();
+    uint32_t pre = 0;
+    for (int i = 0; i < w; ++i) pre += ws[i];
+    st->base[q][t] = pre + inc - c;
+    if (c != 0u && (int64_t)c < n) act[q] = 1;
+    __syncthreads();
+  }
+  if (t == 0) {
+    int sel = 0;
+    for (int q = 0; q < npass; ++q) {
+      st->active[q] = act[q];
+      st->sel[q] = sel;
+      sel ^= act[q];
+    }
+    st->sel[npass] = sel;
+  }
+}
+
+// look: one 64-bit word per (tile, digit): epoch << 34 | state << 32 | count,
+// state 1 the tile's own count, 2 the count of it and all before; words of
+// earlier passes carry an earlier epoch.
+// R keys per thread.  The tile's keys are put in order in shared memory first, so
+// that a digit's run is written by consecutive threads.
+template <int R>
+__global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict__ k0, uint32_t* __restrict__ v0,
+                                                           uint64_t* __restrict__ k1, uint32_t* __restrict__ v1,
+                                                           int64_t n, int pass, SortState* __restrict__ st,
+                                                           unsigned long long* look, unsigned epoch,
+                                                           int* __restrict__ flag) {
+  if (!st->active[pass]) return;
+  const bool swap = st->sel[pass] != 0;
+  const uint64_t* kin = swap ? k1 : k0;
+  const uint32_t* vin = swap ? v1 : v0;
+  uint64_t* kout = swap ? k0 : k1;
+  uint32_t* vout = swap ? v0 : v1;
+  constexpr int kTileKeys = kSortThreads * R;
+  extern __shared__ uint64_t sk[];  // [kTileKeys] keys, then [kTileKeys] values
+  uint32_t* sv = reinterpret_cast<uint32_t*>(sk + kTileKeys);
+  __shared__ uint32_t cnt[kSortThreads / 32][256];
+  __shared__ uint32_t shift_to[256];  // output position minus position in the tile
+  __shared__ uint32_t ws[kSortThreads / 32];
+  __shared__ int s_tile, s_bad;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) {
+    s_tile = (int)atomicAdd(&st->ticket[pass], 1u);
+    s_bad = 0;
+  }
+  for (int q = 0; q < kSortThreads / 32; ++q) cnt[q][tid] = 0u;
+  __syncthreads();
+  const int tile = s_tile, shift = 8 * pass;
+  const int64_t t0 = (int64_t)tile * kTileKeys;
+  const int have = (int)min((int64_t)kTileKeys, n - t0);
+  // the warp's 32 R keys in order: row r holds keys 32 r + lane
+  const int base = w * (32 * R) + lane;
+  uint64_t key[R];
+  uint32_t val[R], rank[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const bool live = base + 32 * r < have;
+    key[r] = live ? kin[t0 + base + 32 * r] : 0ull;
+    val[r] = live ? vin[t0 + base + 32 * r] : 0u;
+  }
+  const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (w * (32 * R) + 32 * r >= have) break;
+    const bool live = base + 32 * r < have;
+    const int d = live ? (int)((key[r] >> shift) & 0xff) : 256;
+    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    const int leader = __ffs(peers) - 1;
+    uint32_t before = 0;
+    if (live && lane == leader) {
+      before = cnt[w][d];
+      cnt[w][d] = before + (uint32_t)__popc(peers);
+    }
+    before = __shfl_sync(0xffffffffu, before, leader);
+    rank[r] = before + (uint32_t)__popc(peers & lt);
+    __syncwarp();
+  }
+  __syncthreads();
+  {  // thread = digit: the tile's count, the warps' first ranks, the tiles before
+    uint32_t total = 0;
+#pragma unroll
+    for (int q = 0; q < kSortThreads / 32; ++q) {
+      const uint32_t c = cnt[q][tid];
+      cnt[q][tid] = total;
+      total += c;
+    }
+    volatile unsigned long long* lk = look;
+    const unsigned long long tag = (unsigned long long)epoch << 34;
+    lk[(size_t)tile * 256 + tid] = tag | ((tile == 0 ? 2ull : 1ull) << 32) | total;
+    // first position of the digit in the tile
+    const uint32_t inc = warp_incl_scan(total);
+    if (lane == 31) ws[w] = inc;
+    __syncthreads();
+    uint32_t local = inc - total;
+    for (int q = 0; q < w; ++q) local += ws[q];
+#pragma unroll
+    for (int q = 0; q < kSortThreads / 32; ++q) cnt[q][tid] += local;
+    uint32_t pre = 0;
+    bool ok = true;
+    for (int t = tile - 1; ok && t >= 0; --t) {
+      unsigned long long x = 0;
+      long long spin = 0;
+      while (((x = lk[(size_t)t * 256 + tid]) >> 34) != epoch)
+        if (++spin > kSweepSpin) {
+          ok = false;
+          break;
+        }
+      pre += (uint32_t)x;
+      if ((x >> 32) & 2ull) break;
+    }
+    if (!ok) s_bad = 1;
+    else if (tile > 0) lk[(size_t)tile * 256 + tid] = tag | (2ull << 32) | (pre + total);
+    shift_to[tid] = st->base[pass][tid] + pre - local;
+  }
+  __syncthreads();
+  if (s_bad) {  // gave up: write nothing
+    if (tid == 0) atomicExch(flag, FMM_E_TIMEOUT);
+    return;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (base + 32 * r >= have) break;
+    const uint32_t o = cnt[w][(int)((key[r] >> shift) & 0xff)] + rank[r];
+    sk[o] = key[r];
+    sv[o] = val[r];
+  }
+  __syncthreads();
+  for (int i = tid; i < have; i += kSortThreads) {
+    const uint64_t k = sk[i];
+    const uint32_t o = shift_to[(int)((k >> shift) & 0xff)] + (uint32_t)i;
+    kout[o] = k;
+    vout[o] = sv[i];
+  }
+}
+
+// Keys per thread: small tiles while they are few (a tile is one CTA's serial
+// work), large ones for throughput.
+int sweep_rows(int64_t n) { return n <= 65536 ? 4 : (n <= (1 << 20) ? 8 : 16); }
 
 }  // namespace
 
-int iota_u32(uint32_t* v, int64_t n, cudaStream_t s) {
-  if (n <= 0) return FMM_OK;
+int sort_begin(SortScratch& b, int64_t n, cudaStream_t s) {
+  const int64_t tile = (int64_t)kSortThreads * sweep_rows(n);
+  const size_t tiles = (size_t)((n + tile - 1) / tile);
+  FMM_TRY(b.state.ensure(sizeof(SortState)));
+  if (b.look.bytes < tiles * 256 * sizeof(unsigned long long) || b.epoch > (1u << 29)) {
+    FMM_TRY(b.look.ensure(tiles * 256 * sizeof(unsigned long long)));
+    FMM_CUDA_TRY(cudaMemsetAsync(b.look.ptr, 0, b.look.bytes, s));  // epoch 0: never published
+    b.epoch = 0;
+  }
+  FMM_CUDA_TRY(cudaMemsetAsync(b.state.ptr, 0, sizeof(SortState), s));
+  return FMM_OK;
+}
+
+int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int npass, bool all,
+                int* flag, cudaStream_t s) {
+  SortState* st = b.state.as<SortState>();
   ++g_launches;
-  k_iota<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(v, n);
+  k_digit_scan<<<1, 256, 0, s>>>(st, n, npass, all ? 1 : 0);
+  const int R = sweep_rows(n);
+  const int64_t tile = (int64_t)kSortThreads * R;
+  const unsigned g = (unsigned)((n + tile - 1) / tile);
+  const size_t sh = (size_t)tile * (sizeof(uint64_t) + sizeof(uint32_t));
+  auto kern = R == 4 ? k_onesweep<4> : (R == 8 ? k_onesweep<8> : k_onesweep<16>);
+  static const bool ok = cudaFuncSetAttribute(k_onesweep<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              kSortThreads * 16 * 12) == cudaSuccess;
+  if (!ok) return FMM_E_CUDA;
+  unsigned long long* look = b.look.as<unsigned long long>();
+  for (int q = 0; q < npass; ++q) {
+    ++g_launches;
+    kern<<<g, kSortThreads, sh, s>>>(k0, v0, k1, v1, n, q, st, look, ++b.epoch, flag);
+  }
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }
 
-// Sort (keys, vals) by key bits [bit_begin, bit_end).  Input in (k0,v0);
-// on return *in_second says whether the result is in (k1,v1).
-int radix_sort_u64(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bit_begin,
-                   int bit_end, int* in_second, DBuf& hist, DBuf& scan_tmp, cudaStream_t s, uint64_t vary) {
+// Sort (keys, vals) by the lowest `bits` key bits, stable; the result is in
+// (k1, v1) if *in_second.
+int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
+                   int* in_second, int* flag, cudaStream_t s) {
   *in_second = 0;
-  if (n <= 1) return FMM_OK;
-  int ntiles = (int)((n + kSortTile - 1) / kSortTile);
-  FMM_TRY(hist.ensure((size_t)256 * ntiles * sizeof(uint32_t)));
-  uint64_t* ka = k0;
-  uint64_t* kb = k1;
-  uint32_t* va = v0;
-  uint32_t* vb = v1;
-  for (int shift = bit_begin; shift < bit_end; shift += 8) {
-    const int w = bit_end - shift < 8 ? bit_end - shift : 8;
-    if (((vary >> shift) & ((1ull << w) - 1ull)) == 0ull) continue;  // constant digit: identity pass
-    ++g_launches;
-    k_sort_hist<<<ntiles, kSortThreads, 0, s>>>(ka, n, shift, ntiles, hist.as<uint32_t>());
-    FMM_TRY(exclusive_scan_u32(hist.as<uint32_t>(), hist.as<uint32_t>(), (int64_t)256 * ntiles, nullptr,
-                               scan_tmp, s));
-    ++g_launches;
-    k_sort_scatter<<<ntiles, kSortThreads, 0, s>>>(ka, va, kb, vb, n, shift, ntiles, hist.as<uint32_t>());
-    FMM_CUDA_TRY(cudaGetLastError());
-    uint64_t* tk = ka;
-    ka = kb;
-    kb = tk;
-    uint32_t* tv = va;
-    va = vb;
-    vb = tv;
-    *in_second ^= 1;
-  }
+  if (n <= 1 || bits <= 0) return FMM_OK;
+  const int npass = (bits + 7) / 8;
+  FMM_TRY(sort_begin(b, n, s));
+  ++g_launches;
+  k_digit_hist<<<(unsigned)std::min<int64_t>(608, (n + 2047) / 2048), 256, 0, s>>>(k0, n, npass,
+                                                                                   &b.state.as<SortState>()->hist[0][0]);
+  FMM_TRY(sort_passes(b, k0, v0, k1, v1, n, npass, true, flag, s));
+  *in_second = npass & 1;
   return FMM_OK;
 }
 

@@ -5,17 +5,27 @@
 namespace fmm {
 int exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dev, DBuf& tmp,
                        cudaStream_t s);
-// Exclusive scans of three arrays of length n in shared passes; total_dev[3]
-// (if given) receives the three sums.  tmp holds the block sums, tmp2 the
-// scratch of their scans when n exceeds 16M.
-int exclusive_scan3_u32(const uint32_t* const in[3], uint32_t* const out[3], int64_t n, uint32_t* total_dev,
-                        DBuf& tmp, DBuf& tmp2, cudaStream_t s);
-int iota_u32(uint32_t* v, int64_t n, cudaStream_t s);
-// vary: the key bits that differ between keys (if known); a pass whose 8-bit
-// digit is the same in every key is the identity and is skipped.
-int radix_sort_u64(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bit_begin,
-                   int bit_end, int* in_second, DBuf& hist, DBuf& scan_tmp, cudaStream_t s,
-                   uint64_t vary = ~0ull);
+constexpr int kSortPasses = 8;  // 8-bit digits of a 64-bit key
+struct SortState {
+  uint32_t hist[kSortPasses][256], base[kSortPasses][256];
+  uint32_t ticket[kSortPasses];
+  int active[kSortPasses], sel[kSortPasses + 1];  // pass q reads buffer sel[q]; the result is in sel[npass]
+};
+// Scratch of the sort: one per stream that sorts.
+struct SortScratch {
+  DBuf state, look;
+  unsigned epoch = 0;
+};
+// A sort in two halves, for a kernel that makes the keys and counts their
+// digits (SortState::hist) itself: sort_begin clears the state; sort_passes
+// sorts by npass digits.  all: every pass runs, so the result is in buffer
+// npass & 1; else passes over a constant digit are left out and the result is
+// in buffer SortState::sel[npass], known on the device alone.
+int sort_begin(SortScratch& b, int64_t n, cudaStream_t s);
+int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int npass, bool all,
+                int* flag, cudaStream_t s);
+int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
+                   int* in_second, int* flag, cudaStream_t s);
 
 // A barrier over the blocks of a cooperative launch.  Every wait is bounded:
 // on expiry the blocks give up together (abort) and the barrier returns false.
@@ -25,6 +35,32 @@ struct GridBar {
 constexpr long long kGridSpin = 1ll << 24;
 
 #ifdef __CUDACC__
+// Adds the warp's keys to the block's digit counts h[npass][256] (all lanes
+// call it; a digit that is the same in every lane takes one atomic).
+__device__ __forceinline__ void count_digits(uint32_t* h, uint64_t key, bool live, int npass) {
+  const unsigned m = __ballot_sync(0xffffffffu, live);
+  if (!m) return;
+  const int lead = __ffs(m) - 1;
+  for (int q = 0; q < npass; ++q) {
+    const int d = (int)((key >> (8 * q)) & 0xff);
+    const int d0 = __shfl_sync(0xffffffffu, d, lead);
+    if (__all_sync(0xffffffffu, !live || d == d0)) {
+      if ((int)(threadIdx.x & 31) == lead) atomicAdd(&h[q * 256 + d0], (uint32_t)__popc(m));
+    } else if (live) {
+      atomicAdd(&h[q * 256 + d], 1u);
+    }
+  }
+}
+__device__ __forceinline__ void clear_digits(uint32_t* h, int npass) {
+  for (int i = threadIdx.x; i < npass * 256; i += blockDim.x) h[i] = 0u;
+  __syncthreads();
+}
+__device__ __forceinline__ void flush_digits(const uint32_t* h, int npass, uint32_t* hist) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < npass * 256; i += blockDim.x)
+    if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
 __device__ __forceinline__ bool grid_barrier(GridBar* st, unsigned nblocks) {
   __syncthreads();
   if (threadIdx.x == 0) {

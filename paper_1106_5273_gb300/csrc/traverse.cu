@@ -340,11 +340,21 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
 
 // ---- P2P CSR
 
-__global__ void k_p2p_keys(const int4* __restrict__ raw, int n, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  keys[i] = (uint64_t)raw[i].x;
-  vals[i] = (uint32_t)i;
+__global__ void __launch_bounds__(256) k_p2p_keys(const int4* __restrict__ raw, int n, uint64_t* __restrict__ keys,
+                                                  uint32_t* __restrict__ vals, int npass,
+                                                  uint32_t* __restrict__ hist) {
+  __shared__ uint32_t h[4 * 256];
+  clear_digits(h, npass);
+  for (int b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
+    const int i = b + threadIdx.x;
+    const uint64_t k = i < n ? (uint64_t)raw[i].x : 0ull;
+    if (i < n) {
+      keys[i] = k;
+      vals[i] = (uint32_t)i;
+    }
+    count_digits(h, k, i < n, npass);
+  }
+  flush_digits(h, npass, hist);
 }
 
 // Entries in leaf order: (first source particle, image) and the source count;
@@ -793,8 +803,8 @@ static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
   k_tile_order_keys<<<gc, T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc, p->lk0.as<uint64_t>(),
                                      p->lv0.as<uint32_t>(), gcount);
   int second = 0;
-  FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
-                         nc, 0, 8, &second, p->sort_hist, p->scan_tmp, s));
+  FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
+                         nc, 8, &second, p->flags.as<int>(), s));
   ++g_launches;
   k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, ntiles, rng);
   ++g_launches;
@@ -823,10 +833,12 @@ static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t
   FMM_CUDA_TRY(cudaMemsetAsync(dpairs, 0, 2 * sizeof(unsigned long long), s));
   const unsigned g = std::max(1u, (unsigned)((n + T - 1) / T));
   ++g_launches;
-  k_p2p_keys<<<g, T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
-  int second = 0;
-  FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
-                         n, 0, bits_for(p->ncells), &second, p->sort_hist, p->scan_tmp, s));
+  const int npass = bits_for(p->ncells) / 8, second = npass & 1;  // at most 4: cells are fewer than 2^27
+  FMM_TRY(sort_begin(p->sort, std::max(n, 1), s));
+  k_p2p_keys<<<std::min(g, 608u), T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(),
+                                             npass, &p->sort.state.as<SortState>()->hist[0][0]);
+  FMM_TRY(sort_passes(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                      p->lv1.as<uint32_t>(), std::max(n, 1), npass, true, p->flags.as<int>(), s));
   uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
   uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
   ++g_launches;
@@ -1075,8 +1087,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
           k_bucket_keys<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(), (int)nkeys, p->lk0.as<uint64_t>(),
                                          p->lv0.as<uint32_t>());
           int second = 0;
-          FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                                 p->lv1.as<uint32_t>(), nkeys, 0, 3, &second, p->sort_hist, p->scan_tmp, s));
+          FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                                 p->lv1.as<uint32_t>(), nkeys, 3, &second, p->flags.as<int>(), s));
           // the sorted bucket numbers are not needed: their buffer takes the keys in the new order
           uint64_t* out = second ? p->lk0.as<uint64_t>() : p->lk1.as<uint64_t>();
           k_bucket_order<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(),
@@ -1132,8 +1144,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
                                    nsub, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       int second = 0;
-      FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), n, 0, tb + kp.bits, &second, p->sort_hist, p->scan_tmp, s));
+      FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, p->flags.as<int>(), s));
       uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
@@ -1161,9 +1173,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       unsigned gs = (unsigned)((ns + T - 1) / T);
       ++g_launches;
       k_copy_u64_iota<<<gs, T, 0, s>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
-      FMM_TRY(radix_sort_u64(p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), ns, 0, std::max(kp.bits, 1), &second, p->sort_hist, p->scan_tmp,
-                             s));
+      FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
+                             p->lv1.as<uint32_t>(), ns, std::max(kp.bits, 1), &second, p->flags.as<int>(), s));
       sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;

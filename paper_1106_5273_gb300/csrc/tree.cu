@@ -174,54 +174,58 @@ __device__ inline uint64_t quantize_axis(float x, double bmin, double f, double 
 }
 
 // kbits Morton bits per axis; a batch puts the problem index above them.
-// span (if given) gathers the AND and the OR of all keys (one atomic each per
-// warp): their XOR marks the key bits that vary.
-__global__ void k_keys(const float* __restrict__ pos, int64_t n, const double* __restrict__ box,
-                       const int* __restrict__ off, int nseg, int kbits, uint64_t* __restrict__ keys,
-                       uint32_t* __restrict__ idx, unsigned long long* __restrict__ span) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long ka = ~0ull, ko = 0ull;
+// hist (if given): the digit counts of the sort.
+__global__ void __launch_bounds__(256) k_keys(const float* __restrict__ pos, int64_t n, const double* __restrict__ box,
+                                              const int* __restrict__ off, int nseg, int kbits,
+                                              uint64_t* __restrict__ keys, uint32_t* __restrict__ idx, int npass,
+                                              uint32_t* __restrict__ hist) {
+  __shared__ uint32_t h[kSortPasses * 256];
+  __shared__ double f0;
   const double scale = ldexp(1.0, kbits);
   // one problem: f once per block (FP64 division is slow)
-  __shared__ double f0;
-  if (!off) {
-    if (threadIdx.x == 0) f0 = __ddiv_rn(scale, box[3]);
-    __syncthreads();
+  if (!off && threadIdx.x == 0) f0 = __ddiv_rn(scale, box[3]);
+  clear_digits(h, npass);
+  for (int64_t b0 = (int64_t)blockIdx.x * blockDim.x; b0 < n; b0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = b0 + threadIdx.x;
+    uint64_t k = 0ull;
+    if (i < n) {
+      const int sg = off ? seg_of(off, nseg, i) : 0;
+      const double* b = box + 4 * sg;
+      const double f = off ? __ddiv_rn(scale, b[3]) : f0;
+      const uint64_t kx = quantize_axis(pos[3 * i + 0], b[0], f, scale);
+      const uint64_t ky = quantize_axis(pos[3 * i + 1], b[1], f, scale);
+      const uint64_t kz = quantize_axis(pos[3 * i + 2], b[2], f, scale);
+      k = ((uint64_t)sg << (3 * kbits)) | (spread3(kx) << 2) | (spread3(ky) << 1) | spread3(kz);
+      keys[i] = k;
+      idx[i] = (uint32_t)i;
+    }
+    if (hist) count_digits(h, k, i < n, npass);
   }
-  if (i < n) {
-    const int sg = off ? seg_of(off, nseg, i) : 0;
-    const double* b = box + 4 * sg;
-    const double f = off ? __ddiv_rn(scale, b[3]) : f0;
-    uint64_t kx = quantize_axis(pos[3 * i + 0], b[0], f, scale);
-    uint64_t ky = quantize_axis(pos[3 * i + 1], b[1], f, scale);
-    uint64_t kz = quantize_axis(pos[3 * i + 2], b[2], f, scale);
-    const uint64_t k = ((uint64_t)sg << (3 * kbits)) | (spread3(kx) << 2) | (spread3(ky) << 1) | spread3(kz);
-    keys[i] = k;
-    idx[i] = (uint32_t)i;
-    ka = ko = k;
-  }
-  if (!span) return;
-  for (int o = 16; o > 0; o >>= 1) {
-    ka &= __shfl_xor_sync(0xffffffffu, ka, o);
-    ko |= __shfl_xor_sync(0xffffffffu, ko, o);
-  }
-  if ((threadIdx.x & 31) == 0 && (int64_t)blockIdx.x * blockDim.x + threadIdx.x < n) {
-    atomicAnd(&span[0], ka);
-    atomicOr(&span[1], ko);
-  }
+  if (hist) flush_digits(h, npass, hist);
 }
 
-// Sorted position i of a batch lies in its problem's input range.
+// Sorted position i of a batch lies in its problem's input range.  The sort
+// left its result in one of two buffers (sel, known on the device); the keys
+// and indices end up in the first.
 __global__ void k_permute(const float* __restrict__ pos, const float* __restrict__ gam,
                           const float* __restrict__ sig, float sig_u, const float* __restrict__ seg_sig,
-                          const int* __restrict__ off, int nseg, const uint32_t* __restrict__ idx,
-                          int64_t n, float4* __restrict__ A, float4* __restrict__ B) {
+                          const int* __restrict__ off, int nseg, uint64_t* __restrict__ k0, uint32_t* __restrict__ v0,
+                          const uint64_t* __restrict__ k1, const uint32_t* __restrict__ v1,
+                          const int* __restrict__ sel, int64_t n, float4* __restrict__ A, float4* __restrict__ B) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  uint32_t j = idx[i];
+  uint32_t j;
+  if (*sel) {
+    j = v1[i];
+    v0[i] = j;
+    k0[i] = k1[i];
+  } else {
+    j = v0[i];
+  }
+  const size_t q = 3 * (size_t)j;
   float s = sig ? sig[j] : (seg_sig ? seg_sig[seg_of(off, nseg, i)] : sig_u);
-  A[i] = make_float4(pos[3 * j], pos[3 * j + 1], pos[3 * j + 2], s);
-  B[i] = make_float4(gam[3 * j], gam[3 * j + 1], gam[3 * j + 2], 0.f);
+  A[i] = make_float4(pos[q], pos[q + 1], pos[q + 2], s);
+  B[i] = make_float4(gam[q], gam[q + 1], gam[q + 2], 0.f);
 }
 
 __global__ void k_sigma_max(const float* __restrict__ sig, int64_t n, unsigned int* __restrict__ out) {
@@ -635,6 +639,24 @@ static int tree_from_sorted(fmm_plan p, int64_t n, int nroot, const int* off, co
   return FMM_OK;
 }
 
+// Keys and their sort; passes over digits that no key changes are left out (a
+// lattice leaves its low bits constant).
+static int sort_particles(fmm_plan p, const float* pos, int64_t n, const double* box, const int* off, int nseg,
+                          int kbits, int bits, cudaStream_t s) {
+  const int npass = (bits + 7) / 8;
+  p->skeys = p->keys0.as<uint64_t>();
+  p->sidx = p->vals0.as<uint32_t>();
+  FMM_TRY(sort_begin(p->sort, n, s));
+  ++g_launches;
+  k_keys<<<(unsigned)std::min<int64_t>(608, (n + 255) / 256), 256, 0, s>>>(
+      pos, n, box, off, nseg, kbits, p->skeys, p->sidx, npass, &p->sort.state.as<SortState>()->hist[0][0]);
+  FMM_CUDA_TRY(cudaGetLastError());
+  return sort_passes(p->sort, p->keys0.as<uint64_t>(), p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(),
+                     p->vals1.as<uint32_t>(), n, npass, false, p->flags.as<int>(), s);
+}
+
+static const int* sorted_sel(fmm_plan p, int bits) { return &p->sort.state.as<SortState>()->sel[(bits + 7) / 8]; }
+
 // Keys, sort, permutation into sorted SoA, octree, centres, radii.
 int build_tree(fmm_plan p, int64_t n, const float* pos, const float* gam, const float* sig, float sig_u,
                cudaStream_t s) {
@@ -663,29 +685,11 @@ int build_tree(fmm_plan p, int64_t n, const float* pos, const float* gam, const 
     ++g_launches;
     k_sigma_max<<<parts, 256, 0, s>>>(sig, n, smax);
   }
-  uint64_t* k0 = p->keys0.as<uint64_t>();
-  uint64_t* k1 = p->keys1.as<uint64_t>();
-  uint32_t* v0 = p->vals0.as<uint32_t>();
-  uint32_t* v1 = p->vals1.as<uint32_t>();
-  unsigned long long* span = reinterpret_cast<unsigned long long*>(box + kScalKeySpan);
-  FMM_CUDA_TRY(cudaMemsetAsync(span, 0xff, sizeof(unsigned long long), s));
-  FMM_CUDA_TRY(cudaMemsetAsync(span + 1, 0, sizeof(unsigned long long), s));
+  FMM_TRY(sort_particles(p, pos, n, box, nullptr, 1, kMaxLevel, 3 * kMaxLevel, s));
   ++g_launches;
-  k_keys<<<nb, T, 0, s>>>(pos, n, box, nullptr, 1, kMaxLevel, k0, v0, span);
-  FMM_CUDA_TRY(cudaGetLastError());
-  // sort passes over digits that no key changes are skipped (a lattice leaves
-  // its low bits constant)
-  unsigned long long* hspan = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 512);
-  FMM_CUDA_TRY(cudaMemcpyAsync(hspan, span, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  FMM_CUDA_TRY(cudaStreamSynchronize(s));
-  const uint64_t vary = hspan[0] ^ hspan[1];
-  int second = 0;
-  FMM_TRY(radix_sort_u64(k0, v0, k1, v1, n, 0, 63, &second, p->sort_hist, p->scan_tmp, s, vary));
-  p->skeys = second ? k1 : k0;
-  p->sidx = second ? v1 : v0;
-  ++g_launches;
-  k_permute<<<nb, T, 0, s>>>(pos, gam, sig, sig_u, nullptr, nullptr, 1, p->sidx, n, p->sortA.as<float4>(),
-                             p->sortB.as<float4>());
+  k_permute<<<nb, T, 0, s>>>(pos, gam, sig, sig_u, nullptr, nullptr, 1, p->keys0.as<uint64_t>(),
+                             p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(), p->vals1.as<uint32_t>(),
+                             sorted_sel(p, 3 * kMaxLevel), n, p->sortA.as<float4>(), p->sortB.as<float4>());
   FMM_CUDA_TRY(cudaGetLastError());
   return tree_from_sorted(p, n, 1, nullptr, box, kMaxLevel, false, s);
 }
@@ -750,29 +754,15 @@ int build_forest(fmm_plan p, int64_t n, const float* pos, const float* gam, cons
     ++g_launches;
     k_sigma_max_seg<<<S, 256, 0, s>>>(sig, off, p->seg_smax.as<unsigned int>());
   }
-  uint64_t* k0 = p->keys0.as<uint64_t>();
-  uint64_t* k1 = p->keys1.as<uint64_t>();
-  uint32_t* v0 = p->vals0.as<uint32_t>();
-  uint32_t* v1 = p->vals1.as<uint32_t>();
-  unsigned long long* span = reinterpret_cast<unsigned long long*>(p->scal.as<double>() + kScalKeySpan);
-  FMM_CUDA_TRY(cudaMemsetAsync(span, 0xff, sizeof(unsigned long long), s));
-  FMM_CUDA_TRY(cudaMemsetAsync(span + 1, 0, sizeof(unsigned long long), s));
-  ++g_launches;
-  k_keys<<<nb, T, 0, s>>>(pos, n, box, off, S, kBatchBits, k0, v0, span);
-  FMM_CUDA_TRY(cudaGetLastError());
-  unsigned long long* hspan = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(p->pinned) + 512);
-  FMM_CUDA_TRY(cudaMemcpyAsync(hspan, span, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  FMM_CUDA_TRY(cudaStreamSynchronize(s));
   int sbits = 0;
   while ((1 << sbits) < S) ++sbits;
-  int second = 0;
-  FMM_TRY(radix_sort_u64(k0, v0, k1, v1, n, 0, 3 * kBatchBits + sbits, &second, p->sort_hist, p->scan_tmp, s,
-                         hspan[0] ^ hspan[1]));
-  p->skeys = second ? k1 : k0;
-  p->sidx = second ? v1 : v0;
+  const int bits = 3 * kBatchBits + sbits;
+  FMM_TRY(sort_particles(p, pos, n, box, off, S, kBatchBits, bits, s));
   ++g_launches;
-  k_permute<<<nb, T, 0, s>>>(pos, gam, sig, 0.f, sig ? nullptr : p->seg_sig.as<float>(), off, S, p->sidx, n,
-                             p->sortA.as<float4>(), p->sortB.as<float4>());
+  k_permute<<<nb, T, 0, s>>>(pos, gam, sig, 0.f, sig ? nullptr : p->seg_sig.as<float>(), off, S,
+                             p->keys0.as<uint64_t>(), p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(),
+                             p->vals1.as<uint32_t>(), sorted_sel(p, bits), n, p->sortA.as<float4>(),
+                             p->sortB.as<float4>());
   FMM_CUDA_TRY(cudaGetLastError());
   return tree_from_sorted(p, n, S, off, box, kBatchBits, true, s);
 }
@@ -796,7 +786,7 @@ int morton_keys_raw(int64_t n, const float* pos, int periodic, const double* box
     k_bbox_final<<<1, 256, 0, s>>>(partials, parts, box);
   }
   ++g_launches;
-  k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, n, box, nullptr, 1, kMaxLevel, keys, idx, nullptr);
+  k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, n, box, nullptr, 1, kMaxLevel, keys, idx, 0, nullptr);
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }
