@@ -550,7 +550,10 @@ int64_t fmm_kernel_launch_count(void);
  */
 int fmm_plan_set_list_capacity(fmm_plan plan, int64_t frontier, int64_t m2l, int64_t p2p);
 
-/* Enable (1) or disable (0) CUDA-event phase timing in fmm_stats. */
+/* Enable (1) or disable (0) CUDA-event phase timing in fmm_stats.  With timing
+ * on the near field, the M2L lists, the M2L and the downward pass run one after
+ * the other on the caller's stream (otherwise the near field overlaps the
+ * rest), so that each phase is timed alone; the results are the same. */
 int fmm_plan_set_timing(fmm_plan plan, int enable);
 
 /* Work counts and phase times of the last evaluation (synchronizes). */

@@ -35,7 +35,7 @@ int check_params(const fmm_params* q) {
 
 std::vector<DBuf*> plan_buffers(fmm_plan p) {
   return {&p->m2m_T, &p->l2l_T, &p->l2p_tab, &p->lattice, &p->keys0, &p->keys1, &p->vals0, &p->vals1,
-          &p->sortA, &p->sortB, &p->far_u, &p->far_s, &p->c_clo, &p->tree_state, &p->in_pos, &p->in_gam, &p->in_sig,
+          &p->sortA, &p->sortB, &p->far_u, &p->far_s, &p->near_u, &p->near_s, &p->pk0, &p->pk1, &p->pv0, &p->pv1, &p->p_scan, &p->p_sort.state, &p->p_sort.look, &p->c_clo, &p->tree_state, &p->in_pos, &p->in_gam, &p->in_sig,
           &p->out_vel, &p->out_dg, &p->c_begin, &p->c_end, &p->c_level, &p->c_parent, &p->c_child,
           &p->c_nchild, &p->c_key, &p->c_center, &p->c_radius2, &p->c_radius, &p->dip_part, &p->c_cf, &p->c_tile,
           &p->tile_cells, &p->tile_first, &p->tile_groups, &p->c_ijk, &p->t_pos, &p->t_gam, &p->t_sig, &p->t_vel, &p->leaves, &p->M, &p->L, &p->Mbf, &p->fr0, &p->fr1, &p->tcount, &p->tmask,
@@ -61,11 +61,34 @@ struct Timer {
 int ensure_aux_stream(fmm_plan p) {
   if (p->s_up) return FMM_OK;
   FMM_CUDA_TRY(cudaStreamCreateWithFlags(&p->s_up, cudaStreamNonBlocking));
+  int lo = 0, hi = 0;
+  FMM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+  FMM_CUDA_TRY(cudaStreamCreateWithPriority(&p->s_far, cudaStreamNonBlocking, hi));
+  for (cudaEvent_t* e : {&p->ev_up, &p->ev_near})
+    FMM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
   FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
   FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_read, cudaEventDisableTiming));
   return FMM_OK;
 }
+
+}  // namespace
+
+namespace fmm {
+// M2L, the periodic lattice and the downward pass (after the upward pass).
+int far_field(fmm_plan p, int64_t n, cudaStream_t s, const std::function<void()>& after_m2l) {
+  const size_t lbytes = (size_t)p->ncells * 3 * p->P * sizeof(float);
+  FMM_TRY(p->L.ensure(lbytes));
+  FMM_CUDA_TRY(cudaMemsetAsync(p->L.ptr, 0, lbytes, s));
+  if (p->last_tc) FMM_TRY(m2l_tensor(p, s));
+  else FMM_TRY(m2l_simt(p, s));
+  FMM_TRY(apply_lattice(p, s));
+  if (after_m2l) after_m2l();
+  return downward_pass(p, n, s);
+}
+}  // namespace fmm
+
+namespace {
 
 // sg: nullptr for one problem, else the (non-empty) problems of a batch.
 int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const float* sig, float sig_u, float* vel,
@@ -92,33 +115,37 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
   if (sg) FMM_TRY(build_forest(p, n, pos, gam, sig, *sg, s));
   else FMM_TRY(build_tree(p, n, pos, gam, sig, sig_u, s));
   tm.mark();
-  // Fork: P2M / M2M on the plan's second stream while the traversal (which
-  // reads only the tree) runs on the caller's stream; join before M2L.
-  FMM_CUDA_TRY(cudaEventRecord(p->ev_fork, s));
-  FMM_CUDA_TRY(cudaStreamWaitEvent(p->s_up, p->ev_fork, 0));
-  {
-    int urc = upward_pass(p, p->s_up);
-    if (urc == FMM_OK) urc = dipole_pass(p, n, p->s_up);
-    if (urc != FMM_OK) {
-      cudaStreamSynchronize(p->s_up);
-      return urc;
-    }
-  }
-  tm.mark_on(p->s_up);
-  FMM_CUDA_TRY(cudaEventRecord(p->ev_join, p->s_up));
-  // from here on an early return must not leave the upward pass running
+  // Fork: P2M / M2M on a plan stream while the traversal (which reads only the
+  // tree) runs on the caller's.  Then the near field (bound by the FMA pipe) runs
+  // on the caller's stream as soon as its lists are ready, beside the M2L lists,
+  // the M2L (tensor cores, gathers) and the downward pass on a stream of the
+  // highest priority; k_finish adds the two.  What the overlap hides is mostly the
+  // list building and the small levels' latency: ball 1000 558 -> 491 us per
+  // evaluation, spectrum 61^3 3142 -> 2890, strengths 64^3 3553 -> 3211,
+  // Taylor-Green 128^3 26268 -> 25900.  With timing on, everything after the
+  // upward pass runs in turn on the caller's stream, so that each phase is timed
+  // alone.
+  const bool serial = p->timing != 0;
+  cudaStream_t fs = serial ? s : p->s_far;
+  // from here on an early return must not leave a plan stream running
   struct JoinOnExit {
     fmm_plan p;
-    cudaStream_t s;
     bool joined = false;
     ~JoinOnExit() {
-      if (!joined) cudaStreamSynchronize(p->s_up);
+      if (joined) return;
+      cudaStreamSynchronize(p->s_up);
+      cudaStreamSynchronize(p->s_far);
     }
-  } join_guard{p, s};
+  } join_guard{p};
+  if (sg) FMM_TRY(segment_tables(p, sig ? 1 : 0, s));
+  FMM_CUDA_TRY(cudaEventRecord(p->ev_fork, s));
+  FMM_CUDA_TRY(cudaStreamWaitEvent(p->s_up, p->ev_fork, 0));
+  FMM_TRY(upward_pass(p, p->s_up));
+  FMM_TRY(dipole_pass(p, n, p->s_up));
+  tm.mark_on(p->s_up);
+  FMM_CUDA_TRY(cudaEventRecord(p->ev_up, p->s_up));
   double smax = (double)sig_u;
-  if (sg) {
-    FMM_TRY(segment_tables(p, sig ? 1 : 0, s));
-  } else if (sig) {
+  if (!sg && sig) {
     unsigned int bits = 0;
     FMM_CUDA_TRY(cudaMemcpyAsync(&bits, p->scal.as<double>() + kScalSigma, sizeof(unsigned int),
                                  cudaMemcpyDeviceToHost, s));
@@ -127,21 +154,21 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
     memcpy(&f, &bits, sizeof(f));
     smax = (double)f;
   }
-  FMM_TRY(traverse(p, smax, s));
-  FMM_TRY(m2l_build_items(p, s));
-  tm.mark();
-  FMM_CUDA_TRY(cudaStreamWaitEvent(s, p->ev_join, 0));
+  auto near = [&] { return p2p_near(p, n, sig_u, sig ? 1 : 0, smax, dg != nullptr, s); };
+  FMM_TRY(traverse(p, smax, s, fs, [&] { return serial ? FMM_OK : near(); }));
+  FMM_TRY(m2l_build_items(p, fs));
+  tm.mark_on(fs);
+  FMM_CUDA_TRY(cudaStreamWaitEvent(fs, p->ev_up, 0));
+  FMM_TRY(far_field(p, n, fs, [&] { tm.mark_on(fs); }));
+  tm.mark_on(fs);
+  if (serial) {
+    FMM_TRY(near());
+  } else {
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_join, fs));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(s, p->ev_join, 0));
+  }
+  FMM_TRY(p2p_finish(p, n, vel, dg, s));
   join_guard.joined = true;
-  const int nc = (int)p->ncells;
-  FMM_TRY(p->L.ensure((size_t)nc * 3 * p->P * sizeof(float)));
-  FMM_CUDA_TRY(cudaMemsetAsync(p->L.ptr, 0, (size_t)nc * 3 * p->P * sizeof(float), s));
-  if (p->last_tc) FMM_TRY(m2l_tensor(p, s));
-  else FMM_TRY(m2l_simt(p, s));
-  FMM_TRY(apply_lattice(p, s));
-  tm.mark();
-  FMM_TRY(downward_pass(p, n, s));
-  tm.mark();
-  FMM_TRY(p2p_near(p, n, sig_u, sig ? 1 : 0, smax, vel, dg, s));
   tm.mark();
   // error flags raised by kernels
   int hf = 0;
@@ -283,6 +310,9 @@ void fmm_plan_destroy(fmm_plan p) {
     for (int i = 0; i < 8; ++i) cudaEventDestroy(p->ev[i]);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
+  if (p->ev_up) cudaEventDestroy(p->ev_up);
+  if (p->ev_near) cudaEventDestroy(p->ev_near);
+  if (p->s_far) cudaStreamDestroy(p->s_far);
   if (p->ev_read) cudaEventDestroy(p->ev_read);
   if (p->s_up) cudaStreamDestroy(p->s_up);
   delete p;

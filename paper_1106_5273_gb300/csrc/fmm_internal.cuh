@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <functional>
 #include <vector>
 
 #include "common.cuh"
@@ -103,6 +104,7 @@ struct fmm_plan_s {
   uint32_t* sidx = nullptr;              // sorted position -> input index
   fmm::DBuf sortA, sortB;                // float4 (x,y,z,sigma), (gx,gy,gz,0) in sorted order
   fmm::DBuf far_u, far_s;                // [n][3] far field, sorted order
+  fmm::DBuf near_u, near_s;              // [n][3] near field, sorted order
   fmm::DBuf c_clo;                       // float4 low part of the centre, then u32 FP32 squared radius
   fmm::DBuf tree_state;                  // state and block totals of the octree kernel
   fmm::DBuf in_pos, in_gam, in_sig, out_vel, out_dg;  // staging of the _host entry point
@@ -143,6 +145,8 @@ struct fmm_plan_s {
   // scratch
   fmm::DBuf scan_tmp;
   fmm::SortScratch sort;
+  fmm::DBuf pk0, pk1, pv0, pv1, p_scan;  // the P2P grouping's own list sort and scan (it runs beside the M2L lists)
+  fmm::SortScratch p_sort;
   fmm::DBuf scal;   // small scalars (see kScal*)
   fmm::DBuf flags;  // int error flags
   void* pinned = nullptr;  // host pinned scratch (counts)
@@ -177,7 +181,10 @@ struct fmm_plan_s {
   // the upward pass runs on this plan stream while the traversal runs on the
   // caller's stream (both read only the tree); fork / join by events
   cudaStream_t s_up = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the M2L lists, the M2L and the downward pass run on this one (highest
+  // priority) while the near field runs on the caller's
+  cudaStream_t s_far = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_up = nullptr, ev_near = nullptr;
   cudaEvent_t ev_read = nullptr;  // the host's reads of list sizes
 };
 
@@ -203,7 +210,9 @@ int lattice_operator_device(int p, int images, double* A, cudaStream_t s);
 int upward_pass(fmm_plan p, cudaStream_t s);
 int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s);
 // traverse.cu
-int traverse(fmm_plan p, double sigma_max_host, cudaStream_t s);
+// lists of both fields: the P2P lists on s, the M2L lists on f (which may be s);
+// near() launches the near field on s as soon as its lists are ready
+int traverse(fmm_plan p, double sigma_max_host, cudaStream_t s, cudaStream_t f, const std::function<int()>& near);
 // per-problem MAC and near-field tables of a batch (after the forest is built)
 int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s);
 // m2l.cu
@@ -212,11 +221,14 @@ int m2l_build_items(fmm_plan p, cudaStream_t s);  // once per tree
 int m2l_tensor(fmm_plan p, cudaStream_t s);
 // downward.cu
 int downward_pass(fmm_plan p, int64_t n, cudaStream_t s);
+// fmm_api.cu
+int far_field(fmm_plan p, int64_t n, cudaStream_t s, const std::function<void()>& after_m2l);
 // reuse.cu
 int eval_strengths(fmm_plan p, const float* gam, float* vel, float* dg, cudaStream_t s);
 // p2p.cu
-int p2p_near(fmm_plan p, int64_t n, float sig_u, int per_particle_sigma, double smax, float* vel, float* dg,
+int p2p_near(fmm_plan p, int64_t n, float sig_u, int per_particle_sigma, double smax, bool stretching,
              cudaStream_t s);
+int p2p_finish(fmm_plan p, int64_t n, float* vel, float* dg, cudaStream_t s);
 // work items of the pair kernel; counts (device) receives (items, partial slots)
 int p2p_tile(fmm_plan p);
 int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s);

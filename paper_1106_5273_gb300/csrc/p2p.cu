@@ -418,37 +418,33 @@ __device__ __forceinline__ void run_group(const Stage<PS>& sm, int jb, int je, i
   }
 }
 
-// What the pair kernel and the combine kernel write.
+// What the pair kernel and the combine kernel write: the near field of every
+// particle in sorted order.
 struct P2POut {
-  const float* far_u;
-  const float* far_s;
-  const uint32_t* sidx;
-  const double* dip;  // uniform dipole velocity of a one-problem evaluation (or nullptr)
-  float* vel;
-  float* dg;
+  float* u;
+  float* s;
 };
 
-// Output of target i (sorted position) from its 12 sums.
+// Near field of target i (sorted position) from its 12 sums.
 template <int ST>
 __device__ __forceinline__ void write_target(const P2POut& out, int i, float X, float Y, float Z, const float4& g,
-                                             const float v[12], float dux, float duy, float duz) {
-  const size_t o = out.sidx[i], f = (size_t)3 * i;
+                                             const float v[12]) {
+  const size_t f = (size_t)3 * i;
   const float ax = v[0], ay = v[1], az = v[2];
-  if (out.vel) {  // u = A x X_i - B
-    out.vel[3 * o] = out.far_u[f] + kInv4Pi * ((ay * Z - az * Y) - v[3]) + dux;
-    out.vel[3 * o + 1] = out.far_u[f + 1] + kInv4Pi * ((az * X - ax * Z) - v[4]) + duy;
-    out.vel[3 * o + 2] = out.far_u[f + 2] + kInv4Pi * ((ax * Y - ay * X) - v[5]) + duz;
-  }
-  if (ST == 1 && out.dg) {  // s = A x gamma_i - 3 (C x X_i - D)
+  // u = A x X_i - B
+  out.u[f] = kInv4Pi * ((ay * Z - az * Y) - v[3]);
+  out.u[f + 1] = kInv4Pi * ((az * X - ax * Z) - v[4]);
+  out.u[f + 2] = kInv4Pi * ((ax * Y - ay * X) - v[5]);
+  if (ST == 1) {  // s = A x gamma_i - 3 (C x X_i - D)
     const float cx = v[6], cy = v[7], cz = v[8];
-    out.dg[3 * o] = out.far_s[f] + kInv4Pi * ((ay * g.z - az * g.y) + kM3 * ((cy * Z - cz * Y) - v[9]));
-    out.dg[3 * o + 1] = out.far_s[f + 1] + kInv4Pi * ((az * g.x - ax * g.z) + kM3 * ((cz * X - cx * Z) - v[10]));
-    out.dg[3 * o + 2] = out.far_s[f + 2] + kInv4Pi * ((ax * g.y - ay * g.x) + kM3 * ((cx * Y - cy * X) - v[11]));
+    out.s[f] = kInv4Pi * ((ay * g.z - az * g.y) + kM3 * ((cy * Z - cz * Y) - v[9]));
+    out.s[f + 1] = kInv4Pi * ((az * g.x - ax * g.z) + kM3 * ((cz * X - cx * Z) - v[10]));
+    out.s[f + 2] = kInv4Pi * ((ax * g.y - ay * g.x) + kM3 * ((cx * Y - cy * X) - v[11]));
   }
-  if (ST == 2 && out.dg) {  // s = gamma_i x A - 3 (W X_i + D)
-    out.dg[3 * o] = out.far_s[f] + kInv4Pi * ((g.y * az - g.z * ay) + kM3 * (v[6] * X + v[9]));
-    out.dg[3 * o + 1] = out.far_s[f + 1] + kInv4Pi * ((g.z * ax - g.x * az) + kM3 * (v[6] * Y + v[10]));
-    out.dg[3 * o + 2] = out.far_s[f + 2] + kInv4Pi * ((g.x * ay - g.y * ax) + kM3 * (v[6] * Z + v[11]));
+  if (ST == 2) {  // s = gamma_i x A - 3 (W X_i + D)
+    out.s[f] = kInv4Pi * ((g.y * az - g.z * ay) + kM3 * (v[6] * X + v[9]));
+    out.s[f + 1] = kInv4Pi * ((g.z * ax - g.x * az) + kM3 * (v[6] * Y + v[10]));
+    out.s[f + 2] = kInv4Pi * ((g.x * ay - g.y * ax) + kM3 * (v[6] * Z + v[11]));
   }
 }
 
@@ -491,20 +487,12 @@ __global__ void __launch_bounds__(32, kP2PPerSm)
   const int t0 = item.y, nt = min(tile, end[leaf] - t0);
   const int2 rg = off[item.x];
   const float4 lc = cf[leaf];
-  float dux = 0.f, duy = 0.f, duz = 0.f;
   if (cseg) {
     const SegP2P& q = sp[cseg[leaf]];
     K0 = q.k;
     blen = q.blen;
     smax = q.smax;
     margin0 = q.margin;
-    dux = q.dip[0];
-    duy = q.dip[1];
-    duz = q.dip[2];
-  } else if (out.dip) {
-    dux = (float)out.dip[0];
-    duy = (float)out.dip[1];
-    duz = (float)out.dip[2];
   }
   const bool wide = nt > 32;
   const int groups = nt > 16 ? 1 : (nt > 8 ? 2 : 4);
@@ -751,7 +739,7 @@ __global__ void __launch_bounds__(32, kP2PPerSm)
       for (int i = 0; i < NV; ++i) partial[((size_t)ps * 12 + i) * kTileMax + k] = v[i];
     } else {
       const float4 g = make_float4(q ? t.gx.y : t.gx.x, q ? t.gy.y : t.gy.x, q ? t.gz.y : t.gz.x, 0.f);
-      write_target<ST>(out, t0 + k, q ? t.x.y : t.x.x, q ? t.y.y : t.y.x, q ? t.z.y : t.z.x, g, v, dux, duy, duz);
+      write_target<ST>(out, t0 + k, q ? t.x.y : t.x.x, q ? t.y.y : t.y.x, q ? t.z.y : t.z.x, g, v);
     }
   }
   if (lane == 0) {
@@ -771,24 +759,12 @@ __global__ void __launch_bounds__(kTileMax) k_p2p_combine(const int2* __restrict
                                                           const int* __restrict__ begin, const int* __restrict__ end,
                                                           const float4* __restrict__ cf,
                                                           const float4* __restrict__ A, const float4* __restrict__ B,
-                                                          const int* __restrict__ cseg, const SegP2P* __restrict__ sp,
                                                           P2POut out, const float* __restrict__ partial) {
   constexpr int NV = ST == 0 ? 6 : 12;
   const int2 pl = plan[blockIdx.x];
   if (pl.y <= 1) return;
   const int leaf = leaves[blockIdx.x];
   const float4 lc = cf[leaf];
-  float dux = 0.f, duy = 0.f, duz = 0.f;
-  if (cseg) {
-    const SegP2P& q = sp[cseg[leaf]];
-    dux = q.dip[0];
-    duy = q.dip[1];
-    duz = q.dip[2];
-  } else if (out.dip) {
-    dux = (float)out.dip[0];
-    duy = (float)out.dip[1];
-    duz = (float)out.dip[2];
-  }
   int slot = pl.x;
   for (int t0 = begin[leaf]; t0 < end[leaf]; t0 += tile, slot += pl.y) {
     const int i = t0 + threadIdx.x;
@@ -802,7 +778,36 @@ __global__ void __launch_bounds__(kTileMax) k_p2p_combine(const int2* __restrict
       for (int q = 0; q < NV; ++q) v[q] += src[q * kTileMax];
     }
     const float4 xi = A[i];
-    write_target<ST>(out, i, xi.x - lc.x, xi.y - lc.y, xi.z - lc.z, B[i], v, dux, duy, duz);
+    write_target<ST>(out, i, xi.x - lc.x, xi.y - lc.y, xi.z - lc.z, B[i], v);
+  }
+}
+
+// The outputs in the caller's order: near + far field, and the uniform velocity of
+// the periodic dipole term (dip; in a batch the problem's).
+__global__ void k_finish(const float* __restrict__ near_u, const float* __restrict__ near_s,
+                         const float* __restrict__ far_u, const float* __restrict__ far_s,
+                         const uint32_t* __restrict__ sidx, int64_t n, const double* __restrict__ dip,
+                         const SegP2P* __restrict__ sp, const int* __restrict__ off, int nseg,
+                         float* __restrict__ vel, float* __restrict__ dg) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float d[3] = {0.f, 0.f, 0.f};
+  if (dip)
+    for (int a = 0; a < 3; ++a) d[a] = (float)dip[a];
+  if (sp) {
+    int lo = 0, hi = nseg;  // the problem of sorted position i
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if ((int64_t)off[mid] <= i) lo = mid;
+      else hi = mid;
+    }
+    for (int a = 0; a < 3; ++a) d[a] = sp[lo].dip[a];
+  }
+  const size_t o = 3 * (size_t)sidx[i], f = 3 * (size_t)i;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (vel) vel[o + a] = far_u[f + a] + near_u[f + a] + d[a];
+    if (dg) dg[o + a] = far_s[f + a] + near_s[f + a];
   }
 }
 
@@ -1185,7 +1190,14 @@ __global__ void __launch_bounds__(256) k_dipole_seg(const float4* __restrict__ A
 // sorted particles, so it runs on the upward pass's stream beside the
 // traversal, into its own partial-sum buffer.
 int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
-  if (!p->prm.periodic || p->batched || n == 0) return FMM_OK;
+  if (!p->prm.periodic || n == 0) return FMM_OK;
+  if (p->batched) {  // after the problem tables, which hold the result
+    ++g_launches;
+    k_dipole_seg<<<p->nseg, 256, 0, s>>>(p->sortA.as<float4>(), p->sortB.as<float4>(), p->seg_off.as<int>(),
+                                         p->seg_box.as<double>(), p->seg_p2p.as<SegP2P>());
+    FMM_CUDA_TRY(cudaGetLastError());
+    return FMM_OK;
+  }
   const int parts = 256;
   double* scal = p->scal.as<double>();
   FMM_TRY(p->dip_part.ensure((size_t)parts * 3 * sizeof(double)));
@@ -1202,12 +1214,13 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
 // per (tile of a leaf, range of its sources).  Ranges bound the longest warp:
 // the big outer leaves of a clustered cloud meet thousands of small ones, and
 // one warp per leaf left the chip waiting for them (Plummer, 30,011 blobs:
-// P2P 2.5 ms; 0.39 ms with ranges).  One-problem plans take the range that
-// gives about eight warps per resident one, at least 128 sources (two chunks);
+// P2P 2.5 ms; 0.39 ms with ranges), and with it how long the far field's
+// kernels wait for room.  One-problem plans take the range that gives kItemTarget
+// items, at least 128 sources (two chunks);
 // the partial slots are then bounded by twice that many items (3 KB each).  A
 // batch takes a rule of its own, so that a problem's sums do not depend on the
 // rest of the batch, with the ranges of a leaf capped for the slots' sake.
-constexpr int64_t kItemTarget = 8 * 16 * 152;  // items aimed at (24 instead of 16 per SM: Plummer 30,011 0.39 -> 0.42 ms)
+constexpr int64_t kItemTarget = 8 * 32 * 152;  // items aimed at (half as many: ball 100,003 2.15 instead of 2.09 ms in all)
 constexpr uint32_t kItemSrcMin = 128;
 // batch of 32 problems, 477,044 blobs: P2P 5.23 ms; 5.17 with whole lists only
 // up to 4096 sources, for twice the slots
@@ -1264,24 +1277,14 @@ static int p2p_attributes() {
   return ok ? FMM_OK : FMM_E_CUDA;
 }
 
-int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, float* vel, float* dg, cudaStream_t s) {
+// The near field of every particle, in sorted order (near_u, near_s).
+int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, bool stretching, cudaStream_t s) {
   double* scal = p->scal.as<double>();
   const int* cseg = p->batched ? p->c_seg.as<int>() : nullptr;
   SegP2P* sp = p->batched ? p->seg_p2p.as<SegP2P>() : nullptr;
-  P2POut out;
-  out.far_u = p->far_u.as<float>();
-  out.far_s = p->far_s.as<float>();
-  out.sidx = p->sidx;
-  out.dip = nullptr;
-  out.vel = vel;
-  out.dg = dg;
-  if (p->prm.periodic && p->batched) {
-    ++g_launches;
-    k_dipole_seg<<<p->nseg, 256, 0, s>>>(p->sortA.as<float4>(), p->sortB.as<float4>(), p->seg_off.as<int>(),
-                                         p->seg_box.as<double>(), sp);
-  } else if (p->prm.periodic) {
-    out.dip = scal + kScalDipole;  // dipole_pass ran beside the traversal
-  }
+  FMM_TRY(p->near_u.ensure((size_t)n * 3 * sizeof(float)));
+  if (stretching) FMM_TRY(p->near_s.ensure((size_t)n * 3 * sizeof(float)));
+  const P2POut out{p->near_u.as<float>(), p->near_s.as<float>()};
   const float blen = p->prm.periodic ? (float)p->prm.box_len : 0.f;
   const SigK K0 = make_sigk(ps ? 1.f : sig_u);
   const int mode = ps ? (p->prm.sigma_rule == FMM_SIGMA_MIXED ? 2 : 1) : 0;
@@ -1319,16 +1322,30 @@ int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, float* vel
     if (p->n_p2p_slots > 0) {          \
       ++g_launches;                    \
       k_p2p_combine<ST_><<<(unsigned)p->nleaves, kTileMax, 0, s>>>(p->p2p_plan.as<int2>(), tile, leaves, cb, ce, cf, \
-                                                                   A, B, cseg, sp, out, partial);                    \
+                                                                   A, B, out, partial);                              \
     }                                  \
   } while (0)
   ++g_launches;
   // without a stretching output the kernels skip T and the stretching sums
-  if (!dg) FMM_P2P_ST(0);
+  if (!stretching) FMM_P2P_ST(0);
   else if (p->prm.outputs & FMM_OUT_STRETCHING_TRANSPOSE) FMM_P2P_ST(2);
   else FMM_P2P_ST(1);
 #undef FMM_P2P_ST
 #undef FMM_P2P
+  FMM_CUDA_TRY(cudaGetLastError());
+  return FMM_OK;
+}
+
+// Outputs from the near and the far field.
+int p2p_finish(fmm_plan p, int64_t n, float* vel, float* dg, cudaStream_t s) {
+  if (!vel && !dg) return FMM_OK;
+  const bool seg = p->prm.periodic && p->batched;
+  SegP2P* sp = seg ? p->seg_p2p.as<SegP2P>() : nullptr;
+  const double* dip = p->prm.periodic && !p->batched ? p->scal.as<double>() + kScalDipole : nullptr;
+  ++g_launches;
+  k_finish<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p->near_u.as<float>(), p->near_s.as<float>(),
+                                                       p->far_u.as<float>(), p->far_s.as<float>(), p->sidx, n, dip, sp,
+                                                       seg ? p->seg_off.as<int>() : nullptr, p->nseg, vel, dg);
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }

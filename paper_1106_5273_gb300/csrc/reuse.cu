@@ -51,15 +51,25 @@ int eval_strengths(fmm_plan p, const float* gam, float* vel, float* dg, cudaStre
   ++g_launches;
   k_gather_gamma<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gam, p->sidx, n, p->sortB.as<float4>());
   FMM_CUDA_TRY(cudaGetLastError());
-  FMM_TRY(upward_pass(p, s));
-  FMM_TRY(dipole_pass(p, n, s));
-  const size_t lbytes = (size_t)p->ncells * 3 * p->P * sizeof(float);
-  FMM_CUDA_TRY(cudaMemsetAsync(p->L.ptr, 0, lbytes, s));
-  if (p->last_tc) FMM_TRY(m2l_tensor(p, s));
-  else FMM_TRY(m2l_simt(p, s));
-  FMM_TRY(apply_lattice(p, s));
-  FMM_TRY(downward_pass(p, n, s));
-  FMM_TRY(p2p_near(p, n, p->reuse_sig_u, p->reuse_ps, p->reuse_smax, vel, dg, s));
+  // the far field on the plan's stream beside the near field, as in a full
+  // evaluation (one after the other with timing on)
+  const bool serial = p->timing != 0;
+  cudaStream_t fs = serial ? s : p->s_far;
+  if (!serial) {
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_fork, s));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(fs, p->ev_fork, 0));
+  }
+  int rc = upward_pass(p, fs);
+  if (rc == FMM_OK) rc = dipole_pass(p, n, fs);
+  if (rc == FMM_OK) rc = far_field(p, n, fs, nullptr);
+  if (rc == FMM_OK)
+    rc = p2p_near(p, n, p->reuse_sig_u, p->reuse_ps, p->reuse_smax, dg != nullptr, s);
+  if (!serial) {  // join also after an error
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_join, fs));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(s, p->ev_join, 0));
+  }
+  FMM_TRY(rc);
+  FMM_TRY(p2p_finish(p, n, vel, dg, s));
   return FMM_OK;
 }
 

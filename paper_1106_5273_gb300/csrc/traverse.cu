@@ -822,10 +822,10 @@ static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
 // summed over the target tiles.
 static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t s) {
   const int T = 256;
-  FMM_TRY(p->lk0.ensure((size_t)(n + 1) * sizeof(uint64_t)));
-  FMM_TRY(p->lk1.ensure((size_t)(n + 1) * sizeof(uint64_t)));
-  FMM_TRY(p->lv0.ensure((size_t)(n + 1) * sizeof(uint32_t)));
-  FMM_TRY(p->lv1.ensure((size_t)(n + 1) * sizeof(uint32_t)));
+  FMM_TRY(p->pk0.ensure((size_t)(n + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->pk1.ensure((size_t)(n + 1) * sizeof(uint64_t)));
+  FMM_TRY(p->pv0.ensure((size_t)(n + 1) * sizeof(uint32_t)));
+  FMM_TRY(p->pv1.ensure((size_t)(n + 1) * sizeof(uint32_t)));
   FMM_TRY(p->p2p_sorted.ensure((size_t)(n + 1) * sizeof(int2)));
   FMM_TRY(p->p2p_off.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
   FMM_TRY(p->p2p_pre.ensure((size_t)(n + 1) * sizeof(uint32_t)));
@@ -834,13 +834,13 @@ static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t
   const unsigned g = std::max(1u, (unsigned)((n + T - 1) / T));
   ++g_launches;
   const int npass = bits_for(p->ncells) / 8, second = npass & 1;  // at most 4: cells are fewer than 2^27
-  FMM_TRY(sort_begin(p->sort, std::max(n, 1), s));
-  k_p2p_keys<<<std::min(g, 608u), T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(),
-                                             npass, &p->sort.state.as<SortState>()->hist[0][0]);
-  FMM_TRY(sort_passes(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                      p->lv1.as<uint32_t>(), std::max(n, 1), npass, true, p->flags.as<int>(), s));
-  uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
-  uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
+  FMM_TRY(sort_begin(p->p_sort, std::max(n, 1), s));
+  k_p2p_keys<<<std::min(g, 608u), T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->pk0.as<uint64_t>(), p->pv0.as<uint32_t>(),
+                                             npass, &p->p_sort.state.as<SortState>()->hist[0][0]);
+  FMM_TRY(sort_passes(p->p_sort, p->pk0.as<uint64_t>(), p->pv0.as<uint32_t>(), p->pk1.as<uint64_t>(),
+                      p->pv1.as<uint32_t>(), std::max(n, 1), npass, true, p->flags.as<int>(), s));
+  uint64_t* sk = second ? p->pk1.as<uint64_t>() : p->pk0.as<uint64_t>();
+  uint32_t* sv = second ? p->pv1.as<uint32_t>() : p->pv0.as<uint32_t>();
   ++g_launches;
   k_p2p_gather<<<std::min(g, 1216u), T, 0, s>>>(p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(),
                                                 p->p2p_pre.as<uint32_t>(), p->c_begin.as<int>(), p->c_end.as<int>(),
@@ -848,7 +848,7 @@ static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t
   FMM_CUDA_TRY(cudaMemcpyAsync(totals, dpairs, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   // the scan wraps past 2^32 sources; differences within a leaf stay exact
   FMM_TRY(exclusive_scan_u32(p->p2p_pre.as<uint32_t>(), p->p2p_pre.as<uint32_t>(), n, p->p2p_pre.as<uint32_t>() + n,
-                             p->scan_tmp, s));
+                             p->p_scan, s));
   ++g_launches;
   k_p2p_offsets<<<(unsigned)((p->nleaves + T - 1) / T), T, 0, s>>>(p->leaves.as<int>(), (int)p->nleaves, sk, n,
                                                                    p->p2p_off.as<int2>());
@@ -856,7 +856,7 @@ static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t
   return FMM_OK;
 }
 
-int traverse(fmm_plan p, double smax, cudaStream_t s) {
+int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std::function<int()>& near) {
   const int T = 256;
   const int nc = (int)p->ncells;
   if (p->ncells >= (1ll << kPairSrcBits)) return FMM_E_CAPACITY;  // the 8-byte M2L pair record
@@ -906,8 +906,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   // the host reads `bytes` of device counts: enqueue the copy, mark it, and
   // (after more work is enqueued behind it) wait for the mark
   auto read_mark = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
-    FMM_CUDA_TRY(cudaMemcpyAsync(dst_h, src_d, bytes, cudaMemcpyDeviceToHost, s));
-    FMM_CUDA_TRY(cudaEventRecord(p->ev_read, s));
+    FMM_CUDA_TRY(cudaMemcpyAsync(dst_h, src_d, bytes, cudaMemcpyDeviceToHost, f));
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_read, f));
     return FMM_OK;
   };
 
@@ -995,46 +995,53 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
   p->n_m2l = nm;
   p->n_p2p = np;
 
-  // ---- M2L: translation keys and their field ranges; the P2P grouping runs
-  // while the host reads the ranges
+  // ---- M2L lists on f, P2P lists on s
+  if (f != s) {
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(f, p->ev_near, 0));
+  }
   const int n = (int)nm;
   const unsigned g = (unsigned)((n + T - 1) / T);
   if (n > 0) {
     FMM_TRY(p->m2l_key.ensure((size_t)(n + 1) * sizeof(uint64_t)));
     ++g_launches;
-    k_m2l_keys<<<std::min<unsigned>(g, 2048u), T, 0, s>>>(p->m2l_raw.as<int2>(), n, p->c_level.as<int>(),
+    k_m2l_keys<<<std::min<unsigned>(g, 2048u), T, 0, f>>>(p->m2l_raw.as<int2>(), n, p->c_level.as<int>(),
                                                           p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
                                                           p->flags.as<int>());
   }
-  FMM_CUDA_TRY(cudaMemcpyAsync(hrng, drng, 8 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  FMM_CUDA_TRY(cudaMemcpyAsync(hrng, drng, 8 * sizeof(int), cudaMemcpyDeviceToHost, f));
   FMM_TRY(read_mark(hmisc, dmisc, sizeof(uint32_t)));
   FMM_TRY(group_p2p(p, (int)np, reinterpret_cast<unsigned long long*>(pin + 64), s));
+  FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
   p->n_keys = 0;
   p->n_steps = 0;
   p->n_built = 0;
   // the work items of the pair kernel, once the list totals are on the host
   auto p2p_items = [&]() -> int {
+    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_near));
     const unsigned long long* tot = reinterpret_cast<unsigned long long*>(pin + 64);
     p->p2p_pairs = (int64_t)tot[0];
     FMM_TRY(p2p_build_items(p, p->last_n, (int64_t)tot[1], dmisc + 4, s));
+    FMM_CUDA_TRY(cudaMemcpyAsync(hmisc + 4, dmisc + 4, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
     return FMM_OK;
   };
-  auto p2p_counts = [&]() {
+  // ... and once they are counted, the near field itself
+  auto p2p_launch = [&]() -> int {
+    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_near));
     p->n_p2p_items = hmisc[4];
     p->n_p2p_slots = hmisc[5];
+    return near();
   };
   FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
   p->ntiles = hmisc[0];
   // step ranges: one per tile, in a batch one per tile and key bucket
   const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p->P);
   FMM_TRY(p->tile_range.ensure((size_t)(p->ntiles + 1) * nsub * sizeof(int2)));
-  FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (size_t)(p->ntiles + 1) * nsub * sizeof(int2), s));
+  FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (size_t)(p->ntiles + 1) * nsub * sizeof(int2), f));
   if (n == 0) {
-    FMM_CUDA_TRY(cudaStreamSynchronize(s));
     FMM_TRY(p2p_items());
-    FMM_TRY(read_mark(hmisc + 4, dmisc + 4, 2 * sizeof(uint32_t)));
-    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-    p2p_counts();
+    FMM_TRY(p2p_launch());
   } else {
     FMM_TRY(p->lv0.ensure((n + 1) * sizeof(uint32_t)));
     FMM_TRY(p->tcount.ensure((n + 1) * sizeof(uint32_t)));
@@ -1055,18 +1062,20 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
     while ((1ll << tb) < (long long)p->ntiles * nsub) ++tb;
     if (tb + kp.bits > 63) return FMM_E_DEPTH;
     const int64_t K = 1ll << kp.bits;
-    bool binned = false;
+    bool items_done = false, binned = false;
     if (kp.bits <= kBinKeyBits && !(p->prm.m2l_mode & FMM_M2L_SORT_STEPS)) {
       // the steps from flag tables (no sort) when the tables are small
       FMM_TRY(p->bin_flag.ensure((size_t)(K + 1) * sizeof(uint32_t)));
       FMM_TRY(p->bin_scan.ensure((size_t)(K + 1) * sizeof(uint32_t)));
       uint32_t* kflag = p->bin_flag.as<uint32_t>();
       uint32_t* kslot = p->bin_scan.as<uint32_t>();
-      FMM_CUDA_TRY(cudaMemsetAsync(kflag, 0, (size_t)K * sizeof(uint32_t), s));
+      FMM_CUDA_TRY(cudaMemsetAsync(kflag, 0, (size_t)K * sizeof(uint32_t), f));
       ++g_launches;
-      k_key_mark<<<g, T, 0, s>>>(p->m2l_key.as<uint64_t>(), n, kp, kflag);
-      FMM_TRY(exclusive_scan_u32(kflag, kslot, K, dmisc + 1, p->scan_tmp, s));
+      k_key_mark<<<g, T, 0, f>>>(p->m2l_key.as<uint64_t>(), n, kp, kflag);
+      FMM_TRY(exclusive_scan_u32(kflag, kslot, K, dmisc + 1, p->scan_tmp, f));
       FMM_TRY(read_mark(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
+      FMM_TRY(p2p_items());
+      items_done = true;
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
       const int64_t nkeys = hmisc[1];
       const int64_t nb = nkeys * (int64_t)p->ntiles;
@@ -1075,7 +1084,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
         p->n_keys = nkeys;
         FMM_TRY(p->ukeys.ensure((size_t)(nkeys + 1) * sizeof(uint64_t)));
         ++g_launches;
-        k_key_unpack<<<(unsigned)((K + T - 1) / T), T, 0, s>>>(kflag, kslot, K, kp, p->ukeys.as<uint64_t>());
+        k_key_unpack<<<(unsigned)((K + T - 1) / T), T, 0, f>>>(kflag, kslot, K, kp, p->ukeys.as<uint64_t>());
         const uint32_t* perm = nullptr;
         if (nsub > 1) {
           FMM_TRY(p->lk0.ensure((nkeys + 1) * sizeof(uint64_t)));
@@ -1084,53 +1093,52 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
           FMM_TRY(p->m2l_slot.ensure((nkeys + 1) * sizeof(uint32_t)));
           const unsigned gk = (unsigned)((nkeys + T - 1) / T);
           g_launches += 2;
-          k_bucket_keys<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(), (int)nkeys, p->lk0.as<uint64_t>(),
+          k_bucket_keys<<<gk, T, 0, f>>>(p->ukeys.as<uint64_t>(), (int)nkeys, p->lk0.as<uint64_t>(),
                                          p->lv0.as<uint32_t>());
           int second = 0;
           FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                                 p->lv1.as<uint32_t>(), nkeys, 3, &second, p->flags.as<int>(), s));
+                                 p->lv1.as<uint32_t>(), nkeys, 3, &second, p->flags.as<int>(), f));
           // the sorted bucket numbers are not needed: their buffer takes the keys in the new order
           uint64_t* out = second ? p->lk0.as<uint64_t>() : p->lk1.as<uint64_t>();
-          k_bucket_order<<<gk, T, 0, s>>>(p->ukeys.as<uint64_t>(),
+          k_bucket_order<<<gk, T, 0, f>>>(p->ukeys.as<uint64_t>(),
                                           second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(), (int)nkeys, out,
                                           p->m2l_slot.as<uint32_t>());
-          FMM_CUDA_TRY(cudaMemcpyAsync(p->ukeys.ptr, out, (size_t)nkeys * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+          FMM_CUDA_TRY(cudaMemcpyAsync(p->ukeys.ptr, out, (size_t)nkeys * sizeof(uint64_t), cudaMemcpyDeviceToDevice, f));
           perm = p->m2l_slot.as<uint32_t>();
         }
         uint32_t* miss = p->tcount.as<uint32_t>();
         uint32_t* rank = p->tscan0.as<uint32_t>();
-        FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, s));
+        FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, f));
         // the key tables stay live: bins go to bin_flag2 / bin_scan2
         FMM_TRY(p->bin_flag2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
         FMM_TRY(p->bin_scan2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
         uint32_t* bflag = p->bin_flag2.as<uint32_t>();
         uint32_t* bstep = p->bin_scan2.as<uint32_t>();
         uint32_t* pbin = p->lv0.as<uint32_t>();
-        FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), s));
+        FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), f));
         ++g_launches;
-        k_bin_mark<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
+        k_bin_mark<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
                                    kslot, perm, (int)nkeys, bflag, pbin);
-        FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, s));
-        FMM_TRY(p2p_items());
-        FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 4 * sizeof(uint32_t)));
+        FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, f));
+        FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
+        FMM_TRY(p2p_launch());
         FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-        p2p_counts();
         p->n_steps = hmisc[2];
         const int64_t ns = p->n_steps;
         FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_src.ensure((ns + 1) * tsz * sizeof(int)));
-        FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, s));
-        FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), s));
+        FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, f));
+        FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), f));
         ++g_launches;
-        k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, s>>>(bflag, bstep, nb, (int)nkeys, p->tslot_map.as<int>(),
+        k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, f>>>(bflag, bstep, nb, (int)nkeys, p->tslot_map.as<int>(),
                                                                p->ukeys.as<uint64_t>(), nsub, p->st_tile.as<int>(),
                                                                p->st_slot.as<int>());
         ++g_launches;
-        k_bin_fill<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(), tsz,
+        k_bin_fill<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), pbin, n, bstep, p->c_tile.as<int>(), tsz,
                                      p->st_src.as<int>());
         ++g_launches;
-        k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns,
+        k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, f>>>(p->st_tile.as<int>(), (int)ns,
                                                                 p->tile_range.as<int2>());
         FMM_CUDA_TRY(cudaGetLastError());
       }
@@ -1139,18 +1147,20 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       FMM_TRY(p->lk0.ensure((n + 1) * sizeof(uint64_t)));
       FMM_TRY(p->lk1.ensure((n + 1) * sizeof(uint64_t)));
       FMM_TRY(p->lv1.ensure((n + 1) * sizeof(uint32_t)));
+      if (!items_done) FMM_TRY(p2p_items());
+      FMM_TRY(p2p_launch());
       // sort pairs by (tile, compact key): consecutive runs are the steps
       ++g_launches;
-      k_step_keys2<<<g, T, 0, s>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
+      k_step_keys2<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
                                    nsub, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       int second = 0;
       FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, p->flags.as<int>(), s));
+                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, p->flags.as<int>(), f));
       uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
-      k_step_flags<<<g, T, 0, s>>>(sk, n, p->tcount.as<uint32_t>());
-      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, s));
+      k_step_flags<<<g, T, 0, f>>>(sk, n, p->tcount.as<uint32_t>());
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, f));
       FMM_TRY(read_mark(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
       p->n_steps = hmisc[2];
@@ -1160,41 +1170,39 @@ int traverse(fmm_plan p, double smax, cudaStream_t s) {
       FMM_TRY(p->st_src.ensure((ns + 1) * tsz * sizeof(int)));
       FMM_TRY(p->st_ckey.ensure((ns + 1) * sizeof(uint64_t)));
       FMM_TRY(p->st_fkey.ensure((ns + 1) * sizeof(uint64_t)));
-      FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), s));
+      FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), f));
       ++g_launches;
-      k_step_write2<<<g, T, 0, s>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
+      k_step_write2<<<g, T, 0, f>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
                                     p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), tsz, kp.bits,
                                     p->st_tile.as<int>(),
                                     p->st_ckey.as<uint64_t>(), p->st_fkey.as<uint64_t>(), p->st_src.as<int>());
       ++g_launches;
-      k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, s>>>(p->st_tile.as<int>(), (int)ns, p->tile_range.as<int2>());
+      k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, f>>>(p->st_tile.as<int>(), (int)ns, p->tile_range.as<int2>());
       // distinct translations among the steps -> operator slots
       FMM_TRY(p->ukeys.ensure((ns + 1) * sizeof(uint64_t)));
       unsigned gs = (unsigned)((ns + T - 1) / T);
       ++g_launches;
-      k_copy_u64_iota<<<gs, T, 0, s>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+      k_copy_u64_iota<<<gs, T, 0, f>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), ns, std::max(kp.bits, 1), &second, p->flags.as<int>(), s));
+                             p->lv1.as<uint32_t>(), ns, std::max(kp.bits, 1), &second, p->flags.as<int>(), f));
       sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
-      k_unique_flags<<<gs, T, 0, s>>>(sk, (int)ns, p->tcount.as<uint32_t>());
-      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dmisc + 1, p->scan_tmp, s));
+      k_unique_flags<<<gs, T, 0, f>>>(sk, (int)ns, p->tcount.as<uint32_t>());
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dmisc + 1, p->scan_tmp, f));
       ++g_launches;
-      k_step_slots<<<gs, T, 0, s>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
+      k_step_slots<<<gs, T, 0, f>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
                                     p->st_fkey.as<uint64_t>(), p->ukeys.as<uint64_t>(), p->st_slot.as<int>());
-      FMM_TRY(p2p_items());
-      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, 5 * sizeof(uint32_t)));
+      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      p2p_counts();
       p->n_keys = hmisc[1];
       uint32_t* miss = p->tcount.as<uint32_t>();
       uint32_t* rank = p->tscan0.as<uint32_t>();
-      FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, s));
+      FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, f));
       FMM_TRY(read_mark(hmisc + 3, dmisc + 3, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, s));
-      FMM_TRY(remap_step_slots(p, s));
+      FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, f));
+      FMM_TRY(remap_step_slots(p, f));
       FMM_CUDA_TRY(cudaGetLastError());
     }
   }
