@@ -97,6 +97,7 @@ struct fmm_plan_s {
   fmm::DBuf m2m_T;    // [8][P(k)][P(r)] FP32 transposed M2M matrices by child octant
   fmm::DBuf l2l_T;    // [8][P(k)][P(r)] FP32 transposed L2L matrices by child octant
   fmm::DBuf l2p_tab;  // [5][P] int4 L2P gather table (indices into L~, signed weights)
+  fmm::DBuf m2l_inu;  // [P] FP64 1 / nu of every coefficient (M2L operators)
   fmm::DBuf lattice;  // [P][P] FP64 periodic lattice operator (row = output)
   // particles
   fmm::DBuf keys0, keys1, vals0, vals1;  // radix sort ping-pong

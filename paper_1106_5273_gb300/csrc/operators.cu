@@ -147,24 +147,57 @@ __device__ __forceinline__ float round_tf32(float x) {
   return __uint_as_float(u & 0xFFFFE000u);
 }
 
+// v or -v, by its sign bit.
+__device__ __forceinline__ double flip(double v, bool neg) {
+  return __longlong_as_double(__double_as_longlong(v) ^ ((long long)neg << 63));
+}
+
+// M2L operators of new translations, one CTA each, in FP64.
 // kind 0: BF16 tiles [key][hi/lo][nkc K chunks of 64][rows][64];
 // kind 1: TF32 tiles [key][hi/lo][nkc K chunks of 32][rows][32]; both 128-byte
-// rows with 16-byte groups in the 128-byte swizzle order (group j at j ^ (row & 7)).
-__global__ void k_build_m2l(const uint64_t* __restrict__ keys, const int* __restrict__ slots, int nkeys, int p,
-                            float* __restrict__ T32, uint8_t* __restrict__ Tb, int nkc, int kind) {
+// rows with 16-byte groups in the 128-byte swizzle order (group j at j ^ (row & 7)),
+// padding rows and columns zero; nkc = 0: FP32 [key][P][P].
+// FP64 runs at a 64th of the FP32 rate, so an entry takes one addition, two
+// multiplications and one conversion: the factors 1 / nu come from a table, the
+// irregular harmonics are built by one thread per order m, and a thread writes
+// 16 bytes of a row at a time.  The first evaluation of Plummer 1,000,000 (49,141
+// operators, p = 12) spent 57.4 ms here with a division and the conversions per
+// entry and one thread for the harmonics, now 11.7.
+__global__ void __launch_bounds__(256) k_build_m2l(const uint64_t* __restrict__ keys, const int* __restrict__ slots,
+                                                   int nkeys, int p, const double* __restrict__ inu,
+                                                   float* __restrict__ T32, uint8_t* __restrict__ Tb, int nkc,
+                                                   int kind) {
   __shared__ cd I[(2 * kPMax - 1) * (2 * kPMax) / 2];
-  __shared__ double nu[kNCoefMax];
-  __shared__ double rp[kPMax];
-  __shared__ int nmp[kNCoefMax];  // real index -> (n, m, part) packed
+  __shared__ double ar[kNCoefMax], bc[kNCoefMax];  // (-1)^n / nu of a row, ratio^j / nu of a column
+  __shared__ int nmp[kNCoefMax];                   // real index -> (n, m, part) packed
   const int kid = blockIdx.x;
   if (kid >= nkeys) return;
   const int key_id = slots[kid];  // cache slot written by this block
-  const int P = p * p;
-  uint64_t key = keys[kid];
+  const int P = p * p, D = 2 * p - 1;
   int delta;
   double tau[3];
-  m2l_key_decode(key, &delta, tau);
-  if (threadIdx.x == 0) irregular_table_d(tau[0], tau[1], tau[2], 2 * p - 1, I);
+  m2l_key_decode(keys[kid], &delta, tau);
+  if ((int)threadIdx.x < D) {
+    // thread = order m: the diagonal I_m^m, then up the column (the recurrences
+    // and their order of irregular_table_d)
+    const int m = threadIdx.x;
+    const double x = tau[0], y = tau[1], z = tau[2], r2 = x * x + y * y + z * z, inv_r2 = 1.0 / r2;
+    cd d = {1.0 / sqrt(r2), 0.0};
+    for (int q = 1; q <= m; ++q) d = cscale(cmul(d, cd{x, y}), (2.0 * q - 1.0) * inv_r2);
+    I[cidx(m, m)] = d;
+    cd b1 = {0.0, 0.0}, b0 = d;  // I_{n-2}^m, I_{n-1}^m
+    for (int n = m + 1; n < D; ++n) {
+      cd a = cscale(b0, (2.0 * n - 1.0) * z);
+      if (n - 2 >= m) {
+        const cd b = cscale(b1, (double)((n - 1) * (n - 1) - m * m));
+        a.re -= b.re;
+        a.im -= b.im;
+      }
+      b1 = b0;
+      b0 = cscale(a, inv_r2);
+      I[cidx(n, m)] = b0;
+    }
+  }
   for (int r = threadIdx.x; r < P; r += blockDim.x) {
     int n = (int)sqrtf((float)r);
     while (n * n > r) --n;
@@ -172,49 +205,66 @@ __global__ void k_build_m2l(const uint64_t* __restrict__ keys, const int* __rest
     int o = r - n * n;
     int m = (o + 1) / 2, part = (o == 0) ? 0 : ((o - 1) & 1);
     nmp[r] = (n << 16) | (m << 8) | part;
-    nu[r] = nu_d(n, m);
-  }
-  if (threadIdx.x < (unsigned)p) rp[threadIdx.x] = ldexp(1.0, delta * (int)threadIdx.x);
-  const int rows = m2l_cols(P);  // output rows of the operator tiles
-  const size_t chunk_bytes = (size_t)rows * 128;
-  if (nkc) {  // zero this slot's tiles (padding rows and columns stay zero)
-    uint4* z = reinterpret_cast<uint4*>(Tb + (size_t)key_id * 2 * nkc * chunk_bytes);
-    for (size_t i = threadIdx.x; i < 2 * nkc * chunk_bytes / 16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    const double v = inu[r];
+    ar[r] = (n & 1) ? -v : v;
+    bc[r] = ldexp(v, delta * n);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < P * P; e += blockDim.x) {
-    int r = e / P, c = e % P;
-    int a = nmp[r], b = nmp[c];
-    int n = a >> 16, m = (a >> 8) & 0xff, po = a & 1;
-    int j = b >> 16, k = (b >> 8) & 0xff, pi = b & 1;
-    double s = ((n & 1) ? -1.0 : 1.0) * rp[j] / (nu[r] * nu[c]);
-    cd A = cconj(harm_get(I, j + n, k + m));
-    cd B = {0.0, 0.0};
-    if (k > 0) {
-      B = cconj(harm_get(I, j + n, m - k));
-      if (k & 1) B = {-B.re, -B.im};
+  // entry (r, c): output (n, m, po), input (j, k, pi); A = conj I_{j+n}^{k+m},
+  // B = (-1)^k conj I_{j+n}^{m-k} (0 for k = 0); the real parts of
+  // s [a (A + B) + i b (B - A)]
+  auto entry = [&](int r, int c) -> double {
+    if (r >= P || c >= P) return 0.0;
+    const int a = nmp[r], b = nmp[c];
+    const int n = a >> 16, m = (a >> 8) & 0xff, po = a & 1;
+    const int j = b >> 16, k = (b >> 8) & 0xff, pi = b & 1;
+    const bool im = po != pi;  // the imaginary parts enter
+    const cd* Ia = &I[cidx(j + n, k + m)];
+    const double va = flip(im ? Ia->im : Ia->re, im);
+    const int q = m - k;
+    const cd* Ib = &I[cidx(j + n, q < 0 ? -q : q)];
+    // (-1)^k, and for q < 0 I^{q} = (-1)^q conj I^{-q}
+    const bool neg = ((k & 1) != 0) != (q < 0 && (((q & 1) != 0) != im));
+    const double vb = k > 0 ? flip(im ? Ib->im : Ib->re, neg != im) : 0.0;
+    // one form for all parts (signs flipped, no divergence): pi = 0 takes va + vb,
+    // pi = 1 va - vb (po = 0) or vb - va
+    return ar[r] * bc[c] * (flip(va, pi && po) + flip(vb, pi && !po));
+  };
+  if (!nkc) {  // the SIMT path's FP32 copy
+    for (int e = threadIdx.x; e < P * P; e += blockDim.x) T32[(size_t)key_id * P * P + e] = (float)entry(e / P, e % P);
+    return;
+  }
+  const int rows = m2l_cols(P);  // output rows of the operator tiles
+  const size_t chunk_bytes = (size_t)rows * 128;
+  uint8_t* T = Tb + (size_t)key_id * 2 * nkc * chunk_bytes;
+  for (int u = threadIdx.x; u < rows * nkc * 8; u += blockDim.x) {
+    const int r = u / (nkc * 8), kc = (u >> 3) % nkc, g = u & 7;
+    uint32_t hi[4], lo[4];
+    if (kind == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        hi[q] = lo[q] = 0u;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float v = (float)entry(r, kc * 64 + g * 8 + 2 * q + e);
+          const __nv_bfloat16 h = __float2bfloat16(v);
+          const __nv_bfloat16 l = __float2bfloat16(v - __bfloat162float(h));
+          hi[q] |= (uint32_t)__bfloat16_as_ushort(h) << (16 * e);
+          lo[q] |= (uint32_t)__bfloat16_as_ushort(l) << (16 * e);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double v = entry(r, kc * 32 + g * 4 + q);
+        const float h = round_tf32((float)v);
+        hi[q] = __float_as_uint(h);
+        lo[q] = __float_as_uint(round_tf32((float)(v - (double)h)));
+      }
     }
-    double v;
-    if (pi == 0) v = po == 0 ? s * (A.re + B.re) : s * (A.im + B.im);
-    else v = po == 0 ? -s * (B.im - A.im) : s * (B.re - A.re);
-    if (!nkc) T32[(size_t)key_id * P * P + e] = (float)v;  // FP32 copy for the SIMT path only
-    if (nkc && kind == 0) {
-      __nv_bfloat16* Tbf = reinterpret_cast<__nv_bfloat16*>(Tb);
-      __nv_bfloat16 hi = __double2bfloat16(v);
-      __nv_bfloat16 lo = __double2bfloat16(v - (double)__bfloat162float(hi));
-      const int kc = c >> 6, j = (c & 63) >> 3, el = c & 7;
-      const size_t within = (size_t)r * 64 + (size_t)(((j ^ (r & 7)) << 3) + el);
-      Tbf[(((size_t)key_id * 2 + 0) * nkc + kc) * ((size_t)rows * 64) + within] = hi;
-      Tbf[(((size_t)key_id * 2 + 1) * nkc + kc) * ((size_t)rows * 64) + within] = lo;
-    } else if (nkc) {
-      float* Ttf = reinterpret_cast<float*>(Tb);
-      const float hi = round_tf32((float)v);
-      const float lo = round_tf32((float)(v - (double)hi));
-      const int kc = c >> 5, j = (c & 31) >> 2, el = c & 3;
-      const size_t within = (size_t)r * 32 + (size_t)(((j ^ (r & 7)) << 2) + el);
-      Ttf[(((size_t)key_id * 2 + 0) * nkc + kc) * ((size_t)rows * 32) + within] = hi;
-      Ttf[(((size_t)key_id * 2 + 1) * nkc + kc) * ((size_t)rows * 32) + within] = lo;
-    }
+    uint8_t* dst = T + (size_t)kc * chunk_bytes + (size_t)r * 128 + (size_t)((g ^ (r & 7)) << 4);
+    *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(dst + (size_t)nkc * chunk_bytes) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
 }
 
@@ -295,6 +345,12 @@ int build_constant_operators(fmm_plan p) {
       }
   FMM_TRY(p->l2p_tab.ensure(tab.size() * sizeof(int4)));
   FMM_CUDA_TRY(cudaMemcpy(p->l2p_tab.ptr, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  std::vector<double> inu(P);
+  for (int n = 0; n < pp; ++n)
+    for (int m = 0; m <= n; ++m)
+      for (int part = 0; part < (m ? 2 : 1); ++part) inu[ridx(n, m, part)] = 1.0 / nu_d(n, m);
+  FMM_TRY(p->m2l_inu.ensure(inu.size() * sizeof(double)));
+  FMM_CUDA_TRY(cudaMemcpy(p->m2l_inu.ptr, inu.data(), inu.size() * sizeof(double), cudaMemcpyHostToDevice));
   if (p->prm.periodic) {  // the lattice operator, in FP64 on the device
     FMM_TRY(p->lattice.ensure((size_t)P * P * sizeof(double)));
     FMM_TRY(lattice_operator_device(pp, p->prm.images, p->lattice.as<double>(), 0));
@@ -439,7 +495,8 @@ int build_m2l_operators(fmm_plan p, int64_t nmiss, uint32_t* miss, uint32_t* ran
       p->tmiss_slots.as<int>());
   ++g_launches;
   k_build_m2l<<<(unsigned)nmiss, 256, 0, s>>>(p->tmiss_keys.as<uint64_t>(), p->tmiss_slots.as<int>(), (int)nmiss,
-                                              p->prm.p, p->T32.as<float>(), p->Tbf.as<uint8_t>(),
+                                              p->prm.p, p->m2l_inu.as<double>(), p->T32.as<float>(),
+                                              p->Tbf.as<uint8_t>(),
                                               tc ? m2l_kchunks(P, p->tc_kind) : 0, p->tc_kind);
   FMM_CUDA_TRY(cudaGetLastError());
   p->tc_size = need;
