@@ -21,9 +21,9 @@
 // A stage is one step and one 64-wide K chunk: the operator (rows pre-swizzled
 // in global memory in the 128-byte-swizzle K-major layout) arrives by 1-D bulk
 // copies on mbarrier fullA, issued by a warp of their own; 8 producer warps
-// gather the rows of B (128 B each) by 16-byte cp.async into the same swizzle and
-// arrive on fullB; one thread issues the MMAs and commits them to the stage's
-// empty barrier.  Every wait is bounded; on expiry the kernel records
+// load the rows of B (128 B each) into registers, store them in the same swizzle
+// once the buffer is free and arrive on fullB; one thread issues the MMAs and
+// commits them to the empty barrier.  Every wait is bounded; on expiry the kernel records
 // FMM_E_TIMEOUT, waits (bounded) for its own copies, frees its tensor memory
 // and returns.
 //
@@ -32,7 +32,8 @@
 // the 128 rows, and an MMA costs about 20-40 cycles on top of N / 2, so fewer
 // and wider MMAs win (Taylor-Green 128^3, p = 10: 4.09 ms against 4.74 with the
 // cells as rows).  Elsewhere the cells win: Plummer 1,000,000 at p = 12 38.3 ->
-// 26.3 ms, Plummer 30,011 at p = 8 0.89 -> 0.56 ms.
+// 26.3 ms, Plummer 30,011 at p = 8 0.89 -> 0.56 ms (one stage of cp.async gathers; with the
+// gathers in registers while the buffer is still read, 23.9 -> 20.1 and 0.54).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -48,7 +49,6 @@ constexpr int kProducerWarps = 8;
 constexpr int kThreads = (kProducerWarps + 2) * 32;  // + MMA warp, + operator copy warp
 constexpr int kMmaWarp = kProducerWarps, kCopyWarp = kProducerWarps + 1;
 constexpr uint32_t kBBytes = kRows * 128;   // one K chunk of the gathered rows, hi or lo
-constexpr int kStagesMax = 2;
 constexpr long long kSpin = 1ll << 24;
 static_assert(3 * kTileCells <= kRows, "a tile's rows fit one MMA");
 // operator-row form
@@ -168,9 +168,9 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 16-byte asynchronous copy to shared memory; zeros if !live.
-__device__ __forceinline__ void gather16(uint32_t dst, const uint8_t* src, bool live) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+__device__ __forceinline__ void store16(uint32_t dst, const uint4& v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
 }
 
 // ---- Cell rows (P <= 64 or P > 128).
@@ -183,12 +183,16 @@ __device__ __forceinline__ void gather16(uint32_t dst, const uint8_t* src, bool 
 // writes the local expansions (slot -1), the others write D to their partial
 // slot, summed by k_m2l_combine.  items == nullptr (batches): CTA x runs the
 // steps of range range0 + x, i.e. of one key bucket of one tile, into slot x.
-template <int KIND>
-__global__ void __launch_bounds__(kThreads, 3)
+// CTAS per SM: three up to N = 64; two with N > 128, whose 256 tensor-memory
+// columns admit no more, which leaves the gathers 78 registers a thread instead
+// of 64 (Plummer 1,000,000 at p = 12 22.9 -> 20.1 ms; at p = 8 two CTAs are 20%
+// slower than three).
+template <int KIND, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS)
     k_m2l_cells(const int2* __restrict__ tile_range, int range0, const int4* __restrict__ items,
              const uint32_t* __restrict__ nitems, const uint32_t* __restrict__ order, const int* __restrict__ tfirst, const int* __restrict__ st_slot,
              const int* __restrict__ st_src, const uint8_t* __restrict__ Tb, const uint8_t* __restrict__ Mb, int P,
-             int N, int nkc, int nkc3, int ksteps_last, int nstages, uint32_t tmem_cols,
+             int N, int nkc, int nkc3, int ksteps_last, uint32_t tmem_cols,
              const int* __restrict__ tcell, float* __restrict__ L, float* __restrict__ partial,
              int* __restrict__ flag) {
   extern __shared__ uint8_t smem_raw[];
@@ -210,22 +214,16 @@ __global__ void __launch_bounds__(kThreads, 3)
   constexpr int NB = 2;  // blocks of each operand per stage: hi and lo
   const uint32_t abytes = (uint32_t)N * 128u;
   const uint32_t stage_bytes = (uint32_t)NB * (kBBytes + abytes);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nstages * stage_bytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStagesMax + 1);
-  volatile int* abort = reinterpret_cast<volatile int*>(bars + 3 * kStagesMax + 2);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + stage_bytes);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
+  volatile int* abort = reinterpret_cast<volatile int*>(bars + 5);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sbase = smem_u32(smem);
-  const uint32_t bar0 = smem_u32(bars);
-  auto fullA = [&](int s) { return bar0 + 8u * (uint32_t)s; };
-  auto fullB = [&](int s) { return bar0 + 8u * (uint32_t)(kStagesMax + s); };
-  auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(2 * kStagesMax + s); };
-  const uint32_t done = bar0 + 8u * (uint32_t)(3 * kStagesMax);
+  const uint32_t fullA = smem_u32(bars), fullB = fullA + 8u, empty = fullA + 16u, done = fullA + 24u;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < nstages; ++s) {
-      mbar_init(fullA(s), 1);
-      mbar_init(fullB(s), kProducerWarps);
-      mbar_init(empty(s), 1);
-    }
+    mbar_init(fullA, 1);
+    mbar_init(fullB, kProducerWarps);
+    mbar_init(empty, 1);
     mbar_init(done, 1);
     *abort = 0;
     fence_mbar_init();
@@ -243,130 +241,97 @@ __global__ void __launch_bounds__(kThreads, 3)
   const int niter = (rg.y - rg.x) * nkc;
 
   if (warp < kProducerWarps) {
-    // ---- producers: thread t copies 16-byte chunk j = t % 8 of rows t/8 + 32 q
-    // (q = 0..3), i.e. of component row % 3 of the source in slot row / 3
+    // ---- producers: thread t moves 16-byte chunk j = t % 8 of rows t/8 + 32 q
+    // (q = 0..3), i.e. of component row % 3 of the source in slot row / 3, hi and
+    // lo; a step's rows are loaded before its buffer is waited for
     const int j = threadIdx.x & 7, r0 = threadIdx.x >> 3;
-    int src[4], nxt[4];
-    // pieces of the ring that hold a source's values: a piece without a source
+    int nxt[4];
+    // pieces of the buffer that hold a source's values: a piece without a source
     // is cleared only if it does (adaptive trees pair few of a tile's cells
     // under one translation)
-    uint32_t dirty[kStagesMax];
-#pragma unroll
-    for (int q = 0; q < kStagesMax; ++q) dirty[q] = 0xffffffffu;
-    auto sources = [&](int st, int* v) {
+    uint32_t held = 0xffu;
+    auto sources = [&](int st) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int r = r0 + 32 * q;
-        v[q] = r < 3 * kTileCells ? __ldg(st_src + (size_t)st * kTileCells + r / 3) : -1;
+        nxt[q] = r < 3 * kTileCells ? __ldg(st_src + (size_t)st * kTileCells + r / 3) : -1;
       }
     };
-    sources(rg.x, nxt);
-    const int ahead = nstages - 1;  // iterations in flight behind the one being loaded
-    int st = rg.x, kc = 0, stage = 0, astage = 0;
+    sources(rg.x);
+    const uint32_t dst = sbase + (uint32_t)r0 * 128u + (uint32_t)((j ^ (r0 & 7)) << 4);
+    int st = rg.x, kc = 0;
     uint32_t ph = 0u;
-    bool ok = true;
-    for (int it = 0; it < niter + ahead; ++it) {
-      if (it < niter) {
-        if (kc == 0) {
+    for (int it = 0; it < niter; ++it) {
+      const bool need = j < 2 * (kc == nkc - 1 ? ksteps_last : 4), lo = kc < nkc3;
+      uint4 v[8];
+      uint32_t live = 0u;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) src[q] = nxt[q];
-          if (st + 1 < rg.y) sources(st + 1, nxt);
-        }
-        // the warp goes on or gives up as one
-        if (!__all_sync(0xffffffffu, mbar_wait(empty(stage), ph ^ 1u, abort))) {
-          ok = false;
-          break;
-        }
-        const uint32_t dst = sbase + (uint32_t)stage * stage_bytes + (uint32_t)r0 * 128u + (uint32_t)((j ^ (r0 & 7)) << 4);
-        uint32_t held = 0u;
-#pragma unroll
-        for (int q = 0; q < kStagesMax; ++q)
-          if (q == stage) held = dirty[q];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          const bool need = (b == 0 || kc < nkc3) && j < 2 * (kc == nkc - 1 ? ksteps_last : 4);
-          if (!need) continue;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int r = r0 + 32 * q;
-            if (r >= 3 * kTileCells) continue;
-            const bool live = src[q] >= 0;
-            const uint32_t bit = 1u << (b * 4 + q);
-            if (!live && !(held & bit)) continue;
-            held = live ? held | bit : held & ~bit;
-            const uint8_t* p = Mb + ((((size_t)(live ? src[q] : 0) * 2 + b) * 3 + r % 3) * nkc + kc) * 128 + j * 16;
-            gather16(dst + (uint32_t)b * kBBytes + (uint32_t)q * 4096u, p, live);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < kStagesMax; ++q)
-          if (q == stage) dirty[q] = held;
-        if (++kc == nkc) {
-          kc = 0;
-          ++st;
-        }
-        if (++stage == nstages) {
-          stage = 0;
-          ph ^= 1u;
-        }
+      for (int q = 0; q < 4; ++q) {
+        if (!need || nxt[q] < 0) continue;
+        const uint8_t* p = Mb + ((((size_t)nxt[q] * 2) * 3 + (r0 + 32 * q) % 3) * nkc + kc) * 128 + j * 16;
+        v[q] = __ldg(reinterpret_cast<const uint4*>(p));
+        if (lo) v[4 + q] = __ldg(reinterpret_cast<const uint4*>(p + (size_t)3 * nkc * 128));
+        live |= (lo ? 0x11u : 0x1u) << q;
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      if (it >= ahead) {  // the rows of iteration it - ahead have landed
-        if (ahead == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
-        else asm volatile("cp.async.wait_group 1;" ::: "memory");
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(fullB(astage));
-        if (++astage == nstages) astage = 0;
+      if (++kc == nkc) {
+        kc = 0;
+        if (++st < rg.y) sources(st);
       }
+      // the warp goes on or gives up as one
+      if (!__all_sync(0xffffffffu, mbar_wait(empty, ph ^ 1u, abort))) break;
+      ph ^= 1u;
+      const uint32_t clear = need ? held & ~live & (lo ? 0xffu : 0x0fu) : 0u;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const uint32_t at = dst + (uint32_t)(q >> 2) * kBBytes + (uint32_t)(q & 3) * 4096u;
+        if (live & (1u << q)) store16(at, v[q]);
+        else if (clear & (1u << q)) store16(at, make_uint4(0u, 0u, 0u, 0u));
+      }
+      held = (held & ~clear) | live;
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(fullB);
     }
-    if (!ok) asm volatile("cp.async.wait_group 0;" ::: "memory");
   } else if (warp == kCopyWarp) {
     // ---- operator copies
     if (lane == 0) {
-      int issued = 0, stage = 0, st = rg.x, kc = 0;
-      uint32_t ph = 0u;
+      int issued = 0, st = rg.x, kc = 0;
       bool ok = true;
       for (int it = 0; it < niter; ++it) {
-        if (!mbar_wait(empty(stage), ph ^ 1u, abort)) {
+        if (!mbar_wait(empty, ((uint32_t)it & 1u) ^ 1u, abort)) {
           ok = false;
           break;
         }
         const uint8_t* T = Tb + (size_t)st_slot[st] * 2 * nkc * abytes;
-        const uint32_t a0 = sbase + (uint32_t)stage * stage_bytes + (uint32_t)NB * kBBytes;
+        const uint32_t a0 = sbase + (uint32_t)NB * kBBytes;
         const bool lo = kc < nkc3;  // chunks from nkc3 on take the hi.hi product only
-        mbar_arrive_tx(fullA(stage), lo ? 2u * abytes : abytes);
-        bulk_g2s(a0, T + (size_t)kc * abytes, abytes, fullA(stage));
-        if (lo) bulk_g2s(a0 + abytes, T + (size_t)(nkc + kc) * abytes, abytes, fullA(stage));
+        mbar_arrive_tx(fullA, lo ? 2u * abytes : abytes);
+        bulk_g2s(a0, T + (size_t)kc * abytes, abytes, fullA);
+        if (lo) bulk_g2s(a0 + abytes, T + (size_t)(nkc + kc) * abytes, abytes, fullA);
         issued = it + 1;
         if (++kc == nkc) {
           kc = 0;
           ++st;
         }
-        if (++stage == nstages) {
-          stage = 0;
-          ph ^= 1u;
-        }
       }
-      if (!ok) {  // let the copies in flight land before the CTA exits
+      if (!ok && issued) {  // let the copies in flight land before the CTA exits
         volatile int never = 0;
-        for (int it = issued > nstages ? issued - nstages : 0; it < issued; ++it)
-          mbar_wait(fullA(it % nstages), (uint32_t)(it / nstages) & 1u, &never);
+        mbar_wait(fullA, (uint32_t)(issued - 1) & 1u, &never);
       }
     }
   } else if (lane == 0) {
     // ---- MMA issue
     const uint32_t id = idesc(KIND, N);
-    int stage = 0, kc = 0;
-    uint32_t ph = 0u;
+    int kc = 0;
     bool ok = true;
     for (int it = 0; it < niter; ++it) {
-      if (!mbar_wait(fullA(stage), ph, abort) || !mbar_wait(fullB(stage), ph, abort)) {
+      const uint32_t ph = (uint32_t)it & 1u;
+      if (!mbar_wait(fullA, ph, abort) || !mbar_wait(fullB, ph, abort)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      const uint32_t b_hi = sbase + (uint32_t)stage * stage_bytes, b_lo = b_hi + kBBytes;
+      const uint32_t b_hi = sbase, b_lo = b_hi + kBBytes;
       const uint32_t a_hi = b_hi + (uint32_t)NB * kBBytes, a_lo = a_hi + abytes;
       const int ks = (kc == nkc - 1) ? ksteps_last : 4;
       const bool three = kc < nkc3;
@@ -379,11 +344,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         }
       }
       if (++kc == nkc) kc = 0;
-      umma_commit(empty(stage));
-      if (++stage == nstages) {
-        stage = 0;
-        ph ^= 1u;
-      }
+      umma_commit(empty);
     }
     umma_commit(done);
     if (!ok) {
@@ -826,7 +787,7 @@ __global__ void k_wait_selftest(long long spins, int arrive, int* status) {
 struct M2lForm {
   const void* kern;
   size_t smem;
-  int threads, nstages, rows, ld;
+  int threads, rows, ld;
   uint32_t tmem_cols;
   bool m2;
 };
@@ -849,17 +810,17 @@ static M2lForm m2l_form(fmm_plan p, int nkc, int nkc3) {
     return f;
   }
   f.m2 = false;
-  f.kern = kind ? (const void*)k_m2l_cells<1> : (const void*)k_m2l_cells<0>;
+  const bool two = N > 128;
+  f.kern = kind ? (two ? (const void*)k_m2l_cells<1, 2> : (const void*)k_m2l_cells<1, 3>)
+                : (two ? (const void*)k_m2l_cells<0, 2> : (const void*)k_m2l_cells<0, 3>);
   f.tmem_cols = 32;
   while ((int)f.tmem_cols < N) f.tmem_cols *= 2;
-  const size_t stage = 2 * (kBBytes + (size_t)N * 128);
   // One stage per CTA and as many CTAs per SM as registers, TMEM and the stage
-  // memory allow (three at p <= 8, two at p >= 12): the CTAs hide each other's
-  // gathers, and more gathering threads run.  Rings of 2 and 3 stages in fewer
-  // CTAs were slower: Plummer 1,000,000 at p = 12 26.3 / 34.1 / 34.4 ms for 1 /
-  // 2 / 3 stages, the batch of 32 at p = 8 1.17 / 1.42 / 2.39 ms.
-  f.nstages = 1;
-  f.smem = f.nstages * stage + (3 * kStagesMax + 4) * 8 + 1024;
+  // memory allow: the CTAs hide each other's gathers, and more gathering threads
+  // run.  Rings of 2 and 3 stages of cp.async gathers in fewer CTAs were slower:
+  // Plummer 1,000,000 at p = 12 26.3 / 34.1 / 34.4 ms for 1 / 2 / 3 stages, the
+  // batch of 32 at p = 8 1.17 / 1.42 / 2.39 ms.
+  f.smem = 2 * (kBBytes + (size_t)N * 128) + 64 + 1024;
   f.threads = kThreads;
   f.rows = kRows;
   f.ld = N;
@@ -942,7 +903,8 @@ int m2l_tensor(fmm_plan p, cudaStream_t s) {
   const M2lForm f = m2l_form(p, nkc, nkc3);
   p->m2l_stage_chunks = f.m2 ? 2 : 1;
   static const bool attr_ok = [] {
-    const void* k[5] = {(const void*)k_m2l_cells<1>, (const void*)k_m2l_cells<0>,
+    const void* k[7] = {(const void*)k_m2l_cells<1, 2>, (const void*)k_m2l_cells<1, 3>,
+                        (const void*)k_m2l_cells<0, 2>, (const void*)k_m2l_cells<0, 3>,
                         (const void*)k_m2l_rows<0, true>, (const void*)k_m2l_rows<1, false>,
                         (const void*)k_m2l_rows<0, false>};
     for (const void* q : k)
@@ -966,14 +928,14 @@ int m2l_tensor(fmm_plan p, cudaStream_t s) {
     const uint8_t* Mb = p->Mbf.as<uint8_t>();
     float* partial = p->m2l_partial.as<float>();
     int* flag = p->flags.as<int>();
-    int P = p->P, NN = N, a = nkc, b = nkc3, c = last, d = f.nstages;
+    int P = p->P, NN = N, a = nkc, b = nkc3, c = last;
     uint32_t e = f.tmem_cols;
     void* cells[] = {&ranges, &range0, &items, &nitems, &order, &tfirst, &slot, &src, &Tb, &Mb, &P, &NN,
-                     &a, &b, &c, &d, &e, &tcell, &L, &partial, &flag};
+                     &a, &b, &c, &e, &tcell, &L, &partial, &flag};
     void* rows[] = {&ranges, &range0, &items, &nitems, &order, &tfirst, &slot, &src, &Tb, &Mb, &P, &NN,
                     &a, &b, &c, &tcell, &L, &partial, &flag};
     ++g_launches;
-    FMM_CUDA_TRY(cudaLaunchKernel(f.kern, dim3(grid), dim3(f.threads), f.nstages ? cells : rows, f.smem, s));
+    FMM_CUDA_TRY(cudaLaunchKernel(f.kern, dim3(grid), dim3(f.threads), f.rows == kRows ? cells : rows, f.smem, s));
     return FMM_OK;
   };
   if (p->batched) {
