@@ -811,12 +811,6 @@ __global__ void k_finish(const float* __restrict__ near_u, const float* __restri
   }
 }
 
-// How a leaf's F sources are cut into ranges: none up to `whole`, else ranges of
-// at most `range` sources, but at most `cap` of them.
-struct RangeRule {
-  uint32_t whole, range, cap;
-};
-
 // ---- work items: per leaf, tiles x ranges, the longest ranges first (four
 // length classes, leaf order within each), so that the last warps to start
 // are short: in leaf order the batch of 32 problems waited for its longest
@@ -830,7 +824,7 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
                                                             const int* __restrict__ begin,
                                                             const int* __restrict__ end,
                                                             const int2* __restrict__ off,
-                                                            const uint32_t* __restrict__ epre, int tile, RangeRule rr,
+                                                            const uint32_t* __restrict__ epre, int tile, uint32_t range,
                                                             int4* __restrict__ items, int* __restrict__ islot,
                                                             int2* __restrict__ plan, uint32_t* __restrict__ counts,
                                                             uint32_t* blk, GridBar* bar) {
@@ -852,7 +846,7 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
       q.tb = begin[leaf];
       q.te = end[leaf];
       q.F = epre[rg.y] - epre[rg.x];
-      q.nsp = q.F <= rr.whole ? 1u : min(rr.cap, (q.F + rr.range - 1) / rr.range);
+      q.nsp = q.F <= range ? 1u : (q.F + range - 1) / range;
       q.nit = q.nsp * (uint32_t)((q.te - q.tb + tile - 1) / tile);
       const uint32_t len = q.F / q.nsp;
       q.cls = len >= 8192u ? 0 : (len >= 4096u ? 1 : (len >= 2048u ? 2 : 3));
@@ -1218,27 +1212,27 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
 // kernels wait for room.  One-problem plans take the range that gives kItemTarget
 // items, at least 128 sources (two chunks);
 // the partial slots are then bounded by twice that many items (3 KB each).  A
-// batch takes a rule of its own, so that a problem's sums do not depend on the
-// rest of the batch, with the ranges of a leaf capped for the slots' sake.
+// batch keeps whole lists: a problem's sums may not depend on the rest of the
+// batch, its many problems fill the chip, and the long lists start first.
+// Ranges of 2048 sources for lists above 8192 gave 2% (batch of 32 problems,
+// 477,044 blobs: 7.79 ms instead of 7.95) but moved single values by up to
+// 1.6e-3 of the largest component from those of one running sum; the sums of a
+// batch stay those of one running sum (3.6e-4).
 constexpr int64_t kItemTarget = 8 * 32 * 152;  // items aimed at (half as many: ball 100,003 2.15 instead of 2.09 ms in all)
 constexpr uint32_t kItemSrcMin = 128;
-// batch of 32 problems, 477,044 blobs: P2P 5.23 ms; 5.17 with whole lists only
-// up to 4096 sources, for twice the slots
-constexpr RangeRule kBatchRule = {8192u, 2048u, 16u};
 
 int p2p_tile(fmm_plan p) { return p->prm.p2p_tpl == 1 ? 32 : kTileMax; }
 
 int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s) {
   const int tile = p2p_tile(p);
-  RangeRule rr = kBatchRule;
+  uint32_t range = 0xffffffffu;
   if (!p->batched) {
     const int64_t q = (tile_sources / kItemTarget + kCh - 1) / kCh * kCh;
-    rr.whole = rr.range = (uint32_t)std::min<int64_t>(0xffffffffll - kCh, std::max<int64_t>(kItemSrcMin, q));
-    rr.cap = 0xffffffffu;
+    range = (uint32_t)std::min<int64_t>(0xffffffffll - kCh, std::max<int64_t>(kItemSrcMin, q));
   }
   // at most one partly filled range and one partly filled tile per leaf
   const int64_t tiles = p->nleaves + n / tile + 1;
-  const int64_t items = tiles + std::min<int64_t>(tile_sources / rr.range + 1, tiles * (int64_t)rr.cap);
+  const int64_t items = tiles + tile_sources / range + 1;
   FMM_TRY(p->p2p_items.ensure((size_t)items * sizeof(int4)));
   FMM_TRY(p->p2p_islot.ensure((size_t)items * sizeof(int)));
   FMM_TRY(p->p2p_plan.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
@@ -1256,7 +1250,7 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* count
   int2* plan = p->p2p_plan.as<int2>();
   int nl = (int)p->nleaves, tl = tile;
   const unsigned G = (unsigned)std::min<int64_t>(kItemBlocks, (nl + kItemThreads - 1) / kItemThreads);
-  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &rr, &it, &is, &plan, &counts, &blk, &bar};
+  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &range, &it, &is, &plan, &counts, &blk, &bar};
   ++g_launches;
   FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_p2p_items, dim3(G), dim3(kItemThreads), args, 0, s));
   FMM_CUDA_TRY(cudaGetLastError());
