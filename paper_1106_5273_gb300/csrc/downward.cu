@@ -2,6 +2,8 @@
 // giving grad and Hessian of the three vector-potential components, hence
 //   u = (1/4pi) curl psi,  s = (gamma_i . grad) u          (Eqs. 1 and 3)
 // for the far field, written in sorted particle order.
+#include <type_traits>
+
 #include "expansions.cuh"
 #include "fmm_internal.cuh"
 
@@ -35,8 +37,19 @@ __global__ void __launch_bounds__(128) k_l2l(int lb, const int* __restrict__ par
   }
 }
 
-// One CTA per leaf, one thread per particle.
-__global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, const int* __restrict__ begin,
+// One CTA per leaf.  Leaves of more than 32 particles take one thread each.
+// Leaves of at most 32, 16 or 8 are served by 2, 4 or 8 groups of threads that
+// share the columns m of the expansion (folded, so that long and short columns
+// pair up) and add their sums at the end (p >= 8): adaptive trees have leaves
+// of about 20 particles, and a thread's chain over all columns was the kernel's
+// time.  Bound by the shared-memory reads of the coefficients and that chain.
+// Plummer 1,000,000 at p = 12 1.41 -> 0.90 ms, Taylor-Green 128^3 (full leaves)
+// 0.55 -> 0.49 ms.
+constexpr int kL2PThreads = 64;
+// floats before the recurrence factors: the coefficients and the expansion, or
+// the groups' sums
+__host__ __device__ inline int l2p_floats(int P) { return 33 * P + (P & 1) > 30 * 32 ? 33 * P + (P & 1) : 30 * 32; }
+__global__ void __launch_bounds__(kL2PThreads) k_l2p(const int* __restrict__ leaves, const int* __restrict__ begin,
                                             const int* __restrict__ end, const int* __restrict__ level,
                                             const double* __restrict__ center, const double* __restrict__ box,
                                             const int* __restrict__ cseg,
@@ -47,8 +60,12 @@ __global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, cons
   const int P = p * p;
   float2* sD = reinterpret_cast<float2*>(sm);  // [3][5][P] complex, see below
   float* sL = sm + 2 * 15 * P;                 // [3][P]
+  float2* sC = reinterpret_cast<float2*>(sm + l2p_floats(P));  // recurrence factors
   const int leaf = leaves[blockIdx.x];
   for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) sL[i] = L[(size_t)leaf * 3 * P + i];
+  const int b = begin[leaf], e = end[leaf];
+  const int width = column_width(e - b, p, kL2PThreads), G = kL2PThreads / width;
+  if (G > 1) fill_recurrence(sC, p, threadIdx.x, kL2PThreads);
   __syncthreads();
   const int on[5] = {1, 1, 2, 2, 2};
   // The leaf's coefficients of the derivative expansions, once per leaf:
@@ -63,11 +80,16 @@ __global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, cons
     for (int q = 0; q < 3; ++q) sD[q * 5 * P + e] = make_float2(cre * sL[q * P + t.x], cim * sL[q * P + t.y]);
   }
   __syncthreads();
-  const int b = begin[leaf], e = end[leaf];
   const double a = box[4 * (cseg ? cseg[leaf] : 0) + 3] * ldexp(1.0, -level[leaf]);
   const float inv_a = (float)(1.0 / a);
   const double cx = center[3 * leaf], cy = center[3 * leaf + 1], cz = center[3 * leaf + 2];
-  for (int j = b + threadIdx.x; j < e; j += blockDim.x) {
+  const int grp = threadIdx.x / width, tl = threadIdx.x % width;
+  auto eval = [&](auto grouped) {
+  constexpr bool GR = decltype(grouped)::value;
+  for (int j0 = b; j0 < e; j0 += width) {  // once when there are groups
+    const bool live = j0 + tl < e;
+    if (!GR && !live) continue;
+    const int j = live ? j0 + tl : b;
     float4 x = A[j];
     float4 g = B[j];
     const float X = (float)((double)x.x - cx) * inv_a;
@@ -80,28 +102,32 @@ __global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, cons
 #pragma unroll
       for (int o = 0; o < 5; ++o) acc[q][o][0] = acc[q][o][1] = 0.f;
     float dre = 1.f, dim = 0.f;  // R~_m^m
-    for (int m = 0; m < p - 1; ++m) {
-      if (m > 0) {
-        float f = sqrtf((2.f * m - 1.f) / (2.f * m));
-        float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
+    int at = 0;
+    for (int i = 0; (GR ? i * G : i) < p - 1; ++i) {
+      const int m = GR ? folded_column(i, grp, G) : i;
+      if (m >= p - 1) continue;
+      while (at < m) {
+        ++at;
+        const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
+        const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
         dre = nr;
         dim = ni;
       }
       float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{k-1}, R~_k
       for (int k = m; k < p - 1; ++k) {
         if (k > m) {
-          float inv = rsqrtf((float)((k + m) * (k - m)));
+          const float2 cf = GR ? sC[k * (k + 1) / 2 + m] : recurrence(k, m);
           float aa = (2.f * k - 1.f) * Z;
           float vr = aa * r0r, vi = aa * r0i;
           if (k - 2 >= m) {
-            float bb = r2 * sqrtf((float)((k + m - 1) * (k - m - 1)));
+            float bb = r2 * cf.y;
             vr -= bb * r1r;
             vi -= bb * r1i;
           }
           r1r = r0r;
           r1i = r0i;
-          r0r = vr * inv;
-          r0i = vi * inv;
+          r0r = vr * cf.x;
+          r0i = vi * cf.x;
         }
         // contributions of R~_k^{+m} and R~_k^{-m}
 #pragma unroll
@@ -124,6 +150,21 @@ __global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, cons
         }
       }
     }
+    if (GR) {  // the groups' sums: within the warps, then the second warp's to the first
+      __syncthreads();
+      float* red = sm;  // [30][32]; the coefficients have been used
+#pragma unroll
+      for (int i = 0; i < 30; ++i) {
+        float& v = acc[i / 10][i / 2 % 5][i & 1];
+        for (int o = width; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x >= 32) red[i * 32 + (threadIdx.x & 31)] = v;
+      }
+      __syncthreads();
+      if (threadIdx.x >= 32) return;
+#pragma unroll
+      for (int i = 0; i < 30; ++i) acc[i / 10][i / 2 % 5][i & 1] += red[i * 32 + threadIdx.x];
+    }
+    if (GR && (!live || grp)) continue;
     // grad / Hessian of Phi_q (unnormalized: L'_n' = a^-(n'+1) acc)
     const float s2 = inv_a * inv_a, s3 = s2 * inv_a;
     float G[3][3], H[3][3][3];
@@ -169,6 +210,9 @@ __global__ void __launch_bounds__(64) k_l2p(const int* __restrict__ leaves, cons
     far_s[3 * j + 1] = sy * c4;
     far_s[3 * j + 2] = sz * c4;
   }
+  };
+  if (G > 1) eval(std::true_type{});
+  else eval(std::false_type{});
 }
 
 }  // namespace
@@ -185,7 +229,7 @@ int downward_pass(fmm_plan p, int64_t n, cudaStream_t s) {
   FMM_TRY(p->far_u.ensure((size_t)n * 3 * sizeof(float)));
   FMM_TRY(p->far_s.ensure((size_t)n * 3 * sizeof(float)));
   ++g_launches;
-  k_l2p<<<(unsigned)p->nleaves, 64, (2 * 15 + 3) * P * sizeof(float), s>>>(
+  k_l2p<<<(unsigned)p->nleaves, kL2PThreads, l2p_floats(P) * sizeof(float) + recurrence_bytes(p->prm.p), s>>>(
       p->leaves.as<int>(), p->c_begin.as<int>(), p->c_end.as<int>(), p->c_level.as<int>(), p->c_center.as<double>(),
       p->batched ? p->seg_box.as<double>() : p->scal.as<double>(), p->batched ? p->c_seg.as<int>() : nullptr,
       p->sortA.as<float4>(), p->sortB.as<float4>(), p->L.as<float>(), p->l2p_tab.as<int4>(),

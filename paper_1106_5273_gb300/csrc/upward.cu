@@ -3,6 +3,8 @@
 // Three potentials (one per component of gamma) share the expansions.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "expansions.cuh"
 #include "fmm_internal.cuh"
 
@@ -13,7 +15,11 @@ namespace {
 constexpr int kP2MThreads = 64;  // particles per pass of k_p2m (one per thread)
 constexpr int kP2MRows = 4;      // output rows per thread: P <= 256 (p <= 16)
 
-// One CTA per leaf; threads own coefficients r = tid, tid + 128.
+// One CTA per leaf; threads own coefficients r = tid, tid + 64, ...  The harmonics
+// of a chunk of at most 32, 16 or 8 particles are built by 2, 4 or 8 groups of
+// threads, which share the columns m (p >= 8).  Bound by the recurrences' chain
+// and the row stores: Plummer 1,000,000 at p = 12 took 0.76 ms with one thread
+// per particle and the empty rows cleared, now 0.55.
 __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ leaves, const int* __restrict__ begin,
                                                      const int* __restrict__ end, const int* __restrict__ level,
                                                      const double* __restrict__ center,
@@ -25,6 +31,8 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
   const int PS = P | 1;                          // odd row stride: the per-thread row stores hit distinct banks
   float* sR = sm;                                // [kP2MThreads][PS] conj(R~) real-packed
   float4* sG = reinterpret_cast<float4*>(sm + ((kP2MThreads * PS + 3) & ~3));  // [kP2MThreads]
+  // recurrence factors of a grouped chunk, in the rows that it leaves free
+  float2* sC = reinterpret_cast<float2*>(sR + 32 * PS);
   const int leaf = leaves[blockIdx.x];
   const int b = begin[leaf], e = end[leaf];
   const double a = box[4 * (cseg ? cseg[leaf] : 0) + 3] * ldexp(1.0, -level[leaf]);
@@ -35,22 +43,29 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
 #pragma unroll
   for (int q = 0; q < kP2MRows; ++q) acc[0][q] = acc[1][q] = acc[2][q] = 0.f;
   for (int c0 = b; c0 < e; c0 += kP2MThreads) {
-    // one particle per thread: the regular solid harmonics R~_n^m by the
-    // recurrences in registers (the diagonal m = n, then up each column m),
-    // stored conjugated in real-packed order
-    const int j = c0 + t;
-    float* row = sR + t * PS;
-    if (j < e) {
-      const float4 x = A[j];
-      const float4 g = B[j];
+    const int cnt = min(kP2MThreads, e - c0);
+    const int width = column_width(cnt, p, kP2MThreads), G = kP2MThreads / width;
+    const int grp = t / width, tl = t % width;
+    // the regular solid harmonics R~_n^m of a particle by the recurrences in
+    // registers (the diagonal m = n, then up each column m), stored conjugated
+    // in real-packed order
+    auto rows = [&](auto grouped) {
+    constexpr bool GR = decltype(grouped)::value;
+    if (tl < cnt) {
+      float* row = sR + tl * PS;
+      const float4 x = A[c0 + tl];
       const float X = (float)((double)x.x - cx) * inv_a;
       const float Y = (float)((double)x.y - cy) * inv_a;
       const float Z = (float)((double)x.z - cz) * inv_a;
       const float r2 = X * X + Y * Y + Z * Z;
       float dre = 1.f, dim = 0.f;  // R~_m^m
-      for (int m = 0; m < p; ++m) {
-        if (m > 0) {
-          const float f = sqrtf((2.f * m - 1.f) / (2.f * m));
+      int at = 0;
+      for (int i = 0; (GR ? i * G : i) < p; ++i) {
+        const int m = GR ? folded_column(i, grp, G) : i;
+        if (m >= p) continue;
+        while (at < m) {
+          ++at;
+          const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
           const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
           dre = nr;
           dim = ni;
@@ -58,18 +73,18 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
         float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{n-1}^m, R~_n^m
         for (int n = m; n < p; ++n) {
           if (n > m) {
-            const float inv = rsqrtf((float)((n + m) * (n - m)));
+            const float2 cf = GR ? sC[n * (n + 1) / 2 + m] : recurrence(n, m);
             const float aa = (2.f * n - 1.f) * Z;
             float vr = aa * r0r, vi = aa * r0i;
             if (n - 2 >= m) {
-              const float bb = r2 * sqrtf((float)((n + m - 1) * (n - m - 1)));
+              const float bb = r2 * cf.y;
               vr -= bb * r1r;
               vi -= bb * r1i;
             }
             r1r = r0r;
             r1i = r0i;
-            r0r = vr * inv;
-            r0i = vi * inv;
+            r0r = vr * cf.x;
+            r0i = vi * cf.x;
           }
           if (m == 0) {
             row[n * n] = r0r;
@@ -79,14 +94,21 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
           }
         }
       }
-      sG[t] = make_float4(g.x, g.y, g.z, 0.f);
+      if (grp == 0) {
+        const float4 g = B[c0 + tl];
+        sG[tl] = make_float4(g.x, g.y, g.z, 0.f);
+      }
+    }
+    };
+    if (G > 1) {
+      fill_recurrence(sC, p, t, kP2MThreads);
+      __syncthreads();
+      rows(std::true_type{});
     } else {
-      for (int r = 0; r < P; ++r) row[r] = 0.f;
-      sG[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+      rows(std::false_type{});
     }
     __syncthreads();
     // M_c[r] += sum over the chunk's particles of gamma_c R~*[r]
-    const int cnt = min(kP2MThreads, e - c0);
 #pragma unroll
     for (int q = 0; q < kP2MRows; ++q) {
       const int r = t + kP2MThreads * q;
@@ -109,51 +131,86 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
   }
 }
 
-// One CTA per cell of the level; leaves keep their P2M result.  The cell's
-// expansion is the sum, in child order, of each child's term.
-__global__ void __launch_bounds__(128) k_m2m(int lb, const int* __restrict__ child, const int* __restrict__ nchild,
-                                             const uint64_t* __restrict__ ckey, const float* __restrict__ opT, int P,
-                                             float* __restrict__ M) {
-  extern __shared__ float sMc[];  // [3][P]
-  const int c = lb + blockIdx.x;
-  const int nch = nchild[c];
-  if (nch == 0) return;
-  float acc[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (int q = 0; q < nch; ++q) {
-    const int ch = child[c] + q;
-    const int oct = (int)(ckey[ch] & 7ull);
-    for (int i = threadIdx.x; i < 3 * P; i += blockDim.x) sMc[i] = M[(size_t)ch * 3 * P + i];
-    __syncthreads();
-    const float* W = opT + (size_t)oct * P * P;
-    for (int h = 0; h < 2; ++h) {
-      int r = threadIdx.x + 128 * h;
-      if (r >= P) break;
-      // the child's term, then added to the sum of the earlier children's
-      // (the order and rounding of k_m2m8)
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+// Four consecutive cells of the level per CTA; leaves keep their P2M result.  The
+// cell's expansion is the sum, in child order, of each child's term.  Each of
+// four groups of threads (thread = output row) applies two octants' operators
+// to the four cells' children there: an operator row comes from L2 once for
+// four cells, which is what one CTA per cell was bound by (Plummer 1,000,000
+// at p = 12: 1.33 -> 0.86 ms, Taylor-Green 128^3 0.25 -> 0.15 ms, ball of
+// 100,003 0.077 -> 0.021).  L2L in the same form (four parents per CTA and
+// octant) gained nothing: half of those children do not exist.
+constexpr int kMCells = 4, kMGroups = 4;
+__global__ void __launch_bounds__(kMGroups * 256) k_m2m(int lb, int le, const int* __restrict__ child,
+                                                        const int* __restrict__ nchild,
+                                                        const uint64_t* __restrict__ ckey,
+                                                        const float* __restrict__ opT, int P, float* __restrict__ M) {
+  extern __shared__ float4 sM4[];  // [8 octants][3][P] x the cells: the children's expansions, then their terms
+  __shared__ int kid[8][kMCells];
+  float* sMf = reinterpret_cast<float*>(sM4);
+  const int c0 = lb + kMCells * (int)blockIdx.x;
+  if (threadIdx.x < 8 * kMCells) kid[threadIdx.x / kMCells][threadIdx.x % kMCells] = -1;
+  __syncthreads();
+  if (threadIdx.x < 8 * kMCells) {
+    const int q = threadIdx.x / 8, i = threadIdx.x % 8, c = c0 + q;
+    if (c < le && i < nchild[c]) kid[(int)(ckey[child[c] + i] & 7ull)][q] = child[c] + i;
+  }
+  __syncthreads();
+  const int W0 = blockDim.x / kMGroups, g = threadIdx.x / W0, r = threadIdx.x % W0;
+  for (int o = 2 * g; o < 2 * g + 2; ++o)
+#pragma unroll
+    for (int q = 0; q < kMCells; ++q) {
+      const int ch = kid[o][q];
+      for (int i = r; i < 3 * P; i += W0) sMf[kMCells * (o * 3 * P + i) + q] = ch >= 0 ? M[(size_t)ch * 3 * P + i] : 0.f;
+    }
+  __syncthreads();
+  float acc[2][3][kMCells];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int q = 0; q < kMCells; ++q) acc[h][c][q] = 0.f;
+    const int o = 2 * g + h;
+    if (r >= P || (kid[o][0] & kid[o][1] & kid[o][2] & kid[o][3]) < 0) {
+      // all four absent: -1 & -1 & -1 & -1 < 0 (one present index clears the sign bit)
+      continue;
+    }
+    const float* W = opT + (size_t)o * P * P + r;
+    const float4* x4 = sM4 + o * 3 * P;
 #pragma unroll 8
-      for (int k = 0; k < P; ++k) {
-        float w = W[(size_t)k * P + r];
-        a0 = fmaf(w, sMc[k], a0);
-        a1 = fmaf(w, sMc[P + k], a1);
-        a2 = fmaf(w, sMc[2 * P + k], a2);
-      }
-      if (q == 0) {
-        acc[0][h] = a0;
-        acc[1][h] = a1;
-        acc[2][h] = a2;
-      } else {
-        acc[0][h] += a0;
-        acc[1][h] += a1;
-        acc[2][h] += a2;
+    for (int k = 0; k < P; ++k) {
+      const float w = W[(size_t)k * P];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float4 x = x4[c * P + k];
+        acc[h][c][0] = fmaf(w, x.x, acc[h][c][0]);
+        acc[h][c][1] = fmaf(w, x.y, acc[h][c][1]);
+        acc[h][c][2] = fmaf(w, x.z, acc[h][c][2]);
+        acc[h][c][3] = fmaf(w, x.w, acc[h][c][3]);
       }
     }
-    __syncthreads();
   }
-  for (int h = 0; h < 2; ++h) {
-    int r = threadIdx.x + 128 * h;
-    if (r >= P) break;
-    for (int cc = 0; cc < 3; ++cc) M[((size_t)c * 3 + cc) * P + r] = acc[cc][h];
+  __syncthreads();
+  if (r < P)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        sM4[((2 * g + h) * 3 + c) * P + r] = make_float4(acc[h][c][0], acc[h][c][1], acc[h][c][2], acc[h][c][3]);
+  __syncthreads();
+  // group g sums cell g's terms in child order (the order and rounding of k_m2m8)
+  const int c = c0 + g;
+  if (c >= le || nchild[c] == 0) return;
+  for (int e = r; e < 3 * P; e += W0) {
+    float sum = 0.f;
+    bool first = true;
+    for (int o = 0; o < 8; ++o) {
+      if (kid[o][g] < 0) continue;
+      const float v = sMf[kMCells * (o * 3 * P + e) + g];
+      sum = first ? v : sum + v;
+      first = false;
+    }
+    M[(size_t)c * 3 * P + e] = sum;
   }
 }
 
@@ -164,7 +221,7 @@ __global__ void __launch_bounds__(128) k_m2m(int lb, const int* __restrict__ chi
 // and the cell's expansion is the sum of the children's terms in child
 // order (a fixed order, so the result is deterministic).
 constexpr int kM2MGroup = 128;
-constexpr int kM2MWide = 1024;  // levels of at least this many cells use k_m2m (one 128-thread CTA per cell)
+constexpr int kM2MWide = 1024;  // levels of at least this many cells use k_m2m
 __global__ void __launch_bounds__(8 * kM2MGroup) k_m2m8(int lb, const int* __restrict__ child,
                                                        const int* __restrict__ nchild,
                                                        const uint64_t* __restrict__ ckey,
@@ -266,13 +323,15 @@ int upward_pass(fmm_plan p, cudaStream_t s) {
   const size_t sh_m2m = (size_t)2 * 8 * 3 * P * sizeof(float);  // 48 KB at P = 256
   if (sh_m2m > 48 * 1024)
     FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_m2m));
+  if (2 * sh_m2m > 48 * 1024)
+    FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * sh_m2m)));
   for (int l = p->nlevels - 2; l >= 0; --l) {
     int lb = p->level_begin[l], le = p->level_begin[l + 1];
     ++g_launches;
     if (le - lb >= kM2MWide)
-      k_m2m<<<le - lb, 128, 3 * P * sizeof(float), s>>>(lb, p->c_child.as<int>(), p->c_nchild.as<int>(),
-                                                        p->c_key.as<uint64_t>(), p->m2m_T.as<float>(), P,
-                                                        p->M.as<float>());
+      k_m2m<<<(le - lb + kMCells - 1) / kMCells, kMGroups * ((P + 31) & ~31), kMCells * 8 * 3 * P * sizeof(float), s>>>(
+          lb, le, p->c_child.as<int>(), p->c_nchild.as<int>(), p->c_key.as<uint64_t>(), p->m2m_T.as<float>(), P,
+          p->M.as<float>());
     else
       k_m2m8<<<le - lb, 8 * kM2MGroup, 2 * 8 * 3 * P * sizeof(float), s>>>(
           lb, p->c_child.as<int>(), p->c_nchild.as<int>(), p->c_key.as<uint64_t>(), p->m2m_T.as<float>(), P,
