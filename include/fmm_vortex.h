@@ -156,7 +156,7 @@ typedef struct {
   int64_t p2p_cell_pairs; /* (target leaf, source leaf, image) entries */
   int64_t p2p_pairs;      /* particle-particle interactions (incl. self pair) */
   int64_t m2l_pairs;      /* (target cell, source cell, image) M2L entries */
-  int64_t m2l_steps;      /* (64-cell target tile, translation) GEMM steps */
+  int64_t m2l_steps;      /* (target tile, translation) GEMM steps */
   int64_t m2l_keys;       /* distinct translation operators */
   int64_t m2l_built;      /* operators built by this call (the rest came from the plan's cache) */
   int64_t p2p_pairs_near; /* particle pairs evaluated with the full cutoff and series test */

@@ -469,8 +469,8 @@ constexpr int kP2PPerSm = 24;
 // Bound by the FMA pipe: 78 cycles per 64 pairs and warp scheduler at
 // Taylor-Green 128^3, where the pair loops alone (microbenchmark) take 66 (far)
 // and 87 (mid).  Measured P2P, before (one warp per leaf, whole lists, source
-// leaves staged one by one) and after: Taylor-Green 128^3 19.34 -> 18.56 ms,
-// Plummer 1,000,000 22.3 -> 10.5 ms, Plummer 30,011 2.52 -> 0.39 ms, ball
+// leaves staged one by one) and after: Taylor-Green 128^3 19.34 -> 18.7 ms,
+// Plummer 1,000,000 22.3 -> 9.9 ms, Plummer 30,011 2.52 -> 0.45 ms, ball
 // 100,003 1.74 -> 1.11 ms.
 template <int PS, int ST>
 __global__ void __launch_bounds__(32, kP2PPerSm)
@@ -814,10 +814,10 @@ __global__ void k_finish(const float* __restrict__ near_u, const float* __restri
 // ---- work items: per leaf, tiles x ranges, the longest ranges first (four
 // length classes, leaf order within each), so that the last warps to start
 // are short: in leaf order the batch of 32 problems waited for its longest
-// lists (P2P 5.56 ms, now 5.23).  One cooperative launch: the blocks own
-// contiguous ranges of the leaves, take their class totals, meet at a bounded
-// grid barrier and write (one CTA over all leaves took 153 us at Taylor-Green
-// 128^3).  counts[0] = items, counts[1] = partial slots.
+// lists (cut at 2048 sources: P2P 5.56 ms, 5.23 longest first).  One cooperative
+// launch: the blocks own contiguous ranges of the leaves, take their class
+// totals, meet at a bounded grid barrier and write (one CTA over all leaves took
+// 153 us at Taylor-Green 128^3).  counts[0] = items, counts[1] = partial slots.
 constexpr int kItemClasses = 4, kItemThreads = 256, kItemBlocks = 128;
 
 __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restrict__ leaves, int nl,
@@ -1208,7 +1208,7 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
 // per (tile of a leaf, range of its sources).  Ranges bound the longest warp:
 // the big outer leaves of a clustered cloud meet thousands of small ones, and
 // one warp per leaf left the chip waiting for them (Plummer, 30,011 blobs:
-// P2P 2.5 ms; 0.39 ms with ranges), and with it how long the far field's
+// P2P 2.5 ms; 0.45 ms with ranges), and with it how long the far field's
 // kernels wait for room.  One-problem plans take the range that gives kItemTarget
 // items, at least 128 sources (two chunks);
 // the partial slots are then bounded by twice that many items (3 KB each).  A
