@@ -170,6 +170,13 @@ __device__ inline void split_of(const TravArgs& t, int a, int b, bool& split_a, 
 // level.
 
 constexpr int kTravThreads = 256;
+// Pairs per block from which a thread classifies a whole pair instead of one
+// child.  Below, a thread's chain over up to eight children with dependent loads
+// is the level's time (Plummer 30,011: 2.01 -> 1.91 ms per evaluation with eight
+// lanes per pair, ball 100,003 2.10 -> 2.08); above, the loads of the pair itself,
+// repeated by every lane, cost more than that (Taylor-Green 128^3: 25.90 ms, 26.02
+// with lanes only; 512 and 8192 are within 0.1% of 2048 but on that case).
+constexpr uint32_t kTravWide = 2048;
 constexpr int kTravMaxIter = 128;         // > 2 x the 22 levels a pair can descend
 
 struct TravState {
@@ -224,9 +231,11 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
   for (; nf > 0 && iter < kTravMaxIter; ++iter) {
     const uint32_t chunk = (nf + G - 1) / G;
     const uint32_t i0 = min(nf, b * chunk), i1 = min(nf, i0 + chunk);
-    // phase A: classify the block's pairs, block totals
+    // phase A: classify the block's pairs, block totals.  Mask of a pair: bit q
+    // child q is a P2P pair, bit 8 + q it goes on, bits 16 up the children.
     uint32_t c[3] = {0u, 0u, 0u};
-    for (uint32_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    const bool wide = chunk > kTravWide;
+    for (uint32_t i = i0 + threadIdx.x; wide && i < i1; i += blockDim.x) {
       const int4 pr = cur[i];
       bool sa;
       int c0, ncc;
@@ -235,10 +244,32 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
       for (int q = 0; q < ncc; ++q) {
         const int ch = c0 + q;
         const int ty = sa ? interact(t, ch, pr.y, pr.z) : interact(t, pr.x, ch, pr.z);
-        msk |= (uint32_t)ty << (2 * q);
+        msk |= (uint32_t)((ty & 1) | (ty & 2) << 7) << q;
         c[ty] += 1u;
       }
-      mask[i] = msk | ((uint32_t)ncc << 16);
+      mask[i] = msk | (uint32_t)ncc << 16;
+    }
+    for (uint32_t base = i0; !wide && base < i1; base += kTravThreads / 8) {
+      const uint32_t i = base + threadIdx.x / 8;
+      const int q = threadIdx.x & 7;
+      int ncc = 0, ty = -1;
+      if (i < i1) {
+        const int4 pr = cur[i];
+        bool sa;
+        int c0;
+        split_of(t, pr.x, pr.y, sa, c0, ncc);
+        if (q < ncc) {
+          const int ch = c0 + q;
+          ty = interact(t, sa ? ch : pr.x, sa ? pr.y : ch, pr.z);
+          c[0] += ty == 0;
+          c[1] += ty == 1;
+          c[2] += ty == 2;
+        }
+      }
+      const int sh = threadIdx.x & 24;
+      const uint32_t is1 = __ballot_sync(0xffffffffu, ty == 1) >> sh & 0xffu;
+      const uint32_t is2 = __ballot_sync(0xffffffffu, ty == 2) >> sh & 0xffu;
+      if (i < i1 && q == 0) mask[i] = is1 | is2 << 8 | (uint32_t)ncc << 16;
     }
     {
       const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -298,7 +329,9 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
       if (i < i1) {
         msk = mask[i];
         ncc = msk >> 16;
-        for (uint32_t q = 0; q < ncc; ++q) v[(msk >> (2 * q)) & 3u] += 1u;
+        v[1] = __popc(msk & 0xffu);
+        v[2] = __popc(msk & 0xff00u);
+        v[0] = ncc - v[1] - v[2];
       }
       uint32_t tot[3];
       block_scan3(v, tot);
@@ -311,7 +344,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
         for (uint32_t q = 0; q < ncc; ++q) {
           const int ch = c0 + (int)q;
           const int4 val = sa ? make_int4(ch, pr.y, pr.z, 0) : make_int4(pr.x, ch, pr.z, 0);
-          const uint32_t ty = (msk >> (2 * q)) & 3u;
+          const uint32_t ty = (msk >> q & 1u) | (msk >> (q + 7) & 2u);
           if (ty == 0) m2l[im++] = pack_m2l(val.x, val.y, val.z);
           else if (ty == 1) p2p[ip++] = val;
           else nxt[iff++] = val;
