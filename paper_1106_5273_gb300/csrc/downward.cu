@@ -85,131 +85,131 @@ __global__ void __launch_bounds__(kL2PThreads) k_l2p(const int* __restrict__ lea
   const double cx = center[3 * leaf], cy = center[3 * leaf + 1], cz = center[3 * leaf + 2];
   const int grp = threadIdx.x / width, tl = threadIdx.x % width;
   auto eval = [&](auto grouped) {
-  constexpr bool GR = decltype(grouped)::value;
-  for (int j0 = b; j0 < e; j0 += width) {  // once when there are groups
-    const bool live = j0 + tl < e;
-    if (!GR && !live) continue;
-    const int j = live ? j0 + tl : b;
-    float4 x = A[j];
-    float4 g = B[j];
-    const float X = (float)((double)x.x - cx) * inv_a;
-    const float Y = (float)((double)x.y - cy) * inv_a;
-    const float Z = (float)((double)x.z - cz) * inv_a;
-    const float r2 = X * X + Y * Y + Z * Z;
-    float acc[3][5][2];
+    constexpr bool GR = decltype(grouped)::value;
+    for (int j0 = b; j0 < e; j0 += width) {  // once when there are groups
+      const bool live = j0 + tl < e;
+      if (!GR && !live) continue;
+      const int j = live ? j0 + tl : b;
+      float4 x = A[j];
+      float4 g = B[j];
+      const float X = (float)((double)x.x - cx) * inv_a;
+      const float Y = (float)((double)x.y - cy) * inv_a;
+      const float Z = (float)((double)x.z - cz) * inv_a;
+      const float r2 = X * X + Y * Y + Z * Z;
+      float acc[3][5][2];
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
+      for (int q = 0; q < 3; ++q)
 #pragma unroll
-      for (int o = 0; o < 5; ++o) acc[q][o][0] = acc[q][o][1] = 0.f;
-    float dre = 1.f, dim = 0.f;  // R~_m^m
-    int at = 0;
-    for (int i = 0; (GR ? i * G : i) < p - 1; ++i) {
-      const int m = GR ? folded_column(i, grp, G) : i;
-      if (m >= p - 1) continue;
-      while (at < m) {
-        ++at;
-        const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
-        const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
-        dre = nr;
-        dim = ni;
-      }
-      float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{k-1}, R~_k
-      for (int k = m; k < p - 1; ++k) {
-        if (k > m) {
-          const float2 cf = GR ? sC[k * (k + 1) / 2 + m] : recurrence(k, m);
-          float aa = (2.f * k - 1.f) * Z;
-          float vr = aa * r0r, vi = aa * r0i;
-          if (k - 2 >= m) {
-            float bb = r2 * cf.y;
-            vr -= bb * r1r;
-            vi -= bb * r1i;
-          }
-          r1r = r0r;
-          r1i = r0i;
-          r0r = vr * cf.x;
-          r0i = vi * cf.x;
+        for (int o = 0; o < 5; ++o) acc[q][o][0] = acc[q][o][1] = 0.f;
+      float dre = 1.f, dim = 0.f;  // R~_m^m
+      int at = 0;
+      for (int i = 0; (GR ? i * G : i) < p - 1; ++i) {
+        const int m = GR ? folded_column(i, grp, G) : i;
+        if (m >= p - 1) continue;
+        while (at < m) {
+          ++at;
+          const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
+          const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
+          dre = nr;
+          dim = ni;
         }
-        // contributions of R~_k^{+m} and R~_k^{-m}
-#pragma unroll
-        for (int o = 0; o < 5; ++o) {
-          if (on[o] + k > p - 1) continue;
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const float2 d = sD[(q * 5 + o) * P + k * k + k + m];
-            acc[q][o][0] = fmaf(d.x, r0r, fmaf(-d.y, r0i, acc[q][o][0]));
-            acc[q][o][1] = fmaf(d.x, r0i, fmaf(d.y, r0r, acc[q][o][1]));
+        float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{k-1}, R~_k
+        for (int k = m; k < p - 1; ++k) {
+          if (k > m) {
+            const float2 cf = GR ? sC[k * (k + 1) / 2 + m] : recurrence(k, m);
+            float aa = (2.f * k - 1.f) * Z;
+            float vr = aa * r0r, vi = aa * r0i;
+            if (k - 2 >= m) {
+              float bb = r2 * cf.y;
+              vr -= bb * r1r;
+              vi -= bb * r1i;
+            }
+            r1r = r0r;
+            r1i = r0i;
+            r0r = vr * cf.x;
+            r0i = vi * cf.x;
           }
-          if (m > 0) {
+          // contributions of R~_k^{+m} and R~_k^{-m}
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {  // conj(R~_k^m)
-              const float2 d = sD[(q * 5 + o) * P + k * k + k - m];
-              acc[q][o][0] = fmaf(d.x, r0r, fmaf(d.y, r0i, acc[q][o][0]));
-              acc[q][o][1] = fmaf(-d.x, r0i, fmaf(d.y, r0r, acc[q][o][1]));
+          for (int o = 0; o < 5; ++o) {
+            if (on[o] + k > p - 1) continue;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const float2 d = sD[(q * 5 + o) * P + k * k + k + m];
+              acc[q][o][0] = fmaf(d.x, r0r, fmaf(-d.y, r0i, acc[q][o][0]));
+              acc[q][o][1] = fmaf(d.x, r0i, fmaf(d.y, r0r, acc[q][o][1]));
+            }
+            if (m > 0) {
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {  // conj(R~_k^m)
+                const float2 d = sD[(q * 5 + o) * P + k * k + k - m];
+                acc[q][o][0] = fmaf(d.x, r0r, fmaf(d.y, r0i, acc[q][o][0]));
+                acc[q][o][1] = fmaf(-d.x, r0i, fmaf(d.y, r0r, acc[q][o][1]));
+              }
             }
           }
         }
       }
-    }
-    if (GR) {  // the groups' sums: within the warps, then the second warp's to the first
-      __syncthreads();
-      float* red = sm;  // [30][32]; the coefficients have been used
+      if (GR) {  // the groups' sums: within the warps, then the second warp's to the first
+        __syncthreads();
+        float* red = sm;  // [30][32]; the coefficients have been used
 #pragma unroll
-      for (int i = 0; i < 30; ++i) {
-        float& v = acc[i / 10][i / 2 % 5][i & 1];
-        for (int o = width; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x >= 32) red[i * 32 + (threadIdx.x & 31)] = v;
+        for (int i = 0; i < 30; ++i) {
+          float& v = acc[i / 10][i / 2 % 5][i & 1];
+          for (int o = width; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (threadIdx.x >= 32) red[i * 32 + (threadIdx.x & 31)] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x >= 32) return;
+#pragma unroll
+        for (int i = 0; i < 30; ++i) acc[i / 10][i / 2 % 5][i & 1] += red[i * 32 + threadIdx.x];
       }
-      __syncthreads();
-      if (threadIdx.x >= 32) return;
+      if (GR && (!live || grp)) continue;
+      // grad / Hessian of Phi_q (unnormalized: L'_n' = a^-(n'+1) acc)
+      const float s2 = inv_a * inv_a, s3 = s2 * inv_a;
+      float G[3][3], H[3][3][3];
 #pragma unroll
-      for (int i = 0; i < 30; ++i) acc[i / 10][i / 2 % 5][i & 1] += red[i * 32 + threadIdx.x];
-    }
-    if (GR && (!live || grp)) continue;
-    // grad / Hessian of Phi_q (unnormalized: L'_n' = a^-(n'+1) acc)
-    const float s2 = inv_a * inv_a, s3 = s2 * inv_a;
-    float G[3][3], H[3][3][3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      G[q][0] = acc[q][1][0] * s2;
-      G[q][1] = -acc[q][1][1] * s2;
-      G[q][2] = acc[q][0][0] * s2;
-      float L0 = acc[q][2][0] * s3, a1 = acc[q][3][0] * s3, b1 = acc[q][3][1] * s3;
-      float a2 = acc[q][4][0] * s3, b2 = acc[q][4][1] * s3;
-      H[q][0][0] = 0.5f * (a2 - L0);
-      H[q][1][1] = 0.5f * (-a2 - L0);
-      H[q][2][2] = L0;
-      H[q][0][1] = H[q][1][0] = -0.5f * b2;
-      H[q][0][2] = H[q][2][0] = a1;
-      H[q][1][2] = H[q][2][1] = -b1;
-    }
-    const float c4 = 0.0795774715459476679f;
-    float ux = G[2][1] - G[1][2], uy = G[0][2] - G[2][0], uz = G[1][0] - G[0][1];
-    const float gv[3] = {g.x, g.y, g.z};
-    float sx = 0.f, sy = 0.f, sz = 0.f;
-    if (transpose) {  // s_d = sum_l gamma_l d u_l / d x_d
-      float sd[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-        sd[d] = gv[0] * (H[2][d][1] - H[1][d][2]) + gv[1] * (H[0][d][2] - H[2][d][0]) +
-                gv[2] * (H[1][d][0] - H[0][d][1]);
-      sx = sd[0];
-      sy = sd[1];
-      sz = sd[2];
-    } else {  // s_l = sum_d gamma_d d u_l / d x_d
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        sx += gv[d] * (H[2][d][1] - H[1][d][2]);
-        sy += gv[d] * (H[0][d][2] - H[2][d][0]);
-        sz += gv[d] * (H[1][d][0] - H[0][d][1]);
+      for (int q = 0; q < 3; ++q) {
+        G[q][0] = acc[q][1][0] * s2;
+        G[q][1] = -acc[q][1][1] * s2;
+        G[q][2] = acc[q][0][0] * s2;
+        float L0 = acc[q][2][0] * s3, a1 = acc[q][3][0] * s3, b1 = acc[q][3][1] * s3;
+        float a2 = acc[q][4][0] * s3, b2 = acc[q][4][1] * s3;
+        H[q][0][0] = 0.5f * (a2 - L0);
+        H[q][1][1] = 0.5f * (-a2 - L0);
+        H[q][2][2] = L0;
+        H[q][0][1] = H[q][1][0] = -0.5f * b2;
+        H[q][0][2] = H[q][2][0] = a1;
+        H[q][1][2] = H[q][2][1] = -b1;
       }
+      const float c4 = 0.0795774715459476679f;
+      float ux = G[2][1] - G[1][2], uy = G[0][2] - G[2][0], uz = G[1][0] - G[0][1];
+      const float gv[3] = {g.x, g.y, g.z};
+      float sx = 0.f, sy = 0.f, sz = 0.f;
+      if (transpose) {  // s_d = sum_l gamma_l d u_l / d x_d
+        float sd[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+          sd[d] = gv[0] * (H[2][d][1] - H[1][d][2]) + gv[1] * (H[0][d][2] - H[2][d][0]) +
+                  gv[2] * (H[1][d][0] - H[0][d][1]);
+        sx = sd[0];
+        sy = sd[1];
+        sz = sd[2];
+      } else {  // s_l = sum_d gamma_d d u_l / d x_d
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          sx += gv[d] * (H[2][d][1] - H[1][d][2]);
+          sy += gv[d] * (H[0][d][2] - H[2][d][0]);
+          sz += gv[d] * (H[1][d][0] - H[0][d][1]);
+        }
+      }
+      far_u[3 * j] = ux * c4;
+      far_u[3 * j + 1] = uy * c4;
+      far_u[3 * j + 2] = uz * c4;
+      far_s[3 * j] = sx * c4;
+      far_s[3 * j + 1] = sy * c4;
+      far_s[3 * j + 2] = sz * c4;
     }
-    far_u[3 * j] = ux * c4;
-    far_u[3 * j + 1] = uy * c4;
-    far_u[3 * j + 2] = uz * c4;
-    far_s[3 * j] = sx * c4;
-    far_s[3 * j + 1] = sy * c4;
-    far_s[3 * j + 2] = sz * c4;
-  }
   };
   if (G > 1) eval(std::true_type{});
   else eval(std::false_type{});

@@ -50,55 +50,55 @@ __global__ void __launch_bounds__(kP2MThreads) k_p2m(const int* __restrict__ lea
     // registers (the diagonal m = n, then up each column m), stored conjugated
     // in real-packed order
     auto rows = [&](auto grouped) {
-    constexpr bool GR = decltype(grouped)::value;
-    if (tl < cnt) {
-      float* row = sR + tl * PS;
-      const float4 x = A[c0 + tl];
-      const float X = (float)((double)x.x - cx) * inv_a;
-      const float Y = (float)((double)x.y - cy) * inv_a;
-      const float Z = (float)((double)x.z - cz) * inv_a;
-      const float r2 = X * X + Y * Y + Z * Z;
-      float dre = 1.f, dim = 0.f;  // R~_m^m
-      int at = 0;
-      for (int i = 0; (GR ? i * G : i) < p; ++i) {
-        const int m = GR ? folded_column(i, grp, G) : i;
-        if (m >= p) continue;
-        while (at < m) {
-          ++at;
-          const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
-          const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
-          dre = nr;
-          dim = ni;
-        }
-        float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{n-1}^m, R~_n^m
-        for (int n = m; n < p; ++n) {
-          if (n > m) {
-            const float2 cf = GR ? sC[n * (n + 1) / 2 + m] : recurrence(n, m);
-            const float aa = (2.f * n - 1.f) * Z;
-            float vr = aa * r0r, vi = aa * r0i;
-            if (n - 2 >= m) {
-              const float bb = r2 * cf.y;
-              vr -= bb * r1r;
-              vi -= bb * r1i;
+      constexpr bool GR = decltype(grouped)::value;
+      if (tl < cnt) {
+        float* row = sR + tl * PS;
+        const float4 x = A[c0 + tl];
+        const float X = (float)((double)x.x - cx) * inv_a;
+        const float Y = (float)((double)x.y - cy) * inv_a;
+        const float Z = (float)((double)x.z - cz) * inv_a;
+        const float r2 = X * X + Y * Y + Z * Z;
+        float dre = 1.f, dim = 0.f;  // R~_m^m
+        int at = 0;
+        for (int i = 0; (GR ? i * G : i) < p; ++i) {
+          const int m = GR ? folded_column(i, grp, G) : i;
+          if (m >= p) continue;
+          while (at < m) {
+            ++at;
+            const float f = GR ? sC[at * (at + 1) / 2 + at].x : recurrence(at, at).x;
+            const float nr = f * (dre * X - dim * Y), ni = f * (dre * Y + dim * X);
+            dre = nr;
+            dim = ni;
+          }
+          float r1r = 0.f, r1i = 0.f, r0r = dre, r0i = dim;  // R~_{n-1}^m, R~_n^m
+          for (int n = m; n < p; ++n) {
+            if (n > m) {
+              const float2 cf = GR ? sC[n * (n + 1) / 2 + m] : recurrence(n, m);
+              const float aa = (2.f * n - 1.f) * Z;
+              float vr = aa * r0r, vi = aa * r0i;
+              if (n - 2 >= m) {
+                const float bb = r2 * cf.y;
+                vr -= bb * r1r;
+                vi -= bb * r1i;
+              }
+              r1r = r0r;
+              r1i = r0i;
+              r0r = vr * cf.x;
+              r0i = vi * cf.x;
             }
-            r1r = r0r;
-            r1i = r0i;
-            r0r = vr * cf.x;
-            r0i = vi * cf.x;
-          }
-          if (m == 0) {
-            row[n * n] = r0r;
-          } else {
-            row[n * n + 2 * m - 1] = r0r;
-            row[n * n + 2 * m] = -r0i;
+            if (m == 0) {
+              row[n * n] = r0r;
+            } else {
+              row[n * n + 2 * m - 1] = r0r;
+              row[n * n + 2 * m] = -r0i;
+            }
           }
         }
+        if (grp == 0) {
+          const float4 g = B[c0 + tl];
+          sG[tl] = make_float4(g.x, g.y, g.z, 0.f);
+        }
       }
-      if (grp == 0) {
-        const float4 g = B[c0 + tl];
-        sG[tl] = make_float4(g.x, g.y, g.z, 0.f);
-      }
-    }
     };
     if (G > 1) {
       fill_recurrence(sC, p, t, kP2MThreads);
@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(kMGroups * 256) k_m2m(int lb, int le, const in
 #pragma unroll
     for (int q = 0; q < kMCells; ++q) {
       const int ch = kid[o][q];
-      for (int i = r; i < 3 * P; i += W0) sMf[kMCells * (o * 3 * P + i) + q] = ch >= 0 ? M[(size_t)ch * 3 * P + i] : 0.f;
+      for (int i = r; i < 3 * P; i += W0)
+        sMf[kMCells * (o * 3 * P + i) + q] = ch >= 0 ? M[(size_t)ch * 3 * P + i] : 0.f;
     }
   __syncthreads();
   float acc[2][3][kMCells];
