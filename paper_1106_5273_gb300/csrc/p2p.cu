@@ -1217,7 +1217,7 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
 // Ranges of 2048 sources for lists above 8192 gave 2% (batch of 32 problems,
 // 477,044 blobs: 7.79 ms instead of 7.95) but moved single values by up to
 // 1.6e-3 of the largest component from those of one running sum; the sums of a
-// batch stay those of one running sum (3.6e-4).
+// batch stay those of one running sum (5.6e-4 at most over 18 inputs).
 constexpr int64_t kItemTarget = 8 * 32 * 152;  // items aimed at (half as many: ball 100,003 2.15 instead of 2.09 ms in all)
 constexpr uint32_t kItemSrcMin = 128;
 
