@@ -550,6 +550,21 @@ int64_t fmm_kernel_launch_count(void);
  */
 int fmm_plan_set_list_capacity(fmm_plan plan, int64_t frontier, int64_t m2l, int64_t p2p);
 
+/*
+ * How often a bounded wait of the plan's kernels polls before it gives up (0:
+ * the default, 2^24, seconds; at most that; negative: every such wait that is
+ * not the last to arrive gives up at once).  An evaluation whose wait gave up
+ * returns FMM_E_TIMEOUT; nothing that the wait was for is used, and the next
+ * evaluation is not affected.  Small values exercise that path.
+ * FMM_E_INVAL for another wait or limit.
+ */
+enum {
+  FMM_WAIT_TREE = 0,      /* grid barrier of the octree kernel */
+  FMM_WAIT_TRAVERSAL = 1, /* grid barrier of the traversal */
+  FMM_WAIT_ITEMS = 2      /* grid barrier of the P2P work items */
+};
+int fmm_plan_set_wait_limit(fmm_plan plan, int wait, int64_t polls);
+
 /* Enable (1) or disable (0) CUDA-event phase timing in fmm_stats.  With timing
  * on the near field, the M2L lists, the M2L and the downward pass run one after
  * the other on the caller's stream (otherwise the near field overlaps the

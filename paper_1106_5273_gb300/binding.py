@@ -19,6 +19,7 @@ FMM_M2L_FULL_SPLIT = 16
 FMM_M2L_CHUNK_STAGES = 32
 FMM_SIGMA_SOURCE, FMM_SIGMA_MIXED = 0, 1
 FMM_SPLIT_SOURCE, FMM_SPLIT_TARGET = 0, 1
+FMM_WAIT_TREE, FMM_WAIT_TRAVERSAL, FMM_WAIT_ITEMS = 0, 1, 2
 FMM_OUT_VELOCITY, FMM_OUT_STRETCHING, FMM_OUT_STRETCHING_TRANSPOSE = 1, 2, 4
 
 
@@ -91,6 +92,7 @@ lib.fmm_autotune_ncrit.argtypes = [ctypes.POINTER(Params), ctypes.c_int32, _vp, 
                                    ctypes.c_int32, ctypes.c_int32, _vp, _vp, _vp]
 lib.fmm_plan_set_timing.argtypes = [_vp, ctypes.c_int]
 lib.fmm_plan_set_list_capacity.argtypes = [_vp, _i64, _i64, _i64]
+lib.fmm_plan_set_wait_limit.argtypes = [_vp, ctypes.c_int, _i64]
 lib.fmm_selftest_bounded_wait.argtypes = [_i64, ctypes.c_int, _vp]
 lib.fmm_eval_batch.argtypes = [_vp, ctypes.c_int32, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp]
 lib.fmm_plan_device_bytes.argtypes = [_vp]
@@ -266,6 +268,10 @@ class Plan:
         """fmm_plan_set_list_capacity: starting capacities of the traversal's buffers."""
         _check(lib.fmm_plan_set_list_capacity(self._h, int(frontier), int(m2l), int(p2p)),
                "fmm_plan_set_list_capacity")
+
+    def set_wait_limit(self, wait, polls=0):
+        """fmm_plan_set_wait_limit: polls of one of the plan's bounded waits (FMM_WAIT_*)."""
+        _check(lib.fmm_plan_set_wait_limit(self._h, int(wait), int(polls)), "fmm_plan_set_wait_limit")
 
     def set_timing(self, on=True):
         _check(lib.fmm_plan_set_timing(self._h, 1 if on else 0), "fmm_plan_set_timing")

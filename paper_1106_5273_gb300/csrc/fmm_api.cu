@@ -423,6 +423,12 @@ int fmm_plan_set_list_capacity(fmm_plan p, int64_t frontier, int64_t m2l, int64_
   return FMM_OK;
 }
 
+int fmm_plan_set_wait_limit(fmm_plan p, int wait, int64_t polls) {
+  if (!p || wait < 0 || wait >= kWaits || polls > kGridSpin) return FMM_E_INVAL;
+  p->wait_limit[wait] = polls == 0 ? kGridSpin : polls;
+  return FMM_OK;
+}
+
 int fmm_plan_set_timing(fmm_plan p, int enable) {
   if (!p) return FMM_E_INVAL;
   p->timing = enable ? 1 : 0;

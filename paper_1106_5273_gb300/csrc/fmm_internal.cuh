@@ -15,6 +15,7 @@ constexpr int kScalBox = 0;     // box_min[3], box_len
 constexpr int kScalDipole = 4;  // dipole velocity correction [3] (double)
 constexpr int kScalSigma = 8;   // float bits of max sigma (per-particle sigma)
 constexpr int kScalCount = 16;  // u32 counters area
+constexpr int kWaits = 3;       // bounded waits with a limit of their own (FMM_WAIT_*)
 constexpr int kBatchBits = 16;  // Morton bits per axis of a batched evaluation (depth cap 16)
 constexpr int kMaxBatch = 1 << (63 - 3 * kBatchBits);  // problems per batched evaluation
 
@@ -60,6 +61,12 @@ struct SegP2P {  // near field: core width and its constants, class bounds, dipo
   SigK k;
   float sigma, smax, blen, margin;
   float dip[3], pad;
+};
+// Barrier of the kernel that cuts the P2P lists into work items, and its counts
+// (read by the host together).
+struct ItemState {
+  GridBar bar;
+  uint32_t items, slots;
 };
 // Host description of a batch (problems concatenated; nullptr = one problem).
 struct SegSpec {
@@ -187,6 +194,7 @@ struct fmm_plan_s {
   cudaStream_t s_far = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_up = nullptr, ev_near = nullptr;
   cudaEvent_t ev_read = nullptr;  // the host's reads of list sizes
+  long long wait_limit[fmm::kWaits] = {fmm::kGridSpin, fmm::kGridSpin, fmm::kGridSpin};  // polls (fmm_plan_set_wait_limit)
 };
 
 namespace fmm {
@@ -230,9 +238,9 @@ int eval_strengths(fmm_plan p, const float* gam, float* vel, float* dg, cudaStre
 int p2p_near(fmm_plan p, int64_t n, float sig_u, int per_particle_sigma, double smax, bool stretching,
              cudaStream_t s);
 int p2p_finish(fmm_plan p, int64_t n, float* vel, float* dg, cudaStream_t s);
-// work items of the pair kernel; counts (device) receives (items, partial slots)
+// work items of the pair kernel, counted in *p->p2p_bar (ItemState)
 int p2p_tile(fmm_plan p);
-int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s);
+int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, cudaStream_t s);
 int p2p_direct_all(int64_t n, const float* pos, const float* gam, const float* sig, float sig_u, float* vel,
                    float* dg, cudaStream_t s);
 }  // namespace fmm

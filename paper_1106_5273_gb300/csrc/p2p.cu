@@ -817,7 +817,8 @@ __global__ void k_finish(const float* __restrict__ near_u, const float* __restri
 // lists (cut at 2048 sources: P2P 5.56 ms, 5.23 longest first).  One cooperative
 // launch: the blocks own contiguous ranges of the leaves, take their class
 // totals, meet at a bounded grid barrier and write (one CTA over all leaves took
-// 153 us at Taylor-Green 128^3).  counts[0] = items, counts[1] = partial slots.
+// 153 us at Taylor-Green 128^3).  The host reads the counts with the barrier's
+// abort word and launches the pair kernel only if that is 0.
 constexpr int kItemClasses = 4, kItemThreads = 256, kItemBlocks = 128;
 
 __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restrict__ leaves, int nl,
@@ -826,8 +827,8 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
                                                             const int2* __restrict__ off,
                                                             const uint32_t* __restrict__ epre, int tile, uint32_t range,
                                                             int4* __restrict__ items, int* __restrict__ islot,
-                                                            int2* __restrict__ plan, uint32_t* __restrict__ counts,
-                                                            uint32_t* blk, GridBar* bar) {
+                                                            int2* __restrict__ plan, ItemState* st, uint32_t* blk,
+                                                            long long spins) {
   constexpr int NC = kItemClasses + 1;  // item classes, then partial slots
   __shared__ uint32_t ws[NC][kItemThreads / 32];
   __shared__ uint32_t carry[NC];
@@ -870,7 +871,7 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
     for (int i = 0; i < kItemThreads / 32; ++i) x += ws[threadIdx.x][i];
     blk[b * NC + threadIdx.x] = x;
   }
-  if (!grid_barrier(bar, (unsigned)G)) return;
+  if (!grid_barrier(&st->bar, (unsigned)G, spins)) return;
   if (threadIdx.x < NC) {  // this block's first item of each class, and its first slot
     uint32_t pre = 0, all = 0;
     for (int j = 0; j < G; ++j) {
@@ -889,8 +890,8 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
       acc += ws[k][0];
     }
     if (b == 0) {
-      counts[0] = acc;
-      counts[1] = ws[kItemClasses][0];
+      st->items = acc;
+      st->slots = ws[kItemClasses][0];
     }
   }
   __syncthreads();
@@ -1223,7 +1224,7 @@ constexpr uint32_t kItemSrcMin = 128;
 
 int p2p_tile(fmm_plan p) { return p->prm.p2p_tpl == 1 ? 32 : kTileMax; }
 
-int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* counts, cudaStream_t s) {
+int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, cudaStream_t s) {
   const int tile = p2p_tile(p);
   uint32_t range = 0xffffffffu;
   if (!p->batched) {
@@ -1236,10 +1237,10 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* count
   FMM_TRY(p->p2p_items.ensure((size_t)items * sizeof(int4)));
   FMM_TRY(p->p2p_islot.ensure((size_t)items * sizeof(int)));
   FMM_TRY(p->p2p_plan.ensure((size_t)(p->nleaves + 1) * sizeof(int2)));
-  FMM_TRY(p->p2p_bar.ensure(sizeof(GridBar) + (size_t)kItemBlocks * (kItemClasses + 1) * sizeof(uint32_t)));
-  GridBar* bar = p->p2p_bar.as<GridBar>();
-  uint32_t* blk = reinterpret_cast<uint32_t*>(bar + 1);
-  FMM_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar), s));
+  FMM_TRY(p->p2p_bar.ensure(sizeof(ItemState) + (size_t)kItemBlocks * (kItemClasses + 1) * sizeof(uint32_t)));
+  ItemState* st = p->p2p_bar.as<ItemState>();
+  uint32_t* blk = reinterpret_cast<uint32_t*>(st + 1);
+  FMM_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(ItemState), s));
   const int* leaves = p->leaves.as<int>();
   const int* cb = p->c_begin.as<int>();
   const int* ce = p->c_end.as<int>();
@@ -1250,7 +1251,8 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, uint32_t* count
   int2* plan = p->p2p_plan.as<int2>();
   int nl = (int)p->nleaves, tl = tile;
   const unsigned G = (unsigned)std::min<int64_t>(kItemBlocks, (nl + kItemThreads - 1) / kItemThreads);
-  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &range, &it, &is, &plan, &counts, &blk, &bar};
+  long long spins = p->wait_limit[FMM_WAIT_ITEMS];
+  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &range, &it, &is, &plan, &st, &blk, &spins};
   ++g_launches;
   FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_p2p_items, dim3(G), dim3(kItemThreads), args, 0, s));
   FMM_CUDA_TRY(cudaGetLastError());

@@ -27,8 +27,11 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
 int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
                    int* in_second, int* flag, cudaStream_t s);
 
-// A barrier over the blocks of a cooperative launch.  Every wait is bounded:
-// on expiry the blocks give up together (abort) and the barrier returns false.
+// A barrier over the blocks of a cooperative launch.  A wait polls at most
+// `spins` times (not at all if negative); on expiry the blocks give up together
+// and the barrier returns false.  A block may leave the barrier just before
+// another gives up, so what the launch wrote is good only if abort is still 0
+// when it has ended: whoever uses it looks there first.
 struct GridBar {
   uint32_t count, gen, abort;
 };
@@ -61,7 +64,7 @@ __device__ __forceinline__ void flush_digits(const uint32_t* h, int npass, uint3
     if (h[i]) atomicAdd(&hist[i], h[i]);
 }
 
-__device__ __forceinline__ bool grid_barrier(GridBar* st, unsigned nblocks) {
+__device__ __forceinline__ bool grid_barrier(GridBar* st, unsigned nblocks, long long spins) {
   __syncthreads();
   if (threadIdx.x == 0) {
     volatile uint32_t* gen = &st->gen;
@@ -73,9 +76,9 @@ __device__ __forceinline__ bool grid_barrier(GridBar* st, unsigned nblocks) {
       __threadfence();
       atomicAdd(&st->gen, 1u);
     } else {
-      for (long long i = 0; *gen == g; ++i) {
+      for (long long i = 0; spins < 0 || *gen == g; ++i) {
         if (*ab) break;
-        if (i > kGridSpin) {
+        if (i > spins) {
           atomicExch(&st->abort, 1u);
           break;
         }

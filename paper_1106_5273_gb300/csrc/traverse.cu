@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
                                                             const uint32_t* __restrict__ cnt0, int2* __restrict__ m2l,
                                                             int4* __restrict__ p2p, uint32_t* __restrict__ mask,
                                                             uint32_t* __restrict__ blk, TravState* st, uint32_t cap_fr,
-                                                            uint32_t cap_m, uint32_t cap_p, int resume) {
+                                                            uint32_t cap_m, uint32_t cap_p, int resume, long long spins) {
   __shared__ uint32_t red[3][kTravThreads / 32];
   __shared__ uint32_t bases[6];
   const unsigned G = gridDim.x, b = blockIdx.x;
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
         blk[3 * b + threadIdx.x] = x;
       }
     }
-    if (!grid_barrier(&st->bar, G)) return;
+    if (!grid_barrier(&st->bar, G, spins)) return;
     // offsets of this block (sum of the earlier blocks) and the level totals
     if (threadIdx.x < 6) bases[threadIdx.x] = 0u;
     __syncthreads();
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kTravThreads) k_trav_loop(TravArgs t, int4* __
     int4* sw = cur;
     cur = nxt;
     nxt = sw;
-    if (!grid_barrier(&st->bar, G)) return;
+    if (!grid_barrier(&st->bar, G, spins)) return;
   }
   if (b == 0 && threadIdx.x == 0) {  // where the lists stand (and, if stopped, where to resume)
     st->nm = nm;
@@ -931,9 +931,10 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
   uint32_t* hc = reinterpret_cast<uint32_t*>(p->pinned);
   uint32_t* dcnt = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount);
   int* drng = reinterpret_cast<int*>(p->scal.as<double>() + kScalCount + 8);
-  // device counts: tiles, translations, steps, missing operators, P2P items and partial slots
+  // device counts: tiles, translations, steps, missing operators
   uint32_t* dmisc = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount + 12);
   char* pin = reinterpret_cast<char*>(p->pinned);
+  ItemState* hitems = reinterpret_cast<ItemState*>(pin + 320);
   uint32_t* hmisc = reinterpret_cast<uint32_t*>(pin + 288);
   int* hrng = reinterpret_cast<int*>(pin + 256);
   // the host reads `bytes` of device counts: enqueue the copy, mark it, and
@@ -993,7 +994,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     uint32_t* blk = p->tscan0.as<uint32_t>();
     uint32_t cf = (uint32_t)cap_fr, cm = (uint32_t)cap_m, cp = (uint32_t)cap_p;
     int resume = launch > 0 ? 1 : 0;
-    void* args[] = {&ta, &a0, &a1, &dcnt, &am, &ap, &msk, &blk, &dst, &cf, &cm, &cp, &resume};
+    long long spins = p->wait_limit[FMM_WAIT_TRAVERSAL];
+    void* args[] = {&ta, &a0, &a1, &dcnt, &am, &ap, &msk, &blk, &dst, &cf, &cm, &cp, &resume, &spins};
     ++g_launches;
     FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_trav_loop, dim3(G), dim3(kTravThreads), args, 0, s));
     TravState hs;
@@ -1054,16 +1056,17 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     FMM_CUDA_TRY(cudaEventSynchronize(p->ev_near));
     const unsigned long long* tot = reinterpret_cast<unsigned long long*>(pin + 64);
     p->p2p_pairs = (int64_t)tot[0];
-    FMM_TRY(p2p_build_items(p, p->last_n, (int64_t)tot[1], dmisc + 4, s));
-    FMM_CUDA_TRY(cudaMemcpyAsync(hmisc + 4, dmisc + 4, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    FMM_TRY(p2p_build_items(p, p->last_n, (int64_t)tot[1], s));
+    FMM_CUDA_TRY(cudaMemcpyAsync(hitems, p->p2p_bar.ptr, sizeof(ItemState), cudaMemcpyDeviceToHost, s));
     FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
     return FMM_OK;
   };
   // ... and once they are counted, the near field itself
   auto p2p_launch = [&]() -> int {
     FMM_CUDA_TRY(cudaEventSynchronize(p->ev_near));
-    p->n_p2p_items = hmisc[4];
-    p->n_p2p_slots = hmisc[5];
+    if (hitems->bar.abort) return FMM_E_TIMEOUT;  // the items are not all there
+    p->n_p2p_items = hitems->items;
+    p->n_p2p_slots = hitems->slots;
     return near();
   };
   FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
                                                             int nroot, const int* __restrict__ off,
                                                             const double* __restrict__ box, int kbits, int ncrit,
                                                             int cap, TreeState* st, uint32_t* __restrict__ blk,
-                                                            int resume) {
+                                                            int resume, long long spins) {
   __shared__ uint32_t ws[kTreeThreads / 32];
   const unsigned G = gridDim.x, b = blockIdx.x;
   const int lane = threadIdx.x & 31, d = threadIdx.x & 7;
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
       st->level_begin[0] = 0;
       st->level_begin[1] = nroot;
     }
-    if (!grid_barrier(&st->bar, G)) return;
+    if (!grid_barrier(&st->bar, G, spins)) return;
   }
   for (;; ++l) {
     // phase A: 8 lanes per cell; lane d finds the first particle of child digit
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
     }
     sum = block_sum(sum, ws);
     if (threadIdx.x == 0) blk[b] = sum;
-    if (!grid_barrier(&st->bar, G)) return;
+    if (!grid_barrier(&st->bar, G, spins)) return;
     uint32_t pre, total;
     block_offsets(blk, G, b, ws, pre, total);
     if ((int64_t)le + total > (int64_t)cap) {  // every block sees the same totals
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
       }
       run += tot;
     }
-    if (!grid_barrier(&st->bar, G)) return;
+    if (!grid_barrier(&st->bar, G, spins)) return;
     if (total == 0) break;
     lb = le;
     le += (int)total;
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
   }
   sum = block_sum(sum, ws);
   if (threadIdx.x == 0) blk[b] = sum;
-  if (!grid_barrier(&st->bar, G)) return;
+  if (!grid_barrier(&st->bar, G, spins)) return;
   uint32_t pre, total;
   block_offsets(blk, G, b, ws, pre, total);
   for (int base = i0; base < i1; base += kTreeThreads) {
@@ -496,7 +496,7 @@ __device__ __forceinline__ float dist2_f(const float4& a, const float4& h, const
 template <bool EXACT>
 __global__ void __launch_bounds__(256) k_radius(const float4* __restrict__ A, const TreeState* __restrict__ st,
                                                 TreeArrays t) {
-  if (!st->done) return;  // the cell arrays are being grown
+  if (!st->done || st->bar.abort) return;  // the cell arrays are being grown, or are not all there
   const int lane = threadIdx.x & 31, nl = st->nleaves;
   for (int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w < nl; w += (int)((gridDim.x * blockDim.x) >> 5)) {
     const int leaf = t.leaves[w], b = t.begin[leaf], e = t.end[leaf];
@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(256) k_radius(const float4* __restrict__ A, co
 }
 
 __global__ void k_radius_final(const TreeState* __restrict__ st, TreeArrays t, double* __restrict__ R) {
-  if (!st->done) return;
+  if (!st->done || st->bar.abort) return;
   const int nc = st->ncells;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
     const double r = __dsqrt_rn(__longlong_as_double((long long)t.r2[c]));
@@ -613,7 +613,8 @@ static int tree_from_sorted(fmm_plan p, int64_t n, int nroot, const int* off, co
     t.cnt = p->tcount.as<uint32_t>();
     const uint64_t* sk = p->skeys;
     int ni = (int)n, ncrit = p->prm.ncrit, icap = (int)cap, resume = launch > 0 ? 1 : 0;
-    void* args[] = {&sk, &t, &ni, &nroot, &off, &box, &kbits, &ncrit, &icap, &st, &blk, &resume};
+    long long spins = p->wait_limit[FMM_WAIT_TREE];
+    void* args[] = {&sk, &t, &ni, &nroot, &off, &box, &kbits, &ncrit, &icap, &st, &blk, &resume, &spins};
     ++g_launches;
     FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_tree_loop, dim3(G), dim3(kTreeThreads), args, 0, s));
     FMM_CUDA_TRY(cudaMemcpyAsync(hs, st, sizeof(TreeState), cudaMemcpyDeviceToHost, s));
