@@ -561,7 +561,9 @@ int fmm_plan_set_list_capacity(fmm_plan plan, int64_t frontier, int64_t m2l, int
 enum {
   FMM_WAIT_TREE = 0,      /* grid barrier of the octree kernel */
   FMM_WAIT_TRAVERSAL = 1, /* grid barrier of the traversal */
-  FMM_WAIT_ITEMS = 2      /* grid barrier of the P2P work items */
+  FMM_WAIT_ITEMS = 2,     /* grid barrier of the P2P work items */
+  FMM_WAIT_SORT = 3,      /* look-back of the particle, cell and M2L sorts */
+  FMM_WAIT_LIST_SORT = 4  /* look-back of the P2P list sort */
 };
 int fmm_plan_set_wait_limit(fmm_plan plan, int wait, int64_t polls);
 

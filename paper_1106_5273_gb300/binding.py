@@ -19,7 +19,7 @@ FMM_M2L_FULL_SPLIT = 16
 FMM_M2L_CHUNK_STAGES = 32
 FMM_SIGMA_SOURCE, FMM_SIGMA_MIXED = 0, 1
 FMM_SPLIT_SOURCE, FMM_SPLIT_TARGET = 0, 1
-FMM_WAIT_TREE, FMM_WAIT_TRAVERSAL, FMM_WAIT_ITEMS = 0, 1, 2
+FMM_WAIT_TREE, FMM_WAIT_TRAVERSAL, FMM_WAIT_ITEMS, FMM_WAIT_SORT, FMM_WAIT_LIST_SORT = 0, 1, 2, 3, 4
 FMM_OUT_VELOCITY, FMM_OUT_STRETCHING, FMM_OUT_STRETCHING_TRANSPOSE = 1, 2, 4
 
 

@@ -283,6 +283,9 @@ int fmm_plan_create(const fmm_params* prm, int64_t n_max, fmm_plan* out) {
         (rc = p->scal.ensure(64 * sizeof(double))) ||
         (rc = p->flags.ensure(16 * sizeof(int))))
       break;
+    p->sort.error = p->p_sort.error = p->flags.as<int>();
+    p->sort.failed = p->flags.as<int>() + 1;
+    p->p_sort.failed = p->flags.as<int>() + 2;
     if (cudaMallocHost(&p->pinned, 4096) != cudaSuccess) {
       rc = FMM_E_NOMEM;
       break;
@@ -424,8 +427,11 @@ int fmm_plan_set_list_capacity(fmm_plan p, int64_t frontier, int64_t m2l, int64_
 }
 
 int fmm_plan_set_wait_limit(fmm_plan p, int wait, int64_t polls) {
-  if (!p || wait < 0 || wait >= kWaits || polls > kGridSpin) return FMM_E_INVAL;
-  p->wait_limit[wait] = polls == 0 ? kGridSpin : polls;
+  static_assert(kGridSpin == kSweepSpin, "one default for all waits");
+  if (!p || wait < 0 || wait > FMM_WAIT_LIST_SORT || polls > kGridSpin) return FMM_E_INVAL;
+  const long long v = polls == 0 ? kGridSpin : polls;
+  if (wait < kBarriers) p->wait_limit[wait] = v;
+  else (wait == FMM_WAIT_SORT ? p->sort : p->p_sort).spins = v;
   return FMM_OK;
 }
 

@@ -15,7 +15,7 @@ constexpr int kScalBox = 0;     // box_min[3], box_len
 constexpr int kScalDipole = 4;  // dipole velocity correction [3] (double)
 constexpr int kScalSigma = 8;   // float bits of max sigma (per-particle sigma)
 constexpr int kScalCount = 16;  // u32 counters area
-constexpr int kWaits = 3;       // bounded waits with a limit of their own (FMM_WAIT_*)
+constexpr int kBarriers = 3;    // grid barriers with a limit of their own (the first of FMM_WAIT_*)
 constexpr int kBatchBits = 16;  // Morton bits per axis of a batched evaluation (depth cap 16)
 constexpr int kMaxBatch = 1 << (63 - 3 * kBatchBits);  // problems per batched evaluation
 
@@ -156,7 +156,7 @@ struct fmm_plan_s {
   fmm::DBuf pk0, pk1, pv0, pv1, p_scan;  // the P2P grouping's own list sort and scan (it runs beside the M2L lists)
   fmm::SortScratch p_sort;
   fmm::DBuf scal;   // small scalars (see kScal*)
-  fmm::DBuf flags;  // int error flags
+  fmm::DBuf flags;  // int: error code, then whether a sort with sort / p_sort failed
   void* pinned = nullptr;  // host pinned scratch (counts)
   // host mirror of the last tree / lists
   std::vector<int> level_begin;  // cells of level l: [level_begin[l], level_begin[l+1])
@@ -194,7 +194,7 @@ struct fmm_plan_s {
   cudaStream_t s_far = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_up = nullptr, ev_near = nullptr;
   cudaEvent_t ev_read = nullptr;  // the host's reads of list sizes
-  long long wait_limit[fmm::kWaits] = {fmm::kGridSpin, fmm::kGridSpin, fmm::kGridSpin};  // polls (fmm_plan_set_wait_limit)
+  long long wait_limit[fmm::kBarriers] = {fmm::kGridSpin, fmm::kGridSpin, fmm::kGridSpin};  // polls (fmm_plan_set_wait_limit)
 };
 
 namespace fmm {

@@ -710,6 +710,14 @@ __global__ void k_m2l_item_keys(const int4* __restrict__ items, const uint32_t* 
   vals[i] = (uint32_t)i;
 }
 
+// The sorted items (in their own order if the sort failed, so that the M2L stays
+// within them; the evaluation then ends with FMM_E_TIMEOUT).
+__global__ void k_m2l_item_order(const uint32_t* __restrict__ sorted, const int* __restrict__ failed, int n,
+                                 uint32_t* __restrict__ order) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) order[i] = *failed ? (uint32_t)i : sorted[i];
+}
+
 __global__ void k_m2l_item_fill(const int2* __restrict__ tr, int ntiles, int S, const uint32_t* __restrict__ cnt,
                                 const uint32_t* __restrict__ ioff, const uint32_t* __restrict__ poff,
                                 int4* __restrict__ items) {
@@ -884,9 +892,10 @@ int m2l_build_items(fmm_plan p, cudaStream_t s) {
                                                               p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
     int second = 0;
     FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                           p->lv1.as<uint32_t>(), (int64_t)k, 32, &second, p->flags.as<int>(), s));
-    FMM_CUDA_TRY(cudaMemcpyAsync(w.order, second ? p->lv1.ptr : p->lv0.ptr, k * sizeof(uint32_t),
-                                 cudaMemcpyDeviceToDevice, s));
+                           p->lv1.as<uint32_t>(), (int64_t)k, 32, &second, s));
+    ++g_launches;
+    k_m2l_item_order<<<(unsigned)((k + T - 1) / T), T, 0, s>>>(
+        second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(), p->sort.failed, (int)k, w.order);
   }
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;

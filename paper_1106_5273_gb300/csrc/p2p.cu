@@ -828,12 +828,16 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
                                                             const uint32_t* __restrict__ epre, int tile, uint32_t range,
                                                             int4* __restrict__ items, int* __restrict__ islot,
                                                             int2* __restrict__ plan, ItemState* st, uint32_t* blk,
-                                                            long long spins) {
+                                                            long long spins, const int* __restrict__ sort_failed) {
   constexpr int NC = kItemClasses + 1;  // item classes, then partial slots
   __shared__ uint32_t ws[NC][kItemThreads / 32];
   __shared__ uint32_t carry[NC];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int G = (int)gridDim.x, b = (int)blockIdx.x;
+  if (*sort_failed) {  // no lists to cut: give up as after an expired wait
+    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
+    return;
+  }
   const int chunk = (nl + G - 1) / G, l0 = min(nl, b * chunk), l1 = min(nl, l0 + chunk);
   struct Leaf {
     uint32_t nit, nsp, F;
@@ -1252,7 +1256,7 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, cudaStream_t s)
   int nl = (int)p->nleaves, tl = tile;
   const unsigned G = (unsigned)std::min<int64_t>(kItemBlocks, (nl + kItemThreads - 1) / kItemThreads);
   long long spins = p->wait_limit[FMM_WAIT_ITEMS];
-  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &range, &it, &is, &plan, &st, &blk, &spins};
+  void* args[] = {&leaves, &nl, &cb, &ce, &off, &pre, &tl, &range, &it, &is, &plan, &st, &blk, &spins, &p->p_sort.failed};
   ++g_launches;
   FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_p2p_items, dim3(G), dim3(kItemThreads), args, 0, s));
   FMM_CUDA_TRY(cudaGetLastError());

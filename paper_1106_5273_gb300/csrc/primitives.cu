@@ -200,7 +200,6 @@ __global__ void k_sort_scatter(const uint64_t* __restrict__ kin, const uint32_t*
 // kernels per pass and a host read of the varying digits before: the tree phase
 // of 1000 blobs took 0.23 ms, now 0.14, of 100,003 0.44 -> 0.24, of 1,000,000
 // 0.82 -> 0.67.
-constexpr long long kSweepSpin = 1ll << 24;
 
 // Counts of digit q (8 bits from bit 8 q) of every key, q < npass.
 __global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__ keys, int64_t n, int npass,
@@ -254,8 +253,10 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
                                                            uint64_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                            int64_t n, int pass, SortState* __restrict__ st,
                                                            unsigned long long* look, unsigned epoch,
-                                                           int* __restrict__ flag) {
-  if (!st->active[pass]) return;
+                                                           long long spins, int* error, volatile int* failed) {
+  // after a wait that ran out the input of this pass is not all there; a tile
+  // of the pass where it does may go on, its input is
+  if (!st->active[pass] || *failed) return;
   const bool swap = st->sel[pass] != 0;
   const uint64_t* kin = swap ? k1 : k0;
   const uint32_t* vin = swap ? v1 : v0;
@@ -330,8 +331,8 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
     for (int t = tile - 1; ok && t >= 0; --t) {
       unsigned long long x = 0;
       long long spin = 0;
-      while (((x = lk[(size_t)t * 256 + tid]) >> 34) != epoch)
-        if (++spin > kSweepSpin) {
+      while (spins < 0 || ((x = lk[(size_t)t * 256 + tid]) >> 34) != epoch)
+        if (++spin > spins || ((spin & 255) == 0 && *failed)) {
           ok = false;
           break;
         }
@@ -344,7 +345,10 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
   }
   __syncthreads();
   if (s_bad) {  // gave up: write nothing
-    if (tid == 0) atomicExch(flag, FMM_E_TIMEOUT);
+    if (tid == 0) {
+      *failed = 1;
+      atomicExch(error, FMM_E_TIMEOUT);
+    }
     return;
   }
 #pragma unroll
@@ -383,7 +387,7 @@ int sort_begin(SortScratch& b, int64_t n, cudaStream_t s) {
 }
 
 int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int npass, bool all,
-                int* flag, cudaStream_t s) {
+                cudaStream_t s) {
   SortState* st = b.state.as<SortState>();
   ++g_launches;
   k_digit_scan<<<1, 256, 0, s>>>(st, n, npass, all ? 1 : 0);
@@ -398,7 +402,7 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
   unsigned long long* look = b.look.as<unsigned long long>();
   for (int q = 0; q < npass; ++q) {
     ++g_launches;
-    kern<<<g, kSortThreads, sh, s>>>(k0, v0, k1, v1, n, q, st, look, ++b.epoch, flag);
+    kern<<<g, kSortThreads, sh, s>>>(k0, v0, k1, v1, n, q, st, look, ++b.epoch, b.spins, b.error, b.failed);
   }
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
@@ -407,7 +411,7 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
 // Sort (keys, vals) by the lowest `bits` key bits, stable; the result is in
 // (k1, v1) if *in_second.
 int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
-                   int* in_second, int* flag, cudaStream_t s) {
+                   int* in_second, cudaStream_t s) {
   *in_second = 0;
   if (n <= 1 || bits <= 0) return FMM_OK;
   const int npass = (bits + 7) / 8;
@@ -415,7 +419,7 @@ int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uin
   ++g_launches;
   k_digit_hist<<<(unsigned)std::min<int64_t>(608, (n + 2047) / 2048), 256, 0, s>>>(k0, n, npass,
                                                                                    &b.state.as<SortState>()->hist[0][0]);
-  FMM_TRY(sort_passes(b, k0, v0, k1, v1, n, npass, true, flag, s));
+  FMM_TRY(sort_passes(b, k0, v0, k1, v1, n, npass, true, s));
   *in_second = npass & 1;
   return FMM_OK;
 }

@@ -11,10 +11,17 @@ struct SortState {
   uint32_t ticket[kSortPasses];
   int active[kSortPasses], sel[kSortPasses + 1];  // pass q reads buffer sel[q]; the result is in sel[npass]
 };
-// Scratch of the sort: one per stream that sorts.
+// Scratch of the sort: one per stream that sorts.  A look-back wait polls at
+// most `spins` times (not at all if negative).  When one runs out, *error
+// becomes FMM_E_TIMEOUT and *failed 1: that pass and all later sorts with the
+// same *failed leave their output unwritten, so whoever uses it looks there
+// first (the words are cleared at the start of an evaluation).
+constexpr long long kSweepSpin = 1ll << 24;
 struct SortScratch {
   DBuf state, look;
   unsigned epoch = 0;
+  int *error = nullptr, *failed = nullptr;
+  long long spins = kSweepSpin;
 };
 // A sort in two halves, for a kernel that makes the keys and counts their
 // digits (SortState::hist) itself: sort_begin clears the state; sort_passes
@@ -23,9 +30,9 @@ struct SortScratch {
 // in buffer SortState::sel[npass], known on the device alone.
 int sort_begin(SortScratch& b, int64_t n, cudaStream_t s);
 int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int npass, bool all,
-                int* flag, cudaStream_t s);
+                cudaStream_t s);
 int radix_sort_u64(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
-                   int* in_second, int* flag, cudaStream_t s);
+                   int* in_second, cudaStream_t s);
 
 // A barrier over the blocks of a cooperative launch.  A wait polls at most
 // `spins` times (not at all if negative); on expiry the blocks give up together

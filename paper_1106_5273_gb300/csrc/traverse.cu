@@ -396,7 +396,9 @@ __global__ void __launch_bounds__(256) k_p2p_keys(const int4* __restrict__ raw, 
 __global__ void __launch_bounds__(256) k_p2p_gather(const int4* __restrict__ raw, const uint32_t* __restrict__ order,
                                                     int n, int2* __restrict__ out, uint32_t* __restrict__ count,
                                                     const int* __restrict__ begin, const int* __restrict__ end,
-                                                    int tile, unsigned long long* __restrict__ totals) {
+                                                    int tile, const int* __restrict__ failed,
+                                                    unsigned long long* __restrict__ totals) {
+  if (*failed) return;  // the list is not sorted
   unsigned long long pairs = 0, srcs = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int4 v = raw[order[i]];
@@ -598,9 +600,10 @@ __global__ void k_bucket_keys(const uint64_t* __restrict__ ukeys, int nk, uint64
 }
 
 __global__ void k_bucket_order(const uint64_t* __restrict__ ukeys, const uint32_t* __restrict__ order, int nk,
-                               uint64_t* __restrict__ out, uint32_t* __restrict__ perm) {
+                               const int* __restrict__ failed, uint64_t* __restrict__ out,
+                               uint32_t* __restrict__ perm) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nk) return;
+  if (i >= nk || *failed) return;
   out[i] = ukeys[order[i]];
   perm[order[i]] = (uint32_t)i;
 }
@@ -608,10 +611,10 @@ __global__ void k_bucket_order(const uint64_t* __restrict__ ukeys, const uint32_
 // bin of pair i = tile * nkeys + slot; flags the bin and keeps it per pair.
 __global__ void k_bin_mark(const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys, int n,
                            const int* __restrict__ ctile, int tsz, KeyPack kp, const uint32_t* __restrict__ kslot,
-                           const uint32_t* __restrict__ perm, int nkeys, uint32_t* __restrict__ bflag,
-                           uint32_t* __restrict__ pbin) {
+                           const uint32_t* __restrict__ perm, const int* __restrict__ failed, int nkeys,
+                           uint32_t* __restrict__ bflag, uint32_t* __restrict__ pbin) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *failed) return;
   uint32_t slot = kslot[compact_key(fkeys[i], kp)];
   if (perm) slot = perm[slot];
   const uint32_t b = (uint32_t)(ctile[raw[i].x] / tsz) * (uint32_t)nkeys + slot;
@@ -658,10 +661,10 @@ __global__ void k_step_write2(const uint64_t* __restrict__ k, const uint32_t* __
 
 __global__ void k_step_slots(const uint64_t* __restrict__ sk, const uint32_t* __restrict__ sidx, int ns,
                              const uint32_t* __restrict__ f, const uint32_t* __restrict__ e,
-                             const uint64_t* __restrict__ st_fkey, uint64_t* __restrict__ ukeys,
-                             int* __restrict__ st_slot) {
+                             const uint64_t* __restrict__ st_fkey, const int* __restrict__ failed,
+                             uint64_t* __restrict__ ukeys, int* __restrict__ st_slot) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ns) return;
+  if (i >= ns || *failed) return;
   const uint32_t slot = e[i] + f[i] - 1u;
   if (f[i]) ukeys[slot] = st_fkey[sidx[i]];
   st_slot[sidx[i]] = (int)slot;
@@ -708,10 +711,11 @@ __global__ void __launch_bounds__(256) k_tile_order_keys(const int* __restrict__
 }
 
 // gofs[g] = first sorted position of (level, octant) group g, gtile[g] = its
-// first tile; *ntiles the number of tiles.  Also starts the key ranges.
+// first tile; misc[0] the number of tiles, misc[1] whether a sort of the plan has
+// failed so far (for the host).  Also starts the key ranges.
 __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int tsz, int* __restrict__ gofs,
-                                                     int* __restrict__ gtile, uint32_t* __restrict__ ntiles,
-                                                     int* __restrict__ rng) {
+                                                     int* __restrict__ gtile, const int* __restrict__ failed,
+                                                     uint32_t* __restrict__ misc, int* __restrict__ rng) {
   __shared__ int cells[256], tiles[256];
   const int g = threadIdx.x;
   const int c = g < kGroups ? gcount[g] : 0, t = (c + tsz - 1) / tsz;
@@ -729,16 +733,20 @@ __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gco
     gofs[g] = cells[g] - c;
     gtile[g] = tiles[g] - t;
   }
-  if (g == 255) *ntiles = (uint32_t)tiles[255];
+  if (g == 255) {
+    misc[0] = (uint32_t)tiles[255];
+    misc[1] = (uint32_t)*failed;
+  }
   if (g < 8) rng[g] = (g & 1) ? INT_MIN : INT_MAX;
 }
 
 __global__ void k_cell_tiles(int nc, int tsz, const uint32_t* __restrict__ ntiles, const uint32_t* __restrict__ order,
                              const int* __restrict__ level, const uint64_t* __restrict__ ckey,
-                             const int* __restrict__ gofs, const int* __restrict__ gtile, int* __restrict__ ctile,
-                             int* __restrict__ tcell, int* __restrict__ tfirst) {
+                             const int* __restrict__ gofs, const int* __restrict__ gtile,
+                             const int* __restrict__ failed, int* __restrict__ ctile, int* __restrict__ tcell,
+                             int* __restrict__ tfirst) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nc) return;
+  if (q >= nc || *failed) return;
   const int c = (int)order[q];
   const int g = level[c] * 8 + (int)(ckey[c] & 7ull);
   const int r = q - gofs[g];
@@ -814,8 +822,9 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
 }
 
 // Tiles: at most m2l_tile cells of one (level, octant) group each; and the cells'
-// integer coordinates.  ntiles and the key ranges stay on the device.
-static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
+// integer coordinates.  The number of tiles (misc[0]), the sorts' status (misc[1])
+// and the key ranges stay on the device.
+static int cell_tiles(fmm_plan p, uint32_t* misc, int* rng, cudaStream_t s) {
   const int T = 256;
   const int nc = (int)p->ncells, tsz = m2l_tile(p->P);
   FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
@@ -837,13 +846,13 @@ static int cell_tiles(fmm_plan p, uint32_t* ntiles, int* rng, cudaStream_t s) {
                                      p->lv0.as<uint32_t>(), gcount);
   int second = 0;
   FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
-                         nc, 8, &second, p->flags.as<int>(), s));
+                         nc, 8, &second, s));
   ++g_launches;
-  k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, ntiles, rng);
+  k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, p->sort.failed, misc, rng);
   ++g_launches;
-  k_cell_tiles<<<gc, T, 0, s>>>(nc, tsz, ntiles, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
-                                p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs, gtile, p->c_tile.as<int>(),
-                                p->tile_cells.as<int>(), p->tile_first.as<int>());
+  k_cell_tiles<<<gc, T, 0, s>>>(nc, tsz, misc, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
+                                p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs, gtile, p->sort.failed,
+                                p->c_tile.as<int>(), p->tile_cells.as<int>(), p->tile_first.as<int>());
   ++g_launches;
   k_cell_ijk<<<gc, T, 0, s>>>(p->c_level.as<int>(), p->c_key.as<uint64_t>(), nc, p->c_ijk.as<uint64_t>());
   FMM_CUDA_TRY(cudaGetLastError());
@@ -871,13 +880,13 @@ static int group_p2p(fmm_plan p, int n, unsigned long long* totals, cudaStream_t
   k_p2p_keys<<<std::min(g, 608u), T, 0, s>>>(p->p2p_raw.as<int4>(), n, p->pk0.as<uint64_t>(), p->pv0.as<uint32_t>(),
                                              npass, &p->p_sort.state.as<SortState>()->hist[0][0]);
   FMM_TRY(sort_passes(p->p_sort, p->pk0.as<uint64_t>(), p->pv0.as<uint32_t>(), p->pk1.as<uint64_t>(),
-                      p->pv1.as<uint32_t>(), std::max(n, 1), npass, true, p->flags.as<int>(), s));
+                      p->pv1.as<uint32_t>(), std::max(n, 1), npass, true, s));
   uint64_t* sk = second ? p->pk1.as<uint64_t>() : p->pk0.as<uint64_t>();
   uint32_t* sv = second ? p->pv1.as<uint32_t>() : p->pv0.as<uint32_t>();
   ++g_launches;
   k_p2p_gather<<<std::min(g, 1216u), T, 0, s>>>(p->p2p_raw.as<int4>(), sv, n, p->p2p_sorted.as<int2>(),
                                                 p->p2p_pre.as<uint32_t>(), p->c_begin.as<int>(), p->c_end.as<int>(),
-                                                p2p_tile(p), dpairs);
+                                                p2p_tile(p), p->p_sort.failed, dpairs);
   FMM_CUDA_TRY(cudaMemcpyAsync(totals, dpairs, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   // the scan wraps past 2^32 sources; differences within a leaf stay exact
   FMM_TRY(exclusive_scan_u32(p->p2p_pre.as<uint32_t>(), p->p2p_pre.as<uint32_t>(), n, p->p2p_pre.as<uint32_t>() + n,
@@ -936,13 +945,20 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
   char* pin = reinterpret_cast<char*>(p->pinned);
   ItemState* hitems = reinterpret_cast<ItemState*>(pin + 320);
   uint32_t* hmisc = reinterpret_cast<uint32_t*>(pin + 288);
-  int* hrng = reinterpret_cast<int*>(pin + 256);
+  int* hrng = reinterpret_cast<int*>(pin + 256);  // the ranges, and behind them hmisc as on the device
+  int* hfailed = reinterpret_cast<int*>(pin + 352);  // whether a sort of the plan has failed
   // the host reads `bytes` of device counts: enqueue the copy, mark it, and
   // (after more work is enqueued behind it) wait for the mark
   auto read_mark = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
     FMM_CUDA_TRY(cudaMemcpyAsync(dst_h, src_d, bytes, cudaMemcpyDeviceToHost, f));
     FMM_CUDA_TRY(cudaEventRecord(p->ev_read, f));
     return FMM_OK;
+  };
+
+  // the same for counts behind a sort; the caller looks at *hfailed before it uses them
+  auto read_mark_sorted = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
+    FMM_CUDA_TRY(cudaMemcpyAsync(hfailed, p->sort.failed, sizeof(int), cudaMemcpyDeviceToHost, f));
+    return read_mark(dst_h, src_d, bytes);
   };
 
   // Frontier loop: one cooperative launch for all levels; the host reads the
@@ -1044,8 +1060,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
                                                           p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
                                                           p->flags.as<int>());
   }
-  FMM_CUDA_TRY(cudaMemcpyAsync(hrng, drng, 8 * sizeof(int), cudaMemcpyDeviceToHost, f));
-  FMM_TRY(read_mark(hmisc, dmisc, sizeof(uint32_t)));
+  FMM_TRY(read_mark(hrng, drng, 8 * sizeof(int) + 2 * sizeof(uint32_t)));
   FMM_TRY(group_p2p(p, (int)np, reinterpret_cast<unsigned long long*>(pin + 64), s));
   FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
   p->n_keys = 0;
@@ -1070,7 +1085,9 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     return near();
   };
   FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+  if (hmisc[1]) return FMM_E_TIMEOUT;  // the cells were not sorted into tiles
   p->ntiles = hmisc[0];
+  *hfailed = 0;
   // step ranges: one per tile, in a batch one per tile and key bucket
   const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p->P);
   FMM_TRY(p->tile_range.ensure((size_t)(p->ntiles + 1) * nsub * sizeof(int2)));
@@ -1133,12 +1150,12 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
                                          p->lv0.as<uint32_t>());
           int second = 0;
           FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                                 p->lv1.as<uint32_t>(), nkeys, 3, &second, p->flags.as<int>(), f));
+                                 p->lv1.as<uint32_t>(), nkeys, 3, &second, f));
           // the sorted bucket numbers are not needed: their buffer takes the keys in the new order
           uint64_t* out = second ? p->lk0.as<uint64_t>() : p->lk1.as<uint64_t>();
           k_bucket_order<<<gk, T, 0, f>>>(p->ukeys.as<uint64_t>(),
-                                          second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(), (int)nkeys, out,
-                                          p->m2l_slot.as<uint32_t>());
+                                          second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(), (int)nkeys,
+                                          p->sort.failed, out, p->m2l_slot.as<uint32_t>());
           FMM_CUDA_TRY(cudaMemcpyAsync(p->ukeys.ptr, out, (size_t)nkeys * sizeof(uint64_t), cudaMemcpyDeviceToDevice, f));
           perm = p->m2l_slot.as<uint32_t>();
         }
@@ -1154,11 +1171,13 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
         FMM_CUDA_TRY(cudaMemsetAsync(bflag, 0, (size_t)nb * sizeof(uint32_t), f));
         ++g_launches;
         k_bin_mark<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
-                                   kslot, perm, (int)nkeys, bflag, pbin);
+                                   kslot, perm, p->sort.failed, (int)nkeys, bflag, pbin);
         FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, f));
-        FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
+        if (perm) FMM_TRY(read_mark_sorted(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
+        else FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
         FMM_TRY(p2p_launch());
         FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+        if (*hfailed) return FMM_E_TIMEOUT;
         p->n_steps = hmisc[2];
         const int64_t ns = p->n_steps;
         FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
@@ -1191,14 +1210,15 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
                                    nsub, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       int second = 0;
       FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, p->flags.as<int>(), f));
+                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, f));
       uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
       k_step_flags<<<g, T, 0, f>>>(sk, n, p->tcount.as<uint32_t>());
       FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, f));
-      FMM_TRY(read_mark(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
+      FMM_TRY(read_mark_sorted(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      if (*hfailed) return FMM_E_TIMEOUT;
       p->n_steps = hmisc[2];
       const int64_t ns = p->n_steps;
       FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
@@ -1220,7 +1240,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       ++g_launches;
       k_copy_u64_iota<<<gs, T, 0, f>>>(p->st_ckey.as<uint64_t>(), (int)ns, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
       FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), ns, std::max(kp.bits, 1), &second, p->flags.as<int>(), f));
+                             p->lv1.as<uint32_t>(), ns, std::max(kp.bits, 1), &second, f));
       sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
       sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
@@ -1228,9 +1248,11 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dmisc + 1, p->scan_tmp, f));
       ++g_launches;
       k_step_slots<<<gs, T, 0, f>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
-                                    p->st_fkey.as<uint64_t>(), p->ukeys.as<uint64_t>(), p->st_slot.as<int>());
-      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
+                                    p->st_fkey.as<uint64_t>(), p->sort.failed, p->ukeys.as<uint64_t>(),
+                                    p->st_slot.as<int>());
+      FMM_TRY(read_mark_sorted(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+      if (*hfailed) return FMM_E_TIMEOUT;
       p->n_keys = hmisc[1];
       uint32_t* miss = p->tcount.as<uint32_t>();
       uint32_t* rank = p->tscan0.as<uint32_t>();

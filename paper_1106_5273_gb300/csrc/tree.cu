@@ -206,14 +206,15 @@ __global__ void __launch_bounds__(256) k_keys(const float* __restrict__ pos, int
 
 // Sorted position i of a batch lies in its problem's input range.  The sort
 // left its result in one of two buffers (sel, known on the device); the keys
-// and indices end up in the first.
+// and indices end up in the first.  Nothing if the sort failed.
 __global__ void k_permute(const float* __restrict__ pos, const float* __restrict__ gam,
                           const float* __restrict__ sig, float sig_u, const float* __restrict__ seg_sig,
                           const int* __restrict__ off, int nseg, uint64_t* __restrict__ k0, uint32_t* __restrict__ v0,
                           const uint64_t* __restrict__ k1, const uint32_t* __restrict__ v1,
-                          const int* __restrict__ sel, int64_t n, float4* __restrict__ A, float4* __restrict__ B) {
+                          const int* __restrict__ sel, const int* __restrict__ failed, int64_t n,
+                          float4* __restrict__ A, float4* __restrict__ B) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *failed) return;
   uint32_t j;
   if (*sel) {
     j = v1[i];
@@ -323,11 +324,16 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
                                                             int nroot, const int* __restrict__ off,
                                                             const double* __restrict__ box, int kbits, int ncrit,
                                                             int cap, TreeState* st, uint32_t* __restrict__ blk,
-                                                            int resume, long long spins) {
+                                                            int resume, long long spins,
+                                                            const int* __restrict__ sort_failed) {
   __shared__ uint32_t ws[kTreeThreads / 32];
   const unsigned G = gridDim.x, b = blockIdx.x;
   const int lane = threadIdx.x & 31, d = threadIdx.x & 7;
   int lb = 0, le = nroot, l = 0;
+  if (*sort_failed) {  // no sorted keys: give up as after an expired wait
+    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
+    return;
+  }
   if (resume) {
     lb = st->lb;
     le = st->le;
@@ -614,7 +620,7 @@ static int tree_from_sorted(fmm_plan p, int64_t n, int nroot, const int* off, co
     const uint64_t* sk = p->skeys;
     int ni = (int)n, ncrit = p->prm.ncrit, icap = (int)cap, resume = launch > 0 ? 1 : 0;
     long long spins = p->wait_limit[FMM_WAIT_TREE];
-    void* args[] = {&sk, &t, &ni, &nroot, &off, &box, &kbits, &ncrit, &icap, &st, &blk, &resume, &spins};
+    void* args[] = {&sk, &t, &ni, &nroot, &off, &box, &kbits, &ncrit, &icap, &st, &blk, &resume, &spins, &p->sort.failed};
     ++g_launches;
     FMM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_tree_loop, dim3(G), dim3(kTreeThreads), args, 0, s));
     FMM_CUDA_TRY(cudaMemcpyAsync(hs, st, sizeof(TreeState), cudaMemcpyDeviceToHost, s));
@@ -653,7 +659,7 @@ static int sort_particles(fmm_plan p, const float* pos, int64_t n, const double*
       pos, n, box, off, nseg, kbits, p->skeys, p->sidx, npass, &p->sort.state.as<SortState>()->hist[0][0]);
   FMM_CUDA_TRY(cudaGetLastError());
   return sort_passes(p->sort, p->keys0.as<uint64_t>(), p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(),
-                     p->vals1.as<uint32_t>(), n, npass, false, p->flags.as<int>(), s);
+                     p->vals1.as<uint32_t>(), n, npass, false, s);
 }
 
 static const int* sorted_sel(fmm_plan p, int bits) { return &p->sort.state.as<SortState>()->sel[(bits + 7) / 8]; }
@@ -690,7 +696,7 @@ int build_tree(fmm_plan p, int64_t n, const float* pos, const float* gam, const 
   ++g_launches;
   k_permute<<<nb, T, 0, s>>>(pos, gam, sig, sig_u, nullptr, nullptr, 1, p->keys0.as<uint64_t>(),
                              p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(), p->vals1.as<uint32_t>(),
-                             sorted_sel(p, 3 * kMaxLevel), n, p->sortA.as<float4>(), p->sortB.as<float4>());
+                             sorted_sel(p, 3 * kMaxLevel), p->sort.failed, n, p->sortA.as<float4>(), p->sortB.as<float4>());
   FMM_CUDA_TRY(cudaGetLastError());
   return tree_from_sorted(p, n, 1, nullptr, box, kMaxLevel, false, s);
 }
@@ -762,7 +768,7 @@ int build_forest(fmm_plan p, int64_t n, const float* pos, const float* gam, cons
   ++g_launches;
   k_permute<<<nb, T, 0, s>>>(pos, gam, sig, 0.f, sig ? nullptr : p->seg_sig.as<float>(), off, S,
                              p->keys0.as<uint64_t>(), p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(),
-                             p->vals1.as<uint32_t>(), sorted_sel(p, bits), n, p->sortA.as<float4>(),
+                             p->vals1.as<uint32_t>(), sorted_sel(p, bits), p->sort.failed, n, p->sortA.as<float4>(),
                              p->sortB.as<float4>());
   FMM_CUDA_TRY(cudaGetLastError());
   return tree_from_sorted(p, n, S, off, box, kBatchBits, true, s);

@@ -49,6 +49,31 @@ def test_expired_grid_barrier_is_an_error(wait, batch):
         _expires_and_recovers(plan, wait, lambda: plan.eval(pos, gam, sigma_uniform=sig))
 
 
+@pytest.mark.parametrize("case", ["particles", "particles-batch", "list", "list-batch", "cells", "steps", "buckets"])
+def test_expired_look_back_is_an_error(case):
+    """A sort waits from its second tile (1024 keys or more) on, so problems of
+    at most 1024 particles reach the sorts behind the first."""
+    import numpy as np
+    from paper_1106_5273_gb300 import Params, Plan
+    big = case.startswith(("particles", "list"))
+    n = 20000 if big else 1000
+    w = workloads.plummer(n)
+    pos, gam, sig = to_dev(w["pos"]), to_dev(w["gamma"]), 1e-4
+    plan = Plan(n, Params.default(p=4, theta=0.5, ncrit=16 if big else (1 if case == "cells" else 3),
+                                  m2l_mode=8 if case == "steps" else 0))
+    if case.endswith("batch") or case == "buckets":
+        off, sp = np.array([0, 3 * n // 10, n]), np.full(2, sig, np.float32)
+        run = lambda: plan.eval_batch(off, pos, gam, sigma_prob=sp)
+    else:
+        run = lambda: plan.eval(pos, gam, sigma_uniform=sig)
+    run()
+    st = plan.stats()
+    if not big:
+        assert (st.ncells > 1024) == (case == "cells")
+        assert st.m2l_keys > 1024 and st.m2l_pairs > 1024
+    _expires_and_recovers(plan, 4 if case.startswith("list") else 3, run)
+
+
 def test_bad_limits_are_refused():
     from paper_1106_5273_gb300 import FmmError, Params, Plan
     plan = Plan(8, Params.default())
