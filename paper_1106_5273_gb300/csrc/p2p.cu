@@ -1282,8 +1282,9 @@ int p2p_near(fmm_plan p, int64_t n, float sig_u, int ps, double smax, bool stret
   double* scal = p->scal.as<double>();
   const int* cseg = p->batched ? p->c_seg.as<int>() : nullptr;
   SegP2P* sp = p->batched ? p->seg_p2p.as<SegP2P>() : nullptr;
+  // both whatever the outputs: fmm_eval_strengths may ask for others and must not allocate
   FMM_TRY(p->near_u.ensure((size_t)n * 3 * sizeof(float)));
-  if (stretching) FMM_TRY(p->near_s.ensure((size_t)n * 3 * sizeof(float)));
+  FMM_TRY(p->near_s.ensure((size_t)n * 3 * sizeof(float)));
   const P2POut out{p->near_u.as<float>(), p->near_s.as<float>()};
   const float blen = p->prm.periodic ? (float)p->prm.box_len : 0.f;
   const SigK K0 = make_sigk(ps ? 1.f : sig_u);
