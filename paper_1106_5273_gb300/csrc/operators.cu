@@ -429,15 +429,17 @@ __global__ void k_cache_insert(const uint64_t* __restrict__ ukeys, int64_t nk, c
   mslots[rank[i]] = slot;
 }
 
-// Empty table for at least nk keys.
+// Empty table for at least nk keys.  Until it is all there the plan has none
+// (tc_cap 0): an allocation may fail with the old arrays already released.
 static int cache_clear(fmm_plan p, int64_t nk, cudaStream_t s) {
   int64_t cap = 2 * kCacheSlots;
   while (cap < 2 * nk) cap *= 2;
+  p->tc_cap = 0;
+  p->tc_size = 0;
   FMM_TRY(p->tc_key.ensure((size_t)cap * sizeof(uint64_t)));
   FMM_TRY(p->tc_slot.ensure((size_t)cap * sizeof(int)));
-  p->tc_cap = cap;
-  p->tc_size = 0;
   FMM_CUDA_TRY(cudaMemsetAsync(p->tc_key.ptr, 0xff, (size_t)cap * sizeof(uint64_t), s));
+  p->tc_cap = cap;
   return FMM_OK;
 }
 
