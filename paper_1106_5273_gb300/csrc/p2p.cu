@@ -521,6 +521,7 @@ __global__ void __launch_bounds__(32, kP2PPerSm)
       sm.box = b;
       sm.centre = lc;
     }
+    __syncwarp();  // every lane reads them when it classifies its sources
     t.x = make_float2(xs[0], xs[1]);
     t.y = make_float2(ys[0], ys[1]);
     t.z = make_float2(zs[0], zs[1]);
