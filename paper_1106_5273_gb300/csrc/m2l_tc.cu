@@ -804,20 +804,27 @@ static M2lForm m2l_form(fmm_plan p, int nkc, int nkc3) {
   const int kind = p->tc_kind;
   const int N = m2l_cols(p->P);
   M2lForm f{};
-  // A whole step per stage when it has two BF16 K chunks, the second with one
-  // product (p = 9 and 10 at theta <= 0.42): one operator-copy latency per
-  // step instead of one per chunk.
-  f.m2 = kind == 0 && nkc == 2 && nkc3 == 1 && !(p->prm.m2l_mode & FMM_M2L_CHUNK_STAGES);
   if (m2l_tile(p->P) == kTileRows) {
+    // A whole step per stage when it has two BF16 K chunks, the second with one
+    // product, and two such CTAs still fit an SM (p = 9 and 10 at theta <= 0.42):
+    // one operator-copy latency per step instead of one per chunk.  At p = 11 the
+    // stage takes 121 KB, one CTA would run where two do with a chunk per stage
+    // (M2L of Plummer 30,011 at theta = 0.4 2.86 ms against 2.56, of Taylor-Green
+    // 64^3 1.14 against 1.05).
+    const size_t step = 3 * (size_t)((p->P + 7) & ~7) * 128 + 3 * (size_t)kColBytes + 128 + 1024;
+    int smem_sm = 0, reserve = 0;
+    f.m2 = kind == 0 && nkc == 2 && nkc3 == 1 && !(p->prm.m2l_mode & FMM_M2L_CHUNK_STAGES) &&
+           cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, p->device) == cudaSuccess &&
+           cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, p->device) == cudaSuccess &&
+           2 * (step + (size_t)reserve) <= (size_t)smem_sm;
     f.kern = f.m2 ? (const void*)k_m2l_rows<0, true>
                   : (kind ? (const void*)k_m2l_rows<1, false> : (const void*)k_m2l_rows<0, false>);
-    f.smem = (f.m2 ? 3 * (size_t)((p->P + 7) & ~7) * 128 + 3 * (size_t)kColBytes : (size_t)kBarOff) + 128 + 1024;
+    f.smem = f.m2 ? step : (size_t)kBarOff + 128 + 1024;
     f.threads = kRowThreads;
     f.rows = kColsB;
     f.ld = kRowLd;
     return f;
   }
-  f.m2 = false;
   const bool two = N > 128;
   f.kern = kind ? (two ? (const void*)k_m2l_cells<1, 2> : (const void*)k_m2l_cells<1, 3>)
                 : (two ? (const void*)k_m2l_cells<0, 2> : (const void*)k_m2l_cells<0, 3>);
