@@ -558,14 +558,18 @@ __device__ inline uint64_t compact_key(uint64_t k, const KeyPack& kp) {
 // (tile, compact key) sort keys of the M2L pairs (batches: tile and key
 // bucket): a run of equal keys is one step.  A target has at most one source per translation, so the pairs of a
 // step have distinct slots and their order within the run does not matter.
+// parts: the compact key (1), the tile (2) or both in one word (3); order (if
+// given): the pairs in an order already sorted by the other part.
 __global__ void k_step_keys2(const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys, int n,
-                             const int* __restrict__ ctile, int tsz, KeyPack kp, int nsub, uint64_t* __restrict__ keys,
-                             uint32_t* __restrict__ vals) {
+                             const int* __restrict__ ctile, int tsz, KeyPack kp, int nsub, int parts,
+                             const uint32_t* __restrict__ order, const int* __restrict__ failed,
+                             uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t tile = (uint64_t)(ctile[raw[i].x] / tsz) * nsub + (nsub > 1 ? m2l_bucket(fkeys[i]) : 0);
-  keys[i] = (tile << kp.bits) | compact_key(fkeys[i], kp);
-  vals[i] = (uint32_t)i;
+  if (i >= n || (order && *failed)) return;
+  const uint32_t j = order ? order[i] : (uint32_t)i;
+  const uint64_t tile = (uint64_t)(ctile[raw[j].x] / tsz) * nsub + (nsub > 1 ? m2l_bucket(fkeys[j]) : 0);
+  keys[i] = parts == 2 ? tile : (parts == 3 ? tile << kp.bits : 0ull) | compact_key(fkeys[j], kp);
+  vals[i] = j;
 }
 
 // Binned step build.  With K = 2^bits compact keys, the translations present
@@ -643,17 +647,17 @@ __global__ void k_bin_fill(const int2* __restrict__ raw, const uint32_t* __restr
 __global__ void k_step_write2(const uint64_t* __restrict__ k, const uint32_t* __restrict__ idx, int n,
                               const uint32_t* __restrict__ f, const uint32_t* __restrict__ e,
                               const int2* __restrict__ raw, const uint64_t* __restrict__ fkeys,
-                              const int* __restrict__ ctile, int tsz, int kbits, int* __restrict__ st_tile,
-                              uint64_t* __restrict__ st_ckey, uint64_t* __restrict__ st_fkey,
+                              const int* __restrict__ ctile, int tsz, KeyPack kp, int tile_shift,
+                              int* __restrict__ st_tile, uint64_t* __restrict__ st_ckey, uint64_t* __restrict__ st_fkey,
                               int* __restrict__ st_src) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t s = e[i] + f[i] - 1u;
-  const uint64_t key = k[i];
   if (f[i]) {
-    st_tile[s] = (int)(key >> kbits);
-    st_ckey[s] = key & ((1ull << kbits) - 1ull);
-    st_fkey[s] = fkeys[idx[i]];
+    const uint64_t fk = fkeys[idx[i]];
+    st_tile[s] = (int)(k[i] >> tile_shift);
+    st_ckey[s] = compact_key(fk, kp);
+    st_fkey[s] = fk;
   }
   const int2 v = raw[idx[i]];
   st_src[(size_t)s * tsz + (ctile[v.x] % tsz)] = m2l_src(v);
@@ -712,12 +716,14 @@ __global__ void __launch_bounds__(256) k_tile_order_keys(const int* __restrict__
 
 // gofs[g] = first sorted position of (level, octant) group g, gtile[g] = its
 // first tile; misc[0] the number of tiles, misc[1] whether a sort of the plan has
-// failed so far (for the host).  Also starts the key ranges.
+// failed so far, misc[2] the number of tiles if they took 64 cells (for the
+// host).  Also starts the key ranges.
 __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int tsz, int* __restrict__ gofs,
                                                      int* __restrict__ gtile, const int* __restrict__ failed,
                                                      uint32_t* __restrict__ misc, int* __restrict__ rng) {
-  __shared__ int cells[256], tiles[256];
+  __shared__ int cells[256], tiles[256], wide;
   const int g = threadIdx.x;
+  if (g == 0) wide = 0;
   const int c = g < kGroups ? gcount[g] : 0, t = (c + tsz - 1) / tsz;
   cells[g] = c;
   tiles[g] = t;
@@ -729,6 +735,8 @@ __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gco
     tiles[g] += y;
     __syncthreads();
   }
+  if (c) atomicAdd(&wide, (c + kTileRows - 1) / kTileRows);
+  __syncthreads();
   if (g < kGroups) {
     gofs[g] = cells[g] - c;
     gtile[g] = tiles[g] - t;
@@ -736,6 +744,7 @@ __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gco
   if (g == 255) {
     misc[0] = (uint32_t)tiles[255];
     misc[1] = (uint32_t)*failed;
+    misc[2] = (uint32_t)wide;
   }
   if (g < 8) rng[g] = (g & 1) ? INT_MIN : INT_MAX;
 }
@@ -757,9 +766,13 @@ __global__ void k_cell_tiles(int nc, int tsz, const uint32_t* __restrict__ ntile
   if (q == 0) tfirst[*ntiles] = nc;
 }
 
-__global__ void k_step_flags(const uint64_t* __restrict__ k, int n, uint32_t* __restrict__ f) {
+// fkeys (if given): k holds the tiles alone, and the translations are compared too.
+__global__ void k_step_flags(const uint64_t* __restrict__ k, const uint32_t* __restrict__ idx, int n,
+                             const uint64_t* __restrict__ fkeys, const int* __restrict__ failed,
+                             uint32_t* __restrict__ f) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) f[i] = (i == 0 || k[i] != k[i - 1]) ? 1u : 0u;
+  if (i >= n || *failed) return;
+  f[i] = (i == 0 || k[i] != k[i - 1] || (fkeys && fkeys[idx[i]] != fkeys[idx[i - 1]])) ? 1u : 0u;
 }
 
 __global__ void k_tile_ranges(const int* __restrict__ st_tile, int ns, int2* __restrict__ tr) {
@@ -822,8 +835,8 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
 }
 
 // Tiles: at most m2l_tile cells of one (level, octant) group each; and the cells'
-// integer coordinates.  The number of tiles (misc[0]), the sorts' status (misc[1])
-// and the key ranges stay on the device.
+// integer coordinates.  What the host needs of them (misc, see k_tile_groups) and
+// the key ranges stay on the device.
 static int cell_tiles(fmm_plan p, uint32_t* misc, int* rng, cudaStream_t s) {
   const int T = 256;
   const int nc = (int)p->ncells, tsz = m2l_tile(p->P);
@@ -1060,7 +1073,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
                                                           p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
                                                           p->flags.as<int>());
   }
-  FMM_TRY(read_mark(hrng, drng, 8 * sizeof(int) + 2 * sizeof(uint32_t)));
+  FMM_TRY(read_mark(hrng, drng, 8 * sizeof(int) + 3 * sizeof(uint32_t)));
   FMM_TRY(group_p2p(p, (int)np, reinterpret_cast<unsigned long long*>(pin + 64), s));
   FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
   p->n_keys = 0;
@@ -1111,9 +1124,17 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       sh += b;
     }
     kp.bits = sh;
-    int tb = 1;
-    while ((1ll << tb) < (long long)p->ntiles * nsub) ++tb;
-    if (tb + kp.bits > 63) return FMM_E_DEPTH;
+    // Deeper trees than a word of (tile of 64 cells, translation) encodes are
+    // refused.  Smaller tiles and a batch's buckets take up to four bits more;
+    // where those do not fit, the steps are sorted by one part after the other.
+    auto bits_of = [](long long count) {
+      int b = 1;
+      while ((1ll << b) < count) ++b;
+      return b;
+    };
+    if (bits_of(hmisc[2]) + kp.bits > 63) return FMM_E_DEPTH;
+    const int tb = bits_of((long long)p->ntiles * nsub);
+    const bool two = tb + kp.bits > 63;
     const int64_t K = 1ll << kp.bits;
     bool items_done = false, binned = false;
     if (kp.bits <= kBinKeyBits && !(p->prm.m2l_mode & FMM_M2L_SORT_STEPS)) {
@@ -1205,16 +1226,31 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       if (!items_done) FMM_TRY(p2p_items());
       FMM_TRY(p2p_launch());
       // sort pairs by (tile, compact key): consecutive runs are the steps
-      ++g_launches;
-      k_step_keys2<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
-                                   nsub, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>());
+      const int2* raw = p->m2l_raw.as<int2>();
+      const uint64_t* fkeys = p->m2l_key.as<uint64_t>();
+      const int* ctile = p->c_tile.as<int>();
+      const int* failed = p->sort.failed;
+      uint64_t *sk = p->lk0.as<uint64_t>(), *sk1 = p->lk1.as<uint64_t>();
+      uint32_t *sv = p->lv0.as<uint32_t>(), *sv1 = p->lv1.as<uint32_t>();
       int second = 0;
-      FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(),
-                             p->lv1.as<uint32_t>(), n, tb + kp.bits, &second, f));
-      uint64_t* sk = second ? p->lk1.as<uint64_t>() : p->lk0.as<uint64_t>();
-      uint32_t* sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
-      k_step_flags<<<g, T, 0, f>>>(sk, n, p->tcount.as<uint32_t>());
+      k_step_keys2<<<g, T, 0, f>>>(raw, fkeys, n, ctile, tsz, kp, nsub, two ? 1 : 3, nullptr, failed, sk, sv);
+      FMM_TRY(radix_sort_u64(p->sort, sk, sv, sk1, sv1, n, two ? kp.bits : tb + kp.bits, &second, f));
+      if (second) {
+        std::swap(sk, sk1);
+        std::swap(sv, sv1);
+      }
+      if (two) {  // the sort is stable: by translation, then by tile
+        ++g_launches;
+        k_step_keys2<<<g, T, 0, f>>>(raw, fkeys, n, ctile, tsz, kp, nsub, 2, sv, failed, sk1, sv1);
+        FMM_TRY(radix_sort_u64(p->sort, sk1, sv1, sk, sv, n, tb, &second, f));
+        if (!second) {
+          std::swap(sk, sk1);
+          std::swap(sv, sv1);
+        }
+      }
+      ++g_launches;
+      k_step_flags<<<g, T, 0, f>>>(sk, sv, n, two ? fkeys : nullptr, failed, p->tcount.as<uint32_t>());
       FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, f));
       FMM_TRY(read_mark_sorted(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
       FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
@@ -1228,9 +1264,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       FMM_TRY(p->st_fkey.ensure((ns + 1) * sizeof(uint64_t)));
       FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), f));
       ++g_launches;
-      k_step_write2<<<g, T, 0, f>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
-                                    p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), p->c_tile.as<int>(), tsz, kp.bits,
-                                    p->st_tile.as<int>(),
+      k_step_write2<<<g, T, 0, f>>>(sk, sv, n, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), raw, fkeys, ctile,
+                                    tsz, kp, two ? 0 : kp.bits, p->st_tile.as<int>(),
                                     p->st_ckey.as<uint64_t>(), p->st_fkey.as<uint64_t>(), p->st_src.as<int>());
       ++g_launches;
       k_tile_ranges<<<(unsigned)((ns + T - 1) / T), T, 0, f>>>(p->st_tile.as<int>(), (int)ns, p->tile_range.as<int2>());
