@@ -152,7 +152,24 @@ __device__ __forceinline__ double flip(double v, bool neg) {
   return __longlong_as_double(__double_as_longlong(v) ^ ((long long)neg << 63));
 }
 
-// M2L operators of new translations, one CTA each, in FP64.
+// v rounded once to BF16 (to nearest, ties to even): its bits, and in r the
+// rounded value.  On the upper word of the pattern, since an FP64 conversion costs
+// what 64 FP32 operations do; bad is set where the result is neither zero nor
+// normal in BF16 (round_bf16_any serves those).
+__device__ __forceinline__ uint32_t round_bf16(double v, double& r, bool& bad) {
+  const uint32_t hi = (uint32_t)__double2hiint(v);
+  const uint32_t up = ((hi >> 13) | min((uint32_t)__double2loint(v), 1u)) & 1u;  // odd, or beyond the half
+  const uint32_t h = (hi + 0xfffu + up) & 0xffffe000u;                           // 7 of 52 mantissa bits stay
+  const uint32_t x = (h & 0x7fffffffu) >> 13;                                    // exponent and mantissa
+  constexpr uint32_t bias = (1023 - 127) << 7;
+  bad = bad || (x != 0u && x - (bias + 128u) >= (254u << 7));
+  r = __hiloint2double((int)h, 0);
+  return (h >> 16 & 0x8000u) | (uint32_t)max((int)(x - bias), 0);
+}
+__device__ __noinline__ uint32_t round_bf16_any(double v) { return (uint32_t)__bfloat16_as_ushort(__double2bfloat16(v)); }
+
+// M2L operators of new translations, one CTA each, in FP64; both BF16 halves come
+// from the FP64 entry.
 // kind 0: BF16 tiles [key][hi/lo][nkc K chunks of 64][rows][64];
 // kind 1: TF32 tiles [key][hi/lo][nkc K chunks of 32][rows][32]; both 128-byte
 // rows with 16-byte groups in the 128-byte swizzle order (group j at j ^ (row & 7)),
@@ -162,7 +179,8 @@ __device__ __forceinline__ double flip(double v, bool neg) {
 // irregular harmonics are built by one thread per order m, and a thread writes
 // 16 bytes of a row at a time.  The first evaluation of Plummer 1,000,000 (49,141
 // operators, p = 12) spent 57.4 ms here with a division and the conversions per
-// entry and one thread for the harmonics, now 11.7.
+// entry and one thread for the harmonics, now 12.1 (11.7 with the entry rounded to
+// FP32 before the split).
 __global__ void __launch_bounds__(256) k_build_m2l(const uint64_t* __restrict__ keys, const int* __restrict__ slots,
                                                    int nkeys, int p, const double* __restrict__ inu,
                                                    float* __restrict__ T32, uint8_t* __restrict__ Tb, int nkc,
@@ -241,16 +259,31 @@ __global__ void __launch_bounds__(256) k_build_m2l(const uint64_t* __restrict__ 
     const int r = u / (nkc * 8), kc = (u >> 3) % nkc, g = u & 7;
     uint32_t hi[4], lo[4];
     if (kind == 0) {
+      const int c = kc * 64 + g * 8;
+      bool bad = false;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         hi[q] = lo[q] = 0u;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const float v = (float)entry(r, kc * 64 + g * 8 + 2 * q + e);
-          const __nv_bfloat16 h = __float2bfloat16(v);
-          const __nv_bfloat16 l = __float2bfloat16(v - __bfloat162float(h));
-          hi[q] |= (uint32_t)__bfloat16_as_ushort(h) << (16 * e);
-          lo[q] |= (uint32_t)__bfloat16_as_ushort(l) << (16 * e);
+          const double v = entry(r, c + 2 * q + e);
+          double h, l;
+          hi[q] |= round_bf16(v, h, bad) << (16 * e);
+          lo[q] |= round_bf16(v - h, l, bad) << (16 * e);
+        }
+      }
+      if (bad) {
+#pragma unroll 1
+        for (int q = 0; q < 8; ++q) {
+          const double v = entry(r, c + q);
+          const uint32_t h = round_bf16_any(v), sh = 16 * (q & 1);
+          const uint32_t l = round_bf16_any(v - (double)__uint_as_float(h << 16));
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i == q >> 1) {
+              hi[i] = (hi[i] & ~(0xffffu << sh)) | h << sh;
+              lo[i] = (lo[i] & ~(0xffffu << sh)) | l << sh;
+            }
         }
       }
     } else {
