@@ -804,7 +804,7 @@ static M2lForm m2l_form(fmm_plan p, int nkc, int nkc3) {
   const int kind = p->tc_kind;
   const int N = m2l_cols(p->P);
   M2lForm f{};
-  if (m2l_tile(p->P) == kTileRows) {
+  if (m2l_tile(p) == kTileRows) {
     // A whole step per stage when it has two BF16 K chunks, the second with one
     // product, and two such CTAs still fit an SM (p = 9 and 10 at theta <= 0.42):
     // one operator-copy latency per step instead of one per chunk.  At p = 11 the

@@ -839,7 +839,7 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
 // the key ranges stay on the device.
 static int cell_tiles(fmm_plan p, uint32_t* misc, int* rng, cudaStream_t s) {
   const int T = 256;
-  const int nc = (int)p->ncells, tsz = m2l_tile(p->P);
+  const int nc = (int)p->ncells, tsz = m2l_tile(p);
   FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
   FMM_TRY(p->tile_cells.ensure((nc + 1) * sizeof(int)));
   FMM_TRY(p->tile_groups.ensure(3 * kGroups * sizeof(int)));
@@ -1102,7 +1102,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
   p->ntiles = hmisc[0];
   *hfailed = 0;
   // step ranges: one per tile, in a batch one per tile and key bucket
-  const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p->P);
+  const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p);
   FMM_TRY(p->tile_range.ensure((size_t)(p->ntiles + 1) * nsub * sizeof(int2)));
   FMM_CUDA_TRY(cudaMemsetAsync(p->tile_range.ptr, 0, (size_t)(p->ntiles + 1) * nsub * sizeof(int2), f));
   if (n == 0) {

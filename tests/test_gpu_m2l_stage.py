@@ -23,3 +23,14 @@ def test_whole_step_stage_where_two_ctas_fit(p, chunks):
     assert np.array_equal(u, uc) and np.array_equal(s, sc)
     _, us, ss = run_fmm(w, p, 0.4, 24, m2l_mode=1)
     assert rel_l2(u, us) < 1e-5 and rel_l2(s, ss) < 3e-5
+
+
+def test_simt_tiles_are_wide_at_every_p():
+    """The SIMT M2L takes tiles of 64 cells whatever P is, so the steps are the
+    same at every order (the tensor-core M2L takes smaller ones at p = 12)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    w = dict(workloads.plummer(12000), sigma=np.float32(workloads.plummer_sigma(12000)))
+    steps = {(p, mode): run_fmm(w, p, 0.5, 16, m2l_mode=mode)[0].stats().m2l_steps
+             for p, mode in ((4, 1), (10, 1), (12, 1), (12, 2))}
+    assert steps[4, 1] == steps[10, 1] == steps[12, 1] < steps[12, 2]
