@@ -34,6 +34,21 @@ constexpr int kImageZero = 13;     // image index of the zero shift, (ox+1)*9+(o
     if (r_ != FMM_OK) return r_;                   \
   } while (0)
 
+// Runs set() (cudaFuncSetAttribute calls with constant values, so that threads and
+// plans of any parameters agree on them) once for the current device; done is a
+// static array of the caller.  A failure is not remembered.
+constexpr int kMaxDevices = 64;
+template <class F>
+int once_per_device(std::atomic<bool> (&done)[kMaxDevices], F set) {
+  int dev = 0;
+  FMM_CUDA_TRY(cudaGetDevice(&dev));
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  if (known && done[dev].load(std::memory_order_acquire)) return FMM_OK;
+  if (!set()) return FMM_E_CUDA;
+  if (known) done[dev].store(true, std::memory_order_release);
+  return FMM_OK;
+}
+
 // A device-byte budget shared by a group of host threads (the serving loop
 // installs one on its worker threads with set_thread_budget).  Every DBuf
 // allocation made by such a thread is charged to it before cudaMalloc is

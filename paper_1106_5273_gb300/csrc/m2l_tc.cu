@@ -918,7 +918,8 @@ int m2l_tensor(fmm_plan p, cudaStream_t s) {
   const int N = m2l_cols(p->P);
   const M2lForm f = m2l_form(p, nkc, nkc3);
   p->m2l_stage_chunks = f.m2 ? 2 : 1;
-  static const bool attr_ok = [] {
+  static std::atomic<bool> done[kMaxDevices];
+  FMM_TRY(once_per_device(done, [] {
     const void* k[7] = {(const void*)k_m2l_cells<1, 2>, (const void*)k_m2l_cells<1, 3>,
                         (const void*)k_m2l_cells<0, 2>, (const void*)k_m2l_cells<0, 3>,
                         (const void*)k_m2l_rows<0, true>, (const void*)k_m2l_rows<1, false>,
@@ -928,8 +929,7 @@ int m2l_tensor(fmm_plan p, cudaStream_t s) {
           cudaFuncSetAttribute(q, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
         return false;
     return true;
-  }();
-  if (!attr_ok) return FMM_E_CUDA;
+  }));
   const int nt = (int)p->ntiles;
   const int T = 256;
   const int2* ranges = p->tile_range.as<int2>();

@@ -42,7 +42,7 @@ constexpr size_t kScratchBytes = align256(kOffScan + kScanWords * sizeof(uint32_
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-constexpr int kMaxDevices = 64;
+using fmm::kMaxDevices;
 // Device address of the scratch array, per device.  Atomic so that two host
 // threads making their first call on one device at once do not race: both
 // look the same address up and store it (release), readers load it (acquire).

@@ -1267,15 +1267,15 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, cudaStream_t s)
 // The staging memory (7.5 to 13 KB a warp, 16 warps per SM) needs the largest
 // shared-memory carveout.
 static int p2p_attributes() {
-  static const bool ok = [] {
+  static std::atomic<bool> done[kMaxDevices];
+  return once_per_device(done, [] {
     const void* k[9] = {(const void*)k_p2p<0, 0>, (const void*)k_p2p<0, 1>, (const void*)k_p2p<0, 2>,
                         (const void*)k_p2p<1, 0>, (const void*)k_p2p<1, 1>, (const void*)k_p2p<1, 2>,
                         (const void*)k_p2p<2, 0>, (const void*)k_p2p<2, 1>, (const void*)k_p2p<2, 2>};
     for (const void* f : k)
       if (cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) return false;
     return true;
-  }();
-  return ok ? FMM_OK : FMM_E_CUDA;
+  });
 }
 
 // The near field of every particle, in sorted order (near_u, near_s).

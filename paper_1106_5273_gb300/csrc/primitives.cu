@@ -396,9 +396,11 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
   const unsigned g = (unsigned)((n + tile - 1) / tile);
   const size_t sh = (size_t)tile * (sizeof(uint64_t) + sizeof(uint32_t));
   auto kern = R == 4 ? k_onesweep<4> : (R == 8 ? k_onesweep<8> : k_onesweep<16>);
-  static const bool ok = cudaFuncSetAttribute(k_onesweep<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              kSortThreads * 16 * 12) == cudaSuccess;
-  if (!ok) return FMM_E_CUDA;
+  static std::atomic<bool> done[kMaxDevices];
+  FMM_TRY(once_per_device(done, [] {
+    return cudaFuncSetAttribute(k_onesweep<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortThreads * 16 * 12) ==
+           cudaSuccess;
+  }));
   unsigned long long* look = b.look.as<unsigned long long>();
   for (int q = 0; q < npass; ++q) {
     ++g_launches;

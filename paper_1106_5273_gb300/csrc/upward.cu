@@ -312,8 +312,16 @@ int upward_pass(fmm_plan p, cudaStream_t s) {
   const int P = p->P, pp = p->prm.p;
   const int nc = (int)p->ncells;
   FMM_TRY(p->M.ensure((size_t)nc * 3 * P * sizeof(float)));
-  const size_t sh = ((size_t)((kP2MThreads * (P | 1) + 3) & ~3) + 4 * kP2MThreads) * sizeof(float);
-  if (sh > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(k_p2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+  auto p2m_bytes = [](int P) { return ((size_t)((kP2MThreads * (P | 1) + 3) & ~3) + 4 * kP2MThreads) * sizeof(float); };
+  auto m2m_bytes = [](int P) { return (size_t)kMCells * 8 * 3 * P * sizeof(float); };  // k_m2m8: half, at most 48 KB
+  static std::atomic<bool> done[kMaxDevices];
+  FMM_TRY(once_per_device(done, [&] {  // the most that any p needs
+    return cudaFuncSetAttribute(k_p2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2m_bytes(kNCoefMax)) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m2m_bytes(kNCoefMax)) ==
+               cudaSuccess;
+  }));
+  const size_t sh = p2m_bytes(P);
   ++g_launches;
   k_p2m<<<(unsigned)p->nleaves, kP2MThreads, sh, s>>>(p->leaves.as<int>(), p->c_begin.as<int>(), p->c_end.as<int>(),
                                               p->c_level.as<int>(), p->c_center.as<double>(),
@@ -321,16 +329,11 @@ int upward_pass(fmm_plan p, cudaStream_t s) {
                                               p->batched ? p->c_seg.as<int>() : nullptr,
                                               p->sortA.as<float4>(), p->sortB.as<float4>(), pp, p->M.as<float>());
   FMM_CUDA_TRY(cudaGetLastError());
-  const size_t sh_m2m = (size_t)2 * 8 * 3 * P * sizeof(float);  // 48 KB at P = 256
-  if (sh_m2m > 48 * 1024)
-    FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_m2m));
-  if (2 * sh_m2m > 48 * 1024)
-    FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * sh_m2m)));
   for (int l = p->nlevels - 2; l >= 0; --l) {
     int lb = p->level_begin[l], le = p->level_begin[l + 1];
     ++g_launches;
     if (le - lb >= kM2MWide)
-      k_m2m<<<(le - lb + kMCells - 1) / kMCells, kMGroups * ((P + 31) & ~31), kMCells * 8 * 3 * P * sizeof(float), s>>>(
+      k_m2m<<<(le - lb + kMCells - 1) / kMCells, kMGroups * ((P + 31) & ~31), m2m_bytes(P), s>>>(
           lb, le, p->c_child.as<int>(), p->c_nchild.as<int>(), p->c_key.as<uint64_t>(), p->m2m_T.as<float>(), P,
           p->M.as<float>());
     else
