@@ -516,10 +516,11 @@ __global__ void __launch_bounds__(256) k_radius(const float4* __restrict__ A, co
         if (lane == 0 && bits > ((volatile uint32_t*)t.r2f)[c]) atomicMax(&t.r2f[c], bits);
         continue;
       }
-      // twice the rounding of dist2_f: 8 2^-24 relative, and the 2^-48 |c| of the centre
+      // twice the rounding of dist2_f: 8 2^-24 relative, and the 2^-48 |c| of the centre;
+      // squares near the end of the FP32 range screen nothing
       const float top = __uint_as_float(t.r2f[c]);
       const float cm = fmaxf(fmaxf(fabsf(h.x), fabsf(h.y)), fabsf(h.z));
-      const float low = top - (4e-6f * top + sqrtf(top) * (2e-13f * cm));
+      const float low = top < 1e-30f ? 0.f : top - (4e-6f * top + sqrtf(top) * (2e-13f * cm));
       if (m < low) continue;
       const double cx = t.center[3 * (size_t)c], cy = t.center[3 * (size_t)c + 1], cz = t.center[3 * (size_t)c + 2];
       unsigned long long v = 0ull;
