@@ -56,19 +56,17 @@ struct Timer {
   }
 };
 
-// The plan's second stream and its fork / join events (created on the plan's
-// device by its first evaluation).
-int ensure_aux_stream(fmm_plan p) {
-  if (p->s_up) return FMM_OK;
-  FMM_CUDA_TRY(cudaStreamCreateWithFlags(&p->s_up, cudaStreamNonBlocking));
-  int lo = 0, hi = 0;
-  FMM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-  FMM_CUDA_TRY(cudaStreamCreateWithPriority(&p->s_far, cudaStreamNonBlocking, hi));
-  for (cudaEvent_t* e : {&p->ev_up, &p->ev_near})
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-  FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
-  FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
-  FMM_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_read, cudaEventDisableTiming));
+// The plan's two streams and its fork / join events (created on the plan's
+// device by its first evaluation; what a failed one left out, by the next).
+int ensure_aux_streams(fmm_plan p) {
+  if (!p->s_up) FMM_CUDA_TRY(cudaStreamCreateWithFlags(&p->s_up, cudaStreamNonBlocking));
+  if (!p->s_far) {
+    int lo = 0, hi = 0;
+    FMM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    FMM_CUDA_TRY(cudaStreamCreateWithPriority(&p->s_far, cudaStreamNonBlocking, hi));
+  }
+  for (cudaEvent_t* e : {&p->ev_up, &p->ev_near, &p->ev_fork, &p->ev_join, &p->ev_read})
+    if (!*e) FMM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   return FMM_OK;
 }
 
@@ -109,7 +107,7 @@ int eval_device(fmm_plan p, int64_t n, const float* pos, const float* gam, const
   const int m2l_kind = p->prm.m2l_mode & 3;
   p->last_tc = (m2l_kind == FMM_M2L_SIMT) ? 0 : p->tc_ok;
   if ((m2l_kind == FMM_M2L_TENSOR || m2l_kind == FMM_M2L_TENSOR_TF32) && !p->tc_ok) return FMM_E_INVAL;
-  FMM_TRY(ensure_aux_stream(p));
+  FMM_TRY(ensure_aux_streams(p));
   Timer tm{p, s};
   tm.mark();
   if (sg) FMM_TRY(build_forest(p, n, pos, gam, sig, *sg, s));
