@@ -568,8 +568,9 @@ int grow_cells(fmm_plan p, int64_t need, cudaStream_t s) {
 // Octree over the sorted keys (one root per problem), centres, leaves, radii.
 static int tree_from_sorted(fmm_plan p, int64_t n, int nroot, const int* off, const double* box, int kbits,
                             bool with_seg, cudaStream_t s) {
-  int64_t cap = std::max<int64_t>({64 + 4 * n / std::max(1, p->prm.ncrit) + 2 * (int64_t)nroot,
-                                   p->cell_cap});
+  // at most 2^27 to begin with: more cells are not traversed
+  int64_t cap = std::max<int64_t>(
+      std::min<int64_t>(64 + 4 * n / std::max(1, p->prm.ncrit) + 2 * (int64_t)nroot, 1ll << 27), p->cell_cap);
   static int grid_blocks[64] = {0};
   const int dev = p->device >= 0 && p->device < 64 ? p->device : 0;
   if (!grid_blocks[dev]) {
