@@ -660,6 +660,7 @@ static int sort_particles(fmm_plan p, const float* pos, int64_t n, const double*
   k_keys<<<(unsigned)std::min<int64_t>(608, (n + 255) / 256), 256, 0, s>>>(
       pos, n, box, off, nseg, kbits, p->skeys, p->sidx, npass, &p->sort.state.as<SortState>()->hist[0][0]);
   FMM_CUDA_TRY(cudaGetLastError());
+  if (n == 1) return FMM_OK;  // in order, in the first buffer (sel is 0)
   return sort_passes(p->sort, p->keys0.as<uint64_t>(), p->vals0.as<uint32_t>(), p->keys1.as<uint64_t>(),
                      p->vals1.as<uint32_t>(), n, npass, false, s);
 }
