@@ -654,7 +654,8 @@ __global__ void __launch_bounds__(kRowThreads, 2)
   }
   // ---- epilogue: warps 0-3 own TMEM lanes 0-127 (rows = output coefficients)
   if (warp < 4) {
-    if (mbar_wait(done, 0u, abort)) {
+    // the warp reads the tensor memory or gives up as one
+    if (__all_sync(0xffffffffu, mbar_wait(done, 0u, abort))) {
       tc_fence_after();
       const int first = tfirst[tile];
       const int ncell = tfirst[tile + 1] - first;
