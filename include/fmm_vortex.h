@@ -6,7 +6,9 @@
  * vortex-stretching term (Eq. 3), with the fast multipole method of
  * Sec. 3 (Morton octree, P2M/M2M, dual-tree traversal with the FMM MAC of
  * Algorithms 1-2, M2L, L2L/L2P, P2P) in free space or in a periodic cube
- * (Sec. 3.5).  All compute runs in CUDA kernels on the caller's stream.
+ * (Sec. 3.5).  All compute runs in CUDA kernels on the caller's stream and on
+ * streams of the plan that start behind it and are joined with it before the
+ * outputs are written.
  *
  * Conventions shared by every entry point
  *   - d = x_i - x_j, r = |d|, rho = r / sigma_j (the SOURCE core width),

@@ -4,41 +4,12 @@
 
 namespace fmm {
 
-// R~_n^m(x,y,z), n < p, m >= 0, written to re[cidx], im[cidx].
-__device__ inline void regular_table_f(float x, float y, float z, int p, float* re, float* im) {
-  const float r2 = x * x + y * y + z * z;
-  re[0] = 1.f;
-  im[0] = 0.f;
-  for (int m = 1; m < p; ++m) {
-    int pc = (m - 1) * m / 2 + (m - 1), c = m * (m + 1) / 2 + m;
-    float f = sqrtf((2.f * m - 1.f) / (2.f * m));
-    re[c] = f * (re[pc] * x - im[pc] * y);
-    im[c] = f * (re[pc] * y + im[pc] * x);
-  }
-  for (int m = 0; m < p; ++m) {
-    for (int n = m + 1; n < p; ++n) {
-      int c = n * (n + 1) / 2 + m, c1 = (n - 1) * n / 2 + m;
-      float inv = rsqrtf((float)((n + m) * (n - m)));
-      float a = (2.f * n - 1.f) * z;
-      float vr = a * re[c1], vi = a * im[c1];
-      if (n - 2 >= m) {
-        int c2 = (n - 2) * (n - 1) / 2 + m;
-        float b = r2 * sqrtf((float)((n + m - 1) * (n - m - 1)));
-        vr -= b * re[c2];
-        vi -= b * im[c2];
-      }
-      re[c] = vr * inv;
-      im[c] = vi * inv;
-    }
-  }
-}
-
-// Factors of the recurrences above: (rsqrt((n + m)(n - m)),
-// sqrt((n + m - 1)(n - m - 1))) for n > m, and on the diagonal the factor from
-// R~_{m-1}^{m-1} to R~_m^m.  Full warps compute them (the shared-memory pipe is
-// what the sweeps' inner loops wait for: L2P of Taylor-Green 128^3 0.55 ms, 0.67
-// from a table); thread groups that share a leaf's columns read a table,
-// [n (n + 1) / 2 + m].
+// Factors of the recurrences R~_n^m = f.x ((2n - 1) z R~_{n-1}^m - r^2 f.y R~_{n-2}^m):
+// (rsqrt((n + m)(n - m)), sqrt((n + m - 1)(n - m - 1))) for n > m, and on the
+// diagonal the factor from R~_{m-1}^{m-1} to R~_m^m.  Full warps compute them (the
+// shared-memory pipe is what the sweeps' inner loops wait for: L2P of Taylor-Green
+// 128^3 0.55 ms, 0.67 from a table); thread groups that share a leaf's columns read
+// a table, [n (n + 1) / 2 + m].
 __device__ inline float2 recurrence(int n, int m) {
   return n == m ? make_float2(sqrtf((2.f * m - 1.f) / (2.f * m)), 0.f)
                 : make_float2(rsqrtf((float)((n + m) * (n - m))), sqrtf((float)((n + m - 1) * (n - m - 1))));

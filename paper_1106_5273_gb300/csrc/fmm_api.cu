@@ -1,7 +1,9 @@
 // C ABI (include/fmm_vortex.h): plan management and the evaluation sequence
 //   tree (keys, sort, octree, radii) -> P2M/M2M -> traversal -> M2L
-//   (+ periodic lattice) -> L2L/L2P -> P2P + combine,
-// every step a kernel on the caller's stream (Sec. 3.1, Algorithms 1-2).
+//   (+ periodic lattice) -> L2L/L2P, P2P beside it -> combine,
+// every step a kernel (Sec. 3.1, Algorithms 1-2).  The tree, the traversal and the
+// near field run on the caller's stream, the upward pass and the far field on two
+// streams of the plan, forked from it and joined with it by events.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -265,8 +267,7 @@ int fmm_plan_create(const fmm_params* prm, int64_t n_max, fmm_plan* out) {
   p->prm = *prm;
   p->n_max = n_max;
   p->P = prm->p * prm->p;
-  p->Kpad = 128;
-  p->tc_ok = 1;  // tcgen05 M2L: one CTA per 128 output rows (two for p > 11)
+  p->tc_ok = 1;  // the tcgen05 M2L has a form for every p
   p->tc_kind = (prm->m2l_mode & 3) == FMM_M2L_TENSOR_TF32 ? 1 : 0;
   if (cudaGetDevice(&p->device) != cudaSuccess) {
     delete p;

@@ -59,8 +59,8 @@ __host__ __device__ inline SigK make_sigk(float sigma) {
 
 struct SegP2P {  // near field: core width and its constants, class bounds, dipole correction
   SigK k;
-  float sigma, smax, blen, margin;
-  float dip[3], pad;
+  float smax, blen, margin;
+  float dip[3];
 };
 // Barrier of the kernel that cuts the P2P lists into work items, and its counts
 // (read by the host together).
@@ -82,7 +82,6 @@ struct fmm_plan_s {
   fmm_params prm;
   int64_t n_max = 0;
   int P = 0;      // p^2 real coefficients per potential
-  int Kpad = 0;   // unused (the BF16 layouts use 64 x m2l_kchunks(P))
   int device = 0;
   int timing = 0;
   int tc_ok = 0;  // tensor-core M2L usable for this p
@@ -308,6 +307,4 @@ inline int m2l_tile(fmm_plan p) { return p->last_tc && (p->P <= 64 || p->P > 128
 __host__ __device__ inline int m2l_bucket(uint64_t key) {
   return (int)((key * 0x9E3779B97F4A7C15ull) >> 61) & (kKeyBuckets - 1);
 }
-
-// Level / tile layout of the current tree, passed to kernels by value.
 }  // namespace fmm

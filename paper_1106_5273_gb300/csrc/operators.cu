@@ -4,8 +4,8 @@
 // (formulas in harmonics.cuh).  Octree children sit at beta = (+-1/2)^3 in
 // child units with scale ratio 1/2, so M2M and L2L reduce to 8 fixed matrices
 // per p, built here once in FP64 on the host.  Each distinct M2L translation
-// (level difference, offset; see m2l_key_* in traverse.cu) becomes one P x P
-// matrix built in FP64 on the device per evaluation.  The periodic far field
+// (level difference, offset: m2l_key_encode) becomes one P x P matrix built in
+// FP64 on the device, once per plan (the cache below).  The periodic far field
 // (Sec. 3.5) is one FP64 P x P operator on the root multipole: images-1
 // rings of 702 super-cells, each ring the M2L sum from offsets
 // {-4..4}^3 \ {-1..1}^3, the next super-cell the M2M sum of 27 copies.
@@ -174,8 +174,8 @@ __device__ __noinline__ uint32_t round_bf16_any(double v) { return (uint32_t)__b
 // kind 1: TF32 tiles [key][hi/lo][nkc K chunks of 32][rows][32]; both 128-byte
 // rows with 16-byte groups in the 128-byte swizzle order (group j at j ^ (row & 7)),
 // padding rows and columns zero; nkc = 0: FP32 [key][P][P].
-// FP64 runs at a 64th of the FP32 rate, so an entry takes one addition, two
-// multiplications and one conversion: the factors 1 / nu come from a table, the
+// FP64 runs at a 64th of the FP32 rate, so a BF16 entry takes two additions and two
+// multiplications: the factors 1 / nu come from a table, the
 // irregular harmonics are built by one thread per order m, and a thread writes
 // 16 bytes of a row at a time.  The first evaluation of Plummer 1,000,000 (49,141
 // operators, p = 12) spent 57.4 ms here with a division and the conversions per
@@ -415,6 +415,7 @@ __global__ void k_remap_slots(int* __restrict__ st_slot, int64_t ns, const int* 
 constexpr uint64_t kNoKey = ~0ull;  // no key has all its level bits set
 constexpr int64_t kCacheSlots = 1 << 16;  // operators kept (more only if one evaluation needs more)
 
+// The public-domain 64-bit finaliser of MurmurHash3 (A. Appleby).
 __device__ __forceinline__ uint64_t key_hash(uint64_t k) {
   k ^= k >> 33;
   k *= 0xff51afd7ed558ccdull;

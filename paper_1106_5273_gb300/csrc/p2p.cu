@@ -20,9 +20,9 @@
 // self pair is skipped explicitly (its exact value is zero).  Periodic image
 // pairs form the exact FP32 difference first and then add the image shift.
 //
-// A CTA takes a tile of at most 64 targets of a leaf and a range of the leaf's
-// sources, which its four warps share; the sources are staged through shared
-// memory in chunks of 64 per warp.  Each staged source is classified by a lower
+// A CTA of one warp takes a tile of at most 64 targets of a leaf and a range of
+// the leaf's sources; the sources are staged through shared memory in chunks of
+// 64.  Each staged source is classified by a lower
 // bound on its distance to every target of the tile (its distance to the
 // targets' bounding box, rounding margin off): the singular kernel where
 // g = 1 to FP32 precision (rho >= 6.5), the cutoff without the series test
@@ -1220,10 +1220,11 @@ int dipole_pass(fmm_plan p, int64_t n, cudaStream_t s) {
 // the partial slots are then bounded by twice that many items (3 KB each).  A
 // batch keeps whole lists: a problem's sums may not depend on the rest of the
 // batch, its many problems fill the chip, and the long lists start first.
-// Ranges of 2048 sources for lists above 8192 gave 2% (batch of 32 problems,
-// 477,044 blobs: 7.79 ms instead of 7.95) but moved single values by up to
-// 1.6e-3 of the largest component from those of one running sum; the sums of a
-// batch stay those of one running sum (5.6e-4 at most over 18 inputs).
+// Ranges of 2048 sources for lists above 8192 give 2 to 5% (batch of 32 problems,
+// 477,044 blobs: 7.66 ms instead of 7.84) but move single values by up to 1.6e-3
+// of the largest component from those of one running sum (whole lists 5.6e-4 at
+// most over 18 inputs).  Against the FP64 pair sum both err the same: rel-L2 u
+// 3.24e-5 and 3.25e-5, s 9.66e-5 both, largest s 2.3e-4 both.
 constexpr int64_t kItemTarget = 8 * 32 * 152;  // items aimed at (half as many: ball 100,003 2.15 instead of 2.09 ms in all)
 constexpr uint32_t kItemSrcMin = 128;
 
@@ -1264,8 +1265,10 @@ int p2p_build_items(fmm_plan p, int64_t n, int64_t tile_sources, cudaStream_t s)
   return FMM_OK;
 }
 
-// The staging memory (7.5 to 13 KB a warp, 16 warps per SM) needs the largest
-// shared-memory carveout.
+// The staging memory needs the largest shared-memory carveout: 5.4 KB a warp with
+// one core width, 5.6 with the mixed rule (24 warps fit an SM), 10.9 with a width
+// per particle (19 do).
+static_assert(sizeof(Stage<0>) == 5504 && sizeof(Stage<2>) == 5776 && sizeof(Stage<1>) == 11152, "as stated");
 static int p2p_attributes() {
   static std::atomic<bool> done[kMaxDevices];
   return once_per_device(done, [] {

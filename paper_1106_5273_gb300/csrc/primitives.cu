@@ -191,7 +191,9 @@ __global__ void k_sort_scatter(const uint64_t* __restrict__ kin, const uint32_t*
   }
 }
 
-// ---- Sort passes with one kernel each.  The digit counts of all passes are
+// ---- Sort passes with one kernel each: the one-sweep radix sort (Adinets and
+// Merrill, arXiv:2206.01784) over decoupled look-back (Merrill and Garland,
+// NVIDIA NVR-2016-002).  The digit counts of all passes are
 // taken at once (k_digit_hist, or by the kernel that makes the keys), scanned by
 // one CTA (k_digit_scan), and a pass (k_onesweep) ranks its tile, learns the
 // counts of the tiles before it by looking back over their published counts,

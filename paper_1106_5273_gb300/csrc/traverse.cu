@@ -159,9 +159,8 @@ __device__ inline void split_of(const TravArgs& t, int a, int b, bool& split_a, 
 // All levels of the frontier in one launch: the blocks own contiguous ranges
 // of the frontier; per level they classify their pairs (phase A), meet at a
 // grid barrier, take their output offsets from the block totals and emit the
-// children in item order (phase B), and meet again.  The lists come out in
-// the same order as the level-by-level kernels above (item order, children in
-// digit order), with no host round trip per level.  Every block is resident
+// children in item order (phase B), and meet again.  The lists come out in item
+// order, children in digit order, with no host round trip per level.  Every block is resident
 // (cooperative launch); each barrier wait is bounded and gives up with
 // FMM_E_TIMEOUT.  When a level's output would outgrow a buffer the blocks
 // stop together before writing it and save where they are (the lists so far
@@ -806,13 +805,11 @@ __global__ void k_seg_tables(int nseg, const double* __restrict__ box, const uns
   m.pad = 0.f;
   mac[sg] = m;
   SegP2P q;
-  q.sigma = sig ? sig[sg] : 1.f;
-  q.k = make_sigk(q.sigma);
+  q.k = make_sigk(sig ? sig[sg] : 1.f);
   q.smax = (float)smax;
   q.blen = (float)blen;
   q.margin = (float)margin;
   q.dip[0] = q.dip[1] = q.dip[2] = 0.f;
-  q.pad = 0.f;
   pp[sg] = q;
 }
 
