@@ -217,8 +217,10 @@ __global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__
 
 // First output position of every digit of every pass, and which passes do
 // anything: one over a digit that is the same in every key is the identity, and
-// is left out unless `all` (the caller then knows where the result is).
-__global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, int64_t n, int npass, int all) {
+// is left out unless `all` (the caller then knows where the result is); none
+// after a sort that failed.
+__global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, int64_t n, int npass, int all,
+                                                    const int* __restrict__ failed) {
   __shared__ uint32_t ws[8];
   __shared__ int act[kSortPasses];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -236,8 +238,9 @@ __global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, 
   }
   if (t == 0) {
     int sel = 0;
+    const int bad = *failed;
     for (int q = 0; q < npass; ++q) {
-      st->active[q] = act[q];
+      st->active[q] = bad ? 0 : act[q];
       st->sel[q] = sel;
       sel ^= act[q];
     }
@@ -256,9 +259,9 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
                                                            int64_t n, int pass, SortState* __restrict__ st,
                                                            unsigned long long* look, unsigned epoch,
                                                            long long spins, int* error, volatile int* failed) {
-  // after a wait that ran out the input of this pass is not all there; a tile
-  // of the pass where it does may go on, its input is
-  if (!st->active[pass] || *failed) return;
+  // a wait that runs out clears the passes behind, whose input is then not all
+  // there (the tiles of its own pass may go on); the word is read here anyway
+  if (!st->active[pass]) return;
   const bool swap = st->sel[pass] != 0;
   const uint64_t* kin = swap ? k1 : k0;
   const uint32_t* vin = swap ? v1 : v0;
@@ -348,6 +351,7 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
   __syncthreads();
   if (s_bad) {  // gave up: write nothing
     if (tid == 0) {
+      for (int q = pass + 1; q < kSortPasses; ++q) st->active[q] = 0;
       *failed = 1;
       atomicExch(error, FMM_E_TIMEOUT);
     }
@@ -392,7 +396,7 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
                 cudaStream_t s) {
   SortState* st = b.state.as<SortState>();
   ++g_launches;
-  k_digit_scan<<<1, 256, 0, s>>>(st, n, npass, all ? 1 : 0);
+  k_digit_scan<<<1, 256, 0, s>>>(st, n, npass, all ? 1 : 0, b.failed);
   const int R = sweep_rows(n);
   const int64_t tile = (int64_t)kSortThreads * R;
   const unsigned g = (unsigned)((n + tile - 1) / tile);

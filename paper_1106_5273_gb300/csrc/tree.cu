@@ -214,9 +214,10 @@ __global__ void k_permute(const float* __restrict__ pos, const float* __restrict
                           const int* __restrict__ sel, const int* __restrict__ failed, int64_t n,
                           float4* __restrict__ A, float4* __restrict__ B) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || *failed) return;
+  const int second = *sel, bad = *failed;  // both loads in flight
+  if (i >= n || bad) return;
   uint32_t j;
-  if (*sel) {
+  if (second) {
     j = v1[i];
     v0[i] = j;
     k0[i] = k1[i];
