@@ -280,11 +280,11 @@ int fmm_plan_create(const fmm_params* prm, int64_t n_max, fmm_plan* out) {
     if ((rc = p->keys0.ensure(nn * 8)) || (rc = p->keys1.ensure(nn * 8)) || (rc = p->vals0.ensure(nn * 4)) ||
         (rc = p->vals1.ensure(nn * 4)) || (rc = p->sortA.ensure(nn * 16)) || (rc = p->sortB.ensure(nn * 16)) ||
         (rc = p->scal.ensure(64 * sizeof(double))) ||
-        (rc = p->flags.ensure(16 * sizeof(int))))
+        (rc = p->flags.ensure(sizeof(EvalStatus))))
       break;
-    p->sort.error = p->p_sort.error = p->flags.as<int>();
-    p->sort.failed = p->flags.as<int>() + 1;
-    p->p_sort.failed = p->flags.as<int>() + 2;
+    p->sort.error = p->p_sort.error = &p->flags.as<EvalStatus>()->error;
+    p->sort.failed = &p->flags.as<EvalStatus>()->failed;
+    p->p_sort.failed = &p->flags.as<EvalStatus>()->p_failed;
     if (cudaMallocHost(&p->pinned, 4096) != cudaSuccess) {
       rc = FMM_E_NOMEM;
       break;

@@ -62,6 +62,16 @@ struct SegP2P {  // near field: core width and its constants, class bounds, dipo
   float smax, blen, margin;
   float dip[3];
 };
+// Error words and counts of an evaluation: one block on the device (fmm_plan_s::
+// flags), copied whole whenever the host reads one of them.  The first four words
+// are cleared at the start.
+struct EvalStatus {
+  int error;              // FMM_E_* raised by a kernel
+  int failed, p_failed;   // a sort with fmm_plan_s::sort / p_sort failed
+  uint32_t wide_tiles;    // M2L tiles if they took 64 cells
+  uint32_t tiles, keys, steps, missing;  // M2L tiles, translations, steps, operators to build
+  int rng[8];             // min and max of each field of the translation keys
+};
 // Barrier of the kernel that cuts the P2P lists into work items, and its counts
 // (read by the host together).
 struct ItemState {
@@ -155,7 +165,7 @@ struct fmm_plan_s {
   fmm::DBuf pk0, pk1, pv0, pv1, p_scan;  // the P2P grouping's own list sort and scan (it runs beside the M2L lists)
   fmm::SortScratch p_sort;
   fmm::DBuf scal;   // small scalars (see kScal*)
-  fmm::DBuf flags;  // int: error code, then whether a sort with sort / p_sort failed
+  fmm::DBuf flags;  // EvalStatus
   void* pinned = nullptr;  // host pinned scratch (counts)
   // host mirror of the last tree / lists
   std::vector<int> level_begin;  // cells of level l: [level_begin[l], level_begin[l+1])

@@ -835,10 +835,7 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
   __shared__ uint32_t carry[NC];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int G = (int)gridDim.x, b = (int)blockIdx.x;
-  if (*sort_failed) {  // no lists to cut: give up as after an expired wait
-    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
-    return;
-  }
+  const int unsorted = *sort_failed;
   const int chunk = (nl + G - 1) / G, l0 = min(nl, b * chunk), l1 = min(nl, l0 + chunk);
   struct Leaf {
     uint32_t nit, nsp, F;
@@ -877,6 +874,10 @@ __global__ void __launch_bounds__(kItemThreads) k_p2p_items(const int* __restric
     blk[b * NC + threadIdx.x] = x;
   }
   if (!grid_barrier(&st->bar, (unsigned)G, spins)) return;
+  if (unsorted) {  // the counts above mean nothing: give up as after an expired wait
+    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
+    return;
+  }
   if (threadIdx.x < NC) {  // this block's first item of each class, and its first slot
     uint32_t pre = 0, all = 0;
     for (int j = 0; j < G; ++j) {

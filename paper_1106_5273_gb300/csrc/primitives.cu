@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, 
                                                     const int* __restrict__ failed) {
   __shared__ uint32_t ws[8];
   __shared__ int act[kSortPasses];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, bad = *failed;
   for (int q = 0; q < npass; ++q) {
     const uint32_t c = st->hist[q][t];
     if (t == 0) act[q] = all;
@@ -238,7 +238,6 @@ __global__ void __launch_bounds__(256) k_digit_scan(SortState* __restrict__ st, 
   }
   if (t == 0) {
     int sel = 0;
-    const int bad = *failed;
     for (int q = 0; q < npass; ++q) {
       st->active[q] = bad ? 0 : act[q];
       st->sel[q] = sel;
@@ -258,7 +257,7 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
                                                            uint64_t* __restrict__ k1, uint32_t* __restrict__ v1,
                                                            int64_t n, int pass, SortState* __restrict__ st,
                                                            unsigned long long* look, unsigned epoch,
-                                                           long long spins, int* error, volatile int* failed) {
+                                                           int spins, int* error, volatile int* failed) {
   // a wait that runs out clears the passes behind, whose input is then not all
   // there (the tiles of its own pass may go on); the word is read here anyway
   if (!st->active[pass]) return;
@@ -332,12 +331,12 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(uint64_t* __restrict_
 #pragma unroll
     for (int q = 0; q < kSortThreads / 32; ++q) cnt[q][tid] += local;
     uint32_t pre = 0;
-    bool ok = true;
+    bool ok = tile == 0 || spins >= 0;
     for (int t = tile - 1; ok && t >= 0; --t) {
       unsigned long long x = 0;
-      long long spin = 0;
-      while (spins < 0 || ((x = lk[(size_t)t * 256 + tid]) >> 34) != epoch)
-        if (++spin > spins || ((spin & 255) == 0 && *failed)) {
+      int spin = 0;
+      while (((x = lk[(size_t)t * 256 + tid]) >> 34) != epoch)
+        if ((++spin & 1023) == 0 && (spin >= spins || *failed)) {
           ok = false;
           break;
         }
@@ -410,7 +409,7 @@ int sort_passes(SortScratch& b, uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32
   unsigned long long* look = b.look.as<unsigned long long>();
   for (int q = 0; q < npass; ++q) {
     ++g_launches;
-    kern<<<g, kSortThreads, sh, s>>>(k0, v0, k1, v1, n, q, st, look, ++b.epoch, b.spins, b.error, b.failed);
+    kern<<<g, kSortThreads, sh, s>>>(k0, v0, k1, v1, n, q, st, look, ++b.epoch, (int)b.spins, b.error, b.failed);
   }
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;

@@ -12,7 +12,7 @@ struct SortState {
   int active[kSortPasses], sel[kSortPasses + 1];  // pass q reads buffer sel[q]; the result is in sel[npass]
 };
 // Scratch of the sort: one per stream that sorts.  A look-back wait polls at
-// most `spins` times (not at all if negative).  When one runs out, *error
+// most `spins` times, to the next 1024 (not at all if negative).  When one runs out, *error
 // becomes FMM_E_TIMEOUT and *failed 1: that pass and all later sorts with the
 // same *failed leave their output unwritten, so whoever uses it looks there
 // first (the words are cleared at the start of an evaluation).

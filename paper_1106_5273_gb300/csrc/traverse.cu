@@ -714,12 +714,9 @@ __global__ void __launch_bounds__(256) k_tile_order_keys(const int* __restrict__
 }
 
 // gofs[g] = first sorted position of (level, octant) group g, gtile[g] = its
-// first tile; misc[0] the number of tiles, misc[1] whether a sort of the plan has
-// failed so far, misc[2] the number of tiles if they took 64 cells (for the
-// host).  Also starts the key ranges.
+// first tile; counts the tiles, also those of 64 cells, and starts the key ranges.
 __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gcount, int tsz, int* __restrict__ gofs,
-                                                     int* __restrict__ gtile, const int* __restrict__ failed,
-                                                     uint32_t* __restrict__ misc, int* __restrict__ rng) {
+                                                     int* __restrict__ gtile, EvalStatus* __restrict__ status) {
   __shared__ int cells[256], tiles[256], wide;
   const int g = threadIdx.x;
   if (g == 0) wide = 0;
@@ -741,11 +738,10 @@ __global__ void __launch_bounds__(256) k_tile_groups(const int* __restrict__ gco
     gtile[g] = tiles[g] - t;
   }
   if (g == 255) {
-    misc[0] = (uint32_t)tiles[255];
-    misc[1] = (uint32_t)*failed;
-    misc[2] = (uint32_t)wide;
+    status->tiles = (uint32_t)tiles[255];
+    status->wide_tiles = (uint32_t)wide;
   }
-  if (g < 8) rng[g] = (g & 1) ? INT_MIN : INT_MAX;
+  if (g < 8) status->rng[g] = (g & 1) ? INT_MIN : INT_MAX;
 }
 
 __global__ void k_cell_tiles(int nc, int tsz, const uint32_t* __restrict__ ntiles, const uint32_t* __restrict__ order,
@@ -832,9 +828,8 @@ int segment_tables(fmm_plan p, int per_particle_sigma, cudaStream_t s) {
 }
 
 // Tiles: at most m2l_tile cells of one (level, octant) group each; and the cells'
-// integer coordinates.  What the host needs of them (misc, see k_tile_groups) and
-// the key ranges stay on the device.
-static int cell_tiles(fmm_plan p, uint32_t* misc, int* rng, cudaStream_t s) {
+// integer coordinates.  Their number and the key ranges stay on the device.
+static int cell_tiles(fmm_plan p, EvalStatus* status, cudaStream_t s) {
   const int T = 256;
   const int nc = (int)p->ncells, tsz = m2l_tile(p);
   FMM_TRY(p->c_tile.ensure((nc + 1) * sizeof(int)));
@@ -858,9 +853,9 @@ static int cell_tiles(fmm_plan p, uint32_t* misc, int* rng, cudaStream_t s) {
   FMM_TRY(radix_sort_u64(p->sort, p->lk0.as<uint64_t>(), p->lv0.as<uint32_t>(), p->lk1.as<uint64_t>(), p->lv1.as<uint32_t>(),
                          nc, 8, &second, s));
   ++g_launches;
-  k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, p->sort.failed, misc, rng);
+  k_tile_groups<<<1, 256, 0, s>>>(gcount, tsz, gofs, gtile, status);
   ++g_launches;
-  k_cell_tiles<<<gc, T, 0, s>>>(nc, tsz, misc, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
+  k_cell_tiles<<<gc, T, 0, s>>>(nc, tsz, &status->tiles, second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>(),
                                 p->c_level.as<int>(), p->c_key.as<uint64_t>(), gofs, gtile, p->sort.failed,
                                 p->c_tile.as<int>(), p->tile_cells.as<int>(), p->tile_first.as<int>());
   ++g_launches;
@@ -949,26 +944,20 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
   const int img0 = p->prm.periodic ? 0 : kImageZero;
   uint32_t* hc = reinterpret_cast<uint32_t*>(p->pinned);
   uint32_t* dcnt = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount);
-  int* drng = reinterpret_cast<int*>(p->scal.as<double>() + kScalCount + 8);
-  // device counts: tiles, translations, steps, missing operators
-  uint32_t* dmisc = reinterpret_cast<uint32_t*>(p->scal.as<double>() + kScalCount + 12);
+  EvalStatus* st = p->flags.as<EvalStatus>();
   char* pin = reinterpret_cast<char*>(p->pinned);
-  ItemState* hitems = reinterpret_cast<ItemState*>(pin + 320);
-  uint32_t* hmisc = reinterpret_cast<uint32_t*>(pin + 288);
-  int* hrng = reinterpret_cast<int*>(pin + 256);  // the ranges, and behind them hmisc as on the device
-  int* hfailed = reinterpret_cast<int*>(pin + 352);  // whether a sort of the plan has failed
-  // the host reads `bytes` of device counts: enqueue the copy, mark it, and
-  // (after more work is enqueued behind it) wait for the mark
-  auto read_mark = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
-    FMM_CUDA_TRY(cudaMemcpyAsync(dst_h, src_d, bytes, cudaMemcpyDeviceToHost, f));
+  EvalStatus* hst = reinterpret_cast<EvalStatus*>(pin + 256);
+  ItemState* hitems = reinterpret_cast<ItemState*>(pin + 256 + sizeof(EvalStatus));
+  // the host reads the status: enqueue the copy, mark it, and (after more work is
+  // enqueued behind it) wait for the mark; no count behind a failed sort is used
+  auto read_mark = [&]() -> int {
+    FMM_CUDA_TRY(cudaMemcpyAsync(hst, st, sizeof(EvalStatus), cudaMemcpyDeviceToHost, f));
     FMM_CUDA_TRY(cudaEventRecord(p->ev_read, f));
     return FMM_OK;
   };
-
-  // the same for counts behind a sort; the caller looks at *hfailed before it uses them
-  auto read_mark_sorted = [&](void* dst_h, const void* src_d, size_t bytes) -> int {
-    FMM_CUDA_TRY(cudaMemcpyAsync(hfailed, p->sort.failed, sizeof(int), cudaMemcpyDeviceToHost, f));
-    return read_mark(dst_h, src_d, bytes);
+  auto read_wait = [&]() -> int {
+    FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
+    return hst->failed ? FMM_E_TIMEOUT : FMM_OK;
   };
 
   // Frontier loop: one cooperative launch for all levels; the host reads the
@@ -1028,7 +1017,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     FMM_CUDA_TRY(cudaMemcpyAsync(hc, dst, sizeof(TravState), cudaMemcpyDeviceToHost, s));
     FMM_CUDA_TRY(cudaEventRecord(p->ev_read, s));
     // the M2L tiles need the tree alone: they run while the host reads the sizes
-    if (launch == 0) FMM_TRY(cell_tiles(p, dmisc, drng, s));
+    if (launch == 0) FMM_TRY(cell_tiles(p, st, s));
     FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
     memcpy(&hs, hc, sizeof(TravState));
     if (hs.bar.abort) return FMM_E_TIMEOUT;
@@ -1067,10 +1056,10 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     FMM_TRY(p->m2l_key.ensure((size_t)(n + 1) * sizeof(uint64_t)));
     ++g_launches;
     k_m2l_keys<<<std::min<unsigned>(g, 2048u), T, 0, f>>>(p->m2l_raw.as<int2>(), n, p->c_level.as<int>(),
-                                                          p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), drng,
+                                                          p->c_ijk.as<uint64_t>(), p->m2l_key.as<uint64_t>(), st->rng,
                                                           p->flags.as<int>());
   }
-  FMM_TRY(read_mark(hrng, drng, 8 * sizeof(int) + 3 * sizeof(uint32_t)));
+  FMM_TRY(read_mark());
   FMM_TRY(group_p2p(p, (int)np, reinterpret_cast<unsigned long long*>(pin + 64), s));
   FMM_CUDA_TRY(cudaEventRecord(p->ev_near, s));
   p->n_keys = 0;
@@ -1094,10 +1083,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     p->n_p2p_slots = hitems->slots;
     return near();
   };
-  FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-  if (hmisc[1]) return FMM_E_TIMEOUT;  // the cells were not sorted into tiles
-  p->ntiles = hmisc[0];
-  *hfailed = 0;
+  FMM_TRY(read_wait());
+  p->ntiles = hst->tiles;
   // step ranges: one per tile, in a batch one per tile and key bucket
   const int nsub = p->batched ? kKeyBuckets : 1, tsz = m2l_tile(p);
   FMM_TRY(p->tile_range.ensure((size_t)(p->ntiles + 1) * nsub * sizeof(int2)));
@@ -1112,8 +1099,8 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
     KeyPack kp;
     int sh = 0;
     for (int q = 3; q >= 0; --q) {
-      kp.lo[q] = hrng[2 * q];
-      int range = hrng[2 * q + 1] - hrng[2 * q];
+      kp.lo[q] = hst->rng[2 * q];
+      int range = hst->rng[2 * q + 1] - hst->rng[2 * q];
       int b = 0;
       while ((1ll << b) <= (long long)range) ++b;
       kp.shift[q] = sh;
@@ -1129,7 +1116,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       while ((1ll << b) < count) ++b;
       return b;
     };
-    if (bits_of(hmisc[2]) + kp.bits > 63) return FMM_E_DEPTH;
+    if (bits_of(hst->wide_tiles) + kp.bits > 63) return FMM_E_DEPTH;
     const int tb = bits_of((long long)p->ntiles * nsub);
     const bool two = tb + kp.bits > 63;
     const int64_t K = 1ll << kp.bits;
@@ -1143,12 +1130,12 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       FMM_CUDA_TRY(cudaMemsetAsync(kflag, 0, (size_t)K * sizeof(uint32_t), f));
       ++g_launches;
       k_key_mark<<<g, T, 0, f>>>(p->m2l_key.as<uint64_t>(), n, kp, kflag);
-      FMM_TRY(exclusive_scan_u32(kflag, kslot, K, dmisc + 1, p->scan_tmp, f));
-      FMM_TRY(read_mark(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
+      FMM_TRY(exclusive_scan_u32(kflag, kslot, K, &st->keys, p->scan_tmp, f));
+      FMM_TRY(read_mark());
       FMM_TRY(p2p_items());
       items_done = true;
-      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      const int64_t nkeys = hmisc[1];
+      FMM_TRY(read_wait());
+      const int64_t nkeys = hst->keys;
       const int64_t nb = nkeys * (int64_t)p->ntiles;
       if (nb <= kBinMax) {
         binned = true;
@@ -1179,7 +1166,7 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
         }
         uint32_t* miss = p->tcount.as<uint32_t>();
         uint32_t* rank = p->tscan0.as<uint32_t>();
-        FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, f));
+        FMM_TRY(find_m2l_operators(p, miss, rank, &st->missing, f));
         // the key tables stay live: bins go to bin_flag2 / bin_scan2
         FMM_TRY(p->bin_flag2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
         FMM_TRY(p->bin_scan2.ensure((size_t)(nb + 1) * sizeof(uint32_t)));
@@ -1190,18 +1177,16 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
         ++g_launches;
         k_bin_mark<<<g, T, 0, f>>>(p->m2l_raw.as<int2>(), p->m2l_key.as<uint64_t>(), n, p->c_tile.as<int>(), tsz, kp,
                                    kslot, perm, p->sort.failed, (int)nkeys, bflag, pbin);
-        FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, dmisc + 2, p->scan_tmp, f));
-        if (perm) FMM_TRY(read_mark_sorted(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
-        else FMM_TRY(read_mark(hmisc + 2, dmisc + 2, 2 * sizeof(uint32_t)));
+        FMM_TRY(exclusive_scan_u32(bflag, bstep, nb, &st->steps, p->scan_tmp, f));
+        FMM_TRY(read_mark());
         FMM_TRY(p2p_launch());
-        FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-        if (*hfailed) return FMM_E_TIMEOUT;
-        p->n_steps = hmisc[2];
+        FMM_TRY(read_wait());
+        p->n_steps = hst->steps;
         const int64_t ns = p->n_steps;
         FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
         FMM_TRY(p->st_src.ensure((ns + 1) * tsz * sizeof(int)));
-        FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, f));
+        FMM_TRY(build_m2l_operators(p, hst->missing, miss, rank, &st->missing, f));
         FMM_CUDA_TRY(cudaMemsetAsync(p->st_src.ptr, 0xff, (ns + 1) * tsz * sizeof(int), f));
         ++g_launches;
         k_bin_steps<<<(unsigned)((nb + T - 1) / T), T, 0, f>>>(bflag, bstep, nb, (int)nkeys, p->tslot_map.as<int>(),
@@ -1248,11 +1233,10 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       }
       ++g_launches;
       k_step_flags<<<g, T, 0, f>>>(sk, sv, n, two ? fkeys : nullptr, failed, p->tcount.as<uint32_t>());
-      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, dmisc + 2, p->scan_tmp, f));
-      FMM_TRY(read_mark_sorted(hmisc + 2, dmisc + 2, sizeof(uint32_t)));
-      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      if (*hfailed) return FMM_E_TIMEOUT;
-      p->n_steps = hmisc[2];
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), n, &st->steps, p->scan_tmp, f));
+      FMM_TRY(read_mark());
+      FMM_TRY(read_wait());
+      p->n_steps = hst->steps;
       const int64_t ns = p->n_steps;
       FMM_TRY(p->st_tile.ensure((ns + 1) * sizeof(int)));
       FMM_TRY(p->st_slot.ensure((ns + 1) * sizeof(int)));
@@ -1277,21 +1261,20 @@ int traverse(fmm_plan p, double smax, cudaStream_t s, cudaStream_t f, const std:
       sv = second ? p->lv1.as<uint32_t>() : p->lv0.as<uint32_t>();
       ++g_launches;
       k_unique_flags<<<gs, T, 0, f>>>(sk, (int)ns, p->tcount.as<uint32_t>());
-      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, dmisc + 1, p->scan_tmp, f));
+      FMM_TRY(exclusive_scan_u32(p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(), ns, &st->keys, p->scan_tmp, f));
       ++g_launches;
       k_step_slots<<<gs, T, 0, f>>>(sk, sv, (int)ns, p->tcount.as<uint32_t>(), p->tscan0.as<uint32_t>(),
                                     p->st_fkey.as<uint64_t>(), p->sort.failed, p->ukeys.as<uint64_t>(),
                                     p->st_slot.as<int>());
-      FMM_TRY(read_mark_sorted(hmisc + 1, dmisc + 1, sizeof(uint32_t)));
-      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      if (*hfailed) return FMM_E_TIMEOUT;
-      p->n_keys = hmisc[1];
+      FMM_TRY(read_mark());
+      FMM_TRY(read_wait());
+      p->n_keys = hst->keys;
       uint32_t* miss = p->tcount.as<uint32_t>();
       uint32_t* rank = p->tscan0.as<uint32_t>();
-      FMM_TRY(find_m2l_operators(p, miss, rank, dmisc + 3, f));
-      FMM_TRY(read_mark(hmisc + 3, dmisc + 3, sizeof(uint32_t)));
-      FMM_CUDA_TRY(cudaEventSynchronize(p->ev_read));
-      FMM_TRY(build_m2l_operators(p, hmisc[3], miss, rank, dmisc + 3, f));
+      FMM_TRY(find_m2l_operators(p, miss, rank, &st->missing, f));
+      FMM_TRY(read_mark());
+      FMM_TRY(read_wait());
+      FMM_TRY(build_m2l_operators(p, hst->missing, miss, rank, &st->missing, f));
       FMM_TRY(remap_step_slots(p, f));
       FMM_CUDA_TRY(cudaGetLastError());
     }

@@ -331,10 +331,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
   const unsigned G = gridDim.x, b = blockIdx.x;
   const int lane = threadIdx.x & 31, d = threadIdx.x & 7;
   int lb = 0, le = nroot, l = 0;
-  if (*sort_failed) {  // no sorted keys: give up as after an expired wait
-    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
-    return;
-  }
+  const int unsorted = *sort_failed;
   if (resume) {
     lb = st->lb;
     le = st->le;
@@ -352,6 +349,10 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_loop(const uint64_t* __re
       st->level_begin[1] = nroot;
     }
     if (!grid_barrier(&st->bar, G, spins)) return;
+  }
+  if (unsorted) {  // give up as after an expired wait (the same in every block)
+    if (b == 0 && threadIdx.x == 0) st->bar.abort = 1u;
+    return;
   }
   for (;; ++l) {
     // phase A: 8 lanes per cell; lane d finds the first particle of child digit
@@ -503,8 +504,8 @@ __device__ __forceinline__ float dist2_f(const float4& a, const float4& h, const
 template <bool EXACT>
 __global__ void __launch_bounds__(256) k_radius(const float4* __restrict__ A, const TreeState* __restrict__ st,
                                                 TreeArrays t) {
-  if (!st->done || st->bar.abort) return;  // the cell arrays are being grown, or are not all there
-  const int lane = threadIdx.x & 31, nl = st->nleaves;
+  const int lane = threadIdx.x & 31, nl = st->nleaves, done = st->done, bad = st->bar.abort;
+  if (!done || bad) return;  // the cell arrays are being grown, or are not all there
   for (int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w < nl; w += (int)((gridDim.x * blockDim.x) >> 5)) {
     const int leaf = t.leaves[w], b = t.begin[leaf], e = t.end[leaf];
     for (int c = leaf; c >= 0; c = t.parent[c]) {
@@ -543,8 +544,8 @@ __global__ void __launch_bounds__(256) k_radius(const float4* __restrict__ A, co
 }
 
 __global__ void k_radius_final(const TreeState* __restrict__ st, TreeArrays t, double* __restrict__ R) {
-  if (!st->done || st->bar.abort) return;
-  const int nc = st->ncells;
+  const int nc = st->ncells, done = st->done, bad = st->bar.abort;
+  if (!done || bad) return;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
     const double r = __dsqrt_rn(__longlong_as_double((long long)t.r2[c]));
     R[c] = r;
