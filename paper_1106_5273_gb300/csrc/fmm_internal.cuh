@@ -311,8 +311,12 @@ __host__ __device__ inline int m2l_cols(int P) { return (P + 15) & ~15; }
 // MMA's 128 rows (64 cells x 3 components as columns); otherwise the cells are
 // the rows and the P coefficients the columns, which fits any P (both forms
 // measured: m2l_tc.cu).  The SIMT M2L reads an operator once per tile and takes
-// the wide tiles at any P (Plummer 30,011 at p = 12: 465 ms, 518 with 42 cells).
-inline int m2l_tile(fmm_plan p) { return p->last_tc && (p->P <= 64 || p->P > 128) ? kTileCells : kTileRows; }
+// the wide tiles at any P (Plummer 30,011 at p = 12: 465 ms, 518 with 42 cells), but
+// in a batch, where one CTA per tile waits for the longest, the same as the other
+// (32 problems of 20,000 at p = 6: 96 ms, 117 with 64 cells).
+inline int m2l_tile(fmm_plan p) {
+  return (p->last_tc || p->batched) && (p->P <= 64 || p->P > 128) ? kTileCells : kTileRows;
+}
 // Bucket of a translation: a hash of its key, so that it depends on nothing else.
 __host__ __device__ inline int m2l_bucket(uint64_t key) {
   return (int)((key * 0x9E3779B97F4A7C15ull) >> 61) & (kKeyBuckets - 1);

@@ -12,8 +12,10 @@ namespace {
 
 constexpr int kRC = 32;  // output rows per pass
 
-// nsub: step ranges per tile (the key buckets of a batch; contiguous).
-__global__ void __launch_bounds__(3 * kTileRows) k_m2l_simt(const int2* __restrict__ tile_range, int nsub,
+// TSZ target cells per tile; nsub: step ranges per tile (the key buckets of a
+// batch; contiguous).
+template <int TSZ>
+__global__ void __launch_bounds__(3 * TSZ) k_m2l_simt(const int2* __restrict__ tile_range, int nsub,
                                                   const int* __restrict__ tfirst,
                                                   const int* __restrict__ st_slot, const int* __restrict__ st_src,
                                                   const float* __restrict__ T32, const float* __restrict__ M, int P,
@@ -30,7 +32,7 @@ __global__ void __launch_bounds__(3 * kTileRows) k_m2l_simt(const int2* __restri
   if (rg.y <= rg.x) return;
   const int first = tfirst[tile];
   const int ncell = tfirst[tile + 1] - first;
-  const int comp = threadIdx.x / kTileRows, slot = threadIdx.x % kTileRows;
+  const int comp = threadIdx.x / TSZ, slot = threadIdx.x % TSZ;
   for (int r0 = 0; r0 < P; r0 += kRC) {
     const int nr = min(kRC, P - r0);
     float acc[kRC];
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(3 * kTileRows) k_m2l_simt(const int2* __restri
       const float* T = T32 + (size_t)st_slot[st] * P * P;
       for (int i = threadIdx.x; i < nr * P; i += blockDim.x) sT[i] = T[(size_t)r0 * P + i];
       __syncthreads();
-      const int src = st_src[(size_t)st * kTileRows + slot];
+      const int src = st_src[(size_t)st * TSZ + slot];
       if (src >= 0) {
         const float* m = M + ((size_t)src * 3 + comp) * P;
         for (int k = 0; k < P; ++k) {
@@ -62,15 +64,14 @@ __global__ void __launch_bounds__(3 * kTileRows) k_m2l_simt(const int2* __restri
 
 int m2l_simt(fmm_plan p, cudaStream_t s) {
   if (p->n_steps == 0) return FMM_OK;
-  size_t sh = (size_t)kRC * p->P * sizeof(float);
-  if (sh > 48 * 1024) FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2l_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+  const size_t sh = (size_t)kRC * p->P * sizeof(float);  // at most 32 KB
+  const int tsz = m2l_tile(p);
+  auto kern = tsz == kTileRows ? k_m2l_simt<kTileRows> : k_m2l_simt<kTileCells>;
   ++g_launches;
-  k_m2l_simt<<<(unsigned)p->ntiles, 3 * kTileRows, sh, s>>>(p->tile_range.as<int2>(),
-                                                         p->batched ? kKeyBuckets : 1,
-                                                         p->tile_first.as<int>(),
-                                                         p->st_slot.as<int>(),
-                                                         p->st_src.as<int>(), p->T32.as<float>(), p->M.as<float>(),
-                                                         p->P, p->tile_cells.as<int>(), p->L.as<float>());
+  kern<<<(unsigned)p->ntiles, 3 * tsz, sh, s>>>(p->tile_range.as<int2>(), p->batched ? kKeyBuckets : 1,
+                                                p->tile_first.as<int>(), p->st_slot.as<int>(), p->st_src.as<int>(),
+                                                p->T32.as<float>(), p->M.as<float>(), p->P, p->tile_cells.as<int>(),
+                                                p->L.as<float>());
   FMM_CUDA_TRY(cudaGetLastError());
   return FMM_OK;
 }
