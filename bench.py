@@ -186,7 +186,8 @@ def m2l_roofline(st, p, mma_cols=None):
     peak, src = bf16_peak()
     k3 = int(st.m2l_split_coefs) or P
     ach = 2.0 * P * 3 * (3 * k3 + (P - k3)) * st.m2l_pairs / (st.ms_m2l * 1e-3) / 1e12
-    out = {"bound": "tensor", "kernel": "k_m2l_tc", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+    out = {"bound": "tensor", "kernel": "k_m2l_rows" if 64 < P <= 128 else "k_m2l_cells",
+           "achieved": ach, "peak": peak, "unit": "TFLOP/s",
            "frac": ach / peak, "peak_source": src, "ms": st.ms_m2l, "split_coefs": k3,
            "flops": "2 P x 3 components x (3 K3 + (P - K3)) per M2L pair (useful rows only)"}
     if k3 % 16 == 0 or k3 == P:  # BF16 path: K steps of 16
